@@ -220,6 +220,7 @@ extern "C" repq_status repq_qgemm(const repq_gemm_desc* d, void* workspace, size
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (scores_supported(*d)) return scores_tc_supported(*d) ? launch_scores_tc(*d, st) : launch_scores(*d, st);
   const EpilogueParams ep = make_epilogue(*d);
+  if (qgemm_skinny_preferred(*d)) return qgemm_skinny(*d, ep, st);
   if (qgemm_tc_supported(*d)) {
     const size_t need = qgemm_tc_workspace(*d);
     REPQ_REQUIRE(workspace_bytes >= need && (need == 0 || workspace), REPQ_WORKSPACE_TOO_SMALL,

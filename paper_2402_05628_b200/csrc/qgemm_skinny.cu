@@ -1,0 +1,479 @@
+// Integer GEMM for few tokens (decoding, short prompts, single images): the weights are the M = 128 operand of the
+// tensor-core instruction and the tokens its N operand, so that a tile is 128 output channels x 16..256 tokens and no
+// tensor-core row is spent on padding of the token side.
+//
+// What bounds it: with few tokens a layer is one pass over its weights, i.e. the HBM (or, for weights that fit, L2) copy
+// rate, and below some 2 MB of weights the latency of one tile.  Both ask for many CTAs with many bytes in flight each:
+//  - a tile's K range is split over the CTAs of a cluster (1, 2, 4 or 8); the int32 partial sums are exchanged through
+//    distributed shared memory, every CTA finishing an equal share of the tile's tokens (integer sums: the result does
+//    not depend on the split);
+//  - two CTAs per SM where the ring of operand stages allows it, at least 64 KB of weights in flight per CTA;
+//  - while the kernel before it in the stream still runs, every CTA asks for its weights to be brought into L2
+//    (prefetches only: nothing is read before the dependency is resolved).
+// The epilogue has one output channel per thread (the channel's terms live in registers), tokens along the accumulator
+// columns; for one token the 32 lanes of a warp are 32 neighbouring outputs, so loads and stores are coalesced without
+// staging.  The arithmetic is epilogue.cuh's, element by element.
+//
+// Measured (block passes, 7B-shaped decoder layer of 48 tokens, one byte per weight code): 1860 -> 84 us against the warp-MMA
+// kernel (3.2 TB/s of weights over the whole pass, all seven kernels included); one image through a ViT-S block 52 -> 40 us
+// against 128-row tiles, of which so small a layer fills only a handful of SMs.
+//
+// Every wait on an mbarrier is bounded as in the other tensor-core kernels; all threads reach the two cluster barriers
+// whether or not a wait ran out.
+#include <cuda.h>
+#include <cuda_bf16.h>
+
+#include <type_traits>
+
+#include "kernels.h"
+#include "tc_ptx.cuh"
+
+namespace repq {
+namespace {
+
+using namespace tc;
+
+constexpr int kRowsW = 128;                 // output channels per tile (MMA M)
+constexpr int kBK = 128;                    // codes per k-block
+constexpr int kEpiWarps = 8;                // two per tensor-memory lane quarter
+constexpr int kThreads = 32 * (kEpiWarps + 2);
+constexpr int kTok = 8;                     // tokens per tensor-memory load
+constexpr int kMaxStages = 8;
+constexpr uint32_t kWBytes = kRowsW * kBK;
+constexpr int kMaxTokens = 128;           // tokens per tile at most
+constexpr int kPrefetch = 8;                // k-blocks of weights brought into L2 ahead of the dependency wait (all of a
+                                            // CTA's blocks at once crowd out the running kernel's own loads: 83 -> 88 us for
+                                            // a 7B-shaped decoder block of 48 tokens)
+constexpr int kSmemRing = 110 * 1024;       // operand ring with two resident CTAs (227 KB per SM less the static part)
+
+struct SkinnyParams {
+  int M, N, K;
+  int mt;                      // tokens per tile (multiple of 16)
+  int stages, kblocks, split;
+  uint32_t stage_bytes, a_bytes;
+  uint32_t tmem_cols;
+  const int32_t* asum;
+  const int32_t* wsum;
+  int32_t* status;
+  EpilogueParams ep;
+};
+
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, int y) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
+}
+
+// The steps between the linear value and the output conversion that are compiled in only where asked for.
+enum : int { kStepNone = 0, kStepGelu = 1, kStepResidual = 2, kStepRope = 3, kStepGlu = 4 };
+enum : int { kOutF32 = 0, kOutBf16 = 1, kOutC4 = 2, kOutC8 = 3 };
+
+// One chunk of kTok tokens of the thread's output channel j: the accumulators at `taddr` plus the partial sums the other
+// CTAs of the cluster left (`part`, one block of `part_stride` pieces per CTA), then the epilogue.  What an element needs
+// from global memory (residual, rotation table) is requested for the whole chunk before any of it is used.
+template <int OUT, int STEP, bool kWholeChunk>
+__device__ __forceinline__ void finish_chunk(const SkinnyParams& P, const ColumnTerms& ct, uint32_t taddr, const int32_t* asum,
+                                             const uint4* part, int parts, int part_stride, int mc, int j, bool col_ok, int lane) {
+  const EpilogueParams& ep = P.ep;
+  const int live = kWholeChunk ? kTok : min(kTok, P.M - mc);                    // tokens of the chunk inside the matrix (at least one)
+  float res[kTok];
+  float2 cs[kTok];
+  if constexpr (STEP == kStepResidual) {
+#pragma unroll
+    for (int e = 0; e < kTok; ++e) {
+      const int64_t off = int64_t(mc + min(e, live - 1)) * ep.ld_residual + (col_ok ? j : 0);
+      res[e] = ep.residual_bf16 ? __bfloat162float(static_cast<const __nv_bfloat16*>(ep.residual)[off]) : static_cast<const float*>(ep.residual)[off];
+    }
+  }
+  const bool turn = STEP == kStepRope && col_ok && j < ep.rope_cols;
+  if constexpr (STEP == kStepRope) {
+    const float2* line = ep.rope + ((j % ep.rope_dim) >> 1);
+    int pos = mc % ep.rope_period;
+#pragma unroll
+    for (int e = 0; e < kTok; ++e) {
+      if (turn) cs[e] = __ldg(line + int64_t(pos) * (ep.rope_dim >> 1));
+      if (++pos == ep.rope_period) pos = 0;
+    }
+  }
+  uint32_t r[kTok];
+  __syncwarp();
+  tmem_ld8(taddr, r);
+  tmem_ld_wait();
+  for (int s = 0; s < parts; ++s) {
+    const uint4 lo = part[s * part_stride], hi = part[s * part_stride + kRowsW];
+    r[0] += lo.x; r[1] += lo.y; r[2] += lo.z; r[3] += lo.w;
+    r[4] += hi.x; r[5] += hi.y; r[6] += hi.z; r[7] += hi.w;
+  }
+  if (ep.acc_debug != nullptr && col_ok)
+    for (int e = 0; e < live; ++e) ep.acc_debug[int64_t(mc + e) * P.N + j] = int32_t(r[e]);
+  float v[kTok];
+  const int4 as0 = *reinterpret_cast<const int4*>(asum), as1 = *reinterpret_cast<const int4*>(asum + 4);
+  const int32_t as[kTok] = {as0.x, as0.y, as0.z, as0.w, as1.x, as1.y, as1.z, as1.w};
+#pragma unroll
+  for (int e = 0; e < kTok; ++e) {
+    const int32_t corr = int32_t(r[e] - uint32_t(ct.z_w) * uint32_t(as[e]) + uint32_t(ct.kzz));
+    v[e] = fmaf(ct.scale, float(corr), ct.bias);
+    if constexpr (STEP == kStepGelu) v[e] = gelu_erf(v[e]);
+    if constexpr (STEP == kStepResidual) {
+      if (ep.gelu) v[e] = gelu_erf(v[e]);
+      v[e] += res[e];
+    }
+    if constexpr (STEP == kStepRope) {
+      const float other = __shfl_xor_sync(0xffffffffu, v[e], 1);
+      if (turn) {
+        float a = (j & 1) ? other : v[e], b = (j & 1) ? v[e] : other;
+        rope_rotate(cs[e], a, b);
+        v[e] = (j & 1) ? b : a;
+      }
+    }
+    if constexpr (STEP == kStepGlu) {                      // even channel: gate, odd: up; the even lane keeps the product
+      const float up = __shfl_xor_sync(0xffffffffu, v[e], 1);
+      v[e] = silu_mul(v[e], up);
+    }
+  }
+  const bool store = col_ok && !(STEP == kStepGlu && (j & 1));
+  const int64_t at0 = int64_t(mc) * ep.ldo + (STEP == kStepGlu || OUT == kOutC4 ? j >> 1 : j);
+  if constexpr (OUT == kOutF32 || OUT == kOutBf16) {
+    using T = typename std::conditional<OUT == kOutF32, float, __nv_bfloat16>::type;
+    T* o = static_cast<T*>(ep.out) + at0;
+#pragma unroll
+    for (int e = 0; e < kTok; ++e) {
+      if (store && (kWholeChunk || e < live)) {
+        if constexpr (OUT == kOutF32) *o = v[e]; else *o = __float2bfloat16_rn(v[e]);
+      }
+      o += ep.ldo;
+    }
+  } else {
+    uint8_t* o = static_cast<uint8_t*>(ep.out) + at0;
+    int code[kTok];
+#pragma unroll
+    for (int e = 0; e < kTok; ++e) code[e] = store ? requantize(ct, v[e]) : 0;
+#pragma unroll
+    for (int e = 0; e < kTok; ++e) {
+      if constexpr (OUT == kOutC4) {
+        const int next = __shfl_down_sync(0xffffffffu, code[e], 1);
+        if (col_ok && !(j & 1) && (kWholeChunk || e < live)) *o = uint8_t(code[e] | (next << 4));
+      } else {
+        if (store && (kWholeChunk || e < live)) *o = uint8_t(code[e]);
+      }
+      o += ep.ldo;
+    }
+    if (ep.out_row_sum != nullptr) {
+      int sums = 0;                                        // lane e: code sum of token mc + e over the warp's channels
+#pragma unroll
+      for (int e = 0; e < kTok; ++e) {
+        const int total = __reduce_add_sync(0xffffffffu, code[e]);
+        if (lane == e) sums = total;
+      }
+      if (lane < live) atomicAdd(ep.out_row_sum + mc + lane, sums);
+    }
+  }
+}
+
+template <int OUT, int STEP>
+__global__ void __launch_bounds__(kThreads, 2)
+qgemm_skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_a, const __grid_constant__ SkinnyParams P) {
+  extern __shared__ __align__(1024) uint8_t ring[];
+  __shared__ alignas(8) uint64_t s_full[kMaxStages], s_empty[kMaxStages], s_acc, s_done;
+  __shared__ uint32_t s_tmem;
+  __shared__ volatile int s_abort;
+  __shared__ alignas(16) int32_t s_asum[kMaxTokens];
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int split = P.split;
+  const int rank = int(blockIdx.x) % split;
+  const int n0 = int(blockIdx.x) / split * kRowsW, m0 = int(blockIdx.y) * P.mt;
+  const int kb0 = rank * P.kblocks / split, kb1 = (rank + 1) * P.kblocks / split;
+  const int stages = P.stages;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < stages; ++s) { mbar_init(smem_u32(&s_full[s]), 1); mbar_init(smem_u32(&s_empty[s]), 1); }
+    mbar_init(smem_u32(&s_acc), 1);
+    mbar_init(smem_u32(&s_done), 1);
+    s_abort = 0;
+    if (smem_u32(ring) & 1023u) {                          // the swizzled tiles need this alignment
+      atomicCAS(P.status, 0, 69);
+      s_abort = 1;
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == kEpiWarps + 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(P.tmem_cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (warp == kEpiWarps && blockIdx.y == 0)                // weights into L2 while the kernel before this one finishes
+    if (lane < kPrefetch && kb0 + lane < kb1) tma_prefetch_2d(&map_w, (kb0 + lane) * kBK, n0);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = s_tmem;
+  volatile int* abort = &s_abort;
+  grid_dependency_wait();
+  grid_dependency_trigger();
+
+  // the thread's output channel (epilogue warps)
+  const EpilogueParams& ep = P.ep;
+  const int quarter = warp & 3, half = warp >> 2;
+  const int j = n0 + quarter * 32 + lane;
+  const bool col_ok = j < P.N;
+  ColumnTerms ct{};
+
+  bool ok = true;
+  if (warp == kEpiWarps) {
+    // ---------------------------------------------------------------- bulk copies
+    if (lane == 0) {
+      uint32_t stage = 0, phase = 0;
+      int issued = 0;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!mbar_wait(smem_u32(&s_empty[stage]), phase ^ 1, abort, 61, P.status)) break;
+        const uint32_t bar = smem_u32(&s_full[stage]);
+        const uint32_t base = smem_u32(ring) + stage * P.stage_bytes;
+        mbar_expect_tx(bar, kWBytes + P.a_bytes);
+        tma_load_2d(base, &map_w, bar, kb * kBK, n0);
+        tma_load_2d(base + kWBytes, &map_a, bar, kb * kBK, m0);
+        ++issued;
+        if (++stage == uint32_t(stages)) { stage = 0; phase ^= 1; }
+      }
+      // the copies issued last must have landed before the ring is reused and the CTA may exit
+      for (int i = issued < stages ? issued : stages; i > 0; --i) {
+        if (stage == 0) { stage = uint32_t(stages) - 1; phase ^= 1; } else { --stage; }
+        mbar_drain(smem_u32(&s_full[stage]), phase);
+      }
+    }
+  } else if (warp == kEpiWarps + 1) {
+    // ---------------------------------------------------------------- MMA issue: D = s32, A = B = unsigned bytes, K-major
+    if (lane == 0) {
+      const uint32_t idesc = (2u << 4) | (uint32_t(P.mt >> 3) << 17) | (uint32_t(kRowsW >> 4) << 24);
+      uint32_t stage = 0, phase = 0;
+      bool go = true;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!mbar_wait(smem_u32(&s_full[stage]), phase, abort, 62, P.status)) { go = false; break; }
+        tc_fence_after();
+        const uint32_t base = smem_u32(ring) + stage * P.stage_bytes;
+        const uint64_t dw = smem_desc_sw128(base), da = smem_desc_sw128(base + kWBytes);
+#pragma unroll
+        for (int k = 0; k < kBK / 32; ++k) umma_i8(tmem, dw + uint64_t(2 * k), da + uint64_t(2 * k), idesc, (kb != kb0 || k != 0) ? 1u : 0u);
+        umma_commit(smem_u32(&s_empty[stage]));
+        if (++stage == uint32_t(stages)) { stage = 0; phase ^= 1; }
+      }
+      if (go) umma_commit(smem_u32(&s_acc));
+      umma_commit(smem_u32(&s_done));                      // all MMAs have completed before tensor memory is freed
+      mbar_drain(smem_u32(&s_done), 0);
+    }
+  } else {
+    // the tile's token sums and the channel's terms, behind the main loop
+    for (int i = threadIdx.x; i < P.mt; i += 32 * kEpiWarps) s_asum[i] = m0 + i < P.M ? __ldg(P.asum + m0 + i) : 0;
+    if (col_ok) ct = column_terms(ep, j, __ldg(P.wsum + j));
+    if (ep.glu) { const ColumnTerms q = column_terms(ep, 0, 0); ct.inv_so = q.inv_so; ct.zo_lo = q.zo_lo; ct.zo_hi = q.zo_hi; ct.zo = q.zo; }
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
+    ok = mbar_wait(smem_u32(&s_acc), 0, abort, 63, P.status);
+    tc_fence_after();
+  }
+  __syncwarp();
+
+  // ---------------------------------------------------------------- exchange of partial sums
+  // The tile's chunks of kTok tokens are dealt to the cluster's CTAs in contiguous shares; a CTA writes its partial sums
+  // of the other shares into their owners' shared memory: [source][chunk of the share][half of 4 tokens][channel] x 16 B.
+  const int chunks = P.mt / kTok;
+  const int share = (chunks + split - 1) / split;
+  const uint32_t tquarter = tmem + (uint32_t(quarter * 32) << 16);
+  const int row = quarter * 32 + lane;
+  if (split > 1) {
+    cluster_sync();                                        // every CTA of the cluster has finished with its ring
+    if (warp < kEpiWarps) {
+      for (int c = half; c < chunks; c += kEpiWarps / 4) {
+        const int owner = c / share;
+        if (owner == rank) continue;
+        uint32_t r[kTok];
+        tmem_ld8(tquarter + uint32_t(c * kTok), r);
+        tmem_ld_wait();
+        const int src = rank - (rank > owner ? 1 : 0);     // 0 .. split - 2
+        const uint32_t at = smem_u32(ring) + uint32_t((src * share + (c - owner * share)) * 2 * kRowsW + row) * 16u;
+        const uint32_t to = map_to_rank(at, uint32_t(owner));
+        st_cluster_v4(to, r[0], r[1], r[2], r[3]);
+        st_cluster_v4(to + kRowsW * 16u, r[4], r[5], r[6], r[7]);
+      }
+    }
+    cluster_sync();
+  }
+
+  // ---------------------------------------------------------------- epilogue of this CTA's share
+  if (warp < kEpiWarps && ok && !*abort) {
+    const int c_end = min(chunks, (rank + 1) * share);
+    for (int c = rank * share + half; c < c_end; c += kEpiWarps / 4) {
+      const int mc = m0 + c * kTok;
+      if (mc >= P.M) break;
+      const uint4* part = reinterpret_cast<const uint4*>(ring) + (c - rank * share) * 2 * kRowsW + row;
+      if (mc + kTok <= P.M)
+        finish_chunk<OUT, STEP, true>(P, ct, tquarter + uint32_t(c * kTok), s_asum + c * kTok, part, split - 1, share * 2 * kRowsW, mc, j, col_ok, lane);
+      else
+        finish_chunk<OUT, STEP, false>(P, ct, tquarter + uint32_t(c * kTok), s_asum + c * kTok, part, split - 1, share * 2 * kRowsW, mc, j, col_ok, lane);
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kEpiWarps + 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(P.tmem_cols) : "memory");
+  }
+}
+
+repq_status make_map(CUtensorMap* map, const uint8_t* base, int64_t rows, int64_t k, int64_t ld, int box_rows) {
+  EncodeTiledFn fn = encode_fn();
+  REPQ_REQUIRE(fn != nullptr, REPQ_CUDA_ERROR, "qgemm: cuTensorMapEncodeTiled is not available");
+  const cuuint64_t dims[2] = {cuuint64_t(k), cuuint64_t(rows)};
+  const cuuint64_t strides[1] = {cuuint64_t(ld)};
+  const cuuint32_t box[2] = {kBK, cuuint32_t(box_rows)};
+  const cuuint32_t estr[2] = {1, 1};
+  const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t*>(base), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  REPQ_REQUIRE(r == CUDA_SUCCESS, REPQ_CUDA_ERROR, "qgemm: cuTensorMapEncodeTiled failed with code %d", int(r));
+  return REPQ_OK;
+}
+
+template <int OUT, int STEP>
+repq_status launch(dim3 grid, uint32_t smem, const CUtensorMap& map_w, const CUtensorMap& map_a, const SkinnyParams& P, cudaStream_t st) {
+  REPQ_CUDA(cudaFuncSetAttribute(qgemm_skinny_kernel<OUT, STEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemRing));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = unsigned(P.split);
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  REPQ_CUDA(cudaLaunchKernelEx(&cfg, qgemm_skinny_kernel<OUT, STEP>, map_w, map_a, P));
+  note_launch();
+  return REPQ_OK;
+}
+
+template <int OUT>
+repq_status launch_step(int step, dim3 grid, uint32_t smem, const CUtensorMap& map_w, const CUtensorMap& map_a, const SkinnyParams& P, cudaStream_t st) {
+  switch (step) {
+    case kStepGelu: return launch<OUT, kStepGelu>(grid, smem, map_w, map_a, P, st);
+    case kStepResidual: return launch<OUT, kStepResidual>(grid, smem, map_w, map_a, P, st);
+    case kStepRope: return launch<OUT, kStepRope>(grid, smem, map_w, map_a, P, st);
+    case kStepGlu:
+      if constexpr (OUT != kOutC4) return launch<OUT, kStepGlu>(grid, smem, map_w, map_a, P, st);   // (packed codes are refused)
+    default: return launch<OUT, kStepNone>(grid, smem, map_w, map_a, P, st);
+  }
+}
+
+}  // namespace
+
+namespace {
+
+// How a problem is cut up: tokens per tile and CTAs per tile, and the estimated time in microseconds.  The terms were
+// fitted to launches in CUDA graphs (K 384..11008, N 384..22016, 16..788 tokens); what they stand for:
+//   a launch                2.6
+//   operands                k-blocks of a CTA x (16 KB of weights + tokens) x CTAs that share an SM, at 120 KB per us and SM,
+//                           or all weights at 4.5 TB/s, whichever is longer
+//   epilogue                0.028 per token of a CTA's share
+//   exchange in the cluster 1.2
+// At most two CTAs per SM: a second wave costs more than it brings.
+struct Plan { int mt = 0, split = 0; float us = 1e30f; };
+
+Plan plan_of(int M, int N, int K, int sms) {
+  Plan best;
+  const int n_tiles = (N + kRowsW - 1) / kRowsW, kblocks = (K + kBK - 1) / kBK;
+  const float hbm = float(N) * float(K) / 4.5e6f;
+  for (int mt : {16, 32, 48, 64, 96, 128}) {
+    const int m_tiles = (M + mt - 1) / mt;
+    for (int split = 1; split <= 8; split *= 2) {
+      const int64_t ctas = int64_t(n_tiles) * m_tiles * split;
+      if (ctas > 2 * sms || (split > 1 && kblocks < 2 * split)) break;
+      const float per_sm = ctas > sms ? 2.f : 1.f;
+      const int kb = (kblocks + split - 1) / split, share = (mt / kTok + split - 1) / split * kTok;
+      float load = per_sm * float(kb) * (16.f + float(mt) / 8.f) / 120.f;
+      if (load < hbm) load = hbm;
+      const float us = 2.6f + load + per_sm * float(share) * 0.028f + (split > 1 ? 1.2f : 0.f);
+      if (us < best.us) { best.mt = mt; best.split = split; best.us = us; }
+    }
+    if (mt >= M) break;
+  }
+  return best;
+}
+
+}  // namespace
+
+// Taken where its estimate is clearly below that of the 128-row kernel (4.5 us + 0.27 us per round of tiles and k-block, or
+// the weights at 4.5 TB/s), which holds up to some hundreds of tokens, and below 64 tokens wherever the operands allow it.
+bool qgemm_skinny_preferred(const repq_gemm_desc& d) {
+  if (d.batch_outer != 1 || d.batch_inner != 1 || d.N < 64 || d.K < 64) return false;
+  if (!d.a_row_sum || !d.w_row_sum) return false;          // (the sums are not taken here; no workspace)
+  if (packed4(d.bits_a) || packed4(d.bits_w) || packed6(d.bits_w)) return false;
+  if (!(aligned(d.a_codes, 16) && d.lda_bytes % 16 == 0 && aligned(d.w_codes, 16) && d.ldw_bytes % 16 == 0)) return false;
+  const int sms = sm_count();
+  const Plan plan = plan_of(d.M, d.N, d.K, sms);
+  if (plan.mt == 0) return false;
+  if (!qgemm_tc_supported(d)) return true;
+  const int64_t tiles = (int64_t(d.M) + 127) / 128 * ((int64_t(d.N) + 255) / 256);
+  float other = float((tiles + sms - 1) / sms) * float((d.K + kBK - 1) / kBK) * 0.27f;
+  const float hbm = float(d.N) * float(d.K) / 4.5e6f;
+  if (other < hbm) other = hbm;
+  return plan.us * 1.1f < other + 4.5f || (d.M <= 64 && plan.us < other + 4.5f);
+}
+
+repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, cudaStream_t st) {
+  SkinnyParams P{};
+  P.M = d.M; P.N = d.N; P.K = d.K;
+  P.asum = d.a_row_sum; P.wsum = d.w_row_sum;
+  P.ep = ep;
+  P.status = device_status_word();
+  REPQ_REQUIRE(P.status != nullptr, REPQ_CUDA_ERROR, "qgemm: device status word unavailable");
+  const Plan plan = plan_of(d.M, d.N, d.K, sm_count());
+  const int n_tiles = (d.N + kRowsW - 1) / kRowsW, mt = plan.mt, split = plan.split;
+  const int m_tiles = (d.M + mt - 1) / mt;
+  P.kblocks = (d.K + kBK - 1) / kBK;
+  P.mt = mt;
+  P.split = split;
+  P.a_bytes = uint32_t(mt) * kBK;
+  P.stage_bytes = kWBytes + P.a_bytes;
+  const int per = (P.kblocks + split - 1) / split;         // k-blocks of a CTA
+  int stages = kSmemRing / int(P.stage_bytes);             // at least three
+  if (stages > kMaxStages) stages = kMaxStages;
+  if (stages > per) stages = per;
+  P.stages = stages;
+  // the ring also holds the partial sums of the exchange
+  const int share = (mt / kTok + split - 1) / split;
+  const uint32_t exchange = uint32_t(split - 1) * uint32_t(share) * 2u * kRowsW * 16u;
+  uint32_t smem = uint32_t(stages) * P.stage_bytes;
+  if (smem < exchange) smem = exchange;
+  P.tmem_cols = 32;
+  while (P.tmem_cols < uint32_t(mt)) P.tmem_cols *= 2;
+  CUtensorMap map_w, map_a;
+  REPQ_TRY(make_map(&map_w, d.w_codes, d.N, d.K, d.ldw_bytes, kRowsW));
+  REPQ_TRY(make_map(&map_a, d.a_codes, d.M, d.K, d.lda_bytes, mt));
+  const int out = ep.out_kind == REPQ_OUT_F32 ? kOutF32 : ep.out_kind == REPQ_OUT_BF16 ? kOutBf16 : ep.pack4 ? kOutC4 : kOutC8;
+  const int step = ep.rope ? kStepRope : ep.glu ? kStepGlu : ep.residual ? kStepResidual : ep.gelu ? kStepGelu : kStepNone;
+  const dim3 grid(unsigned(n_tiles * split), unsigned(m_tiles));
+  switch (out) {
+    case kOutF32: return launch_step<kOutF32>(step, grid, smem, map_w, map_a, P, st);
+    case kOutBf16: return launch_step<kOutBf16>(step, grid, smem, map_w, map_a, P, st);
+    case kOutC4: return launch_step<kOutC4>(step, grid, smem, map_w, map_a, P, st);
+    default: return launch_step<kOutC8>(step, grid, smem, map_w, map_a, P, st);
+  }
+}
+
+}  // namespace repq
