@@ -201,8 +201,16 @@ def _dtype_code(t: torch.Tensor) -> int:
     raise TypeError("expected a float32 or bfloat16 tensor, got %s" % t.dtype)
 
 
+try:                                    # the raw handle without a Stream object: a microsecond less on every call
+    _raw_stream, _raw_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+except AttributeError:
+    _raw_stream = None
+
+
 def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            return _raw_stream(_raw_device())
         return torch.cuda.current_stream().cuda_stream
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 

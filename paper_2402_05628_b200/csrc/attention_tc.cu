@@ -797,7 +797,7 @@ repq_status make_k_map(CUtensorMap* map, const AttnParams& P, int batch_outer, i
 template <int NB, int kLutBits, int kMode>
 repq_status launch_kernel(const AttnParams& P, int64_t pairs, cudaStream_t st) {
   const size_t smem = sizeof(AttnShared<NB, kLutBits>);
-  REPQ_CUDA(cudaFuncSetAttribute(attention_tc_kernel<NB, kLutBits, kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+  REPQ_TRY((allow_smem<attention_tc_kernel<NB, kLutBits, kMode>>(int(smem))));
   AttnParams Q = P;
   Q.pairs = int(pairs);
   Q.tiles = (P.Lq + kRows - 1) / kRows;

@@ -72,10 +72,10 @@ BlockLayout layout(const repq_block_desc& d) {
   L.off_scores = bump(cur, d.staged_attention ? size_t(rows_s * L.ld_s) * 4 : 0);
   L.off_p = bump(cur, d.staged_attention ? size_t(rows_s * L.ld_p) : 0);
   L.off_attn = bump(cur, size_t(L.M * L.ld_a));
-  L.off_asum_attn = bump(cur, size_t(L.M) * 4);
+  L.off_asum_attn = bump(cur, size_t(L.M) * 4);                    // (neighbours: cleared as one run)
+  L.off_asum_h = bump(cur, size_t(L.M) * 4);
   L.off_xbar = bump(cur, size_t(L.M) * d.dim * act);
   L.off_hidden = bump(cur, size_t(L.M * L.ld_h));
-  L.off_asum_h = bump(cur, size_t(L.M) * 4);
   // scratch of the largest GEMM of the block
   repq_linear_params none{};
   size_t ws = 0;
@@ -135,10 +135,8 @@ static repq_status block_forward_impl(const repq_block_desc* dp, const repq_bloc
   uint8_t* hid_c = ws + L.off_hidden;
   int32_t* asum_h = reinterpret_cast<int32_t*>(ws + L.off_asum_h);
   void* gws = ws + L.off_gemm_ws;
-  // the two row-sum accumulators that kernels add into start at zero; cleared here, ahead of the first kernel,
-  // so that the kernels of the block follow one another in the stream without anything in between
-  REPQ_CUDA(cudaMemsetAsync(asum_attn, 0, size_t(M) * 4, st));
-  REPQ_CUDA(cudaMemsetAsync(asum_h, 0, size_t(M) * 4, st));
+  // the two row-sum accumulators that kernels add into start at zero: the first kernel of the block clears them
+  const ClearWords clear{asum_attn, asum_h + M - asum_attn};
   int n_mark = 0;
 #define REPQ_MARK()                                            \
   do {                                                         \
@@ -147,8 +145,8 @@ static repq_status block_forward_impl(const repq_block_desc* dp, const repq_bloc
   REPQ_MARK();
 
   // ---- X_bar = MSA(LN(X)) + X
-  REPQ_TRY(repq_ln_quant(x, d.act_dtype, M, D, D, p.ln1_gamma_t, p.ln1_beta_t, d.eps, d.norm_kind, p.ln1_s, p.ln1_z,
-                         ab, ln_c, L.ld_a, asum, stream));
+  REPQ_TRY(launch_ln_quant(x, d.act_dtype, M, D, D, p.ln1_gamma_t, p.ln1_beta_t, d.eps, d.norm_kind, p.ln1_s, p.ln1_z,
+                           ab, ln_c, L.ld_a, asum, clear, st));
   REPQ_MARK();
   {
     repq_gemm_desc g = linear_desc(d, M, 3 * D, D, ln_c, L.ld_a, p.ln1_s, p.ln1_z, asum, p.qkv);

@@ -1,6 +1,7 @@
 // Shared host-side plumbing of the repq library: error reporting and argument checks.
 #pragma once
 #include <cuda_runtime.h>
+#include <atomic>
 #include <cstdarg>
 #include <cstdint>
 #include <cstdio>
@@ -65,6 +66,36 @@ void note_launch(int n = 1);
 // memory that an earlier kernel may have written or may still read, and grid_dependency_trigger() once it has
 // started (both are no-ops in a kernel launched the plain way).
 #ifdef __CUDACC__
+// Opt-in of a kernel to more than 48 KB of dynamic shared memory, asked of the runtime once per kernel and device.
+template <auto kKernel>
+repq_status allow_smem(int bytes) {
+  static std::atomic<uint64_t> done{0};                // one bit per device
+  int dev = 0;
+  REPQ_CUDA(cudaGetDevice(&dev));
+  const uint64_t bit = dev < 64 ? uint64_t(1) << dev : 0;
+  if (done.load(std::memory_order_relaxed) & bit) return REPQ_OK;
+  REPQ_CUDA(cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  done.fetch_or(bit, std::memory_order_relaxed);
+  return REPQ_OK;
+}
+
+// Resident blocks per SM of a kernel, remembered per device for the last dynamic shared-memory size asked for.
+struct Residency { std::atomic<uint64_t> last[64]; };   // (bytes << 8) | blocks, 0: nothing yet
+template <typename Kernel>
+repq_status resident_blocks(Residency& memo, Kernel kern, int block, size_t smem, int* out) {
+  int dev = 0;
+  REPQ_CUDA(cudaGetDevice(&dev));
+  const bool keep = dev >= 0 && dev < 64;
+  const uint64_t seen = keep ? memo.last[dev].load(std::memory_order_relaxed) : 0;
+  if (seen != 0 && (seen >> 8) == smem) { *out = int(seen & 0xFF); return REPQ_OK; }
+  int n = 0;
+  REPQ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, block, smem));
+  if (n < 1) n = 1;
+  if (keep) memo.last[dev].store((uint64_t(smem) << 8) | uint64_t(n), std::memory_order_relaxed);
+  *out = n;
+  return REPQ_OK;
+}
+
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

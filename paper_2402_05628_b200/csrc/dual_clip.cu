@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(32 * kWarps, kWarps == 16 ? 2 : 28 / kWarps) d
 template <int kWarps>
 repq_status launch_resident(const ClipParams& P, cudaStream_t st) {
   const size_t smem = size_t(P.n) * sizeof(float);
-  REPQ_CUDA(cudaFuncSetAttribute(dual_clip_resident_kernel<kWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxResident * 4));
+  REPQ_TRY(allow_smem<dual_clip_resident_kernel<kWarps>>(kMaxResident * 4));
   dual_clip_resident_kernel<kWarps><<<P.D, 32 * kWarps, smem, st>>>(P);
   REPQ_CUDA(cudaGetLastError());
   return REPQ_OK;

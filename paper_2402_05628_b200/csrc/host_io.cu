@@ -1,7 +1,14 @@
 // Host-buffer form of the block: a sequence of independent batches whose inputs and outputs live in host
-// memory.  The copies and the block's kernels of neighbouring batches overlap: while batch i is computed,
-// batch i + 1 is copied in and batch i - 1 is copied out, through two device staging buffers per direction
-// and two helper streams.  (Plumbing around the block; the block itself is repq_block_forward.)
+// memory.  The copies and the block's kernels overlap through two device staging buffers per direction and two helper
+// streams.  (Plumbing around the block; the block itself is repq_block_forward.)
+//
+// What bounds it is the host link, one direction each for inputs and outputs; beside that, the first copy in and the last
+// copy out, which nothing overlaps.  The items of a batch are independent, so a batch passes through the pipeline in up to
+// kMaxPieces pieces of whole items: piece c is computed while piece c + 1 is copied in and piece c - 1 copied out, and what
+// nothing overlaps is a piece instead of a batch.  A piece is at least kPieceBytes of input (below, the launches of the
+// block and the small copies take longer than the link does).  Long sequences of batches stay whole: there the ends weigh
+// little and smaller blocks and copies run at lower rates.  64 DeiT-B items per batch: one batch 950 -> 650 us, two
+// 1350 -> 1120, four 2240 -> 2150 (sixteen in pieces would be 7.8 -> 8.4 ms).
 #include <mutex>
 
 #include "kernels.h"
@@ -11,12 +18,15 @@ namespace {
 
 constexpr int kMaxDevices = 64;
 constexpr int kSlots = 2;
+constexpr int kMaxPieces = 8;
+constexpr size_t kPieceBytes = size_t(4) << 20;
+constexpr int kPieceBatches = 4;
 
 struct Pipeline {                 // per device, created on first use, kept for the life of the process
   bool ready = false;
   cudaStream_t in = nullptr, out = nullptr;
   cudaEvent_t start = nullptr;
-  cudaEvent_t copied_in[kSlots] = {}, computed[kSlots] = {}, copied_out[kSlots] = {};
+  cudaEvent_t copied_in[kSlots][kMaxPieces] = {}, computed[kSlots][kMaxPieces] = {}, copied_out[kSlots][kMaxPieces] = {};
 };
 Pipeline g_pipe[kMaxDevices];
 std::mutex g_pipe_mutex;
@@ -31,11 +41,12 @@ repq_status pipeline(Pipeline** out) {
     REPQ_CUDA(cudaStreamCreateWithFlags(&P.in, cudaStreamNonBlocking));
     REPQ_CUDA(cudaStreamCreateWithFlags(&P.out, cudaStreamNonBlocking));
     REPQ_CUDA(cudaEventCreateWithFlags(&P.start, cudaEventDisableTiming));
-    for (int s = 0; s < kSlots; ++s) {
-      REPQ_CUDA(cudaEventCreateWithFlags(&P.copied_in[s], cudaEventDisableTiming));
-      REPQ_CUDA(cudaEventCreateWithFlags(&P.computed[s], cudaEventDisableTiming));
-      REPQ_CUDA(cudaEventCreateWithFlags(&P.copied_out[s], cudaEventDisableTiming));
-    }
+    for (int s = 0; s < kSlots; ++s)
+      for (int c = 0; c < kMaxPieces; ++c) {
+        REPQ_CUDA(cudaEventCreateWithFlags(&P.copied_in[s][c], cudaEventDisableTiming));
+        REPQ_CUDA(cudaEventCreateWithFlags(&P.computed[s][c], cudaEventDisableTiming));
+        REPQ_CUDA(cudaEventCreateWithFlags(&P.copied_out[s][c], cudaEventDisableTiming));
+      }
     P.ready = true;
   }
   *out = &P;
@@ -63,6 +74,7 @@ extern "C" repq_status repq_block_forward_host(const repq_block_desc* d, const r
                "block_forward_host: the two staging buffers of a direction must differ");
   for (int i = 0; i < n_batches; ++i)
     REPQ_REQUIRE(x_host[i] && y_host[i], REPQ_INVALID_ARG, "block_forward_host: NULL host buffer of batch %d", i);
+  REPQ_REQUIRE(d->batch > 0 && d->seq > 0 && d->dim > 0, REPQ_INVALID_ARG, "block_forward_host: sizes must be positive");
   const size_t elems = size_t(d->batch) * size_t(d->seq) * size_t(d->dim);
   const size_t x_bytes = elems * dtype_size(d->act_dtype), y_bytes = elems * dtype_size(d->out_dtype);
   Pipeline* P = nullptr;
@@ -73,24 +85,34 @@ extern "C" repq_status repq_block_forward_host(const repq_block_desc* d, const r
   REPQ_CUDA(cudaEventRecord(P->start, main));
   REPQ_CUDA(cudaStreamWaitEvent(P->in, P->start, 0));
   REPQ_CUDA(cudaStreamWaitEvent(P->out, P->start, 0));
+  int64_t fit = int64_t(x_bytes / kPieceBytes);
+  fit = fit < 1 ? 1 : fit > kMaxPieces ? kMaxPieces : fit;
+  const int pieces = n_batches > kPieceBatches ? 1 : int(fit < d->batch ? fit : d->batch);
+  const size_t x_item = x_bytes / size_t(d->batch), y_item = y_bytes / size_t(d->batch);
+  repq_block_desc piece = *d;
   for (int i = 0; i < n_batches; ++i) {
     const int k = i % kSlots;
-    // copy in: x_dev[k] was last read by the block of batch i - 2
-    if (i >= kSlots) REPQ_CUDA(cudaStreamWaitEvent(P->in, P->computed[k], 0));
-    REPQ_CUDA(cudaMemcpyAsync(s->x_dev[k], x_host[i], x_bytes, cudaMemcpyHostToDevice, P->in));
-    REPQ_CUDA(cudaEventRecord(P->copied_in[k], P->in));
-    // block: y_dev[k] was last read by the copy-out of batch i - 2
-    REPQ_CUDA(cudaStreamWaitEvent(main, P->copied_in[k], 0));
-    if (i >= kSlots) REPQ_CUDA(cudaStreamWaitEvent(main, P->copied_out[k], 0));
-    REPQ_TRY(repq_block_forward(d, p, s->x_dev[k], s->y_dev[k], s->workspace, s->workspace_bytes, stream));
-    REPQ_CUDA(cudaEventRecord(P->computed[k], main));
-    // copy out
-    REPQ_CUDA(cudaStreamWaitEvent(P->out, P->computed[k], 0));
-    REPQ_CUDA(cudaMemcpyAsync(y_host[i], s->y_dev[k], y_bytes, cudaMemcpyDeviceToHost, P->out));
-    REPQ_CUDA(cudaEventRecord(P->copied_out[k], P->out));
+    for (int c = 0; c < pieces; ++c) {
+      const size_t first = size_t(int64_t(d->batch) * c / pieces), end = size_t(int64_t(d->batch) * (c + 1) / pieces);
+      piece.batch = int32_t(end - first);
+      uint8_t* xd = static_cast<uint8_t*>(s->x_dev[k]) + first * x_item;
+      uint8_t* yd = static_cast<uint8_t*>(s->y_dev[k]) + first * y_item;
+      // copy in: this part of x_dev[k] was last read by the same piece of batch i - 2
+      if (i >= kSlots) REPQ_CUDA(cudaStreamWaitEvent(P->in, P->computed[k][c], 0));
+      REPQ_CUDA(cudaMemcpyAsync(xd, static_cast<const uint8_t*>(x_host[i]) + first * x_item, (end - first) * x_item, cudaMemcpyHostToDevice, P->in));
+      REPQ_CUDA(cudaEventRecord(P->copied_in[k][c], P->in));
+      // block: this part of y_dev[k] was last read by the copy-out of the same piece of batch i - 2
+      REPQ_CUDA(cudaStreamWaitEvent(main, P->copied_in[k][c], 0));
+      if (i >= kSlots) REPQ_CUDA(cudaStreamWaitEvent(main, P->copied_out[k][c], 0));
+      REPQ_TRY(repq_block_forward(&piece, p, xd, yd, s->workspace, s->workspace_bytes, stream));
+      REPQ_CUDA(cudaEventRecord(P->computed[k][c], main));
+      // copy out
+      REPQ_CUDA(cudaStreamWaitEvent(P->out, P->computed[k][c], 0));
+      REPQ_CUDA(cudaMemcpyAsync(static_cast<uint8_t*>(y_host[i]) + first * y_item, yd, (end - first) * y_item, cudaMemcpyDeviceToHost, P->out));
+      REPQ_CUDA(cudaEventRecord(P->copied_out[k][c], P->out));
+    }
   }
-  // the caller's stream completes only after the last copies out (and hence after every copy in)
-  for (int i = n_batches > kSlots ? n_batches - kSlots : 0; i < n_batches; ++i)
-    REPQ_CUDA(cudaStreamWaitEvent(main, P->copied_out[i % kSlots], 0));
+  // the caller's stream completes only after the last copy out (and hence, copies leaving in order, after every copy)
+  REPQ_CUDA(cudaStreamWaitEvent(main, P->copied_out[(n_batches - 1) % kSlots][pieces - 1], 0));
   return REPQ_OK;
 }

@@ -5,6 +5,13 @@
 
 namespace repq {
 
+// LayerNorm + quantization (repq_ln_quant), which can also set a run of words to zero: row-sum accumulators that later
+// kernels of a chain add into, without a launch of their own.
+struct ClearWords { int32_t* at = nullptr; int64_t n = 0; };
+repq_status launch_ln_quant(const void* x, int x_dtype, int64_t rows, int D, int64_t ldx, const float* gamma_t,
+                            const float* beta_t, float eps, int norm_kind, float s_t, int z_t, int bits, uint8_t* codes,
+                            int64_t ld_codes_bytes, int32_t* row_sum, ClearWords clear, cudaStream_t st);
+
 // Row sums of a code matrix: out[r] = sum_c codes[r, c] (zero-point correction terms).
 repq_status launch_row_sum(const uint8_t* codes, int bits, int64_t rows, int64_t n, int64_t ld_bytes,
                            int32_t* out, cudaStream_t st);

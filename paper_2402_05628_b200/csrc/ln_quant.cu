@@ -16,8 +16,8 @@
 // instead.  z is added as an integer and the clip of Eq. 4 is the saturation of the packing instruction.
 #include <cuda_bf16.h>
 
-#include "common.h"
 #include "f32x2.cuh"
+#include "kernels.h"
 
 namespace repq {
 namespace {
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__((TPR > 256 ? TPR : 256),
 ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
                 const float* __restrict__ gamma_t, const float* __restrict__ beta_t, float eps, int rms,
                 float inv_s, int z, int qmax, uint8_t* __restrict__ codes, int64_t ldc,
-                int32_t* __restrict__ row_sum) {
+                int32_t* __restrict__ row_sum, int32_t* __restrict__ clear, int64_t n_clear) {
   constexpr int kRows = rows_in_flight(kVPT, TPR);
   constexpr int kBlock = TPR > 256 ? TPR : 256;
   constexpr int kGroups = kBlock / TPR;
@@ -249,6 +249,7 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
   // gamma~ and beta~ are parameters; x and the outputs belong to the chain of kernels
   grid_dependency_wait();
   grid_dependency_trigger();
+  for (int64_t i = int64_t(blockIdx.x) * kBlock + threadIdx.x; i < n_clear; i += int64_t(gridDim.x) * kBlock) clear[i] = 0;
 
   const int tig = threadIdx.x % TPR;             // thread in group
   const int group = threadIdx.x / TPR;
@@ -415,7 +416,7 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
 template <typename T, int TPR, int kVPT>
 repq_status launch(const T* x, int64_t rows, int D, int64_t ldx, const float* g, const float* b, float eps,
                    int rms, float s_t, int z, int bits, uint8_t* codes, int64_t ldc, int32_t* row_sum,
-                   cudaStream_t st) {
+                   ClearWords clear, cudaStream_t st) {
   constexpr int kBlock = TPR > 256 ? TPR : 256;
   constexpr int kRowsPerBlock = kBlock / TPR * rows_in_flight(kVPT, TPR);
   const int64_t need = (rows + kRowsPerBlock - 1) / kRowsPerBlock;
@@ -423,16 +424,18 @@ repq_status launch(const T* x, int64_t rows, int D, int64_t ldx, const float* g,
   const int qmax = code_max(bits);
   const size_t smem = factors_in_registers(kVPT, TPR, sizeof(T)) ? 0 : size_t(D) * 2 * sizeof(float);
   const bool full = D == TPR * kVPT * kChunk;   // the row fills the group exactly: no chunk is predicated
-  auto kern = packed4(bits) ? (full ? ln_quant_kernel<T, TPR, kVPT, true, true> : ln_quant_kernel<T, TPR, kVPT, true, false>)
-                            : (full ? ln_quant_kernel<T, TPR, kVPT, false, true> : ln_quant_kernel<T, TPR, kVPT, false, false>);
+  const bool pack = packed4(bits);
+  auto kern = pack ? (full ? ln_quant_kernel<T, TPR, kVPT, true, true> : ln_quant_kernel<T, TPR, kVPT, true, false>)
+                   : (full ? ln_quant_kernel<T, TPR, kVPT, false, true> : ln_quant_kernel<T, TPR, kVPT, false, false>);
   if (smem > 48 * 1024) REPQ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+  static Residency memo[2][2];
   // persistent grid: exactly the blocks that are resident at once, so that every block keeps its load pipeline
   // running over all of its rows
   int resident = 0;
-  REPQ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kern, kBlock, smem));
-  const int64_t cap = int64_t(sm_count()) * (resident > 0 ? resident : 1);
+  REPQ_TRY(resident_blocks(memo[pack][full], kern, kBlock, smem, &resident));
+  const int64_t cap = int64_t(sm_count()) * resident;
   const int grid = int(need < cap ? need : cap);
-  REPQ_CUDA(launch_chained(kern, dim3(grid), dim3(kBlock), smem, st, x, rows, D, ldx, g, b, eps, rms, inv_s, z, qmax, codes, ldc, row_sum));
+  REPQ_CUDA(launch_chained(kern, dim3(grid), dim3(kBlock), smem, st, x, rows, D, ldx, g, b, eps, rms, inv_s, z, qmax, codes, ldc, row_sum, clear.at, clear.n));
   note_launch();
   return REPQ_OK;
 }
@@ -440,24 +443,24 @@ repq_status launch(const T* x, int64_t rows, int D, int64_t ldx, const float* g,
 template <typename T, int TPR>
 repq_status launch_vpt(int vpt, const T* x, int64_t rows, int D, int64_t ldx, const float* g, const float* b, float eps,
                        int rms, float s_t, int z, int bits, uint8_t* codes, int64_t ldc, int32_t* row_sum,
-                       cudaStream_t st) {
+                       ClearWords clear, cudaStream_t st) {
   switch (vpt) {
-    case 1: return launch<T, TPR, 1>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, st);
-    case 2: return launch<T, TPR, 2>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, st);
-    case 3: return launch<T, TPR, 3>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, st);
-    default: return launch<T, TPR, 4>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, st);
+    case 1: return launch<T, TPR, 1>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
+    case 2: return launch<T, TPR, 2>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
+    case 3: return launch<T, TPR, 3>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
+    default: return launch<T, TPR, 4>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
   }
 }
 
 template <typename T>
 repq_status dispatch(const T* x, int64_t rows, int D, int64_t ldx, const float* g, const float* b, float eps,
                      int rms, float s_t, int z, int bits, uint8_t* codes, int64_t ldc, int32_t* row_sum,
-                     cudaStream_t st) {
+                     ClearWords clear, cudaStream_t st) {
   const int nchunks = D / kChunk;
   // a row that would take four chunks per thread in a group of 128 goes to a whole block with two (measured:
   // D = 4096 runs 9 % faster as 256 x 2 with three resident blocks than as 128 x 4 with one)
 #define REPQ_LN_CASE(TPR) \
-  if (nchunks <= TPR * (TPR == 128 ? 3 : kMaxVPT)) return launch_vpt<T, TPR>((nchunks + TPR - 1) / TPR, x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, st);
+  if (nchunks <= TPR * (TPR == 128 ? 3 : kMaxVPT)) return launch_vpt<T, TPR>((nchunks + TPR - 1) / TPR, x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
   REPQ_LN_CASE(8)
   REPQ_LN_CASE(16)
   REPQ_LN_CASE(32)
@@ -470,14 +473,10 @@ repq_status dispatch(const T* x, int64_t rows, int D, int64_t ldx, const float* 
 }
 
 }  // namespace
-}  // namespace repq
 
-using namespace repq;
-
-extern "C" repq_status repq_ln_quant(const void* x, int x_dtype, int64_t rows, int D, int64_t ldx,
-                                     const float* gamma_t, const float* beta_t, float eps, int norm_kind,
-                                     float s_t, int z_t, int bits, uint8_t* codes, int64_t ld_codes_bytes,
-                                     int32_t* row_sum, void* stream) {
+repq_status launch_ln_quant(const void* x, int x_dtype, int64_t rows, int D, int64_t ldx, const float* gamma_t,
+                            const float* beta_t, float eps, int norm_kind, float s_t, int z_t, int bits, uint8_t* codes,
+                            int64_t ld_codes_bytes, int32_t* row_sum, ClearWords clear, cudaStream_t st) {
   REPQ_REQUIRE(rows >= 0 && D > 0, REPQ_INVALID_ARG, "ln_quant: rows must be >= 0 and D > 0");
   if (rows == 0) return REPQ_OK;
   REPQ_REQUIRE(x && gamma_t && beta_t && codes, REPQ_INVALID_ARG, "ln_quant: NULL pointer");
@@ -495,9 +494,18 @@ extern "C" repq_status repq_ln_quant(const void* x, int x_dtype, int64_t rows, i
   REPQ_REQUIRE(ld_codes_bytes >= code_row_bytes(D, bits), REPQ_INVALID_ARG, "ln_quant: ld_codes_bytes shorter than a row");
   REPQ_REQUIRE(aligned(codes, unit) && ld_codes_bytes % unit == 0, REPQ_ALIGNMENT,
                "ln_quant: codes rows must be %d-byte aligned", int(unit));
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int rms = norm_kind == REPQ_NORM_RMS;
   if (x_dtype == REPQ_F32)
-    return dispatch(static_cast<const float*>(x), rows, D, ldx, gamma_t, beta_t, eps, rms, s_t, z_t, bits, codes, ld_codes_bytes, row_sum, st);
-  return dispatch(static_cast<const __nv_bfloat16*>(x), rows, D, ldx, gamma_t, beta_t, eps, rms, s_t, z_t, bits, codes, ld_codes_bytes, row_sum, st);
+    return dispatch(static_cast<const float*>(x), rows, D, ldx, gamma_t, beta_t, eps, rms, s_t, z_t, bits, codes, ld_codes_bytes, row_sum, clear, st);
+  return dispatch(static_cast<const __nv_bfloat16*>(x), rows, D, ldx, gamma_t, beta_t, eps, rms, s_t, z_t, bits, codes, ld_codes_bytes, row_sum, clear, st);
+}
+
+}  // namespace repq
+
+extern "C" repq_status repq_ln_quant(const void* x, int x_dtype, int64_t rows, int D, int64_t ldx,
+                                     const float* gamma_t, const float* beta_t, float eps, int norm_kind,
+                                     float s_t, int z_t, int bits, uint8_t* codes, int64_t ld_codes_bytes,
+                                     int32_t* row_sum, void* stream) {
+  return repq::launch_ln_quant(x, x_dtype, rows, D, ldx, gamma_t, beta_t, eps, norm_kind, s_t, z_t, bits, codes, ld_codes_bytes,
+                               row_sum, repq::ClearWords{}, static_cast<cudaStream_t>(stream));
 }

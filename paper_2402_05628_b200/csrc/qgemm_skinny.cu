@@ -349,7 +349,7 @@ repq_status make_map(CUtensorMap* map, const uint8_t* base, int64_t rows, int64_
 
 template <int OUT, int STEP>
 repq_status launch(dim3 grid, uint32_t smem, const CUtensorMap& map_w, const CUtensorMap& map_a, const SkinnyParams& P, cudaStream_t st) {
-  REPQ_CUDA(cudaFuncSetAttribute(qgemm_skinny_kernel<OUT, STEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemRing));
+  REPQ_TRY((allow_smem<qgemm_skinny_kernel<OUT, STEP>>(kSmemRing)));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(kThreads);

@@ -980,7 +980,7 @@ repq_status launch_tc_w(const CUtensorMap& map_a, const CUtensorMap& map_b, cons
     map_res = map_out;                                     // not read
   }
   const size_t smem = sizeof(SharedStorage<BN, RES, WP>);
-  REPQ_CUDA(cudaFuncSetAttribute(qgemm_tc_kernel<BN, OUT, RES, PAIR, WP>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+  REPQ_TRY((allow_smem<qgemm_tc_kernel<BN, OUT, RES, PAIR, WP>>(int(smem))));
   const int tiles = ((P.M + BM - 1) / BM) * ((P.N + BN - 1) / BN);
   const int grid = tiles < sms ? tiles : sms;
   REPQ_CUDA(launch_chained(qgemm_tc_kernel<BN, OUT, RES, PAIR, WP>, dim3(grid), dim3(kThreads), smem, st, map_a, map_b, map_out, map_res, P));

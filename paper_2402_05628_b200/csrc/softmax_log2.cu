@@ -388,8 +388,9 @@ repq_status launch(const T* scores, int64_t rows, int L, int64_t ld, bool vec_ok
       if (whole == kVPT - 1) plain = packed4(bits) ? softmax_log2_plain_kernel<T, TPR, kVPT, true, kVPT - 1> : softmax_log2_plain_kernel<T, TPR, kVPT, false, kVPT - 1>;
     }
     int fit = 0;
-    REPQ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, plain, kBlock, 0));
-    const int64_t most = int64_t(sm_count()) * (fit > 0 ? fit : 1);
+    static Residency memo[2][3];
+    REPQ_TRY(resident_blocks(memo[packed4(bits)][TPR > 64 ? 0 : whole == kVPT ? 1 : whole == kVPT - 1 ? 2 : 0], plain, kBlock, 0, &fit));
+    const int64_t most = int64_t(sm_count()) * fit;
     plain<<<int(need < most ? need : most), kBlock, 0, st>>>(scores, rows, L, ld, tail_half, c, log2_s, qmax, codes, ldc);
     REPQ_CUDA(cudaGetLastError());
     note_launch();
@@ -398,8 +399,9 @@ repq_status launch(const T* scores, int64_t rows, int L, int64_t ld, bool vec_ok
   auto kern = packed4(bits) ? softmax_log2_kernel<T, TPR, kVPT, true> : softmax_log2_kernel<T, TPR, kVPT, false>;
   // persistent grid: exactly the blocks that are resident at once (every block keeps its load pipeline running)
   int resident = 0;
-  REPQ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kern, kBlock, 0));
-  const int64_t cap = int64_t(sm_count()) * (resident > 0 ? resident : 1);
+  static Residency memo[2];
+  REPQ_TRY(resident_blocks(memo[packed4(bits)], kern, kBlock, 0, &resident));
+  const int64_t cap = int64_t(sm_count()) * resident;
   const int grid = int(need < cap ? need : cap);
   kern<<<grid, kBlock, 0, st>>>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, qmax, codes, ldc);
   REPQ_CUDA(cudaGetLastError());

@@ -16,8 +16,18 @@ import torch
 from . import binding as B
 
 
+class _Tracked:
+    """Counts assignments to public attributes of any instance, so that what was derived from them can be kept."""
+    changes = 0
+
+    def __setattr__(self, name, value):
+        object.__setattr__(self, name, value)
+        if not name.startswith("_"):
+            _Tracked.changes += 1
+
+
 @dataclasses.dataclass
-class PreparedLinear:
+class PreparedLinear(_Tracked):
     codes: torch.Tensor
     s_w: torch.Tensor
     z_w: torch.Tensor
@@ -38,7 +48,7 @@ def _pack_linear(W: np.ndarray, bias: np.ndarray, bits_w: int, dev) -> PreparedL
     return PreparedLinear(t(codes), t(s_w), t(z_w), t(wsum), t(np.asarray(bias, dtype=np.float32)))
 
 
-class QuantBlock:
+class QuantBlock(_Tracked):
     """Device-resident parameters of one block plus its workspace; `forward` runs the hot path."""
 
     def __init__(self, w, device="cuda:0", out_dtype: Optional[torch.dtype] = None, staged_attention: bool = False,
@@ -96,6 +106,7 @@ class QuantBlock:
         self._ws: Optional[torch.Tensor] = None
         self._staging = None
         self._batch = None
+        self._call = (None, None, None, None)
 
     def desc(self, batch: int) -> B.BlockDesc:
         c = self.cfg
@@ -135,6 +146,15 @@ class QuantBlock:
             self._batch = batch
         return self._ws
 
+    def _prepared(self, batch: int):
+        """Descriptor, parameters and workspace of a pass over `batch` items, kept from the pass before while nothing they
+        were made from has changed (building them takes longer than a small block runs)."""
+        # (attributes of blocks and layers by their assignments; the quantizer dict and the config may be edited in place)
+        key = (batch, _Tracked.changes, tuple(self.act_q.values()), tuple(self.cfg.values()))
+        if self._call[0] != key:
+            self._call = (key, self.desc(batch), self.params(), self.workspace(batch))
+        return self._call[1:]
+
     def forward(self, x: torch.Tensor, y: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
         """x: [batch * seq, dim] on the device, dtype = activation dtype of the config."""
         c = self.cfg
@@ -143,7 +163,8 @@ class QuantBlock:
         assert batch * c["L"] == x.shape[0]
         if y is None:
             y = torch.empty(x.shape, dtype=self.out_dtype, device=x.device)
-        B.repq_block_forward(self.desc(batch), self.params(), x, y, self.workspace(batch), stream)
+        d, p, ws = self._prepared(batch)
+        B.repq_block_forward(d, p, x, y, ws, stream)
         return y
 
     def forward_host(self, x_host: List[torch.Tensor], y_host: List[torch.Tensor], stream=None) -> None:
@@ -162,8 +183,8 @@ class QuantBlock:
         if self._staging is None or self._staging[0][0].shape[0] != rows:
             self._staging = ([torch.empty((rows, c["D"]), dtype=self.act_dtype, device=self.device) for _ in range(2)],
                              [torch.empty((rows, c["D"]), dtype=self.out_dtype, device=self.device) for _ in range(2)])
-        B.repq_block_forward_host(self.desc(batch), self.params(), x_host, y_host, self._staging[0], self._staging[1],
-                                  self.workspace(batch), stream)
+        d, p, ws = self._prepared(batch)
+        B.repq_block_forward_host(d, p, x_host, y_host, self._staging[0], self._staging[1], ws, stream)
 
     def forward_timed(self, x: torch.Tensor, y: torch.Tensor, stream=None) -> List[float]:
         """Same pass with per-stage CUDA-event timing (synchronises); returns milliseconds per stage."""
