@@ -1,0 +1,689 @@
+// Fused attention on integer codes, persistent form (quantizers of at most 7 bits): scores (Eq. 3 with quantized Q and K),
+// Softmax, log-sqrt2 codes (Eq. 15) and P.V with the reparameterized log2 de-quantization (Eqs. 16-17) in one kernel.
+// Scores and codes never leave the SM.  The code of a score depends on the row's final Softmax sum, so the keys are walked
+// twice, a visit being 64 keys (heads of up to 64 channels) or 128 keys (wider heads):
+//   pass 1   S = Q K^T per visit (tcgen05.mma on 8-bit operands into one of two slots of tensor memory), running row
+//            maximum m and sum Z = sum 2^(c (S - m))
+//   pass 2   S again, t = 2 (log2 Z + log2 s) - 2 c (S - m), code p = clip(round(t), 0, 2^b - 1), operand values
+//            2^(-ceil(p/2)) split by the parity of p into E and O, written back over the columns of tensor memory the
+//            scores came from, from where the P.V MMAs take their A operand; O = s s_v (acc_E + sqrt2 acc_O)
+//
+// What bounds it is instruction issue (some 3 instructions per score in pass 1, where ex2 alone takes 8 cycles of a
+// scheduler's special-function unit, and 4 to 6 in pass 2) as long as nothing is waited for, and a tile of 128 queries is
+// a long chain of latencies (launch, Q tile, first K tile, merge of the statistics, last MMA, stores) around only 8 visits
+// when rows have 197 keys.  Hence:
+//  - CTAs are persistent (two per SM for heads of up to 64 channels, one for wider heads) and walk their share of the
+//    tiles; K tiles stream in by bulk tensor copies across tile boundaries, the Q tile of the next tile is staged before
+//    the epilogue of the current one, so that the next tile's first S MMAs run under it;
+//  - a worker thread has one row (its tensor-memory lane) and 32 columns of every visit, which it loads at once: one
+//    barrier wait and one tensor-memory load per 32 scores, all of the warp's arithmetic independent behind it;
+//  - 4-bit codes of 4-bit values (scale s >= 1): the operands 2^(8 - ceil(p/2)) and v - z_v are 8-bit floats (e4m3), exact,
+//    so P.V runs at K = 32 per instruction, and the operand bytes of four keys are formed together in one register from
+//    q = 15 - p (odd q: E = 0x3C + 4 q, even q: O = 0x38 + 4 q) instead of a table look-up per key;
+//  - wider codes take their bf16 operand pair from a per-lane table in shared memory (one bank per lane).
+// Roles: worker warps, then a warp each (one lane) for the S MMAs, the P.V MMAs and the K copies.  Every mbarrier wait is
+// bounded; when one runs out the kernel records a status code, all roles leave their loops, MMAs and copies in flight are
+// drained, tensor memory is freed and the kernel returns.
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <math_constants.h>
+
+#include "attention_common.cuh"
+
+namespace repq {
+namespace attn {
+namespace {
+
+constexpr int kCols = 32;                       // S columns of a thread and visit
+
+template <int NB> struct Shape {
+  static constexpr int kKeys = NB == 1 ? 64 : 128;                  // keys per visit
+  static constexpr int kParts = kKeys / kCols;                      // threads that share a row
+  static constexpr int kWork = 4 * kParts;                          // worker warps
+  static constexpr int kWorkThreads = 32 * kWork;
+  static constexpr int kThreads = kWorkThreads + 96;
+  static constexpr int kCtas = NB == 1 ? 2 : 1;                     // resident per SM
+  static constexpr int kK = NB == 1 ? 3 : 4, kV = 2;                // ring depths
+  static constexpr int kTmem = 256 * NB;                            // 2 S slots + 2 accumulators
+};
+
+template <int NB, int kLutBits>
+struct PipeShared {
+  using Sh = Shape<NB>;
+  static constexpr uint32_t kKBytes = Sh::kKeys * 128;
+  static constexpr uint32_t kVBlockBytes = Sh::kKeys * 128;         // the visit's keys x 128 bytes (64 channels of bf16, or one row of bytes)
+  alignas(1024) uint8_t q[kQBytes];
+  alignas(1024) uint8_t k[Sh::kK][kKBytes];
+  alignas(1024) uint8_t v[Sh::kV][NB * kVBlockBytes];
+  float stat_m[Sh::kParts][kRows], stat_z[Sh::kParts][kRows];
+  static constexpr int kLutEntries = kLutBits ? (1 << kLutBits) + 1 : 1;
+  uint32_t lut[kLutEntries][32];                  // [code][lane] = E value | O value << 16; the last entry repeats the top code
+                                                  // (a clamp at 2^bits that rounds up lands there)
+  alignas(8) uint64_t k_full[Sh::kK];
+  uint64_t k_empty[Sh::kK], v_empty[Sh::kV];
+  uint64_t s_full[2], s_empty[2], s_spent[2], p_full[2];            // s_empty: read in pass 1; s_spent: P.V MMAs have read the operands
+  uint64_t q_full, acc_full, acc_empty, done_s, done_pv, merged[4];   // merged: statistics of a lane quarter's rows are there
+  uint32_t tmem_base;
+  volatile int abort;
+};
+
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr) : "memory");
+}
+// D[tmem] (+)= A[tmem] * B[smem], 8-bit floats, K = 32 (a 32-bit column of A holds four consecutive K elements)
+__device__ __forceinline__ void umma_f8_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ float fma_sat(float a, float b, float c) {       // fma clamped to [0, 1]
+  float d;
+  asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
+// Tile number `it` of CTA `cta` of `ctas`.  Under a causal mask the tiles are dealt longest first (every pair's last tile,
+// then every pair's tile before it, ...), forwards and backwards in turn, so that every CTA gets about the same work;
+// without a mask the tiles of a pair stay neighbours.
+struct Tile { int bo, bi, q0, k_end, nb; };
+template <int kKeys>
+__device__ __forceinline__ bool tile_at(const AttnParams& P, int it, int cta, int ctas, Tile& t) {
+  const int pos = it * ctas + (P.causal && (it & 1) ? ctas - 1 - cta : cta);
+  if (pos >= P.pairs * P.tiles) return false;
+  int pair, tile;
+  if (P.causal) {
+    const int slot = pos / P.pairs;
+    pair = pos - slot * P.pairs;
+    tile = P.tiles - 1 - slot;
+  } else {
+    pair = pos / P.tiles;
+    tile = pos - pair * P.tiles;
+  }
+  t.bo = pair / P.batch_inner;
+  t.bi = pair - t.bo * P.batch_inner;
+  t.q0 = tile * kRows;
+  t.k_end = P.causal ? max(1, min(P.Lk, min(t.q0 + kRows, P.Lq) + P.Lk - P.Lq)) : P.Lk;
+  t.nb = (t.k_end + kKeys - 1) / kKeys;
+  return true;
+}
+
+// kLutBits: width of the table of operand pairs (4, 6, 8; P.V in bf16), or 0: 4-bit codes of 4-bit values, P.V in 8-bit
+// floats.  kF8: 4-bit Q / K codes read as 8-bit floats (a byte below 16 is the e4m3 number byte * 2^-9; the accumulator holds
+// 2^-18 sum (q - z_q) k as a float, exactly); otherwise signed x unsigned bytes.
+template <int NB, int kLutBits, bool kF8>
+__global__ void __launch_bounds__(Shape<NB>::kThreads, Shape<NB>::kCtas)
+attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ AttnParams P) {
+  using Sh = Shape<NB>;
+  using Shared = PipeShared<NB, kLutBits>;
+  constexpr int kKeys = Sh::kKeys, kWork = Sh::kWork, kParts = Sh::kParts, kT = Sh::kWorkThreads, kK = Sh::kK, kV = Sh::kV;
+  constexpr bool kLut = kLutBits != 0;
+  constexpr int kAccCol = 2 * kKeys;
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  Shared& S = *reinterpret_cast<Shared*>(smem_raw);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ksteps = (P.dh + 31) >> 5;                    // S MMAs of K = 32 per visit
+  const int pieces = P.dh >> 4;                           // 16-byte pieces of a Q / K row
+
+  if (tid == 0) {
+    for (int s = 0; s < kK; ++s) { mbar_init(smem_u32(&S.k_full[s]), 1); mbar_init(smem_u32(&S.k_empty[s]), 1); }
+    for (int s = 0; s < kV; ++s) mbar_init(smem_u32(&S.v_empty[s]), 1);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(smem_u32(&S.s_full[s]), 1);
+      mbar_init(smem_u32(&S.s_empty[s]), kWork);
+      mbar_init(smem_u32(&S.s_spent[s]), 1);
+      mbar_init(smem_u32(&S.p_full[s]), kWork);
+    }
+    mbar_init(smem_u32(&S.q_full), kWork);
+    mbar_init(smem_u32(&S.acc_full), 1);
+    for (int s = 0; s < 4; ++s) mbar_init(smem_u32(&S.merged[s]), kParts);
+    mbar_init(smem_u32(&S.acc_empty), kWork);
+    mbar_init(smem_u32(&S.done_s), 1);
+    mbar_init(smem_u32(&S.done_pv), 1);
+    S.abort = 0;
+    if (smem_u32(smem_raw) & 1023u) {                     // the swizzled tiles need this alignment
+      atomicCAS(P.status, 0, 49);
+      S.abort = 1;
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == kWork) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.tmem_base)), "n"(Sh::kTmem) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (kLut && warp < kWork) {
+    for (int i = tid; i < Shared::kLutEntries * 32; i += kT) {
+      const uint32_t code = min(uint32_t(i >> 5), uint32_t(Shared::kLutEntries - 2)), kk = (code + 1u) >> 1;
+      const uint32_t bits16 = kk > 126u ? 0u : (127u - kk) << 7;   // bf16 bits of 2^-ceil(code/2) (0 below the normal range)
+      S.lut[0][i] = (code & 1u) ? bits16 << 16 : bits16;
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = S.tmem_base;
+  volatile int* abort = &S.abort;
+  // everything above touched no global memory of the kernel chain
+  grid_dependency_wait();
+  grid_dependency_trigger();
+
+  Tile t;
+  if (warp == kWork) {
+    // ---------------------------------------------------------------- S MMAs
+    if (lane == 0) {
+      // D = s32 from signed x unsigned bytes, or D = f32 from e4m3 x e4m3; both K-major, M = 128, N = the visit's keys
+      constexpr uint32_t idesc = (kF8 ? (1u << 4) : (2u << 4) | (1u << 7)) | (uint32_t(kKeys >> 3) << 17) | (uint32_t(kRows >> 4) << 24);
+      const uint64_t dq = smem_desc_sw128(smem_u32(S.q));
+      int g = 0;                                          // visits, over both passes and all tiles
+      // a bit per slot: parity of the hand-backs waited for, whether the slot has been used, and by which pass last
+      uint32_t ph_empty = 0, ph_spent = 0, used = 0, pass2 = 0;
+      uint32_t ks = 0, kp = 0;                            // K ring: slot and parity
+      bool ok = true;
+      for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
+        if (!(ok = mbar_wait(smem_u32(&S.q_full), it & 1, abort, 40, P.status))) break;
+#pragma unroll 1
+        for (int b = 0; b < 2 * t.nb; ++b, ++g) {
+          const int slot = g & 1;
+          if (!(ok = mbar_wait(smem_u32(&S.k_full[ks]), kp, abort, 41, P.status))) break;
+          const uint32_t bit = 1u << slot;
+          if (used & bit) {
+            if (pass2 & bit) {
+              if (!(ok = mbar_wait(smem_u32(&S.s_spent[slot]), (ph_spent >> slot) & 1u, abort, 42, P.status))) break;
+              ph_spent ^= bit;
+            } else {
+              if (!(ok = mbar_wait(smem_u32(&S.s_empty[slot]), (ph_empty >> slot) & 1u, abort, 42, P.status))) break;
+              ph_empty ^= bit;
+            }
+          }
+          tc_fence_after();
+          const uint64_t dk = smem_desc_sw128(smem_u32(S.k[ks]));
+          for (int s = 0; s < ksteps; ++s) {
+            if (kF8) umma_f8(tmem_base + uint32_t(slot * kKeys), dq + uint64_t(2 * s), dk + uint64_t(2 * s), idesc, s != 0 ? 1u : 0u);
+            else umma_i8(tmem_base + uint32_t(slot * kKeys), dq + uint64_t(2 * s), dk + uint64_t(2 * s), idesc, s != 0 ? 1u : 0u);
+          }
+          umma_commit(smem_u32(&S.s_full[slot]));
+          umma_commit(smem_u32(&S.k_empty[ks]));
+          used |= bit;
+          pass2 = b >= t.nb ? pass2 | bit : pass2 & ~bit;
+          if (++ks == kK) { ks = 0; kp ^= 1u; }
+        }
+      }
+      umma_commit(smem_u32(&S.done_s));
+      mbar_drain(smem_u32(&S.done_s), 0);
+    }
+  } else if (warp == kWork + 1) {
+    // ---------------------------------------------------------------- P.V MMAs
+    if (lane == 0) {
+      // D = f32, A (tensor memory) and B = bf16 or e4m3, B MN-major, N = n_pad, M = 128
+      const uint32_t idesc = (kLut ? (1u << 4) | (1u << 7) | (1u << 10) : (1u << 4)) | (1u << 16) | (uint32_t(P.n_pad >> 3) << 17) |
+                             (uint32_t(kRows >> 4) << 24);
+      constexpr int kStep = kLut ? 16 : 32;               // keys per MMA
+      int g = 0;
+      uint32_t ph_p = 0, vs = 0;
+      bool ok = true;
+      for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
+        g += t.nb;
+        if (it > 0 && !(ok = mbar_wait(smem_u32(&S.acc_empty), (it - 1) & 1, abort, 50, P.status))) break;
+#pragma unroll 1
+        for (int j = 0; j < t.nb; ++j, ++g) {
+          const int slot = g & 1;
+          if (!(ok = mbar_wait(smem_u32(&S.p_full[slot]), (ph_p >> slot) & 1u, abort, 43, P.status))) break;
+          ph_p ^= 1u << slot;
+          tc_fence_after();
+          const uint64_t dv = smem_desc_sw128(smem_u32(S.v[vs]), Shared::kVBlockBytes);
+          const int steps = (min(kKeys, t.k_end - j * kKeys) + kStep - 1) / kStep;
+          const uint32_t a_base = tmem_base + uint32_t(slot * kKeys);
+          for (int s = 0; s < steps; ++s) {
+            const uint32_t accumulate = (j | s) != 0 ? 1u : 0u;
+            const uint64_t b = dv + uint64_t(kStep * 128 / 16 * s);
+            const uint32_t a_e = a_base + uint32_t(kStep * s);     // E words first, then as many O words
+            if (kLut) {
+              umma_f16_ts(tmem_base + uint32_t(kAccCol), a_e, b, idesc, accumulate);
+              umma_f16_ts(tmem_base + uint32_t(kAccCol + P.n_pad), a_e + 8u, b, idesc, accumulate);
+            } else {
+              umma_f8_ts(tmem_base + uint32_t(kAccCol), a_e, b, idesc, accumulate);
+              umma_f8_ts(tmem_base + uint32_t(kAccCol + P.n_pad), a_e + 8u, b, idesc, accumulate);
+            }
+          }
+          umma_commit(smem_u32(&S.s_spent[slot]));
+          umma_commit(smem_u32(&S.v_empty[vs]));
+          if (++vs == kV) vs = 0;
+        }
+        if (ok) umma_commit(smem_u32(&S.acc_full));
+      }
+      umma_commit(smem_u32(&S.done_pv));
+      mbar_drain(smem_u32(&S.done_pv), 0);
+    }
+  } else if (warp == kWork + 2) {
+    // ---------------------------------------------------------------- K tiles by bulk tensor copies
+    if (lane == 0) {
+      uint32_t ks = 0, kp = 0;
+      int issued = 0;
+      bool ok = true;
+      for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
+#pragma unroll 1
+        for (int b = 0; b < 2 * t.nb; ++b) {
+          if (!(ok = mbar_wait(smem_u32(&S.k_empty[ks]), kp ^ 1u, abort, 48, P.status))) break;
+          const uint32_t bar = smem_u32(&S.k_full[ks]);
+          mbar_expect_tx(bar, Shared::kKBytes);
+          // box: 128 bytes of the head's row (bytes past d_h meet zero bytes of the Q tile), the visit's keys (rows past Lk
+          // are zero-filled), one batch item
+          tma_load_3d(smem_u32(S.k[ks]), &map_k, bar, t.bi * int(P.k_si), (b < t.nb ? b : b - t.nb) * kKeys, t.bo);
+          ++issued;
+          if (++ks == kK) { ks = 0; kp ^= 1u; }
+        }
+      }
+      // the copies issued last must have landed before this CTA may exit
+      for (int i = issued < kK ? issued : kK; i > 0; --i) {
+        if (ks == 0) { ks = kK - 1; kp ^= 1u; } else { --ks; }
+        mbar_drain(smem_u32(&S.k_full[ks]), kp);
+      }
+    }
+  } else {
+    // ---------------------------------------------------------------- Softmax arithmetic, V tiles, epilogue
+    const int quarter = warp & 3, part = warp >> 2;
+    const int r = quarter * 32 + lane;                    // the thread's row inside the tile = its tensor-memory lane
+    const float c = 1.4426950408889634f;
+    const float magic = __uint_as_float(kMagicBits);
+    const uint32_t taddr_s = tmem_base + (uint32_t(quarter * 32) << 16) + uint32_t(part * kCols);
+    const uint32_t lut_addr = smem_u32(&S.lut[0][lane]) - (kMagicBits << 7);
+
+    // ---- Q tile: q - z_q as signed bytes (kF8: sign and magnitude); 4 threads per row (8 when there are 512 workers),
+    // 32 (16) bytes each; the pieces of a tile are requested first and written once the tile before is through its S MMAs
+    constexpr int kQPer = kT == 256 ? 4 : 2;              // pieces per thread: rows of 8 pieces, kT threads
+    const int qrow = tid / (8 / kQPer), qp0 = (tid % (8 / kQPer)) * kQPer;
+    const uint32_t zq4 = uint32_t(P.zq) * 0x01010101u;
+    uint4 qreg[kQPer];
+    auto fetch_q = [&](const Tile& n) {
+      const uint8_t* row = P.q + n.bo * P.q_so + n.bi * P.q_si + int64_t(n.q0 + qrow) * P.ldq;
+#pragma unroll
+      for (int i = 0; i < kQPer; ++i) {
+        qreg[i] = make_uint4(zq4, zq4, zq4, zq4);
+        if (n.q0 + qrow < P.Lq && qp0 + i < pieces) qreg[i] = __ldg(reinterpret_cast<const uint4*>(row) + qp0 + i);
+      }
+    };
+    auto stage_q = [&]() {
+#pragma unroll
+      for (int i = 0; i < kQPer; ++i) {
+        uint4 w = sub_bytes(qreg[i], zq4);
+        if (kF8) w = sign_magnitude(w);
+        if (qp0 + i < 2 * ksteps) *reinterpret_cast<uint4*>(S.q + tile_offset(qrow, qp0 + i)) = w;
+      }
+      fence_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&S.q_full));
+    };
+
+    // ---- V tile of a visit.  8-bit floats: a thread has one key and 16 channels, v - z_v in sign and magnitude.  bf16: a
+    // thread keeps its group of 8 channels and moves down the keys, 32 per step.
+    constexpr int kVItems = kLut ? kKeys / 32 : 1;
+    const int v_g = kLut ? tid % (8 * NB) : tid & 3, v_key0 = kLut ? tid / (8 * NB) : tid >> 2;
+    const bool v_live = v_g * (kLut ? 8 : 16) < P.dh;
+    const uint32_t v_off = kLut ? uint32_t(v_g >> 3) * Shared::kVBlockBytes + tile_offset(v_key0, v_g & 7) : tile_offset(v_key0, v_g);
+    const uint32_t zv4 = uint32_t(P.z_v) * 0x01010101u;
+    const float vz = magic + float(P.z_v);
+    const __nv_bfloat162 vz2 = __float2bfloat162_rn(128.f + float(P.z_v));
+    const uint8_t* v_ptr = nullptr;
+    uint4 v16;
+    uint2 vraw[kVItems];
+    auto fetch_v = [&](int block) {
+      if constexpr (!kLut) {
+        v16 = make_uint4(zv4, zv4, zv4, zv4);
+        const int key = block * kKeys + v_key0;
+        if (v_live && key < t.k_end) v16 = __ldg(reinterpret_cast<const uint4*>(v_ptr + int64_t(block * kKeys) * P.ldv));
+      } else {
+#pragma unroll
+        for (int i = 0; i < kVItems; ++i) {
+          vraw[i] = make_uint2(0u, 0u);
+          const int key = block * kKeys + v_key0 + i * 32;
+          if (v_live && key < t.k_end) vraw[i] = __ldg(reinterpret_cast<const uint2*>(v_ptr + int64_t(block * kKeys + i * 32) * P.ldv));
+        }
+      }
+    };
+    auto stage_v = [&](int block, uint8_t* tile) {
+      if constexpr (!kLut) {
+        *reinterpret_cast<uint4*>(tile + v_off) = sign_magnitude(sub_bytes(v16, zv4));
+      } else {
+#pragma unroll
+        for (int i = 0; i < kVItems; ++i) {
+          uint32_t o4[4] = {0u, 0u, 0u, 0u};
+          if (v_live && block * kKeys + v_key0 + i * 32 < t.k_end) {
+            const uint32_t b03 = vraw[i].x, b47 = vraw[i].y;
+            if (P.v_small) {
+              // v - z_v as bf16: for codes below 128, 128 + v is the bit pattern 0x4300 | v and the bf16 subtraction exact
+              const uint32_t w[4] = {__byte_perm(b03, 0x43434343u, 0x4140), __byte_perm(b03, 0x43434343u, 0x4342),
+                                     __byte_perm(b47, 0x43434343u, 0x4140), __byte_perm(b47, 0x43434343u, 0x4342)};
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const __nv_bfloat162 hh = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&w[e]), vz2);
+                o4[e] = *reinterpret_cast<const uint32_t*>(&hh);
+              }
+            } else {
+              float f[8];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                f[e] = __uint_as_float(__byte_perm(b03, kMagicBits, 0x7650 + e)) - vz;
+                f[4 + e] = __uint_as_float(__byte_perm(b47, kMagicBits, 0x7650 + e)) - vz;
+              }
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const __nv_bfloat162 hh = __floats2bfloat162_rn(f[2 * e], f[2 * e + 1]);
+                o4[e] = *reinterpret_cast<const uint32_t*>(&hh);
+              }
+            }
+          }
+          *reinterpret_cast<uint4*>(tile + v_off + uint32_t(i) * 4096u) = make_uint4(o4[0], o4[1], o4[2], o4[3]);
+        }
+      }
+    };
+
+    // The thread's 32 scores of the visit in `slot`, in units of the score scale, as floats: the accumulators themselves
+    // (kF8) or converted.
+    auto load_scores = [&](int slot, float (&sf)[kCols]) {
+      uint32_t rn[kCols];
+      __syncwarp();
+      tmem_ld32(taddr_s + uint32_t(slot * kKeys), rn);
+      tmem_ld_wait();
+#pragma unroll
+      for (int e = 0; e < kCols; ++e) sf[e] = kF8 ? __uint_as_float(rn[e]) : float(int32_t(rn[e]));
+    };
+
+    float m = -CUDART_INF_F, z = 0.f;       // running maximum (in units of the score scale) and sum of this thread's columns
+    const float sc = P.scale * c;           // exponent of 2 per unit
+    // `seen`: columns e < seen are keys the row sees
+    auto stats = [&](const float (&sf)[kCols], int seen) {
+      if (__builtin_expect(seen >= kCols, 1)) {
+        float b0 = max3(sf[0], sf[1], sf[2]), b1 = max3(sf[3], sf[4], sf[5]);
+#pragma unroll
+        for (int e = 6; e + 3 < kCols; e += 4) { b0 = max3(b0, sf[e], sf[e + 1]); b1 = max3(b1, sf[e + 2], sf[e + 3]); }
+        const float mn = fmaxf(max3(m, b0, b1), fmaxf(sf[kCols - 2], sf[kCols - 1]));
+        const f32x2 sc2 = splat2(sc), nm2 = splat2(-(mn * sc));
+        f32x2 acc[2] = {0ull, 0ull};
+#pragma unroll
+        for (int e = 0; e < kCols; e += 2) {
+          float a0, a1;
+          unpack2(fma2(pack2(sf[e], sf[e + 1]), sc2, nm2), a0, a1);
+          acc[(e >> 1) & 1] = add2(acc[(e >> 1) & 1], pack2(ex2(a0), ex2(a1)));
+        }
+        float z0, z1;
+        unpack2(add2(acc[0], acc[1]), z0, z1);
+        z = z * ex2((m - mn) * sc) + (z0 + z1);        // m = -inf at first: factor 0
+        m = mn;
+      } else if (seen > 0) {
+        float bm = sf[0];
+#pragma unroll
+        for (int e = 1; e < kCols; ++e)
+          if (e < seen) bm = fmaxf(bm, sf[e]);
+        const float mn = fmaxf(m, bm), nm = -(mn * sc);
+        float acc = 0.f;
+#pragma unroll
+        for (int e = 0; e < kCols; ++e)
+          if (e < seen) acc += ex2(fmaf(sf[e], sc, nm));
+        z = z * ex2((m - mn) * sc) + acc;
+        m = mn;
+      }
+    };
+
+    float w1 = 0.f, w0 = 0.f;               // pass 2: value handed to the saturating fma is w1 (sf - m) + w0
+    // Codes and operand words of the thread's 32 columns, stored over the columns the scores came from.
+    auto codes = [&](const float (&sf)[kCols], int seen, uint32_t taddr) {
+      const f32x2 nm2 = splat2(-m), magic2 = splat2(magic);
+      if constexpr (!kLut) {
+        // q = 15 - p = round(16 sat((15 - t) / 16)): t >= 0 (Z >= 1 and s >= 1), so only the lower end is clipped
+        const f32x2 steps2 = splat2(16.f);
+        uint32_t eo[16];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          uint32_t u[4];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            float d0, d1, u0, u1;
+            unpack2(add2(pack2(sf[4 * i + 2 * h], sf[4 * i + 2 * h + 1]), nm2), d0, d1);
+            unpack2(fma2(pack2(fma_sat(d0, w1, w0), fma_sat(d1, w1, w0)), steps2, magic2), u0, u1);
+            u[2 * h] = __float_as_uint(u0);
+            u[2 * h + 1] = __float_as_uint(u1);
+          }
+          const uint32_t q = __byte_perm(__byte_perm(u[0], u[1], 0x0040), __byte_perm(u[2], u[3], 0x0040), 0x5410);
+          const uint32_t odd = q & 0x01010101u, even_key = odd * 0xFFu;       // odd q: even p
+          const uint32_t val = (q + odd) * 4u + 0x38383838u;
+          eo[i] = val & even_key;
+          eo[8 + i] = val & ~even_key;
+        }
+        if (__builtin_expect(seen < kCols, 0)) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int n = seen - 4 * i;
+            const uint32_t keep = n >= 4 ? 0xFFFFFFFFu : n > 0 ? (1u << (8 * n)) - 1u : 0u;
+            eo[i] &= keep;
+            eo[8 + i] &= keep;
+          }
+        }
+        __syncwarp();
+        tmem_st16(taddr, eo);
+      } else {
+        constexpr float kSteps = float(1 << kLutBits);
+        const f32x2 steps2 = splat2(kSteps);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          uint32_t eo[16], eow[16];
+#pragma unroll
+          for (int e = 0; e < 16; e += 2) {
+            float d0, d1, u0, u1;
+            unpack2(add2(pack2(sf[16 * h + e], sf[16 * h + e + 1]), nm2), d0, d1);
+            unpack2(fma2(pack2(fma_sat(d0, w1, w0), fma_sat(d1, w1, w0)), steps2, magic2), u0, u1);
+            asm("ld.shared.u32 %0, [%1];" : "=r"(eo[e]) : "r"(lut_addr + (__float_as_uint(u0) << 7)));
+            asm("ld.shared.u32 %0, [%1];" : "=r"(eo[e + 1]) : "r"(lut_addr + (__float_as_uint(u1) << 7)));
+          }
+          if (__builtin_expect(seen < 16 * h + 16, 0)) {
+#pragma unroll
+            for (int e = 0; e < 16; ++e)
+              if (16 * h + e >= seen) eo[e] = 0u;
+          }
+          // E pairs (even key in the low half) in words 0..7, O pairs in words 8..15
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            eow[e] = __byte_perm(eo[2 * e], eo[2 * e + 1], 0x5410);
+            eow[8 + e] = __byte_perm(eo[2 * e], eo[2 * e + 1], 0x7632);
+          }
+          __syncwarp();
+          tmem_st16(taddr + uint32_t(16 * h), eow);
+        }
+      }
+    };
+
+    bool ok = true, more = tile_at<kKeys>(P, 0, blockIdx.x, gridDim.x, t);
+    int g = 0, jv = 0;                                    // visits and V tiles, over all tiles
+    if (more) { fetch_q(t); stage_q(); }
+    for (int it = 0; more && !*abort; ++it) {
+      const int row = t.q0 + r;
+      const int valid = row < P.Lq ? (P.causal ? max(1, min(P.Lk, row + 1 + P.Lk - P.Lq)) : P.Lk) : 0;   // keys the row sees
+      const int most = __reduce_max_sync(0xffffffffu, valid);                                             // ... any row of the warp
+      v_ptr = P.v + t.bo * P.v_so + t.bi * P.v_si + int64_t(v_key0) * P.ldv + v_g * (kLut ? 8 : 16);
+      fetch_v(0);
+      m = -CUDART_INF_F;
+      z = 0.f;
+      // ---- pass 1
+      for (int b = 0; b < t.nb; ++b, ++g) {
+        const int slot = g & 1, first = b * kKeys + part * kCols;
+        if (!mbar_wait(smem_u32(&S.s_full[slot]), (g >> 1) & 1, abort, 44, P.status)) { ok = false; break; }
+        if (first < most) {                               // (warps whose columns no row sees only hand the slot back)
+          tc_fence_after();
+          float sf[kCols];
+          load_scores(slot, sf);
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&S.s_empty[slot]));
+          stats(sf, valid - first);
+        } else if (lane == 0) {
+          mbar_arrive(smem_u32(&S.s_empty[slot]));
+        }
+      }
+      if (!ok || *abort) break;
+      // merge the column parts of every row: m = max, Z = sum of the rescaled partial sums (same order in every thread of
+      // the row, so that all of them hold the same Z)
+      S.stat_m[part][r] = m;
+      S.stat_z[part][r] = z;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&S.merged[quarter]));
+      if (!mbar_wait(smem_u32(&S.merged[quarter]), it & 1, abort, 45, P.status)) break;
+      float zt = 0.f;
+#pragma unroll
+      for (int q = 0; q < kParts; ++q) m = fmaxf(m, S.stat_m[q][r]);
+#pragma unroll
+      for (int q = 0; q < kParts; ++q) {
+        const float mq = S.stat_m[q][r];
+        if (mq > -CUDART_INF_F) zt += S.stat_z[q][r] * ex2((mq - m) * sc);
+      }
+      {
+        const float k0 = 2.f * (log2f(zt) + P.log2_s);
+        if (kLut) {
+          constexpr float kInv = 1.f / float(1 << (kLut ? kLutBits : 4));
+          w1 = -2.f * sc * kInv;
+          w0 = k0 * kInv;
+        } else {
+          w1 = 2.f * sc * 0.0625f;
+          w0 = (15.f - k0) * 0.0625f;
+        }
+      }
+      // ---- pass 2
+      for (int j = 0; j < t.nb; ++j, ++g, ++jv) {
+        const int slot = g & 1, first = j * kKeys + part * kCols, pb = jv % kV;
+        if (!mbar_wait(smem_u32(&S.v_empty[pb]), ((jv / kV) & 1) ^ 1, abort, 46, P.status)) { ok = false; break; }
+        stage_v(j, S.v[pb]);
+        if (j + 1 < t.nb) fetch_v(j + 1);
+        fence_async_smem();
+        if (!mbar_wait(smem_u32(&S.s_full[slot]), (g >> 1) & 1, abort, 44, P.status)) { ok = false; break; }
+        // columns past the visit's last key are read by the MMAs only inside the step that holds it
+        if (first < t.k_end) {
+          tc_fence_after();
+          const uint32_t taddr = taddr_s + uint32_t(slot * kKeys);
+          if (first < most) {
+            float sf[kCols];
+            load_scores(slot, sf);
+            codes(sf, valid - first, taddr);
+          } else {
+            const uint32_t zero[16] = {};
+            __syncwarp();
+            tmem_st16(taddr, zero);
+            if (kLut) tmem_st16(taddr + 16u, zero);
+          }
+          tmem_st_wait();
+          tc_fence_before();
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&S.p_full[slot]));
+      }
+      if (!ok || *abort) break;
+
+      // ---- the next tile's Q (every S MMA of this tile has completed), then the epilogue: one row per thread, the 16-column
+      // chunks of the accumulators dealt to the parts of a row
+      const Tile cur = t;
+      more = tile_at<kKeys>(P, it + 1, blockIdx.x, gridDim.x, t);
+      if (more) fetch_q(t);
+      if (more) stage_q();
+      if (!mbar_wait(smem_u32(&S.acc_full), it & 1, abort, 47, P.status)) break;
+      tc_fence_after();
+      const float out_scale = kLut ? P.out_scale : 2.f * P.out_scale;   // 8-bit floats: 2^8 A times 2^-9 (v - z_v)
+      const uint32_t taddr = tmem_base + (uint32_t(quarter * 32) << 16) + uint32_t(kAccCol);
+      constexpr int kChunks = NB * 4 / kParts;            // chunks per thread for the widest head
+      float v[kChunks][16];
+#pragma unroll
+      for (int i = 0; i < kChunks; ++i) {
+        const int c0 = (part + i * kParts) * 16;
+        if (c0 < P.dh) {
+          uint32_t re[16], ro[16];
+          __syncwarp();
+          tmem_ld16(taddr + uint32_t(c0), re);
+          tmem_ld16(taddr + uint32_t(P.n_pad + c0), ro);
+          tmem_ld_wait();
+#pragma unroll
+          for (int e = 0; e < 16; ++e)
+            v[i][e] = out_scale * fmaf(1.41421356237309504880f, __uint_as_float(ro[e]), __uint_as_float(re[e]));
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&S.acc_empty));
+      if (row < P.Lq) {
+        int code_sum = 0;
+        const int64_t roff = cur.bo * P.o_so + cur.bi * P.o_si + int64_t(row) * P.ldo;
+#pragma unroll
+        for (int i = 0; i < kChunks; ++i) {
+          const int c0 = (part + i * kParts) * 16;
+          if (c0 < P.dh) store_values(P, v[i], roff, c0, code_sum);
+        }
+        if (P.out_row_sum != nullptr && P.out_kind == REPQ_OUT_CODES && part * 16 < P.dh)
+          atomicAdd(P.out_row_sum + int64_t(cur.bo) * P.Lq + row, code_sum);
+      }
+    }
+  }
+
+  // ------------------------------------------------------------------ teardown
+  if (warp < kWork) tmem_st_wait();               // an error path may leave a tensor-memory store in flight
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kWork) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(Sh::kTmem) : "memory");
+  }
+}
+
+template <int NB, int kLutBits, bool kF8>
+repq_status launch_kernel(const AttnParams& P, int64_t pairs, cudaStream_t st) {
+  using Sh = Shape<NB>;
+  constexpr size_t smem = sizeof(PipeShared<NB, kLutBits>);
+  static_assert(smem <= (NB == 1 ? 113 : 227) * 1024, "shared storage exceeds a CTA's share");
+  REPQ_TRY((allow_smem<attention_pipe_kernel<NB, kLutBits, kF8>>(int(smem))));
+  AttnParams Q = P;
+  Q.pairs = int(pairs);
+  Q.tiles = (P.Lq + kRows - 1) / kRows;
+  if (kF8) Q.scale = P.scale * 262144.f;                  // the accumulators hold 2^-18 sum (q - z_q) k
+  CUtensorMap map_k;
+  REPQ_TRY(make_k_map(&map_k, P, int(pairs / P.batch_inner), Sh::kKeys));
+  const int64_t tiles = int64_t(Q.tiles) * pairs, slots = int64_t(sm_count()) * Sh::kCtas;
+  const dim3 grid{unsigned(tiles < slots ? tiles : slots)};
+  REPQ_CUDA(launch_chained(attention_pipe_kernel<NB, kLutBits, kF8>, grid, dim3(Sh::kThreads), smem, st, map_k, Q));
+  note_launch();
+  return REPQ_OK;
+}
+
+template <bool kF8>
+repq_status launch_form(const AttnParams& P, int64_t pairs, bool small_v, cudaStream_t st) {
+  if (P.dh <= 64) {
+    // 4-bit codes of 4-bit values: P.V in 8-bit floats (V rows by 16-byte loads; s >= 1 keeps t >= 0)
+    if (P.qmax_p <= 15)
+      return small_v && P.log2_s >= 0.f ? launch_kernel<1, 0, kF8>(P, pairs, st) : launch_kernel<1, 4, kF8>(P, pairs, st);
+    if (P.qmax_p <= 63) return launch_kernel<1, 6, kF8>(P, pairs, st);
+    return launch_kernel<1, 8, kF8>(P, pairs, st);
+  }
+  if (P.qmax_p <= 15) return launch_kernel<2, 4, kF8>(P, pairs, st);
+  if (P.qmax_p <= 63) return launch_kernel<2, 6, kF8>(P, pairs, st);
+  return launch_kernel<2, 8, kF8>(P, pairs, st);
+}
+
+}  // namespace
+
+// q - z_q as signed bytes (codes and zero points below 128) and row and batch strides of K usable as tensor-map strides
+bool pipe_supported(const AttnParams& P, int qmax_qk) {
+  return qmax_qk < 128 && P.zq >= 0 && P.zq < 128 && P.zk >= 0 && P.zk < 128 && P.k_so > 0 && P.ldk < (int64_t(1) << 40) &&
+         P.k_so < (int64_t(1) << 40) && int64_t(P.batch_inner - 1) * P.k_si + P.dh <= P.ldk;
+}
+
+repq_status launch_pipe(const AttnParams& P, int64_t pairs, int qmax_qk, cudaStream_t st) {
+  // 4-bit quantizers with the zero point of Q inside the code range: the tiles are also valid 8-bit floats
+  const bool f8 = qmax_qk <= 15 && P.zq <= 15 && !P.no_f8;
+  const bool small_v = qmax_qk <= 15 && P.z_v >= 0 && P.z_v <= 15 && aligned(P.v, 16) && P.ldv % 16 == 0 && P.v_so % 16 == 0 && P.v_si % 16 == 0;
+  return f8 ? launch_form<true>(P, pairs, small_v, st) : launch_form<false>(P, pairs, small_v, st);
+}
+
+}  // namespace attn
+}  // namespace repq

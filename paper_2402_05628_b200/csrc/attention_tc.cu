@@ -40,16 +40,13 @@
 
 #include <cstdlib>
 
-#include "f32x2.cuh"
-#include "kernels.h"
-#include "tc_ptx.cuh"
+#include "attention_common.cuh"
 
 namespace repq {
 namespace {
 
-using namespace tc;
+using namespace attn;
 
-constexpr int kRows = 128;                  // query rows per CTA (MMA M)
 // keys per visit: 64 for heads of up to 64 channels (two CTAs per SM, 256 tensor-memory columns each), 128 for wider
 // heads (one CTA per SM): a tensor-core instruction costs about the same time whether it covers 64 or 128 keys
 template <int NB> struct VisitKeys { static constexpr int value = NB == 1 ? 64 : 128; };
@@ -61,28 +58,6 @@ constexpr int kCols = 16;                     // S columns per tensor-memory loa
 constexpr int kWorkThreads = 32 * kWorkWarps;
 // + S-MMA warp + K-copy warp, and for wide heads a P.V-MMA warp of its own (its waits then do not hold up the S MMAs)
 template <int NB> struct Threads { static constexpr int value = kWorkThreads + (NB == 1 ? 64 : 96); };
-constexpr uint32_t kQBytes = kRows * 128;         // Q tile: rows of 128 bytes (the head's codes, zero-padded)
-constexpr uint32_t kMagicBits = 0x4B400000u;      // float 1.5 * 2^23
-
-struct AttnParams {
-  const uint8_t* q; const uint8_t* k; const uint8_t* v;
-  int64_t ldq, ldk, ldv, q_so, q_si, k_so, k_si, v_so, v_si;
-  int Lq, Lk, dh, batch_inner, causal;
-  float scale;            // alpha s_q s_k
-  int zq, zk;
-  float log2_s;           // log2 of the log-sqrt2 scale
-  int qmax_p;             // 2^bits_p - 1
-  int z_v, v_small;
-  float out_scale;        // s_p s_v
-  int out_kind, qmax, pack4;
-  float inv_so; int zo;
-  void* out; int64_t ldo, o_so, o_si;
-  int32_t* out_row_sum;
-  int n_pad, tmem_cols, vec_store;
-  int no_f8;                                         // keep integer scores where the 8-bit float form would apply
-  int pairs, tiles;                                  // (batch, head) pairs and query tiles of 128 rows: the grid is their product
-  int32_t* status;
-};
 
 // Ring depths.  S: one slot of tensor memory per worker group (2 x 64 or 2 x 128 columns beside the accumulators' 2 x 64
 // or 2 x 128).  Heads of up to 64 channels run two CTAs per SM: two K tiles, one V stage.  Wider heads have the SM to
@@ -113,34 +88,6 @@ struct AttnShared {
   uint32_t tmem_base;
   volatile int abort;
 };
-
-__device__ __forceinline__ uint32_t tile_offset(int row, int piece) {
-  return uint32_t(row >> 3) * 1024u + uint32_t(row & 7) * 128u + (uint32_t(piece ^ (row & 7)) << 4);
-}
-__device__ __forceinline__ int sum_bytes(const uint4& v) {
-  return __dp4a(v.x, 0x01010101u, __dp4a(v.y, 0x01010101u, __dp4a(v.z, 0x01010101u, __dp4a(v.w, 0x01010101u, 0u))));
-}
-// Bytewise c - z (two's complement) for codes and zero points below 128: with the top bit of every byte of c set
-// no borrow crosses a byte, and flipping that bit back leaves c - z mod 256.
-__device__ __forceinline__ uint32_t sub_bytes(uint32_t c, uint32_t z4) { return ((c | 0x80808080u) - z4) ^ 0x80808080u; }
-__device__ __forceinline__ uint4 sub_bytes(const uint4& c, uint32_t z4) {
-  return make_uint4(sub_bytes(c.x, z4), sub_bytes(c.y, z4), sub_bytes(c.z, z4), sub_bytes(c.w, z4));
-}
-// Bytes in two's complement (within [-127, 127]) -> sign bit and magnitude.
-__device__ __forceinline__ uint32_t sign_magnitude(uint32_t x) { return __vabs4(x) | (x & 0x80808080u); }
-__device__ __forceinline__ uint4 sign_magnitude(const uint4& c) {
-  return make_uint4(sign_magnitude(c.x), sign_magnitude(c.y), sign_magnitude(c.z), sign_magnitude(c.w));
-}
-__device__ __forceinline__ float max3(float a, float b, float c) {
-  float d;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
-}
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 
 // NB: 64-channel blocks of the head; kLutBits: width of the Softmax codes when their operand values come from the
 // per-lane table (4, 6, or 8 where one CTA per SM leaves room for 257 entries), 0: integer arithmetic
@@ -778,22 +725,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, AttnParams P) {
   }
 }
 
-// Tensor map of the K codes for the bulk-copy variant: (bytes of a row, keys, batch items); a box is 128 bytes x the keys of a visit.
-repq_status make_k_map(CUtensorMap* map, const AttnParams& P, int batch_outer, int keys) {
-  EncodeTiledFn fn = encode_fn();
-  REPQ_REQUIRE(fn != nullptr, REPQ_CUDA_ERROR, "attention: cuTensorMapEncodeTiled is not available");
-  const cuuint64_t span = cuuint64_t(P.batch_inner - 1) * cuuint64_t(P.k_si) + cuuint64_t(P.dh);    // bytes the heads cover
-  const cuuint64_t dims[3] = {span, cuuint64_t(P.Lk), cuuint64_t(batch_outer)};
-  const cuuint64_t strides[2] = {cuuint64_t(P.ldk), cuuint64_t(P.k_so)};
-  const cuuint32_t box[3] = {128, cuuint32_t(keys), 1};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<uint8_t*>(P.k), dims, strides, box, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  REPQ_REQUIRE(r == CUDA_SUCCESS, REPQ_CUDA_ERROR, "attention: K tensor map failed with code %d", int(r));
-  return REPQ_OK;
-}
-
 template <int NB, int kLutBits, int kMode>
 repq_status launch_kernel(const AttnParams& P, int64_t pairs, cudaStream_t st) {
   const size_t smem = sizeof(AttnShared<NB, kLutBits>);
@@ -827,6 +758,7 @@ repq_status launch(const AttnParams& P, int64_t pairs, int qmax_qk, cudaStream_t
 }  // namespace repq
 
 using namespace repq;
+using namespace repq::attn;
 
 extern "C" repq_status repq_attention(const repq_attention_desc* d, void* stream) {
   REPQ_REQUIRE(d, REPQ_INVALID_ARG, "attention: NULL descriptor");
@@ -887,6 +819,7 @@ extern "C" repq_status repq_attention(const repq_attention_desc* d, void* stream
     P.no_f8 = e && *e && *e != '0';
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (pipe_supported(P, qmax_v) && !getenv("ATT_OLD")) return launch_pipe(P, pairs, qmax_v, st);
   // the per-lane table of the Softmax codes' operand values: 17 / 65 entries everywhere; the 257 entries of 8-bit codes
   // (33 KB) only where the head already limits the SM to one CTA
   if (d->d_h <= 64) {
