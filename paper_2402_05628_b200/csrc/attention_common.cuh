@@ -91,6 +91,26 @@ __device__ __forceinline__ void store_values(const AttnParams& P, const float (&
 #pragma unroll
       for (int e = 0; e < 16; ++e) o[e] = __float2bfloat16_rn(v[e]);
     }
+  } else if (!P.pack4 && P.vec_store) {
+    // t = v / s_o clamped, rounded half to even by the float adder (1.5 * 2^23), z_o added as an integer
+    const float zo_lo = float(-P.zo), zo_hi = float(P.qmax - P.zo);
+    const f32x2 inv2 = splat2(P.inv_so), magic2 = splat2(__uint_as_float(kMagicBits));
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      uint32_t u[4];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        float t0, t1, u0, u1;
+        unpack2(mul2(pack2(v[4 * i + 2 * k], v[4 * i + 2 * k + 1]), inv2), t0, t1);
+        unpack2(add2(pack2(fminf(fmaxf(t0, zo_lo), zo_hi), fminf(fmaxf(t1, zo_lo), zo_hi)), magic2), u0, u1);
+        u[2 * k] = __float_as_uint(u0) + uint32_t(P.zo);
+        u[2 * k + 1] = __float_as_uint(u1) + uint32_t(P.zo);
+      }
+      w[i] = __byte_perm(__byte_perm(u[0], u[1], 0x0040), __byte_perm(u[2], u[3], 0x0040), 0x5410);
+      code_sum = int(__dp4a(w[i], 0x01010101u, uint32_t(code_sum)));
+    }
+    *reinterpret_cast<uint4*>(static_cast<uint8_t*>(P.out) + roff + c0) = make_uint4(w[0], w[1], w[2], w[3]);
   } else {
     const float zo_lo = float(-P.zo), zo_hi = float(P.qmax - P.zo);
     uint32_t q[16];
@@ -111,14 +131,8 @@ __device__ __forceinline__ void store_values(const AttnParams& P, const float (&
         for (int e = 0; e < 4; ++e) { orow[(c0 >> 1) + e] = uint8_t(w0 >> (8 * e)); orow[(c0 >> 1) + 4 + e] = uint8_t(w1 >> (8 * e)); }
       }
     } else {
-      uint32_t w[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) w[e] = q[4 * e] | (q[4 * e + 1] << 8) | (q[4 * e + 2] << 16) | (q[4 * e + 3] << 24);
-      if (P.vec_store) *reinterpret_cast<uint4*>(orow + c0) = make_uint4(w[0], w[1], w[2], w[3]);
-      else {
-#pragma unroll
-        for (int e = 0; e < 16; ++e) orow[c0 + e] = uint8_t(q[e]);
-      }
+      for (int e = 0; e < 16; ++e) orow[c0 + e] = uint8_t(q[e]);
     }
   }
 }

@@ -8,25 +8,36 @@
 //            2^(-ceil(p/2)) split by the parity of p into E and O, written back over the columns of tensor memory the
 //            scores came from, from where the P.V MMAs take their A operand; O = s s_v (acc_E + sqrt2 acc_O)
 //
-// What bounds it is instruction issue (some 3 instructions per score in pass 1, where ex2 alone takes 8 cycles of a
-// scheduler's special-function unit, and 4 to 6 in pass 2) as long as nothing is waited for, and a tile of 128 queries is
-// a long chain of latencies (launch, Q tile, first K tile, merge of the statistics, last MMA, stores) around only 8 visits
-// when rows have 197 keys.  Hence:
+// A byte below 128 is q - z_q as a signed byte in the Q tile and the raw code in the K tile: S' = sum (q - z_q) k differs from
+// the zero-point-corrected sum by a number that is the same for every key of a row and drops out of the Softmax, so K comes
+// by bulk tensor copies untouched.
+//
+// What bounds it: the workers' instructions (ncu, 577 keys, 64 channels: issue slots 58 % busy, a third of the issues spent on
+// waits; ex2 alone takes 8 cycles of a scheduler per 32 scores) and the latency of their chains, not the tensor pipe (13 %).
+// Hence:
 //  - CTAs are persistent (two per SM for heads of up to 64 channels, one for wider heads) and walk their share of the
-//    tiles; K tiles stream in by bulk tensor copies across tile boundaries, the Q tile of the next tile is staged before
-//    the epilogue of the current one, so that the next tile's first S MMAs run under it;
+//    tiles; K tiles stream in by bulk tensor copies across tile boundaries and the Q tile of the next tile is staged during
+//    pass 2 of the present one, so that its S MMAs follow without a gap (a tile of 197 keys is only eight visits: launched one
+//    CTA per tile, half of its time was start and end);
 //  - a worker thread has one row (its tensor-memory lane) and 32 columns of every visit, which it loads at once: one
-//    barrier wait and one tensor-memory load per 32 scores, all of the warp's arithmetic independent behind it;
-//  - 4-bit codes of 4-bit values (scale s >= 1): the operands 2^(8 - ceil(p/2)) and v - z_v are 8-bit floats (e4m3), exact,
+//    barrier wait and one tensor-memory load per 32 scores, all of the warp's arithmetic independent behind it (16 columns at a
+//    time with the next 16 in flight: 20 % slower, more waits and spilled registers);
+//  - warps none of whose rows sees a column of theirs skip it;
+//  - 4-bit codes of 4-bit values (scale s >= 1): the operands 2^(8 - ceil(p/2)) and z_v - v are 8-bit floats (e4m3), exact,
 //    so P.V runs at K = 32 per instruction, and the operand bytes of four keys are formed together in one register from
 //    q = 15 - p (odd q: E = 0x3C + 4 q, even q: O = 0x38 + 4 q) instead of a table look-up per key;
 //  - wider codes take their bf16 operand pair from a per-lane table in shared memory (one bank per lane).
+// Measured against one CTA per tile with two groups of warps on alternate visits: 64 x 12 heads of 64 channels with 197 keys,
+// 4-bit codes, 83 -> 64 us; 32 x 16 heads, 577 keys 240 -> 192; 4 x 32 heads of 128 channels, 2048 causal keys, 8-bit codes,
+// 400 -> 305.  A warp of its own for the V tiles was slower (one warp's chain of loads and conversions per visit).
 // Roles: worker warps, then a warp each (one lane) for the S MMAs, the P.V MMAs and the K copies.  Every mbarrier wait is
 // bounded; when one runs out the kernel records a status code, all roles leave their loops, MMAs and copies in flight are
 // drained, tensor memory is freed and the kernel returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <math_constants.h>
+
+#include <type_traits>
 
 #include "attention_common.cuh"
 
@@ -43,7 +54,7 @@ template <int NB> struct Shape {
   static constexpr int kWorkThreads = 32 * kWork;
   static constexpr int kThreads = kWorkThreads + 96;
   static constexpr int kCtas = NB == 1 ? 2 : 1;                     // resident per SM
-  static constexpr int kK = NB == 1 ? 3 : 4, kV = 2;                // ring depths
+  static constexpr int kK = NB == 1 ? 3 : 4;                        // K tiles in flight
   static constexpr int kTmem = 256 * NB;                            // 2 S slots + 2 accumulators
 };
 
@@ -52,15 +63,16 @@ struct PipeShared {
   using Sh = Shape<NB>;
   static constexpr uint32_t kKBytes = Sh::kKeys * 128;
   static constexpr uint32_t kVBlockBytes = Sh::kKeys * 128;         // the visit's keys x 128 bytes (64 channels of bf16, or one row of bytes)
-  alignas(1024) uint8_t q[kQBytes];
+  alignas(1024) uint8_t q[2][kQBytes];            // of this tile and the next
   alignas(1024) uint8_t k[Sh::kK][kKBytes];
-  alignas(1024) uint8_t v[Sh::kV][NB * kVBlockBytes];
+  static constexpr int kV = NB == 1 && kLutBits != 8 ? 3 : 2;       // V tiles (two where the table takes 33 KB of half an SM)
+  alignas(1024) uint8_t v[kV][NB * kVBlockBytes];
   float stat_m[Sh::kParts][kRows], stat_z[Sh::kParts][kRows];
   static constexpr int kLutEntries = kLutBits ? (1 << kLutBits) + 1 : 1;
   uint32_t lut[kLutEntries][32];                  // [code][lane] = E value | O value << 16; the last entry repeats the top code
                                                   // (a clamp at 2^bits that rounds up lands there)
   alignas(8) uint64_t k_full[Sh::kK];
-  uint64_t k_empty[Sh::kK], v_empty[Sh::kV];
+  uint64_t k_empty[Sh::kK], v_empty[kV];
   uint64_t s_full[2], s_empty[2], s_spent[2], p_full[2];            // s_empty: read in pass 1; s_spent: P.V MMAs have read the operands
   uint64_t q_full, acc_full, acc_empty, done_s, done_pv, merged[4];   // merged: statistics of a lane quarter's rows are there
   uint32_t tmem_base;
@@ -77,6 +89,16 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
         "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr) : "memory");
+}
+// (the registers count as written by the wait: the compiler can neither read nor move them while the load is in flight)
+__device__ __forceinline__ void tmem_ld_wait32(uint32_t (&r)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+                 "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
+                 "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29])
+               :: "memory");
+  asm volatile("" : "+r"(r[30]), "+r"(r[31]));
 }
 // D[tmem] (+)= A[tmem] * B[smem], 8-bit floats, K = 32 (a 32-bit column of A holds four consecutive K elements)
 __device__ __forceinline__ void umma_f8_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
@@ -117,6 +139,47 @@ __device__ __forceinline__ bool tile_at(const AttnParams& P, int it, int cta, in
   return true;
 }
 
+// v - z_v of eight codes as bf16.
+struct VShift {
+  __nv_bfloat162 z2;
+  float z;
+  __device__ __forceinline__ explicit VShift(const AttnParams& P)
+      : z2(__float2bfloat162_rn(128.f + float(P.z_v))), z(12582912.f + float(P.z_v)) {}      // 1.5 * 2^23 + z_v
+  __device__ __forceinline__ uint4 bf16(const uint2& c, int small) const {
+    uint32_t o4[4];
+    if (small) {
+      // for codes below 128, 128 + v is the bit pattern 0x4300 | v and the bf16 subtraction exact
+      const uint32_t w[4] = {__byte_perm(c.x, 0x43434343u, 0x4140), __byte_perm(c.x, 0x43434343u, 0x4342),
+                             __byte_perm(c.y, 0x43434343u, 0x4140), __byte_perm(c.y, 0x43434343u, 0x4342)};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const __nv_bfloat162 hh = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&w[e]), z2);
+        o4[e] = *reinterpret_cast<const uint32_t*>(&hh);
+      }
+    } else {
+      float f[8];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        f[e] = __uint_as_float(__byte_perm(c.x, kMagicBits, 0x7650 + e)) - z;
+        f[4 + e] = __uint_as_float(__byte_perm(c.y, kMagicBits, 0x7650 + e)) - z;
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const __nv_bfloat162 hh = __floats2bfloat162_rn(f[2 * e], f[2 * e + 1]);
+        o4[e] = *reinterpret_cast<const uint32_t*>(&hh);
+      }
+    }
+    return make_uint4(o4[0], o4[1], o4[2], o4[3]);
+  }
+};
+
+// z - v of four 4-bit codes in sign and magnitude (z at most 15, shift4 = 128 - z in every byte): t = 128 + v - z is that
+// byte already where v >= z, and 128 - t is the magnitude where it is not.
+__device__ __forceinline__ uint32_t zero_minus(uint32_t v, uint32_t shift4) {
+  const uint32_t t = v + shift4, low = (~t >> 7) & 0x01010101u;
+  return (t ^ (low * 0x7Fu)) + low;
+}
+
 // kLutBits: width of the table of operand pairs (4, 6, 8; P.V in bf16), or 0: 4-bit codes of 4-bit values, P.V in 8-bit
 // floats.  kF8: 4-bit Q / K codes read as 8-bit floats (a byte below 16 is the e4m3 number byte * 2^-9; the accumulator holds
 // 2^-18 sum (q - z_q) k as a float, exactly); otherwise signed x unsigned bytes.
@@ -125,7 +188,7 @@ __global__ void __launch_bounds__(Shape<NB>::kThreads, Shape<NB>::kCtas)
 attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ AttnParams P) {
   using Sh = Shape<NB>;
   using Shared = PipeShared<NB, kLutBits>;
-  constexpr int kKeys = Sh::kKeys, kWork = Sh::kWork, kParts = Sh::kParts, kT = Sh::kWorkThreads, kK = Sh::kK, kV = Sh::kV;
+  constexpr int kKeys = Sh::kKeys, kWork = Sh::kWork, kParts = Sh::kParts, kT = Sh::kWorkThreads, kK = Sh::kK, kV = Shared::kV;
   constexpr bool kLut = kLutBits != 0;
   constexpr int kAccCol = 2 * kKeys;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -179,89 +242,101 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
   Tile t;
   if (warp == kWork) {
     // ---------------------------------------------------------------- S MMAs
+    // (one lane issues; the loops are kept short, since a visit costs as many issue latencies as they have instructions)
     if (lane == 0) {
-      // D = s32 from signed x unsigned bytes, or D = f32 from e4m3 x e4m3; both K-major, M = 128, N = the visit's keys
-      constexpr uint32_t idesc = (kF8 ? (1u << 4) : (2u << 4) | (1u << 7)) | (uint32_t(kKeys >> 3) << 17) | (uint32_t(kRows >> 4) << 24);
-      const uint64_t dq = smem_desc_sw128(smem_u32(S.q));
-      int g = 0;                                          // visits, over both passes and all tiles
-      // a bit per slot: parity of the hand-backs waited for, whether the slot has been used, and by which pass last
-      uint32_t ph_empty = 0, ph_spent = 0, used = 0, pass2 = 0;
-      uint32_t ks = 0, kp = 0;                            // K ring: slot and parity
-      bool ok = true;
-      for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
-        if (!(ok = mbar_wait(smem_u32(&S.q_full), it & 1, abort, 40, P.status))) break;
+    // D = s32 from signed x unsigned bytes, or D = f32 from e4m3 x e4m3; both K-major, M = 128, N = the visit's keys
+    constexpr uint32_t idesc = (kF8 ? (1u << 4) : (2u << 4) | (1u << 7)) | (uint32_t(kKeys >> 3) << 17) | (uint32_t(kRows >> 4) << 24);
+    const uint64_t dk0 = smem_desc_sw128(smem_u32(S.k[0]));
+    int g = 0;                                            // visits, over both passes and all tiles
+    // a bit per slot: parity of the hand-backs waited for, whether the slot has been used, and by which pass last
+    uint32_t ph_empty = 0, ph_spent = 0, used = 0, pass2 = 0;
+    uint32_t ks = 0, kp = 0;                              // K ring: slot and parity
+    bool ok = true;
+    for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
+      if (!(ok = mbar_wait(smem_u32(&S.q_full), it & 1, abort, 40, P.status))) break;
+      const uint64_t dq = smem_desc_sw128(smem_u32(S.q[it & 1]));
 #pragma unroll 1
-        for (int b = 0; b < 2 * t.nb; ++b, ++g) {
-          const int slot = g & 1;
-          if (!(ok = mbar_wait(smem_u32(&S.k_full[ks]), kp, abort, 41, P.status))) break;
-          const uint32_t bit = 1u << slot;
-          if (used & bit) {
-            if (pass2 & bit) {
-              if (!(ok = mbar_wait(smem_u32(&S.s_spent[slot]), (ph_spent >> slot) & 1u, abort, 42, P.status))) break;
-              ph_spent ^= bit;
-            } else {
-              if (!(ok = mbar_wait(smem_u32(&S.s_empty[slot]), (ph_empty >> slot) & 1u, abort, 42, P.status))) break;
-              ph_empty ^= bit;
+      for (int b = 0; b < 2 * t.nb; ++b, ++g) {
+        const int slot = g & 1;
+        const uint32_t bit = 1u << slot;
+        if (!(ok = mbar_wait(smem_u32(&S.k_full[ks]), kp, abort, 41, P.status))) break;
+        if (used & bit) {
+          const bool spent = (pass2 & bit) != 0;
+          if (!(ok = mbar_wait(spent ? smem_u32(&S.s_spent[slot]) : smem_u32(&S.s_empty[slot]), ((spent ? ph_spent : ph_empty) >> slot) & 1u,
+                               abort, 42, P.status))) break;
+          if (spent) ph_spent ^= bit; else ph_empty ^= bit;
+        }
+        used |= bit;
+        pass2 = b >= t.nb ? pass2 | bit : pass2 & ~bit;
+        tc_fence_after();
+        {
+          const uint64_t dk = dk0 + uint64_t(ks * (Shared::kKBytes >> 4));
+          const uint32_t d = tmem_base + uint32_t(slot * kKeys);
+#pragma unroll
+          for (int s = 0; s < 2 * NB; ++s) {
+            if (s < ksteps) {
+              if (kF8) umma_f8(d, dq + uint64_t(2 * s), dk + uint64_t(2 * s), idesc, s != 0 ? 1u : 0u);
+              else umma_i8(d, dq + uint64_t(2 * s), dk + uint64_t(2 * s), idesc, s != 0 ? 1u : 0u);
             }
-          }
-          tc_fence_after();
-          const uint64_t dk = smem_desc_sw128(smem_u32(S.k[ks]));
-          for (int s = 0; s < ksteps; ++s) {
-            if (kF8) umma_f8(tmem_base + uint32_t(slot * kKeys), dq + uint64_t(2 * s), dk + uint64_t(2 * s), idesc, s != 0 ? 1u : 0u);
-            else umma_i8(tmem_base + uint32_t(slot * kKeys), dq + uint64_t(2 * s), dk + uint64_t(2 * s), idesc, s != 0 ? 1u : 0u);
           }
           umma_commit(smem_u32(&S.s_full[slot]));
           umma_commit(smem_u32(&S.k_empty[ks]));
-          used |= bit;
-          pass2 = b >= t.nb ? pass2 | bit : pass2 & ~bit;
-          if (++ks == kK) { ks = 0; kp ^= 1u; }
         }
+        if (++ks == kK) { ks = 0; kp ^= 1u; }
       }
-      umma_commit(smem_u32(&S.done_s));
-      mbar_drain(smem_u32(&S.done_s), 0);
+    }
+    umma_commit(smem_u32(&S.done_s));
+    mbar_drain(smem_u32(&S.done_s), 0);
     }
   } else if (warp == kWork + 1) {
     // ---------------------------------------------------------------- P.V MMAs
     if (lane == 0) {
-      // D = f32, A (tensor memory) and B = bf16 or e4m3, B MN-major, N = n_pad, M = 128
-      const uint32_t idesc = (kLut ? (1u << 4) | (1u << 7) | (1u << 10) : (1u << 4)) | (1u << 16) | (uint32_t(P.n_pad >> 3) << 17) |
-                             (uint32_t(kRows >> 4) << 24);
-      constexpr int kStep = kLut ? 16 : 32;               // keys per MMA
-      int g = 0;
-      uint32_t ph_p = 0, vs = 0;
-      bool ok = true;
-      for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
-        g += t.nb;
-        if (it > 0 && !(ok = mbar_wait(smem_u32(&S.acc_empty), (it - 1) & 1, abort, 50, P.status))) break;
+    // D = f32, A (tensor memory) and B = bf16 or e4m3, B MN-major, N = n_pad, M = 128
+    const uint32_t idesc = (kLut ? (1u << 4) | (1u << 7) | (1u << 10) : (1u << 4)) | (1u << 16) | (uint32_t(P.n_pad >> 3) << 17) |
+                           (uint32_t(kRows >> 4) << 24);
+    constexpr int kStep = kLut ? 16 : 32;                 // keys per MMA
+    const uint64_t dv0 = smem_desc_sw128(smem_u32(S.v[0]), Shared::kVBlockBytes);
+    const uint32_t d_e = tmem_base + uint32_t(kAccCol), d_o = d_e + uint32_t(P.n_pad);
+    int g = 0;
+    uint32_t ph_p = 0, vs = 0;
+    bool ok = true;
+    for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
+      g += t.nb;
+      if (it > 0 && !(ok = mbar_wait(smem_u32(&S.acc_empty), (it - 1) & 1, abort, 50, P.status))) break;
 #pragma unroll 1
-        for (int j = 0; j < t.nb; ++j, ++g) {
-          const int slot = g & 1;
-          if (!(ok = mbar_wait(smem_u32(&S.p_full[slot]), (ph_p >> slot) & 1u, abort, 43, P.status))) break;
-          ph_p ^= 1u << slot;
-          tc_fence_after();
-          const uint64_t dv = smem_desc_sw128(smem_u32(S.v[vs]), Shared::kVBlockBytes);
-          const int steps = (min(kKeys, t.k_end - j * kKeys) + kStep - 1) / kStep;
+      for (int j = 0; j < t.nb; ++j, ++g) {
+        const int slot = g & 1;
+        if (!(ok = mbar_wait(smem_u32(&S.p_full[slot]), (ph_p >> slot) & 1u, abort, 43, P.status))) break;
+        ph_p ^= 1u << slot;
+        tc_fence_after();
+        const int left = t.k_end - j * kKeys;             // keys from the visit's first on
+        {
+          const uint64_t dv = dv0 + uint64_t(vs * (NB * Shared::kVBlockBytes >> 4));
           const uint32_t a_base = tmem_base + uint32_t(slot * kKeys);
-          for (int s = 0; s < steps; ++s) {
-            const uint32_t accumulate = (j | s) != 0 ? 1u : 0u;
-            const uint64_t b = dv + uint64_t(kStep * 128 / 16 * s);
-            const uint32_t a_e = a_base + uint32_t(kStep * s);     // E words first, then as many O words
-            if (kLut) {
-              umma_f16_ts(tmem_base + uint32_t(kAccCol), a_e, b, idesc, accumulate);
-              umma_f16_ts(tmem_base + uint32_t(kAccCol + P.n_pad), a_e + 8u, b, idesc, accumulate);
-            } else {
-              umma_f8_ts(tmem_base + uint32_t(kAccCol), a_e, b, idesc, accumulate);
-              umma_f8_ts(tmem_base + uint32_t(kAccCol + P.n_pad), a_e + 8u, b, idesc, accumulate);
+#pragma unroll
+          for (int s = 0; s < kKeys / kStep; ++s) {
+            if (s * kStep < left) {
+              const uint32_t accumulate = s != 0 ? 1u : j != 0 ? 1u : 0u;
+              const uint64_t b = dv + uint64_t(kStep * 128 / 16 * s);
+              const uint32_t a_e = a_base + uint32_t(kStep * s);       // E words first, then as many O words
+              if (kLut) {
+                umma_f16_ts(d_e, a_e, b, idesc, accumulate);
+                umma_f16_ts(d_o, a_e + 8u, b, idesc, accumulate);
+              } else {
+                umma_f8_ts(d_e, a_e, b, idesc, accumulate);
+                umma_f8_ts(d_o, a_e + 8u, b, idesc, accumulate);
+              }
             }
           }
           umma_commit(smem_u32(&S.s_spent[slot]));
           umma_commit(smem_u32(&S.v_empty[vs]));
-          if (++vs == kV) vs = 0;
+          if (j + 1 == t.nb) umma_commit(smem_u32(&S.acc_full));
         }
-        if (ok) umma_commit(smem_u32(&S.acc_full));
+        if (++vs == kV) vs = 0;
       }
-      umma_commit(smem_u32(&S.done_pv));
-      mbar_drain(smem_u32(&S.done_pv), 0);
+    }
+    umma_commit(smem_u32(&S.done_pv));
+    mbar_drain(smem_u32(&S.done_pv), 0);
     }
   } else if (warp == kWork + 2) {
     // ---------------------------------------------------------------- K tiles by bulk tensor copies
@@ -297,10 +372,12 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     const uint32_t taddr_s = tmem_base + (uint32_t(quarter * 32) << 16) + uint32_t(part * kCols);
     const uint32_t lut_addr = smem_u32(&S.lut[0][lane]) - (kMagicBits << 7);
 
-    // ---- Q tile: q - z_q as signed bytes (kF8: sign and magnitude); 4 threads per row (8 when there are 512 workers),
-    // 32 (16) bytes each; the pieces of a tile are requested first and written once the tile before is through its S MMAs
-    constexpr int kQPer = kT == 256 ? 4 : 2;              // pieces per thread: rows of 8 pieces, kT threads
-    const int qrow = tid / (8 / kQPer), qp0 = (tid % (8 / kQPer)) * kQPer;
+    // ---- Q tile: q - z_q as signed bytes (kF8: sign and magnitude), two 16-byte pieces per thread.  The next tile's is
+    // requested and written during the first visit of pass 2, into the other of two buffers, so that the next tile's S MMAs
+    // follow this tile's without a gap.
+    constexpr int kQRow = 4 * NB, kQPer = 2;              // pieces of a row (64 or 128 channels) and of a thread
+    static_assert(kRows * kQRow == kQPer * kT, "every piece of the Q tile has a thread");
+    const int qrow = tid / (kQRow / kQPer), qp0 = (tid % (kQRow / kQPer)) * kQPer;
     const uint32_t zq4 = uint32_t(P.zq) * 0x01010101u;
     uint4 qreg[kQPer];
     auto fetch_q = [&](const Tile& n) {
@@ -311,78 +388,44 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
         if (n.q0 + qrow < P.Lq && qp0 + i < pieces) qreg[i] = __ldg(reinterpret_cast<const uint4*>(row) + qp0 + i);
       }
     };
-    auto stage_q = [&]() {
+    auto stage_q = [&](uint8_t* tile) {
 #pragma unroll
       for (int i = 0; i < kQPer; ++i) {
         uint4 w = sub_bytes(qreg[i], zq4);
         if (kF8) w = sign_magnitude(w);
-        if (qp0 + i < 2 * ksteps) *reinterpret_cast<uint4*>(S.q + tile_offset(qrow, qp0 + i)) = w;
+        if (qp0 + i < 2 * ksteps) *reinterpret_cast<uint4*>(tile + tile_offset(qrow, qp0 + i)) = w;
       }
       fence_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&S.q_full));
     };
 
-    // ---- V tile of a visit.  8-bit floats: a thread has one key and 16 channels, v - z_v in sign and magnitude.  bf16: a
-    // thread keeps its group of 8 channels and moves down the keys, 32 per step.
-    constexpr int kVItems = kLut ? kKeys / 32 : 1;
-    const int v_g = kLut ? tid % (8 * NB) : tid & 3, v_key0 = kLut ? tid / (8 * NB) : tid >> 2;
-    const bool v_live = v_g * (kLut ? 8 : 16) < P.dh;
+    // ---- V tile of a visit.  8-bit floats: a thread has one key and 16 channels, z_v - v in sign and magnitude (byte * 2^-9).
+    // bf16: a thread keeps its group of 8 channels and moves down the keys, 32 per step.
+    using VRaw = typename std::conditional<kLut, uint2, uint4>::type;
+    constexpr int kVItems = kLut ? kKeys / 32 : 1, kVChan = kLut ? 8 : 16, kVGroups = 64 * NB / kVChan;
+    const int v_g = tid % kVGroups, v_key0 = tid / kVGroups;
+    const bool v_live = v_g * kVChan < P.dh;
     const uint32_t v_off = kLut ? uint32_t(v_g >> 3) * Shared::kVBlockBytes + tile_offset(v_key0, v_g & 7) : tile_offset(v_key0, v_g);
-    const uint32_t zv4 = uint32_t(P.z_v) * 0x01010101u;
-    const float vz = magic + float(P.z_v);
-    const __nv_bfloat162 vz2 = __float2bfloat162_rn(128.f + float(P.z_v));
+    const VShift vshift(P);
+    const uint32_t shift4 = (128u - uint32_t(P.z_v)) * 0x01010101u;
     const uint8_t* v_ptr = nullptr;
-    uint4 v16;
-    uint2 vraw[kVItems];
+    VRaw vraw[kVItems];
     auto fetch_v = [&](int block) {
-      if constexpr (!kLut) {
-        v16 = make_uint4(zv4, zv4, zv4, zv4);
-        const int key = block * kKeys + v_key0;
-        if (v_live && key < t.k_end) v16 = __ldg(reinterpret_cast<const uint4*>(v_ptr + int64_t(block * kKeys) * P.ldv));
-      } else {
+      const uint8_t* p = v_ptr + int64_t(block * kKeys) * P.ldv;
 #pragma unroll
-        for (int i = 0; i < kVItems; ++i) {
-          vraw[i] = make_uint2(0u, 0u);
-          const int key = block * kKeys + v_key0 + i * 32;
-          if (v_live && key < t.k_end) vraw[i] = __ldg(reinterpret_cast<const uint2*>(v_ptr + int64_t(block * kKeys + i * 32) * P.ldv));
-        }
-      }
+      for (int i = 0; i < kVItems; ++i)
+        if (v_live && block * kKeys + v_key0 + i * 32 < t.k_end) vraw[i] = __ldg(reinterpret_cast<const VRaw*>(p + int64_t(i * 32) * P.ldv));
     };
     auto stage_v = [&](int block, uint8_t* tile) {
-      if constexpr (!kLut) {
-        *reinterpret_cast<uint4*>(tile + v_off) = sign_magnitude(sub_bytes(v16, zv4));
-      } else {
 #pragma unroll
-        for (int i = 0; i < kVItems; ++i) {
-          uint32_t o4[4] = {0u, 0u, 0u, 0u};
-          if (v_live && block * kKeys + v_key0 + i * 32 < t.k_end) {
-            const uint32_t b03 = vraw[i].x, b47 = vraw[i].y;
-            if (P.v_small) {
-              // v - z_v as bf16: for codes below 128, 128 + v is the bit pattern 0x4300 | v and the bf16 subtraction exact
-              const uint32_t w[4] = {__byte_perm(b03, 0x43434343u, 0x4140), __byte_perm(b03, 0x43434343u, 0x4342),
-                                     __byte_perm(b47, 0x43434343u, 0x4140), __byte_perm(b47, 0x43434343u, 0x4342)};
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const __nv_bfloat162 hh = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&w[e]), vz2);
-                o4[e] = *reinterpret_cast<const uint32_t*>(&hh);
-              }
-            } else {
-              float f[8];
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                f[e] = __uint_as_float(__byte_perm(b03, kMagicBits, 0x7650 + e)) - vz;
-                f[4 + e] = __uint_as_float(__byte_perm(b47, kMagicBits, 0x7650 + e)) - vz;
-              }
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const __nv_bfloat162 hh = __floats2bfloat162_rn(f[2 * e], f[2 * e + 1]);
-                o4[e] = *reinterpret_cast<const uint32_t*>(&hh);
-              }
-            }
-          }
-          *reinterpret_cast<uint4*>(tile + v_off + uint32_t(i) * 4096u) = make_uint4(o4[0], o4[1], o4[2], o4[3]);
+      for (int i = 0; i < kVItems; ++i) {
+        uint4 w = make_uint4(0u, 0u, 0u, 0u);
+        if (v_live && block * kKeys + v_key0 + i * 32 < t.k_end) {
+          if constexpr (kLut) w = vshift.bf16(vraw[i], P.v_small);
+          else w = make_uint4(zero_minus(vraw[i].x, shift4), zero_minus(vraw[i].y, shift4), zero_minus(vraw[i].z, shift4), zero_minus(vraw[i].w, shift4));
         }
+        *reinterpret_cast<uint4*>(tile + v_off + uint32_t(i) * 4096u) = w;
       }
     };
 
@@ -392,7 +435,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
       uint32_t rn[kCols];
       __syncwarp();
       tmem_ld32(taddr_s + uint32_t(slot * kKeys), rn);
-      tmem_ld_wait();
+      tmem_ld_wait32(rn);
 #pragma unroll
       for (int e = 0; e < kCols; ++e) sf[e] = kF8 ? __uint_as_float(rn[e]) : float(int32_t(rn[e]));
     };
@@ -500,41 +543,90 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
       }
     };
 
+    // ---- epilogue of tile `it`: one row per thread (`roff`: its output offset, -1: past Lq), the 16-column chunks of the
+    // accumulators dealt to the parts of a row
+    auto finish = [&](int it, int64_t roff, int64_t sum_at) -> bool {
+              if (!mbar_wait(smem_u32(&S.acc_full), it & 1, abort, 47, P.status)) return false;
+              tc_fence_after();
+              const float out_scale = kLut ? P.out_scale : -2.f * P.out_scale;  // 8-bit floats: 2^8 A times 2^-9 (z_v - v)
+              const uint32_t taddr = tmem_base + (uint32_t(quarter * 32) << 16) + uint32_t(kAccCol);
+              int code_sum = 0;
+      #pragma unroll 1
+              for (int c0 = part * 16; c0 < P.dh; c0 += kParts * 16) {
+                uint32_t re[16], ro[16];
+                __syncwarp();
+                tmem_ld16(taddr + uint32_t(c0), re);
+                tmem_ld16(taddr + uint32_t(P.n_pad + c0), ro);
+                tmem_ld_wait(re);
+                tmem_ld_wait(ro);
+                if (c0 + kParts * 16 >= P.dh) {                 // the thread's last chunk: the accumulators may be written again
+                  tc_fence_before();
+                  __syncwarp();
+                  if (lane == 0) mbar_arrive(smem_u32(&S.acc_empty));
+                }
+                float v[16];
+                const f32x2 root2 = splat2(1.41421356237309504880f), scale2 = splat2(out_scale);
+      #pragma unroll
+                for (int e = 0; e < 16; e += 2)
+                  unpack2(mul2(scale2, fma2(root2, pack2(__uint_as_float(ro[e]), __uint_as_float(ro[e + 1])),
+                                            pack2(__uint_as_float(re[e]), __uint_as_float(re[e + 1])))), v[e], v[e + 1]);
+                if (roff >= 0) store_values(P, v, roff, c0, code_sum);
+              }
+              if (part * 16 >= P.dh) {                          // no chunk for this thread
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&S.acc_empty));
+              } else if (roff >= 0 && P.out_row_sum != nullptr && P.out_kind == REPQ_OUT_CODES) {
+                atomicAdd(P.out_row_sum + sum_at, code_sum);
+              }
+      return true;
+    };
+
+    // Where one CTA has the SM (wide heads), the epilogue waits until the next tile's pass 1 is through, under which the tile's
+    // last MMAs complete; where two share it, the other one runs meanwhile and the epilogue follows at once (measured: 64 x 12
+    // heads of 64 channels, 197 keys, 64 against 77 us; 4 x 32 heads of 128 channels, 2048 causal keys, 325 against 310).
+    constexpr bool kDefer = NB != 1;
     bool ok = true, more = tile_at<kKeys>(P, 0, blockIdx.x, gridDim.x, t);
-    int g = 0, jv = 0;                                    // visits and V tiles, over all tiles
-    if (more) { fetch_q(t); stage_q(); }
-    for (int it = 0; more && !*abort; ++it) {
-      const int row = t.q0 + r;
+    int g = 0;                                            // visits, over both passes and all tiles
+    uint32_t vs = 0, vp = 0;                              // V ring: stage and parity
+    int64_t done_row = -1, done_sum = 0;                  // the tile before: output offset and row-sum index of the thread's row, -1: past Lq
+    if (more) { fetch_q(t); stage_q(S.q[0]); }
+    for (int it = 0; !*abort; ++it) {
+      const int row = more ? t.q0 + r : P.Lq;
       const int valid = row < P.Lq ? (P.causal ? max(1, min(P.Lk, row + 1 + P.Lk - P.Lq)) : P.Lk) : 0;   // keys the row sees
       const int most = __reduce_max_sync(0xffffffffu, valid);                                             // ... any row of the warp
-      v_ptr = P.v + t.bo * P.v_so + t.bi * P.v_si + int64_t(v_key0) * P.ldv + v_g * (kLut ? 8 : 16);
-      fetch_v(0);
-      m = -CUDART_INF_F;
-      z = 0.f;
       // ---- pass 1
-      for (int b = 0; b < t.nb; ++b, ++g) {
-        const int slot = g & 1, first = b * kKeys + part * kCols;
-        if (!mbar_wait(smem_u32(&S.s_full[slot]), (g >> 1) & 1, abort, 44, P.status)) { ok = false; break; }
-        if (first < most) {                               // (warps whose columns no row sees only hand the slot back)
-          tc_fence_after();
-          float sf[kCols];
-          load_scores(slot, sf);
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&S.s_empty[slot]));
-          stats(sf, valid - first);
-        } else if (lane == 0) {
-          mbar_arrive(smem_u32(&S.s_empty[slot]));
+      if (more) {
+        v_ptr = P.v + t.bo * P.v_so + t.bi * P.v_si + int64_t(v_key0) * P.ldv + v_g * kVChan;
+        if (kDefer) fetch_v(0);
+        m = -CUDART_INF_F;
+        z = 0.f;
+        for (int b = 0; b < t.nb; ++b, ++g) {
+          const int slot = g & 1, first = b * kKeys + part * kCols;
+          if (!mbar_wait(smem_u32(&S.s_full[slot]), (g >> 1) & 1, abort, 44, P.status)) { ok = false; break; }
+          if (first < most) {                             // (warps whose columns no row sees only hand the slot back)
+            tc_fence_after();
+            float sf[kCols];
+            load_scores(slot, sf);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&S.s_empty[slot]));
+            stats(sf, valid - first);
+          } else if (lane == 0) {
+            mbar_arrive(smem_u32(&S.s_empty[slot]));
+          }
         }
+        if (!ok || *abort) break;
+        if (!kDefer) fetch_v(0);
+        // the column parts of a row are merged below
+        S.stat_m[part][r] = m;
+        S.stat_z[part][r] = z;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&S.merged[quarter]));
       }
-      if (!ok || *abort) break;
-      // merge the column parts of every row: m = max, Z = sum of the rescaled partial sums (same order in every thread of
-      // the row, so that all of them hold the same Z)
-      S.stat_m[part][r] = m;
-      S.stat_z[part][r] = z;
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&S.merged[quarter]));
+      if (kDefer && it > 0 && !finish(it - 1, done_row, done_sum)) break;
+      if (!more) break;
       if (!mbar_wait(smem_u32(&S.merged[quarter]), it & 1, abort, 45, P.status)) break;
+      // m = max, Z = sum of the rescaled partial sums (same order in every thread of the row, so that all hold the same Z)
       float zt = 0.f;
 #pragma unroll
       for (int q = 0; q < kParts; ++q) m = fmaxf(m, S.stat_m[q][r]);
@@ -555,12 +647,18 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
         }
       }
       // ---- pass 2
-      for (int j = 0; j < t.nb; ++j, ++g, ++jv) {
-        const int slot = g & 1, first = j * kKeys + part * kCols, pb = jv % kV;
-        if (!mbar_wait(smem_u32(&S.v_empty[pb]), ((jv / kV) & 1) ^ 1, abort, 46, P.status)) { ok = false; break; }
-        stage_v(j, S.v[pb]);
+      for (int j = 0; j < t.nb; ++j, ++g) {
+        const int slot = g & 1, first = j * kKeys + part * kCols;
+        if (!mbar_wait(smem_u32(&S.v_empty[vs]), vp ^ 1u, abort, 46, P.status)) { ok = false; break; }
+        stage_v(j, S.v[vs]);
         if (j + 1 < t.nb) fetch_v(j + 1);
         fence_async_smem();
+        if (++vs == kV) { vs = 0; vp ^= 1u; }
+        if (j == 0) {
+          Tile next;
+          more = tile_at<kKeys>(P, it + 1, blockIdx.x, gridDim.x, next);
+          if (more) fetch_q(next);
+        }
         if (!mbar_wait(smem_u32(&S.s_full[slot]), (g >> 1) & 1, abort, 44, P.status)) { ok = false; break; }
         // columns past the visit's last key are read by the MMAs only inside the step that holds it
         if (first < t.k_end) {
@@ -581,49 +679,13 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&S.p_full[slot]));
+        if (j == 0 && more) stage_q(S.q[(it + 1) & 1]);   // (the buffer's last reader: the S MMAs of the tile before this one)
       }
       if (!ok || *abort) break;
-
-      // ---- the next tile's Q (every S MMA of this tile has completed), then the epilogue: one row per thread, the 16-column
-      // chunks of the accumulators dealt to the parts of a row
-      const Tile cur = t;
-      more = tile_at<kKeys>(P, it + 1, blockIdx.x, gridDim.x, t);
-      if (more) fetch_q(t);
-      if (more) stage_q();
-      if (!mbar_wait(smem_u32(&S.acc_full), it & 1, abort, 47, P.status)) break;
-      tc_fence_after();
-      const float out_scale = kLut ? P.out_scale : 2.f * P.out_scale;   // 8-bit floats: 2^8 A times 2^-9 (v - z_v)
-      const uint32_t taddr = tmem_base + (uint32_t(quarter * 32) << 16) + uint32_t(kAccCol);
-      constexpr int kChunks = NB * 4 / kParts;            // chunks per thread for the widest head
-      float v[kChunks][16];
-#pragma unroll
-      for (int i = 0; i < kChunks; ++i) {
-        const int c0 = (part + i * kParts) * 16;
-        if (c0 < P.dh) {
-          uint32_t re[16], ro[16];
-          __syncwarp();
-          tmem_ld16(taddr + uint32_t(c0), re);
-          tmem_ld16(taddr + uint32_t(P.n_pad + c0), ro);
-          tmem_ld_wait();
-#pragma unroll
-          for (int e = 0; e < 16; ++e)
-            v[i][e] = out_scale * fmaf(1.41421356237309504880f, __uint_as_float(ro[e]), __uint_as_float(re[e]));
-        }
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&S.acc_empty));
-      if (row < P.Lq) {
-        int code_sum = 0;
-        const int64_t roff = cur.bo * P.o_so + cur.bi * P.o_si + int64_t(row) * P.ldo;
-#pragma unroll
-        for (int i = 0; i < kChunks; ++i) {
-          const int c0 = (part + i * kParts) * 16;
-          if (c0 < P.dh) store_values(P, v[i], roff, c0, code_sum);
-        }
-        if (P.out_row_sum != nullptr && P.out_kind == REPQ_OUT_CODES && part * 16 < P.dh)
-          atomicAdd(P.out_row_sum + int64_t(cur.bo) * P.Lq + row, code_sum);
-      }
+      done_row = row < P.Lq ? t.bo * P.o_so + t.bi * P.o_si + int64_t(row) * P.ldo : -1;
+      done_sum = int64_t(t.bo) * P.Lq + row;
+      if (!kDefer && !finish(it, done_row, done_sum)) break;
+      if (more) tile_at<kKeys>(P, it + 1, blockIdx.x, gridDim.x, t);
     }
   }
 

@@ -1,3 +1,6 @@
+// repq_attention: argument checks, choice of the kernel, and the kernel for 8-bit quantizers (zero points or strides that
+// attention_pipe.cu does not take).
+//
 // Fused attention on integer codes: scores (Eq. 3 with quantized Q and K), Softmax, log-sqrt2 codes (Eq. 15) and
 // P.V with the reparameterized log2 de-quantization (Eqs. 16-17) in one kernel.  Scores and codes never leave the
 // SM.  The code of a score depends on the row's final Softmax sum, so the keys are walked twice, a visit being 64 keys
@@ -23,17 +26,13 @@
 //    computes.  Inside a group a thread has one row (its tensor-memory lane) and half of the visit's columns, handled
 //    in runs of 16 (one tensor-memory load, arithmetic, in pass 2 one tensor-memory store).
 //  - Wide heads use visits of 128 keys (half the instructions per key) and give the P.V MMAs an issuing warp of their
-//    own (warp 18), so that the S MMAs (warp 16) are not held up by the wait for the workers' operands.
+//    own (warp 17), so that the S MMAs (warp 16) are not held up by the wait for the workers' operands.
 //  - The E / O operands never touch shared memory, whose bandwidth the V tiles, the table look-ups and the MMAs' B
 //    operands already share.
-// A group also builds the V tile of its visits (from registers fetched one of its visits ahead) and, for quantizers
-// wider than 7 bits, the K tiles of its visits.  Warp 17 (one lane, quantizers of at most 7 bits): K tiles by bulk
-// tensor copies.  There the Q tile holds q - z_q as signed bytes and the K tile the raw unsigned codes:
-// S' = sum (q - z_q) k differs from the zero-point-corrected sum by -z_k sum (q - z_q), which is the same for every key
-// of a row and drops out of the Softmax (maximum and values are taken on S' alone), so no correction and no pass over
-// the K bytes is needed.  Under a causal mask, key blocks no row of the CTA may see are skipped.  Every mbarrier wait
-// is bounded; when one runs out the kernel records a status code, all roles leave their loops, MMAs in flight are
-// drained, tensor memory is freed and the kernel returns.
+// A group also builds the V and K tiles of its visits (from registers fetched one of its visits ahead), and the score
+// accumulators are corrected by the row and column zero-point terms.  Under a causal mask, key blocks no row of the CTA may
+// see are skipped.  Every mbarrier wait is bounded; when one runs out the kernel records a status code, all roles leave their
+// loops, MMAs in flight are drained, tensor memory is freed and the kernel returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <math_constants.h>
@@ -56,8 +55,8 @@ constexpr int kGroupThreads = 32 * kGroupWarps;
 constexpr int kParts = kWorkWarps / 4;        // threads that share a row: 2 groups x 2 halves of a block's columns
 constexpr int kCols = 16;                     // S columns per tensor-memory load (a run); a thread takes 2 or 4 runs per visit
 constexpr int kWorkThreads = 32 * kWorkWarps;
-// + S-MMA warp + K-copy warp, and for wide heads a P.V-MMA warp of its own (its waits then do not hold up the S MMAs)
-template <int NB> struct Threads { static constexpr int value = kWorkThreads + (NB == 1 ? 64 : 96); };
+// + S-MMA warp, and for wide heads a P.V-MMA warp of its own (its waits then do not hold up the S MMAs)
+template <int NB> struct Threads { static constexpr int value = kWorkThreads + (NB == 1 ? 32 : 64); };
 
 // Ring depths.  S: one slot of tensor memory per worker group (2 x 64 or 2 x 128 columns beside the accumulators' 2 x 64
 // or 2 x 128).  Heads of up to 64 channels run two CTAs per SM: two K tiles, one V stage.  Wider heads have the SM to
@@ -81,7 +80,6 @@ struct AttnShared {
                                                     // lane); the last entry repeats the top code (a clamp at 2^bits that
                                                     // rounds up lands there)
   alignas(8) uint64_t k_full[kK];
-  uint64_t k_empty[kK];                             // K tile read by its S MMAs (bulk-copy variant)
   uint64_t s_full[kS], s_empty[kS], s_spent[kS], p_full[kP], p_empty[kP];   // s_empty: read in pass 1; s_spent: P.V MMAs of a
                                                                             // pass-2 visit have read the operands written over S
   uint64_t stats_ready, acc_full, done, done_pv;
@@ -91,28 +89,15 @@ struct AttnShared {
 
 // NB: 64-channel blocks of the head; kLutBits: width of the Softmax codes when their operand values come from the
 // per-lane table (4, 6, or 8 where one CTA per SM leaves room for 257 entries), 0: integer arithmetic
-// kMode: how the scores are formed.
-//   kCorrected  unsigned Q and K tiles, accumulators corrected by the row and column zero-point terms
-//   kCentred    q - z_q fits a signed byte (quantizers of at most 7 bits): the Q tile holds q - z_q, the K tile the raw
-//               codes, the S MMAs run signed x unsigned and their accumulators need no correction
-//   kCentredF8  4-bit quantizers (|q - z_q| <= 15, k <= 15): the same tiles read as 8-bit floats.  A byte below 16 is
-//               the e4m3 number byte * 2^-9 (subnormals and the first binade are linear in the byte), so the raw K codes
-//               are already such numbers and the Q tile stores sign and magnitude of q - z_q.  Products and sums are
-//               multiples of 2^-18 below 2^-3, exact in the float32 accumulator, which therefore holds
-//               2^-18 sum (q - z_q) k as a float: the int -> float conversion of every score is gone (the factor 2^18 is
-//               folded into the score scale on the host, exactly)
-enum : int { kCorrected = 0, kCentred = 1, kCentredF8 = 2 };
-template <int NB, int kLutBits, int kMode>
+template <int NB, int kLutBits>
 __global__ void __launch_bounds__(Threads<NB>::value, NB == 1 ? 2 : 1)
-attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, AttnParams P) {
+attention_tc_kernel(AttnParams P) {
   using Shared = AttnShared<NB, kLutBits>;
   constexpr int kKeys = Shared::kKeys;
-  constexpr uint32_t kKBytes = Shared::kKBytes, kVBlockBytes = Shared::kVBlockBytes;
+  constexpr uint32_t kVBlockBytes = Shared::kVBlockBytes;
   constexpr bool kSplitIssue = NB != 1;                   // P.V MMAs issued by a warp of their own
   constexpr int kRuns = kKeys / (2 * kCols);              // runs of 16 columns per thread and visit
   constexpr bool kLut = kLutBits != 0;
-  constexpr bool kCentered = kMode != kCorrected;
-  constexpr bool kF8 = kMode == kCentredF8;
   constexpr int kS = Shared::kS, kK = Shared::kK, kP = Shared::kP;      // ring depths (powers of two)
   constexpr int kAccCol = kS * kKeys;                     // first tensor-memory column of the P.V accumulators
   auto ring = [](int i, int depth) { return i & (depth - 1); };
@@ -144,10 +129,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, AttnParams P) {
   const int pieces = P.dh >> 4;                           // 16-byte pieces of a Q / K row
 
   if (tid == 0) {
-    for (int s = 0; s < kK; ++s) {
-      mbar_init(smem_u32(&S.k_full[s]), kCentered ? 1 : kGroupWarps);
-      mbar_init(smem_u32(&S.k_empty[s]), 1);
-    }
+    for (int s = 0; s < kK; ++s) mbar_init(smem_u32(&S.k_full[s]), kGroupWarps);
     for (int s = 0; s < kS; ++s) {
       mbar_init(smem_u32(&S.s_full[s]), 1);
       mbar_init(smem_u32(&S.s_empty[s]), kGroupWarps);
@@ -177,21 +159,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, AttnParams P) {
   grid_dependency_wait();
   grid_dependency_trigger();
 
-  // The first K tiles are asked for before the Q tile is staged (their barriers must be visible first), so that the
-  // copies' latency and the Q loads' run side by side.
-  int k_issued = 0;
-  if (kCentered) {
-    __syncthreads();
-    if (warp == kWorkWarps + 1 && lane == 0) {
-      for (; k_issued < kK && k_issued < 2 * nb; ++k_issued) {
-        const uint32_t bar = smem_u32(&S.k_full[k_issued]);
-        mbar_expect_tx(bar, kKBytes);
-        tma_load_3d(smem_u32(S.k[k_issued]), &map_k, bar, bi * int(P.k_si), (k_issued < nb ? k_issued : k_issued - nb) * kKeys, bo);
-      }
-    }
-  }
-
-  // ---- K rows (quantizers wider than 7 bits): a group stages the K tiles of its own visits, 8 threads per key with one
+  // ---- K rows: a group stages the K tiles of its own visits, 8 threads per key with one
   // 16-byte piece each, two keys per thread; Q rows: 4 threads per row, 2 pieces each
   const uint8_t* k_base = P.k + bo * P.k_so + bi * P.k_si;
   const int gt = tid & (kGroupThreads - 1);       // thread in group
@@ -206,7 +174,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, AttnParams P) {
       if (key < P.Lk && kq < pieces) kreg[u] = __ldg(reinterpret_cast<const uint4*>(k_base + int64_t(key) * P.ldk) + kq);
     }
   };
-  const uint32_t zq4 = uint32_t(P.zq) * 0x01010101u;
   // K tile and column terms of visit g from kreg; then the pieces of the group's visit after that are requested
   auto stage_k = [&](int g) {
     uint8_t* tile = S.k[ring(g, kK)];
@@ -226,7 +193,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, AttnParams P) {
   };
 
   if (warp < kWorkWarps) {
-    if (!kCentered && (tid >> 8) < 2 * nb) fetch_k((tid >> 8) < nb ? (tid >> 8) : (tid >> 8) - nb);   // the group's first visit
+    if ((tid >> 8) < 2 * nb) fetch_k((tid >> 8) < nb ? (tid >> 8) : (tid >> 8) - nb);   // the group's first visit
     const uint8_t* q_base = P.q + bo * P.q_so + bi * P.q_si;
     const int qrow = (tid >> 2) & (kRows - 1), qh = tid & 3;
     int s = 0;
@@ -234,11 +201,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, AttnParams P) {
     for (int j = 0; j < 2; ++j) {
       const int piece = 2 * qh + j;
       uint4 w = make_uint4(0u, 0u, 0u, 0u);
-      if (q0 + qrow < P.Lq && piece < pieces) {
-        w = __ldg(reinterpret_cast<const uint4*>(q_base + int64_t(q0 + qrow) * P.ldq) + piece);
-        if (kCentered) w = sub_bytes(w, zq4);
-        if (kF8) w = sign_magnitude(w);
-      }
+      if (q0 + qrow < P.Lq && piece < pieces) w = __ldg(reinterpret_cast<const uint4*>(q_base + int64_t(q0 + qrow) * P.ldq) + piece);
       if (piece < 2 * ksteps) *reinterpret_cast<uint4*>(S.q + tile_offset(qrow, piece)) = w;
       s += sum_bytes(w);
     }
@@ -288,11 +251,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, AttnParams P) {
     // ---------------------------------------------------------------- MMA issue
     if (lane == 0) {
       // S: D = s32, A = B = unsigned 8-bit, both K-major, N = 64, M = 128
-      // (operand formats: 0 = unsigned, 1 = signed bytes)
-      // kCentredF8: D = f32, A = B = e4m3 (format 0)
-      constexpr uint32_t idesc_s = kF8 ? (1u << 4) | (uint32_t(kKeys >> 3) << 17) | (uint32_t(kRows >> 4) << 24)
-                                       : (2u << 4) | (uint32_t(kCentered) << 7) | (0u << 10) | (uint32_t(kKeys >> 3) << 17) |
-                                             (uint32_t(kRows >> 4) << 24);
+      constexpr uint32_t idesc_s = (2u << 4) | (uint32_t(kKeys >> 3) << 17) | (uint32_t(kRows >> 4) << 24);
       const uint64_t dq = smem_desc_sw128(smem_u32(S.q));
       bool ok = true;
       auto issue_s = [&](int g) {                          // S of key block g % nb, g counted over both passes
@@ -310,11 +269,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, AttnParams P) {
         tc_fence_after();
         const uint64_t dk = smem_desc_sw128(smem_u32(S.k[kb]));
         for (int s = 0; s < ksteps; ++s) {
-          if (kF8) umma_f8(tmem_base + uint32_t(b * kKeys), dq + uint64_t(2 * s), dk + uint64_t(2 * s), idesc_s, s != 0 ? 1u : 0u);
-          else umma_i8(tmem_base + uint32_t(b * kKeys), dq + uint64_t(2 * s), dk + uint64_t(2 * s), idesc_s, s != 0 ? 1u : 0u);
+          umma_i8(tmem_base + uint32_t(b * kKeys), dq + uint64_t(2 * s), dk + uint64_t(2 * s), idesc_s, s != 0 ? 1u : 0u);
         }
         umma_commit(smem_u32(&S.s_full[b]));
-        if (kCentered) umma_commit(smem_u32(&S.k_empty[kb]));     // the K tile may be refilled once these MMAs have read it
         return true;
       };
       if (kSplitIssue) {
@@ -336,7 +293,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, AttnParams P) {
       umma_commit(smem_u32(&S.done));
       mbar_drain(smem_u32(&S.done), 0);
     }
-  } else if (kSplitIssue && warp == kWorkWarps + 2) {
+  } else if (kSplitIssue && warp == kWorkWarps + 1) {
     // ---------------------------------------------------------------- P.V MMA issue (wide heads)
     if (lane == 0) {
       bool ok = true;
@@ -344,23 +301,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, AttnParams P) {
       if (ok && !*abort) umma_commit(smem_u32(&S.acc_full));
       umma_commit(smem_u32(&S.done_pv));
       mbar_drain(smem_u32(&S.done_pv), 0);
-    }
-  } else if (warp == kWorkWarps + 1) {
-    // ---------------------------------------------------------------- K tiles by bulk tensor copies
-    if (kCentered && lane == 0) {
-      int issued = k_issued;
-      for (int g = k_issued; g < 2 * nb && !*abort; ++g) {
-        const int b = ring(g, kK);
-        if (!mbar_wait(smem_u32(&S.k_empty[b]), lap(g, kK) ^ 1u, abort, 48, P.status)) break;
-        const uint32_t bar = smem_u32(&S.k_full[b]);
-        mbar_expect_tx(bar, kKBytes);
-        // box: 128 bytes of the head's row (bytes past d_h meet zero bytes of the Q tile), 64 keys (rows past Lk are
-        // zero-filled), one batch item
-        tma_load_3d(smem_u32(S.k[b]), &map_k, bar, bi * int(P.k_si), (g < nb ? g : g - nb) * kKeys, bo);
-        ++issued;
-      }
-      // the copies issued last must have landed before this CTA may exit
-      for (int i = issued > kK ? issued - kK : 0; i < issued; ++i) mbar_drain(smem_u32(&S.k_full[ring(i, kK)]), lap(i, kK));
     }
   } else {
     // ---------------------------------------------------------------- tiles, Softmax arithmetic, epilogue
@@ -409,12 +349,11 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, AttnParams P) {
     auto begin_visit = [&](int g) -> bool {
       if (!mbar_wait(smem_u32(&S.s_full[ring(g, kS)]), lap(g, kS), abort, 44, P.status)) return false;
       tc_fence_after();
-      if (!kCentered && g + 2 < 2 * nb) stage_k(g + 2);
+      if (g + 2 < 2 * nb) stage_k(g + 2);
       return true;
     };
-    // Run h (16 columns) of the thread's scores of visit g in units of the score scale, as floats: the accumulator
-    // itself (kCentredF8), the converted accumulator (kCentred), or the converted corr = acc - z_k qsum - z_q ksum +
-    // d_h z_q z_k (kCorrected).  The buffer is handed back after the second run.  Keys the row may not see are dealt
+    // Run h (16 columns) of the thread's scores of visit g in units of the score scale, as floats: the converted
+    // corr = acc - z_k qsum - z_q ksum + d_h z_q z_k.  The buffer is handed back after the second run.  Keys the row may not see are dealt
     // with by the callers, in the runs that reach past the keys the thread's row sees: the values themselves are left
     // as they come from tensor memory, so that the common path carries no selects or copies.
     auto read_run = [&](int g, int h, float (&sf)[kCols]) {
@@ -427,22 +366,14 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, AttnParams P) {
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&S.s_empty[ring(g, kS)]));
       }
-      if (kF8) {
+      const int* ct = S.col_term[g & 3] + (half * kRuns + h) * kCols;
 #pragma unroll
-        for (int e = 0; e < kCols; ++e) sf[e] = __uint_as_float(rn[e]);
-      } else if (kCentered) {
-#pragma unroll
-        for (int e = 0; e < kCols; ++e) sf[e] = float(int32_t(rn[e]));
-      } else {
-        const int* ct = S.col_term[g & 3] + (half * kRuns + h) * kCols;
-#pragma unroll
-        for (int e4 = 0; e4 < kCols / 4; ++e4) {
-          const int4 c4 = *reinterpret_cast<const int4*>(ct + 4 * e4);
-          sf[4 * e4 + 0] = float(int32_t(rn[4 * e4 + 0]) + my_row_term + c4.x);
-          sf[4 * e4 + 1] = float(int32_t(rn[4 * e4 + 1]) + my_row_term + c4.y);
-          sf[4 * e4 + 2] = float(int32_t(rn[4 * e4 + 2]) + my_row_term + c4.z);
-          sf[4 * e4 + 3] = float(int32_t(rn[4 * e4 + 3]) + my_row_term + c4.w);
-        }
+      for (int e4 = 0; e4 < kCols / 4; ++e4) {
+        const int4 c4 = *reinterpret_cast<const int4*>(ct + 4 * e4);
+        sf[4 * e4 + 0] = float(int32_t(rn[4 * e4 + 0]) + my_row_term + c4.x);
+        sf[4 * e4 + 1] = float(int32_t(rn[4 * e4 + 1]) + my_row_term + c4.y);
+        sf[4 * e4 + 2] = float(int32_t(rn[4 * e4 + 2]) + my_row_term + c4.z);
+        sf[4 * e4 + 3] = float(int32_t(rn[4 * e4 + 3]) + my_row_term + c4.w);
       }
     };
 
@@ -543,7 +474,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, AttnParams P) {
     };
 
     bool ok = true;
-    if (!kCentered && group < 2 * nb) stage_k(group);          // the K tile of the group's first visit
+    if (group < 2 * nb) stage_k(group);          // the K tile of the group's first visit
     // ---- pass 1 over the group's visits
     for (int g = group; g < nb && !*abort; g += 2) {
       if (!begin_visit(g)) { ok = false; break; }
@@ -725,33 +656,17 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_k, AttnParams P) {
   }
 }
 
-template <int NB, int kLutBits, int kMode>
-repq_status launch_kernel(const AttnParams& P, int64_t pairs, cudaStream_t st) {
+template <int NB, int kLutBits>
+repq_status launch(const AttnParams& P, int64_t pairs, cudaStream_t st) {
   const size_t smem = sizeof(AttnShared<NB, kLutBits>);
-  REPQ_TRY((allow_smem<attention_tc_kernel<NB, kLutBits, kMode>>(int(smem))));
+  REPQ_TRY((allow_smem<attention_tc_kernel<NB, kLutBits>>(int(smem))));
   AttnParams Q = P;
   Q.pairs = int(pairs);
   Q.tiles = (P.Lq + kRows - 1) / kRows;
-  if (kMode == kCentredF8) Q.scale = P.scale * 262144.f;      // the accumulators hold 2^-18 sum (q - z_q) k
-  CUtensorMap map_k{};
-  if (kMode != kCorrected) REPQ_TRY(make_k_map(&map_k, P, int(pairs / P.batch_inner), VisitKeys<NB>::value));
   dim3 grid(unsigned(Q.tiles) * unsigned(pairs));
-  REPQ_CUDA(launch_chained(attention_tc_kernel<NB, kLutBits, kMode>, grid, dim3(Threads<NB>::value), smem, st, map_k, Q));
+  REPQ_CUDA(launch_chained(attention_tc_kernel<NB, kLutBits>, grid, dim3(Threads<NB>::value), smem, st, Q));
   note_launch();
   return REPQ_OK;
-}
-
-template <int NB, int kLutBits>
-repq_status launch(const AttnParams& P, int64_t pairs, int qmax_qk, cudaStream_t st) {
-  // q - z_q and k - z_k as signed bytes: codes and zero points below 128 and differences within [-128, 127]
-  // (the K tiles of this variant come by bulk tensor copies: row and batch strides must be usable as tensor-map strides)
-  const bool centred = qmax_qk < 128 && P.zq >= 0 && P.zq < 128 && P.zk >= 0 && P.zk < 128 && P.k_so > 0 &&
-                       P.ldk < (int64_t(1) << 40) && P.k_so < (int64_t(1) << 40) &&
-                       int64_t(P.batch_inner - 1) * P.k_si + P.dh <= P.ldk;
-  // 4-bit quantizers with the zero point of Q inside the code range: the tiles are also valid 8-bit floats
-  const bool f8 = centred && qmax_qk <= 15 && P.zq <= 15 && !P.no_f8;
-  if (f8) return launch_kernel<NB, kLutBits, kCentredF8>(P, pairs, st);
-  return centred ? launch_kernel<NB, kLutBits, kCentred>(P, pairs, st) : launch_kernel<NB, kLutBits, kCorrected>(P, pairs, st);
 }
 
 }  // namespace
@@ -819,15 +734,15 @@ extern "C" repq_status repq_attention(const repq_attention_desc* d, void* stream
     P.no_f8 = e && *e && *e != '0';
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (pipe_supported(P, qmax_v) && !getenv("ATT_OLD")) return launch_pipe(P, pairs, qmax_v, st);
+  if (pipe_supported(P, qmax_v)) return launch_pipe(P, pairs, qmax_v, st);
   // the per-lane table of the Softmax codes' operand values: 17 / 65 entries everywhere; the 257 entries of 8-bit codes
   // (33 KB) only where the head already limits the SM to one CTA
   if (d->d_h <= 64) {
-    if (P.qmax_p <= 15) return launch<1, 4>(P, pairs, qmax_v, st);
-    if (P.qmax_p <= 63) return launch<1, 6>(P, pairs, qmax_v, st);
-    return launch<1, 0>(P, pairs, qmax_v, st);
+    if (P.qmax_p <= 15) return launch<1, 4>(P, pairs, st);
+    if (P.qmax_p <= 63) return launch<1, 6>(P, pairs, st);
+    return launch<1, 0>(P, pairs, st);
   }
-  if (P.qmax_p <= 15) return launch<2, 4>(P, pairs, qmax_v, st);
-  if (P.qmax_p <= 63) return launch<2, 6>(P, pairs, qmax_v, st);
-  return launch<2, 8>(P, pairs, qmax_v, st);
+  if (P.qmax_p <= 15) return launch<2, 4>(P, pairs, st);
+  if (P.qmax_p <= 63) return launch<2, 6>(P, pairs, st);
+  return launch<2, 8>(P, pairs, st);
 }
