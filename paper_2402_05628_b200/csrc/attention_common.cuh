@@ -12,6 +12,10 @@ namespace attn {
 
 using namespace tc;
 
+__device__ __forceinline__ bool wait_for(uint32_t bar, uint32_t parity, volatile int* abort, int code, int32_t* status) {
+  return tc::mbar_wait<false>(bar, parity, abort, code, status);
+}
+
 constexpr int kRows = 128;                        // query rows per tile (MMA M)
 constexpr uint32_t kQBytes = kRows * 128;         // Q tile: rows of 128 bytes (the head's codes, zero-padded)
 constexpr uint32_t kMagicBits = 0x4B400000u;      // float 1.5 * 2^23

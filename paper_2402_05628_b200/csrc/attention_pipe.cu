@@ -253,16 +253,16 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     uint32_t ks = 0, kp = 0;                              // K ring: slot and parity
     bool ok = true;
     for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
-      if (!(ok = mbar_wait(smem_u32(&S.q_full), it & 1, abort, 40, P.status))) break;
+      if (!(ok = wait_for(smem_u32(&S.q_full), it & 1, abort, 40, P.status))) break;
       const uint64_t dq = smem_desc_sw128(smem_u32(S.q[it & 1]));
 #pragma unroll 1
       for (int b = 0; b < 2 * t.nb; ++b, ++g) {
         const int slot = g & 1;
         const uint32_t bit = 1u << slot;
-        if (!(ok = mbar_wait(smem_u32(&S.k_full[ks]), kp, abort, 41, P.status))) break;
+        if (!(ok = wait_for(smem_u32(&S.k_full[ks]), kp, abort, 41, P.status))) break;
         if (used & bit) {
           const bool spent = (pass2 & bit) != 0;
-          if (!(ok = mbar_wait(spent ? smem_u32(&S.s_spent[slot]) : smem_u32(&S.s_empty[slot]), ((spent ? ph_spent : ph_empty) >> slot) & 1u,
+          if (!(ok = wait_for(spent ? smem_u32(&S.s_spent[slot]) : smem_u32(&S.s_empty[slot]), ((spent ? ph_spent : ph_empty) >> slot) & 1u,
                                abort, 42, P.status))) break;
           if (spent) ph_spent ^= bit; else ph_empty ^= bit;
         }
@@ -302,11 +302,11 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     bool ok = true;
     for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
       g += t.nb;
-      if (it > 0 && !(ok = mbar_wait(smem_u32(&S.acc_empty), (it - 1) & 1, abort, 50, P.status))) break;
+      if (it > 0 && !(ok = wait_for(smem_u32(&S.acc_empty), (it - 1) & 1, abort, 50, P.status))) break;
 #pragma unroll 1
       for (int j = 0; j < t.nb; ++j, ++g) {
         const int slot = g & 1;
-        if (!(ok = mbar_wait(smem_u32(&S.p_full[slot]), (ph_p >> slot) & 1u, abort, 43, P.status))) break;
+        if (!(ok = wait_for(smem_u32(&S.p_full[slot]), (ph_p >> slot) & 1u, abort, 43, P.status))) break;
         ph_p ^= 1u << slot;
         tc_fence_after();
         const int left = t.k_end - j * kKeys;             // keys from the visit's first on
@@ -347,7 +347,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
       for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
 #pragma unroll 1
         for (int b = 0; b < 2 * t.nb; ++b) {
-          if (!(ok = mbar_wait(smem_u32(&S.k_empty[ks]), kp ^ 1u, abort, 48, P.status))) break;
+          if (!(ok = wait_for(smem_u32(&S.k_empty[ks]), kp ^ 1u, abort, 48, P.status))) break;
           const uint32_t bar = smem_u32(&S.k_full[ks]);
           mbar_expect_tx(bar, Shared::kKBytes);
           // box: 128 bytes of the head's row (bytes past d_h meet zero bytes of the Q tile), the visit's keys (rows past Lk
@@ -546,7 +546,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     // ---- epilogue of tile `it`: one row per thread (`roff`: its output offset, -1: past Lq), the 16-column chunks of the
     // accumulators dealt to the parts of a row
     auto finish = [&](int it, int64_t roff, int64_t sum_at) -> bool {
-              if (!mbar_wait(smem_u32(&S.acc_full), it & 1, abort, 47, P.status)) return false;
+              if (!wait_for(smem_u32(&S.acc_full), it & 1, abort, 47, P.status)) return false;
               tc_fence_after();
               const float out_scale = kLut ? P.out_scale : -2.f * P.out_scale;  // 8-bit floats: 2^8 A times 2^-9 (z_v - v)
               const uint32_t taddr = tmem_base + (uint32_t(quarter * 32) << 16) + uint32_t(kAccCol);
@@ -602,7 +602,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
         z = 0.f;
         for (int b = 0; b < t.nb; ++b, ++g) {
           const int slot = g & 1, first = b * kKeys + part * kCols;
-          if (!mbar_wait(smem_u32(&S.s_full[slot]), (g >> 1) & 1, abort, 44, P.status)) { ok = false; break; }
+          if (!wait_for(smem_u32(&S.s_full[slot]), (g >> 1) & 1, abort, 44, P.status)) { ok = false; break; }
           if (first < most) {                             // (warps whose columns no row sees only hand the slot back)
             tc_fence_after();
             float sf[kCols];
@@ -625,7 +625,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
       }
       if (kDefer && it > 0 && !finish(it - 1, done_row, done_sum)) break;
       if (!more) break;
-      if (!mbar_wait(smem_u32(&S.merged[quarter]), it & 1, abort, 45, P.status)) break;
+      if (!wait_for(smem_u32(&S.merged[quarter]), it & 1, abort, 45, P.status)) break;
       // m = max, Z = sum of the rescaled partial sums (same order in every thread of the row, so that all hold the same Z)
       float zt = 0.f;
 #pragma unroll
@@ -649,7 +649,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
       // ---- pass 2
       for (int j = 0; j < t.nb; ++j, ++g) {
         const int slot = g & 1, first = j * kKeys + part * kCols;
-        if (!mbar_wait(smem_u32(&S.v_empty[vs]), vp ^ 1u, abort, 46, P.status)) { ok = false; break; }
+        if (!wait_for(smem_u32(&S.v_empty[vs]), vp ^ 1u, abort, 46, P.status)) { ok = false; break; }
         stage_v(j, S.v[vs]);
         if (j + 1 < t.nb) fetch_v(j + 1);
         fence_async_smem();
@@ -659,7 +659,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
           more = tile_at<kKeys>(P, it + 1, blockIdx.x, gridDim.x, next);
           if (more) fetch_q(next);
         }
-        if (!mbar_wait(smem_u32(&S.s_full[slot]), (g >> 1) & 1, abort, 44, P.status)) { ok = false; break; }
+        if (!wait_for(smem_u32(&S.s_full[slot]), (g >> 1) & 1, abort, 44, P.status)) { ok = false; break; }
         // columns past the visit's last key are read by the MMAs only inside the step that holds it
         if (first < t.k_end) {
           tc_fence_after();

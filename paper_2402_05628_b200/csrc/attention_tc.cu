@@ -230,7 +230,7 @@ attention_tc_kernel(AttnParams P) {
   // B = the V tile in shared memory
   auto issue_pv = [&](int j) {
     const int pb = ring(j, kP);
-    if (!mbar_wait(smem_u32(&S.p_full[pb]), lap(j, kP), abort, 43, P.status)) return false;
+    if (!wait_for(smem_u32(&S.p_full[pb]), lap(j, kP), abort, 43, P.status)) return false;
     tc_fence_after();
     const uint64_t dv = smem_desc_sw128(smem_u32(S.v[pb]), kVBlockBytes);
     const int keys_here = min(kKeys, k_end - j * kKeys);
@@ -256,15 +256,15 @@ attention_tc_kernel(AttnParams P) {
       bool ok = true;
       auto issue_s = [&](int g) {                          // S of key block g % nb, g counted over both passes
         const int b = ring(g, kS), kb = ring(g, kK);
-        if (!mbar_wait(smem_u32(&S.k_full[kb]), lap(g, kK), abort, 41, P.status)) return false;
+        if (!wait_for(smem_u32(&S.k_full[kb]), lap(g, kK), abort, 41, P.status)) return false;
         // the slot's last user: a pass-1 visit (the workers have read it) or a pass-2 visit (its P.V MMAs have read
         // the operands the workers wrote over it)
         const int prev = g - kS;
         if (prev >= nb) {
           const int first = nb + ((b - nb) & (kS - 1));         // the slot's first pass-2 visit
-          if (!mbar_wait(smem_u32(&S.s_spent[b]), lap(prev - first, kS), abort, 42, P.status)) return false;
+          if (!wait_for(smem_u32(&S.s_spent[b]), lap(prev - first, kS), abort, 42, P.status)) return false;
         } else if (prev >= 0) {
-          if (!mbar_wait(smem_u32(&S.s_empty[b]), lap(prev, kS), abort, 42, P.status)) return false;
+          if (!wait_for(smem_u32(&S.s_empty[b]), lap(prev, kS), abort, 42, P.status)) return false;
         }
         tc_fence_after();
         const uint64_t dk = smem_desc_sw128(smem_u32(S.k[kb]));
@@ -347,7 +347,7 @@ attention_tc_kernel(AttnParams P) {
     // Start of a visit: the S MMAs of visit g have completed.  (Where the group stages its own K tiles, the tile of its
     // next visit is written here: with a ring of two it is the tile those MMAs have just finished reading.)
     auto begin_visit = [&](int g) -> bool {
-      if (!mbar_wait(smem_u32(&S.s_full[ring(g, kS)]), lap(g, kS), abort, 44, P.status)) return false;
+      if (!wait_for(smem_u32(&S.s_full[ring(g, kS)]), lap(g, kS), abort, 44, P.status)) return false;
       tc_fence_after();
       if (g + 2 < 2 * nb) stage_k(g + 2);
       return true;
@@ -493,7 +493,7 @@ attention_tc_kernel(AttnParams P) {
       S.stat_z[part][r] = z;
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&S.stats_ready));
-      ok = mbar_wait(smem_u32(&S.stats_ready), 0, abort, 45, P.status);
+      ok = wait_for(smem_u32(&S.stats_ready), 0, abort, 45, P.status);
     }
     const int g2 = nb + ((nb ^ group) & 1);                     // the group's first visit of pass 2
     if (ok && !*abort) {
@@ -528,7 +528,7 @@ attention_tc_kernel(AttnParams P) {
       }
       // the stage of the V tile: the MMAs of the block that used it before must have read it
       const int pb = ring(j, kP);
-      if (!mbar_wait(smem_u32(&S.p_empty[pb]), lap(j, kP) ^ 1u, abort, 46, P.status)) { ok = false; break; }
+      if (!wait_for(smem_u32(&S.p_empty[pb]), lap(j, kP) ^ 1u, abort, 46, P.status)) { ok = false; break; }
 #pragma unroll
       for (int qi = 0; qi < kVItems; ++qi) {
         uint32_t o4[4] = {0u, 0u, 0u, 0u};
@@ -569,7 +569,7 @@ attention_tc_kernel(AttnParams P) {
 
     // ---------------------------------------------------------------- epilogue: one row per thread, the 16-column
     // chunks of the accumulators dealt to the four warps of a lane quarter
-    if (ok && !*abort && mbar_wait(smem_u32(&S.acc_full), 0, abort, 47, P.status)) {
+    if (ok && !*abort && wait_for(smem_u32(&S.acc_full), 0, abort, 47, P.status)) {
       tc_fence_after();
       const float kSqrt2 = 1.41421356237309504880f;
       const float zo_lo = float(-P.zo), zo_hi = float(P.qmax - P.zo);

@@ -3,7 +3,9 @@
 // accumulators back with tcgen05.ld and applies the zero-point correction, scale, bias, GELU, residual
 // and re-quantization of the quantized linear layer.
 //
-// One persistent CTA per SM; roles by warp:
+// One persistent CTA per SM, or a pair of CTAs (a cluster of two) on a 256 x 256 tile where K is long: each CTA copies its
+// own 128 rows of activations and half of the weight tile, one thread of the even CTA issues the MMAs of both
+// (cta_group::2), each CTA holds and finishes the 128 output rows of its own.  Roles by warp:
 //   warp 0       TMA producer (one elected lane): A tile 128 x 128 B, W tile BN x 128 B per stage, 128-byte
 //                swizzle, zero fill outside the matrices
 //   warp 1       tensor-memory allocation and MMA issue (one elected lane): 4 MMAs of K = 32 per stage,
@@ -45,7 +47,6 @@ constexpr int BM = 128, BK = 128;                   // BK in bytes (= codes); BN
 constexpr int kMaxBN = 256;
 constexpr int kChunk = 16;                           // accumulator columns per tcgen05.ld / per store
 constexpr int kEpiWarps = 16;
-constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kThreads = 32 * (2 + kEpiWarps);
 constexpr int kTmemCols = 512;
 constexpr int kAccStride = 256;                      // TMEM columns between the two accumulator buffers
@@ -73,18 +74,19 @@ constexpr uint32_t kResBytes = 32 * 128;            // bf16 residual of one warp
 // copies, one 32 x 64 box per epilogue warp, asked for one tile ahead; the output values are written over the residual
 // values they were computed from and the box leaves by one bulk tensor store (no staging buffer beside it)
 // WP: 0 = weight tiles arrive as bytes; 4 / 6 = packed (64 / 96 bytes per row of 128 codes), expanded by the converters
-template <int BN, bool RES, int WP>
+template <int BN, bool RES, int WP, bool TWO = false>
 struct SharedStorage {
   static constexpr bool W4 = WP != 0;               // (any packed form)
   // kStages: ring of the bulk copies (activation tile + weight tile as it arrives).  kStagesB: ring of byte weight
   // tiles the MMA reads: the same ring when the weights arrive as bytes; with packed weights a short ring of its own
   // (the hop from converter to MMA is short), which leaves room for a deeper copy ring ahead of the converters.
-  static constexpr int kStages = WP == 6 ? 4 : WP == 4 ? 5 : 4;
+  static constexpr int kStages = TWO ? 6 : WP == 4 ? 5 : 4;
   static constexpr int kPackedRow = BK * (WP ? WP : 8) / 8;        // bytes of a packed tile row
   static constexpr int kStagesB = W4 ? 2 : kStages;
   static constexpr int kEpi = W4 ? kEpiWarpsW4 : kEpiWarps;
   alignas(1024) uint8_t a[kStages][kABytes];
-  alignas(1024) uint8_t b[kStagesB][BN * BK];
+  static constexpr int kBRows = TWO ? BN / 2 : BN;                // weight rows of this CTA's stage (a pair: half of the tile's)
+  alignas(1024) uint8_t b[kStagesB][kBRows * BK];
   alignas(1024) uint8_t res[RES ? (BN / kSliceCols) * 4 * kResBytes : 1024];   // one box per active epilogue warp
   uint64_t res_full[kEpiWarps];
   alignas(1024) uint8_t epi[RES ? 1 : kEpi][1024]; // per-warp staging box of the epilogue's bulk stores (RES: the residual box itself)
@@ -102,7 +104,8 @@ struct SharedStorage {
 };
 
 static_assert(sizeof(SharedStorage<kMaxBN, false, 0>) <= 227 * 1024 && sizeof(SharedStorage<kMaxBNW4, false, 4>) <= 227 * 1024 &&
-              sizeof(SharedStorage<kMaxBNW4, false, 6>) <= 227 * 1024 && sizeof(SharedStorage<192, true, 0>) <= 227 * 1024,
+              sizeof(SharedStorage<kMaxBNW4, false, 6>) <= 227 * 1024 && sizeof(SharedStorage<192, true, 0>) <= 227 * 1024 &&
+              sizeof(SharedStorage<kMaxBN, false, 0, true>) <= 227 * 1024,
               "shared storage exceeds the 227 KB a CTA may use");
 
 using namespace tc;
@@ -114,9 +117,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 // Shared-memory matrix descriptor: K-major rows of 128 bytes, 128-byte swizzle, 8-row groups 1024 B apart.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) { return smem_desc_sw128(addr); }
 
-// Instruction descriptor: D = s32, A = B = unsigned 8-bit, both K-major, N = bn, M = 128.
-constexpr uint32_t idesc_for(int bn) {
-  return (2u << 4) | (0u << 7) | (0u << 10) | (uint32_t(bn >> 3) << 17) | (uint32_t(BM >> 4) << 24);
+// Instruction descriptor: D = s32, A = B = unsigned 8-bit, both K-major, N = bn, M = bm.
+constexpr uint32_t idesc_for(int bn, int bm) {
+  return (2u << 4) | (0u << 7) | (0u << 10) | (uint32_t(bn >> 3) << 17) | (uint32_t(bm >> 4) << 24);
 }
 
 // Order of the output tiles.  The row tiles are cut into panels of P.panel; a panel is walked column tile by column
@@ -141,7 +144,7 @@ struct TileOrder {
   FastDiv by_panel, by_last_rows;
 };
 struct TileOrigin { int m0, n0; };
-__device__ __forceinline__ TileOrigin tile_origin(int tile, const TileOrder& T, int bn) {
+__device__ __forceinline__ TileOrigin tile_origin(int tile, const TileOrder& T, int bm, int bn) {
   uint32_t rows = uint32_t(T.panel), first = 0, t = uint32_t(tile);
   uint32_t col;
   if (tile >= T.full) {                                          // the last, shorter panel
@@ -155,7 +158,7 @@ __device__ __forceinline__ TileOrigin tile_origin(int tile, const TileOrder& T, 
     t -= p * T.by_panel_tiles.d;
     col = div_by(t, T.by_panel);
   }
-  return TileOrigin{int(first + (t - col * rows)) * BM, int(col) * bn};
+  return TileOrigin{int(first + (t - col * rows)) * bm, int(col) * bn};
 }
 
 struct TcParams {
@@ -165,6 +168,7 @@ struct TcParams {
   int direct_requant;          // codes out, no GELU, no residual: 1/s_o is folded into the column terms
   int w_packed4;               // weight tiles arrive packed (4: two codes per byte, 6: four in three bytes) and are
                                // expanded in shared memory; 0: byte tiles
+  int pair;                    // 256-row tiles by pairs of CTAs
   TileOrder order;             // panels of row tiles (see TileOrder)
   EpilogueParams ep;
 };
@@ -402,24 +406,28 @@ __device__ __noinline__ void slow_chunk(const EpilogueParams& ep, const TcParams
 // where asked for: kPairNone, kPairRope (rotary embedding), kPairGlu (gated product; byte codes out)
 enum : int { kPairNone = 0, kPairRope = 1, kPairGlu = 2 };
 
-template <int BN, int OUT, bool RES, int PAIR, int WP>
+template <int BN, int OUT, bool RES, int PAIR, int WP, bool TWO>
 __global__ void __launch_bounds__(kThreads, 1)
 qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                 const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res, const __grid_constant__ TcParams P) {
-  using Storage = SharedStorage<BN, RES, WP>;
+  using Storage = SharedStorage<BN, RES, WP, TWO>;
+  constexpr int kTileM = TWO ? 2 * BM : BM;              // rows of a tile (a pair of CTAs: 128 each)
+  static_assert(!TWO || WP == 0, "a pair takes weights stored as bytes");
   constexpr bool W4 = WP != 0;                           // weights arrive packed
   constexpr int kStages = Storage::kStages;
   constexpr int EW = W4 ? kEpiWarpsW4 : kEpiWarps;       // epilogue warps of this variant
   static_assert(!W4 || BN <= kMaxBNW4, "the packed-weight variant has three column slices");
-  constexpr uint32_t kBBytes = BN * BK;
-  constexpr uint32_t kIdesc = idesc_for(BN);
+  constexpr uint32_t kBBytes = Storage::kBRows * BK;
+  constexpr uint32_t kIdesc = idesc_for(BN, kTileM);
+  const int rank = TWO ? int(blockIdx.x) & 1 : 0;        // CTA in the pair; the even one issues the MMAs of both
+  const int tile0 = TWO ? int(blockIdx.x) >> 1 : int(blockIdx.x), tile_step = TWO ? int(gridDim.x) >> 1 : int(gridDim.x);
   // 1024-byte alignment (swizzle atoms) is requested from the declaration so that the compiler keeps
   // treating every access below as a shared-memory access (a hand-aligned generic pointer would not)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   Storage& S = *reinterpret_cast<Storage*>(smem_raw);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m_tiles = (P.M + BM - 1) / BM, n_tiles = (P.N + BN - 1) / BN;
+  const int m_tiles = (P.M + kTileM - 1) / kTileM, n_tiles = (P.N + BN - 1) / BN;
   const int tiles = m_tiles * n_tiles;
   const int kblocks = (P.K + BK - 1) / BK;
 
@@ -429,7 +437,7 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       mbar_init(smem_u32(&S.empty[s]), 1);
     }
     for (int s = 0; s < Storage::kStagesB; ++s) { mbar_init(smem_u32(&S.ready[s]), kConvWarps); mbar_init(smem_u32(&S.bfree[s]), 1); }
-    for (int a = 0; a < 2; ++a) { mbar_init(smem_u32(&S.tmem_full[a]), 1); mbar_init(smem_u32(&S.tmem_empty[a]), EW); }
+    for (int a = 0; a < 2; ++a) { mbar_init(smem_u32(&S.tmem_full[a]), 1); mbar_init(smem_u32(&S.tmem_empty[a]), TWO ? 2 * EW : EW); }
     for (int w = 0; w < kEpiWarps; ++w) mbar_init(smem_u32(&S.res_full[w]), 1);
     mbar_init(smem_u32(&S.done), 1);
     S.abort = 0;
@@ -440,10 +448,16 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.tmem_base)), "n"(kTmemCols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (TWO) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.tmem_base)), "n"(kTmemCols) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.tmem_base)), "n"(kTmemCols) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   tc_fence_before();
+  if (TWO) cluster_sync();                                 // (the barriers of both CTAs are set up)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = S.tmem_base;
@@ -457,12 +471,22 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     if (lane == 0) {
       uint32_t stage = 0, phase = 0;
       long long issued = 0;
-      for (int tile = blockIdx.x; tile < tiles && !*abort; tile += gridDim.x) {
-        const TileOrigin o = tile_origin(tile, P.order, BN);
-        const int m0 = o.m0, n0 = o.n0;
+      for (int tile = tile0; tile < tiles && !*abort; tile += tile_step) {
+        const TileOrigin o = tile_origin(tile, P.order, kTileM, BN);
+        const int m0 = o.m0 + rank * BM, n0 = o.n0 + rank * (BN / 2);
         for (int kb = 0; kb < kblocks; ++kb) {
           if (!mbar_wait(smem_u32(&S.empty[stage]), phase ^ 1, abort, 1)) break;
           const uint32_t bar = smem_u32(&S.full[stage]);
+          if constexpr (TWO) {
+            // both CTAs' copies report to the even one's barrier, which its MMA thread waits on
+            if (rank == 0) mbar_expect_tx(bar, 2 * (kABytes + kBBytes));
+            const uint32_t lead = map_to_rank(bar, 0);
+            tma_load_2d_pair(smem_u32(S.a[stage]), &map_a, lead, kb * BK, m0);
+            tma_load_2d_pair(smem_u32(S.b[stage]), &map_b, lead, kb * BK, n0);
+            ++issued;
+            if (++stage == kStages) { stage = 0; phase ^= 1; }
+            continue;
+          }
           mbar_expect_tx(bar, kABytes + (W4 ? uint32_t(BN * Storage::kPackedRow) : kBBytes));
           tma_load_2d(smem_u32(S.a[stage]), &map_a, bar, kb * BK, m0);
           if constexpr (W4) tma_load_2d(smem_u32(S.bp[stage]), &map_b, bar, kb * Storage::kPackedRow, n0);
@@ -471,8 +495,8 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           if (++stage == kStages) { stage = 0; phase ^= 1; }
         }
       }
-      // drain: the copies issued last must have landed before this CTA may exit
-      const int back = issued < kStages ? int(issued) : kStages;
+      // drain: the copies issued last must have landed before this CTA may exit (a pair: its even CTA waits for both)
+      const int back = rank != 0 ? 0 : issued < kStages ? int(issued) : kStages;
       uint32_t s = stage, ph = phase;
       for (int i = 0; i < back; ++i) {
         if (s == 0) { s = kStages - 1; ph ^= 1; } else { --s; }
@@ -482,10 +506,13 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issue
-    if (lane == 0) {
+    if (lane == 0 && rank == 0) {
+      auto commit = [](uint32_t bar) {
+        if constexpr (TWO) umma_commit_pair(bar); else umma_commit(bar);
+      };
       uint32_t stage = 0, phase = 0, bstage = 0, bphase = 0;
       int it = 0;
-      for (int tile = blockIdx.x; tile < tiles && !*abort; tile += gridDim.x, ++it) {
+      for (int tile = tile0; tile < tiles && !*abort; tile += tile_step, ++it) {
         const uint32_t acc = it & 1, acc_phase = (it >> 1) & 1;
         if (!mbar_wait(smem_u32(&S.tmem_empty[acc]), acc_phase ^ 1, abort, 2)) break;
         tc_fence_after();
@@ -498,20 +525,22 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           tc_fence_after();
           const uint64_t da = smem_desc(smem_u32(S.a[stage])), db = smem_desc(smem_u32(S.b[W4 ? bstage : stage]));
 #pragma unroll
-          for (int k = 0; k < BK / 32; ++k)
-            umma_i8(d_tmem, da + uint64_t(k * 2), db + uint64_t(k * 2), kIdesc, (kb | k) != 0 ? 1u : 0u);
-          umma_commit(smem_u32(&S.empty[stage]));          // frees the stage once these MMAs have read it
+          for (int k = 0; k < BK / 32; ++k) {
+            if constexpr (TWO) umma_i8_pair(d_tmem, da + uint64_t(k * 2), db + uint64_t(k * 2), kIdesc, (kb | k) != 0 ? 1u : 0u);
+            else umma_i8(d_tmem, da + uint64_t(k * 2), db + uint64_t(k * 2), kIdesc, (kb | k) != 0 ? 1u : 0u);
+          }
+          commit(smem_u32(&S.empty[stage]));               // frees the stage once these MMAs have read it
           if (++stage == kStages) { stage = 0; phase ^= 1; }
           if constexpr (W4) {
-            umma_commit(smem_u32(&S.bfree[bstage]));       // and the byte tile for the converters
+            commit(smem_u32(&S.bfree[bstage]));       // and the byte tile for the converters
             if (++bstage == Storage::kStagesB) { bstage = 0; bphase ^= 1; }
           }
         }
         if (!ok) break;
-        umma_commit(smem_u32(&S.tmem_full[acc]));           // accumulator complete
+        commit(smem_u32(&S.tmem_full[acc]));                // accumulator complete
       }
       // all MMAs issued by this thread must have completed before tensor memory is freed
-      umma_commit(smem_u32(&S.done));
+      commit(smem_u32(&S.done));
       const long long t0 = clock64();
       while (!mbar_try_wait(smem_u32(&S.done), 0) && clock64() - t0 < kWaitCycles) {}
     }
@@ -524,7 +553,7 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     const int ct = int(threadIdx.x) - 32 * (2 + EW);
     uint32_t stage = 0, phase = 0, bstage = 0, bphase = 0;
     bool ok = true;
-    for (int tile = blockIdx.x; tile < tiles && ok && !*abort; tile += gridDim.x) {
+    for (int tile = tile0; tile < tiles && ok && !*abort; tile += tile_step) {
       for (int kb = 0; kb < kblocks; ++kb) {
         // the packed tile has landed, and the MMAs that read the byte tile's previous content have completed
         if (!mbar_wait(smem_u32(&S.full[stage]), phase, abort, 7)) { ok = false; break; }
@@ -607,8 +636,8 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     float nx_sw[2] = {0.f, 0.f}, nx_bs[2] = {0.f, 0.f};
     auto fetch_terms = [&](int t) {
       if (t >= tiles || !slice_on) return;
-      const TileOrigin o = tile_origin(t, P.order, BN);
-      const int tm0 = o.m0, tn0 = o.n0;
+      const TileOrigin o = tile_origin(t, P.order, kTileM, BN);
+      const int tm0 = o.m0 + rank * BM, tn0 = o.n0;
       // plain loads from clamped indices: nothing here may consume a loaded value (a select on it would hold the
       // warp until the load returns); rows and columns outside the matrix are dealt with where the values are used
       const int64_t tm = min(int64_t(tm0) + quarter * 32 + lane, int64_t(P.M) - 1);
@@ -628,8 +657,8 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     bool res_pending = false;
     auto fetch_residual = [&](int t) {
       if (!RES || t >= tiles || !slice_on) return;
-      const TileOrigin o = tile_origin(t, P.order, BN);
-      const int tm0 = o.m0, tn0 = o.n0;
+      const TileOrigin o = tile_origin(t, P.order, kTileM, BN);
+      const int tm0 = o.m0 + rank * BM, tn0 = o.n0;
       if (lane == 0) {
         // the box's last content may still be on its way out (the bulk store of the previous tile reads it)
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -638,13 +667,13 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       }
       res_pending = true;
     };
-    fetch_residual(blockIdx.x);
-    fetch_terms(blockIdx.x);
+    fetch_residual(tile0);
+    fetch_terms(tile0);
     int it = 0;
-    for (int tile = blockIdx.x; tile < tiles && !*abort; tile += gridDim.x, ++it) {
+    for (int tile = tile0; tile < tiles && !*abort; tile += tile_step, ++it) {
       const uint32_t acc = it & 1, acc_phase = (it >> 1) & 1;
-      const TileOrigin o = tile_origin(tile, P.order, BN);
-      const int m0 = o.m0, n0 = o.n0;
+      const TileOrigin o = tile_origin(tile, P.order, kTileM, BN);
+      const int m0 = o.m0 + rank * BM, n0 = o.n0;
       const int64_t m = int64_t(m0) + quarter * 32 + lane;
       const bool row_ok = m < P.M;
       // warp-uniform: whole 64-column slice inside the matrix, common epilogue (rows beyond M are clipped by
@@ -690,7 +719,7 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         }
         __syncwarp();
       }
-      fetch_terms(tile + int(gridDim.x));                    // next tile's inputs: in flight during this epilogue
+      fetch_terms(tile + tile_step);                    // next tile's inputs: in flight during this epilogue
       int code_sum = 0;
       // rotary embedding: this row's line of the (cos, sin) table and the slice's first column inside its head
       const float2* rope_row = nullptr;
@@ -846,8 +875,11 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       // accumulator buffer free again
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&S.tmem_empty[acc]));
-      fetch_residual(tile + int(gridDim.x));               // every lane has read this tile's box (the __syncwarp above)
+      if (lane == 0) {
+        if constexpr (TWO) mbar_arrive_cluster(map_to_rank(smem_u32(&S.tmem_empty[acc]), 0));
+        else mbar_arrive(smem_u32(&S.tmem_empty[acc]));
+      }
+      fetch_residual(tile + tile_step);               // every lane has read this tile's box (the __syncwarp above)
       if (ep.out_row_sum != nullptr && row_ok && code_sum != 0) atomicAdd(ep.out_row_sum + m, code_sum);
     }
     if (RES && res_pending) mbar_drain(res_bar, uint32_t(it) & 1u);              // left the loop early: the copy must land
@@ -857,9 +889,11 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   // ------------------------------------------------------------------ teardown
   tc_fence_before();
   __syncthreads();
+  if (TWO) cluster_sync();                                 // neither CTA leaves while the other may still reach its memory
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(kTmemCols) : "memory");
+    if constexpr (TWO) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(kTmemCols) : "memory");
+    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(kTmemCols) : "memory");
   }
 }
 
@@ -933,6 +967,28 @@ int pick_bn(int M, int N, int K, int sms, bool w_packed4, bool res_boxes) {
   return best;
 }
 
+// Whether 256 x 256 tiles by pairs of CTAs beat 128-row tiles of bn columns.  A pair copies a third less operand bytes per
+// operation, so a k-block takes 0.285 us instead of 0.365 (256 columns); an epilogue takes as long as on a 128 x 256 tile, and
+// there are half as many, twice as large pieces to deal out.  (Microseconds; fitted to M 300..16384, N 768..12288, K
+// 768..11008.  8192 x 4096 x 11008 with residual 250 -> 205 us, 8192 x 12288 x 4096 to codes 234 -> 216, 777 x 4096 x 11008 40 ->
+// 35; at K = 768 the epilogue sets the pace and narrow tiles stay.)
+bool pair_is_faster(const TcParams& P, int bn, int sms) {
+  if (P.w_packed4) return false;
+  const float kb = float((P.K + BK - 1) / BK);
+  const bool res16 = P.ep.residual != nullptr && P.ep.residual_bf16;
+  auto rounds = [&](int tm, int tn, int slots) {
+    const long tiles = long((P.M + tm - 1) / tm) * ((P.N + tn - 1) / tn);
+    return float((tiles + slots - 1) / slots);
+  };
+  const float width = float(bn + 160) / 416.f;           // a round's time against that of 256 columns (see pick_bn)
+  const float epi256 = res16 ? 10.2f : 5.2f;             // residual by row-per-lane loads; otherwise
+  const float main1 = (2.0f + 0.365f * kb) * width, epi1 = residual_boxes(P) && bn < kMaxBN ? 5.5f : epi256 * width;
+  const float main2 = 2.2f + 0.285f * kb;
+  const float single = rounds(BM, bn, sms) * (main1 > epi1 ? main1 : epi1);
+  const float pair = rounds(2 * BM, kMaxBN, sms / 2) * (main2 > epi256 ? main2 : epi256);
+  return pair * 1.08f < single;
+}
+
 // Tensor map of the output for the epilogue's bulk stores: boxes of 32 rows x 32 bytes, 32-byte swizzle.
 repq_status make_out_map(CUtensorMap* map, const TcParams& P) {
   EncodeTiledFn fn = encode_fn();
@@ -969,7 +1025,7 @@ repq_status make_box_map(CUtensorMap* map, const TcParams& P, const void* base, 
   return REPQ_OK;
 }
 
-template <int BN, int OUT, bool RES, int PAIR, int WP>
+template <int BN, int OUT, bool RES, int PAIR, int WP, bool TWO = false>
 repq_status launch_tc_w(const CUtensorMap& map_a, const CUtensorMap& map_b, const TcParams& P, int sms, cudaStream_t st) {
   CUtensorMap map_out, map_res;
   if (RES) {
@@ -979,11 +1035,14 @@ repq_status launch_tc_w(const CUtensorMap& map_a, const CUtensorMap& map_b, cons
     REPQ_TRY(make_out_map(&map_out, P));
     map_res = map_out;                                     // not read
   }
-  const size_t smem = sizeof(SharedStorage<BN, RES, WP>);
-  REPQ_TRY((allow_smem<qgemm_tc_kernel<BN, OUT, RES, PAIR, WP>>(int(smem))));
-  const int tiles = ((P.M + BM - 1) / BM) * ((P.N + BN - 1) / BN);
-  const int grid = tiles < sms ? tiles : sms;
-  REPQ_CUDA(launch_chained(qgemm_tc_kernel<BN, OUT, RES, PAIR, WP>, dim3(grid), dim3(kThreads), smem, st, map_a, map_b, map_out, map_res, P));
+  const size_t smem = sizeof(SharedStorage<BN, RES, WP, TWO>);
+  auto kern = qgemm_tc_kernel<BN, OUT, RES, PAIR, WP, TWO>;
+  REPQ_TRY((allow_smem<qgemm_tc_kernel<BN, OUT, RES, PAIR, WP, TWO>>(int(smem))));
+  constexpr int kTileM = TWO ? 2 * BM : BM;
+  const int tiles = ((P.M + kTileM - 1) / kTileM) * ((P.N + BN - 1) / BN);
+  const int slots = TWO ? sms / 2 : sms;
+  const int grid = (tiles < slots ? tiles : slots) * (TWO ? 2 : 1);
+  REPQ_CUDA(launch_chained_cluster(kern, dim3(grid), dim3(kThreads), smem, st, TWO ? 2 : 1, map_a, map_b, map_out, map_res, P));
   note_launch();
   return REPQ_OK;
 }
@@ -993,6 +1052,9 @@ repq_status launch_tc_res(const CUtensorMap& map_a, const CUtensorMap& map_b, co
   if constexpr (!RES && BN <= kMaxBNW4) {
     if (P.w_packed4 == 4) return launch_tc_w<BN, OUT, false, PAIR, 4>(map_a, map_b, P, sms, st);
     if (P.w_packed4 == 6) return launch_tc_w<BN, OUT, false, PAIR, 6>(map_a, map_b, P, sms, st);
+  }
+  if constexpr (!RES && BN == kMaxBN) {
+    if (P.pair) return launch_tc_w<BN, OUT, RES, PAIR, 0, true>(map_a, map_b, P, sms, st);
   }
   return launch_tc_w<BN, OUT, RES, PAIR, 0>(map_a, map_b, P, sms, st);
 }
@@ -1103,15 +1165,19 @@ repq_status qgemm_tc(const repq_gemm_desc& d, const EpilogueParams& ep, void* ws
   P.direct_requant = d.out_kind == REPQ_OUT_CODES && !d.gelu && !d.residual && !d.glu;
   REPQ_REQUIRE(device_status_word() != nullptr, REPQ_CUDA_ERROR, "qgemm: device status word unavailable");
   const int sms = sm_count();
-  const int bn = pick_bn(d.M, d.N, d.K, sms, P.w_packed4 != 0, residual_boxes(P));
+  int bn = pick_bn(d.M, d.N, d.K, sms, P.w_packed4 != 0, residual_boxes(P));
+  P.pair = pair_is_faster(P, bn, sms);
+  if (P.pair) bn = kMaxBN;
   {
     // panels of activations: all row tiles while the activations take at most 40 MB (a third of the L2 capacity),
     // else about 24 MB (measured at 8192 x 4096 x 11008 with residual: 248 us with 40 MB panels, 240-242 with
     // 12..30 MB: the weight tiles and the residual / output rows stream through the same L2), at least 8 row tiles
-    const int m_tiles = (d.M + BM - 1) / BM, n_tiles = (d.N + bn - 1) / bn;
+    const int tile_m = P.pair ? 2 * BM : BM;
+    const int m_tiles = (d.M + tile_m - 1) / tile_m, n_tiles = (d.N + bn - 1) / bn;
     const int64_t a_bytes = int64_t(d.M) * d.K;
-    const int64_t fit = (int64_t(a_bytes <= (int64_t(40) << 20) ? 40 : 24) << 20) / (int64_t(BM) * d.K);
-    int panel = int(fit < 8 ? 8 : fit);
+    const int64_t fit = (int64_t(a_bytes <= (int64_t(40) << 20) ? 40 : 24) << 20) / (int64_t(tile_m) * d.K);
+    const int least = 1024 / tile_m;
+    int panel = int(fit < least ? least : fit);
     if (panel > m_tiles) panel = m_tiles;
     TileOrder& T = P.order;
     T.panel = panel;
@@ -1126,7 +1192,7 @@ repq_status qgemm_tc(const repq_gemm_desc& d, const EpilogueParams& ep, void* ws
   CUtensorMap map_a, map_b;
   REPQ_TRY(make_map(&map_a, a, d.M, d.K, lda, BM));
   if (P.w_packed4) REPQ_TRY(make_map(&map_b, d.w_codes, d.N, code_row_bytes(d.K, d.bits_w), d.ldw_bytes, bn, BK * P.w_packed4 / 8, false));
-  else REPQ_TRY(make_map(&map_b, d.w_codes, d.N, d.K, d.ldw_bytes, bn));
+  else REPQ_TRY(make_map(&map_b, d.w_codes, d.N, d.K, d.ldw_bytes, P.pair ? bn / 2 : bn));
   if (bn == 256) return launch_tc<256>(map_a, map_b, P, sms, st);
   if (bn == 192) return launch_tc<192>(map_a, map_b, P, sms, st);
   return launch_tc<128>(map_a, map_b, P, sms, st);
