@@ -21,7 +21,8 @@
  *    quantizer is unchanged, but its codes are stored one per byte.  That is the operand format of
  *    the 8-bit integer tensor-core instruction, so 4-bit tensors kept this way need no expansion pass
  *    before a GEMM; the packed form is for storage and interchange.  Weight codes of 6 bits may also be
- *    stored four to three bytes (REPQ_PACKED6); the GEMM expands packed weight tiles in shared memory.
+ *    stored four to three bytes (REPQ_PACKED6); the GEMM expands packed weights, into its workspace or tile by tile in shared
+ *    memory.
  *    Code tensors are row-major with a row stride in BYTES; float tensors use strides in ELEMENTS.
  *  - Weights are stored [out features j, in features c] (row j is the paper's column W[:, j]).
  *  - Zero-points are plain integers of any sign (Eq. 6 does not bound them).

@@ -1,6 +1,7 @@
 // repq_block_forward: one quantized transformer block (Eqs. 1-3) as a stream-ordered sequence of the
 // stage kernels.  No host synchronisation, no allocation: every intermediate lives in the caller's
 // workspace.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 
@@ -12,7 +13,7 @@ namespace {
 struct BlockLayout {
   int64_t M, ld_a, ld_qkv, ld_s, ld_p, ld_h;
   size_t off_ln, off_asum, off_qkv, off_scores, off_p, off_attn, off_asum_attn, off_xbar, off_hidden,
-      off_asum_h, off_gemm_ws, gemm_ws, total;
+      off_asum_h, off_gemm_ws, total, least;   // (total: with room for the byte form of packed weights; least: without)
 };
 
 inline size_t bump(size_t& cur, size_t bytes) {
@@ -78,18 +79,20 @@ BlockLayout layout(const repq_block_desc& d) {
   L.off_hidden = bump(cur, size_t(L.M * L.ld_h));
   // scratch of the largest GEMM of the block
   repq_linear_params none{};
-  size_t ws = 0;
+  size_t ws = 0, ws_least = 0;
   const int n_fc1 = d.mlp_kind == REPQ_MLP_SWIGLU ? 2 * d.mlp : d.mlp;
   const int shapes[4][2] = {{3 * d.dim, d.dim}, {d.dim, d.dim}, {n_fc1, d.dim}, {d.dim, d.mlp}};
   for (auto& s : shapes) {
     repq_gemm_desc g = linear_desc(d, L.M, s[0], s[1], nullptr, code_row_bytes(s[1], act_bits(d)), 1.f, 0, nullptr, none);
     g.ldw_bytes = round_up(code_row_bytes(s[1], d.bits_w), 16);
     g.lda_bytes = round_up(code_row_bytes(s[1], act_bits(d)), 16);
-    if (qgemm_tc_supported(g)) ws = ws > qgemm_tc_workspace(g) ? ws : qgemm_tc_workspace(g);
+    g.a_row_sum = g.w_row_sum = reinterpret_cast<const int32_t*>(16);      // (given in a block: not part of the scratch)
+    ws = std::max(ws, qgemm_workspace(g));
+    ws_least = std::max(ws_least, qgemm_workspace_least(g));
   }
-  L.gemm_ws = ws;
-  L.off_gemm_ws = bump(cur, ws);
-  L.total = cur;
+  L.off_gemm_ws = cur;                                  // the last part of the workspace
+  L.total = cur + (ws + 255) / 256 * 256;
+  L.least = cur + (ws_least + 255) / 256 * 256;
   return L;
 }
 
@@ -114,8 +117,8 @@ static repq_status block_forward_impl(const repq_block_desc* dp, const repq_bloc
   REPQ_TRY(validate(d));
   REPQ_REQUIRE(!d.rope || p.rope_cos_sin != nullptr, REPQ_INVALID_ARG, "block_forward: rope is set but rope_cos_sin is NULL");
   const BlockLayout L = layout(d);
-  REPQ_REQUIRE(workspace && workspace_bytes >= L.total, REPQ_WORKSPACE_TOO_SMALL,
-               "block_forward: workspace of %zu bytes given, %zu needed", workspace_bytes, L.total);
+  REPQ_REQUIRE(workspace && workspace_bytes >= L.least, REPQ_WORKSPACE_TOO_SMALL,
+               "block_forward: workspace of %zu bytes given, %zu needed", workspace_bytes, L.least);
   REPQ_REQUIRE(aligned(workspace, 256), REPQ_ALIGNMENT, "block_forward: workspace must be 256-byte aligned");
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -135,6 +138,7 @@ static repq_status block_forward_impl(const repq_block_desc* dp, const repq_bloc
   uint8_t* hid_c = ws + L.off_hidden;
   int32_t* asum_h = reinterpret_cast<int32_t*>(ws + L.off_asum_h);
   void* gws = ws + L.off_gemm_ws;
+  const size_t gws_bytes = workspace_bytes - L.off_gemm_ws;
   // the two row-sum accumulators that kernels add into start at zero: the first kernel of the block clears them
   const ClearWords clear{asum_attn, asum_h + M - asum_attn};
   int n_mark = 0;
@@ -157,7 +161,7 @@ static repq_status block_forward_impl(const repq_block_desc* dp, const repq_bloc
     if (d.rope) {                       // Q and K ranges rotated ahead of their quantizers, V left alone
       g.rope_cos_sin = p.rope_cos_sin; g.rope_period = S; g.rope_dim = dh; g.rope_groups = 2;
     }
-    REPQ_TRY(repq_qgemm(&g, gws, L.gemm_ws, stream));
+    REPQ_TRY(repq_qgemm(&g, gws, gws_bytes, stream));
   }
   REPQ_MARK();
   if (!d.staged_attention) {
@@ -221,7 +225,7 @@ static repq_status block_forward_impl(const repq_block_desc* dp, const repq_bloc
     g.residual = x; g.residual_dtype = d.act_dtype; g.ld_residual = D;
     g.out_kind = d.act_dtype == REPQ_F32 ? REPQ_OUT_F32 : REPQ_OUT_BF16;
     g.out = xbar; g.ldo = D;
-    REPQ_TRY(repq_qgemm(&g, gws, L.gemm_ws, stream));
+    REPQ_TRY(repq_qgemm(&g, gws, gws_bytes, stream));
   }
   REPQ_MARK();
   // ---- Y = MLP(LN(X_bar)) + X_bar
@@ -236,7 +240,7 @@ static repq_status block_forward_impl(const repq_block_desc* dp, const repq_bloc
     g.out_kind = REPQ_OUT_CODES; g.out_bits = ab; g.out_groups = 1;
     g.out_scale[0] = p.s_hidden; g.out_zero[0] = p.z_hidden;
     g.out = hid_c; g.ldo = L.ld_h; g.out_row_sum = asum_h;
-    REPQ_TRY(repq_qgemm(&g, gws, L.gemm_ws, stream));
+    REPQ_TRY(repq_qgemm(&g, gws, gws_bytes, stream));
   }
   REPQ_MARK();
   {
@@ -244,7 +248,7 @@ static repq_status block_forward_impl(const repq_block_desc* dp, const repq_bloc
     g.residual = xbar; g.residual_dtype = d.act_dtype; g.ld_residual = D;
     g.out_kind = d.out_dtype == REPQ_F32 ? REPQ_OUT_F32 : REPQ_OUT_BF16;
     g.out = y; g.ldo = D;
-    REPQ_TRY(repq_qgemm(&g, gws, L.gemm_ws, stream));
+    REPQ_TRY(repq_qgemm(&g, gws, gws_bytes, stream));
   }
   REPQ_MARK();
   return REPQ_OK;
@@ -306,7 +310,7 @@ extern "C" repq_status repq_block_forward_static(const repq_block_desc* d, const
                                                  const void* x, void* y, void* stream) {
   REPQ_REQUIRE(d && p && x && y, REPQ_INVALID_ARG, "block_forward_static: NULL argument");
   REPQ_TRY(validate(*d));
-  const size_t need = layout(*d).total;
+  const size_t need = layout(*d).least;
   REPQ_REQUIRE(need <= size_t(REPQ_STATIC_WORKSPACE_BYTES), REPQ_WORKSPACE_TOO_SMALL,
                "block_forward_static: this block needs %zu bytes of workspace, the built-in scratch holds %zu; "
                "use repq_block_forward with a caller-provided workspace",

@@ -36,6 +36,10 @@ size_t qgemm_tc_workspace(const repq_gemm_desc& d);
 repq_status qgemm_tc(const repq_gemm_desc& d, const EpilogueParams& ep, void* ws, size_t ws_bytes,
                      cudaStream_t st);
 
+// Workspace of a GEMM: with room for a byte copy of packed weights, and the least it can run in.
+size_t qgemm_workspace(const repq_gemm_desc& d);
+size_t qgemm_workspace_least(const repq_gemm_desc& d);
+
 // Integer GEMM for few tokens (weights on the M side of the tensor-core instruction): plain products, byte codes, both
 // row sums given; `preferred` says whether it takes the problem and is the faster one.
 bool qgemm_skinny_preferred(const repq_gemm_desc& d);

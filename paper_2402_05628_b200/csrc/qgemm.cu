@@ -88,6 +88,87 @@ __global__ void expand4_kernel(const uint8_t* __restrict__ src, int64_t rows, in
   }
 }
 
+// Packed weight codes -> one byte per code, 64 codes (32 or 48 bytes) per thread and step.  The packed bytes are requested
+// before the kernel ahead in the stream has finished (weights are parameters), the scratch is written after it.
+template <int kBits>
+__device__ __forceinline__ void expand_words(const uint32_t (&w)[2 * kBits], uint32_t (&o)[16]) {
+  if constexpr (kBits == 4) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t lo = w[i] & 0x0F0F0F0Fu, hi = (w[i] >> 4) & 0x0F0F0F0Fu;
+      o[2 * i] = __byte_perm(lo, hi, 0x5140);
+      o[2 * i + 1] = __byte_perm(lo, hi, 0x7362);
+    }
+  } else {
+    auto spread = [](uint32_t f) {      // four 6-bit fields of f[23:0] -> four bytes
+      return (f & 0x3Fu) | ((f & 0xFC0u) << 2) | ((f & 0x3F000u) << 4) | ((f & 0xFC0000u) << 6);
+    };
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t w0 = w[3 * i], w1 = w[3 * i + 1], w2 = w[3 * i + 2];
+      o[4 * i] = spread(w0);
+      o[4 * i + 1] = spread(__funnelshift_r(w0, w1, 24));
+      o[4 * i + 2] = spread(__funnelshift_r(w1, w2, 16));
+      o[4 * i + 3] = spread(w2 >> 8);
+    }
+  }
+}
+template <int kBits>
+__global__ void __launch_bounds__(256) expand_weights_kernel(const uint8_t* __restrict__ src, int rows, int groups, int64_t ld_src,
+                                                             uint8_t* __restrict__ dst, int64_t ld_dst) {
+  constexpr int kIn = 8 * kBits;                           // packed bytes of 64 codes
+  const int64_t total = int64_t(rows) * groups, stride = int64_t(gridDim.x) * blockDim.x;
+  grid_dependency_trigger();
+  bool waited = false;
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < total; i += stride) {
+    const int64_t r = i / groups;
+    const int g = int(i - r * groups);
+    uint32_t w[2 * kBits], o[16];
+#pragma unroll
+    for (int q = 0; q < kIn / 16; ++q) {                   // (a row ends on a 16-byte boundary)
+      uint4 v = make_uint4(0u, 0u, 0u, 0u);
+      if (int64_t(g) * kIn + 16 * q < ld_src) v = __ldg(reinterpret_cast<const uint4*>(src + r * ld_src + int64_t(g) * kIn) + q);
+      w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
+    }
+    expand_words<kBits>(w, o);
+    if (!waited) { grid_dependency_wait(); waited = true; }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (int64_t(g) * 64 + 16 * q < ld_dst)
+        *(reinterpret_cast<uint4*>(dst + r * ld_dst + int64_t(g) * 64) + q) = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+  }
+  if (!waited) grid_dependency_wait();
+}
+
+// The byte form of packed weights in the caller's workspace, where it has the room (repq_qgemm_workspace_bytes asks for it): one
+// pass over the weights, after which every GEMM kernel takes them.  The GEMM that expands the tiles it copies (bound by its
+// converters' shared-memory traffic, once per row tile) remains for smaller workspaces.  Measured (packed against that form):
+// 3152 tokens through a DeiT-B block with 6-bit weights 125 -> 98 us (bytes: 86), a 7B-shaped decoder block of 48 tokens with
+// 4-bit weights 1860 -> 143 us (bytes: 78).
+struct ByteWeights { size_t offset = 0, total = 0; int64_t ld = 0; };
+bool byte_weights(const repq_gemm_desc& d, repq_gemm_desc* as_bytes, ByteWeights* B) {
+  if (!(packed4(d.bits_w) || packed6(d.bits_w)) || d.batch_outer != 1 || d.batch_inner != 1) return false;
+  if (!aligned(d.w_codes, 16) || d.ldw_bytes % 16 != 0) return false;
+  *as_bytes = d;
+  as_bytes->bits_w = quant_bits(d.bits_w) | REPQ_BYTE_CODES;
+  B->ld = round_up(d.K, 16);
+  as_bytes->ldw_bytes = B->ld;
+  if (!qgemm_skinny_preferred(*as_bytes) && !qgemm_tc_supported(*as_bytes)) return false;
+  B->offset = (qgemm_tc_supported(*as_bytes) ? qgemm_tc_workspace(*as_bytes) : 0);
+  B->offset = (B->offset + 255) / 256 * 256;
+  B->total = B->offset + size_t(d.N) * size_t(B->ld);
+  return true;
+}
+
+repq_status launch_expand_weights(const repq_gemm_desc& d, uint8_t* dst, int64_t ld, cudaStream_t st) {
+  const int groups = int((int64_t(d.K) + 63) / 64);
+  const int64_t blocks = (int64_t(d.N) * groups + 255) / 256, most = int64_t(sm_count()) * 8;
+  auto kern = packed4(d.bits_w) ? expand_weights_kernel<4> : expand_weights_kernel<6>;
+  REPQ_CUDA(launch_chained(kern, dim3(unsigned(blocks < most ? blocks : most)), dim3(256), 0, st, d.w_codes, d.N, groups, d.ldw_bytes, dst, ld));
+  note_launch();
+  return REPQ_OK;
+}
+
 repq_status validate(const repq_gemm_desc& d) {
   REPQ_REQUIRE(d.M >= 0 && d.N > 0 && d.K > 0, REPQ_INVALID_ARG, "qgemm: M >= 0, N > 0, K > 0 required");
   REPQ_REQUIRE(d.batch_outer > 0 && d.batch_inner > 0, REPQ_INVALID_ARG, "qgemm: batch counts must be positive");
@@ -179,6 +260,15 @@ EpilogueParams make_epilogue(const repq_gemm_desc& d) {
 
 }  // namespace
 
+size_t qgemm_workspace_least(const repq_gemm_desc& d) {
+  return !scores_supported(d) && qgemm_tc_supported(d) ? qgemm_tc_workspace(d) : 0;
+}
+size_t qgemm_workspace(const repq_gemm_desc& d) {
+  repq_gemm_desc as_bytes;
+  ByteWeights B;
+  return byte_weights(d, &as_bytes, &B) ? B.total : qgemm_workspace_least(d);
+}
+
 repq_status launch_row_sum(const uint8_t* codes, int bits, int64_t rows, int64_t n, int64_t ld_bytes,
                            int32_t* out, cudaStream_t st) {
   if (rows == 0) return REPQ_OK;
@@ -209,7 +299,7 @@ using namespace repq;
 extern "C" repq_status repq_qgemm_workspace_bytes(const repq_gemm_desc* d, size_t* bytes) {
   REPQ_REQUIRE(d && bytes, REPQ_INVALID_ARG, "qgemm_workspace_bytes: NULL argument");
   REPQ_TRY(validate(*d));
-  *bytes = (d->M > 0 && !scores_supported(*d) && qgemm_tc_supported(*d)) ? qgemm_tc_workspace(*d) : 0;
+  *bytes = d->M > 0 ? qgemm_workspace(*d) : 0;
   return REPQ_OK;
 }
 
@@ -219,6 +309,14 @@ extern "C" repq_status repq_qgemm(const repq_gemm_desc* d, void* workspace, size
   if (d->M == 0) return REPQ_OK;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (scores_supported(*d)) return scores_tc_supported(*d) ? launch_scores_tc(*d, st) : launch_scores(*d, st);
+  repq_gemm_desc as_bytes;
+  ByteWeights B;
+  if (byte_weights(*d, &as_bytes, &B) && workspace && workspace_bytes >= B.total && aligned(workspace, 256)) {
+    uint8_t* w = static_cast<uint8_t*>(workspace) + B.offset;
+    REPQ_TRY(launch_expand_weights(*d, w, B.ld, st));
+    as_bytes.w_codes = w;
+    d = &as_bytes;
+  }
   const EpilogueParams ep = make_epilogue(*d);
   if (qgemm_skinny_preferred(*d)) return qgemm_skinny(*d, ep, st);
   if (qgemm_tc_supported(*d)) {
