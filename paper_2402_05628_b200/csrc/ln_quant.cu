@@ -1,11 +1,17 @@
 // Fused LayerNorm + layer-wise uniform quantization (Eq. 9 with the reparameterized affine factors of
 // Eq. 12, then Eq. 4 with the scalar (s~, z~)).
 //
-// HBM-bound: every input element is read once with 128-bit loads and leaves as a 4-bit (or 8-bit)
-// code.  A row is owned by a group of TPR threads which keeps its slice of the row in registers, so mean
-// and centred variance are two register passes with shuffle reductions.  Each group works on one or two rows
-// at a time, and the rows of its next iteration are requested before the current ones are reduced, so that
-// loads stay in flight all the time.
+// Every input element is read once with 128-bit loads and leaves as a 4-bit (or 8-bit) code.  A row is owned by a group
+// of TPR threads which keeps its slice of the row in registers, so mean and centred variance are two register passes with
+// shuffle reductions.  Each group works on one or two rows at a time, and the rows of its next iteration are requested before
+// the current ones are reduced, so that loads stay in flight all the time.  Rows of several warps meet at one barrier: every
+// warp centres its slice on the slice's own mean, the means and squares are merged behind the barrier, and the code sums wait
+// for the next one.
+//
+// What bounds it: HBM for float input and for rows of one warp (5.1-6.3 TB/s of 6.46), instruction issue and the occupancy
+// the registers leave for longer bf16 rows (ncu, 2048 elements: 10.9 warp instructions per 32 elements, 16 warps per SM, issue
+// slots 59 % busy).  Measured against three barriers per iteration: 32768 bf16 rows of 4096 78 -> 73 us, 65536 of 1536 53 -> 45,
+// 32768 float rows of 2048 83 -> 48, 16384 of 4096 76 -> 49.
 // The per-channel factors gamma~/s~ and beta~/s~ are staged once per CTA in shared memory (halves of the 8-element
 // chunks apart, so that a warp's 16-byte reads are free of bank conflicts), or, for rows of 3080 to 4096 bf16 elements,
 // kept in the registers of the thread that owns their columns.
@@ -25,10 +31,13 @@ namespace {
 constexpr int kChunk = 8;   // elements per 128-bit bf16 load
 constexpr int kMaxVPT = 4;  // chunks per thread: 1..4, chosen per row length
 
-// Rows a thread group works on at a time (the loads of the next ones are always in flight as well): two,
-// except where four chunks per thread would cost a resident block (measured: 16 x 3 / 32 x 3 / 256 x 4 threads x
-// chunks run best with two rows, 32 x 4 / 128 x 4 with one).
-__host__ __device__ constexpr int rows_in_flight(int vpt, int tpr) { return vpt >= 4 && tpr < 256 ? 1 : 2; }
+// Rows a thread group works on at a time (the loads of the next ones are always in flight as well): two, except where the
+// chunks per thread leave the registers for one (measured: bf16 rows of 2048 / 4096 elements, 64 x 4 / 128 x 4 threads x
+// chunks, 69 / 73 us with one row, 97 / 101 with two; whole bf16 rows of 256 x 4 74 and 69; float rows of 768, 32 x 3, 21 and
+// 28).
+__host__ __device__ constexpr int rows_in_flight(int vpt, int tpr, bool full, int elem_bytes) {
+  return vpt < (elem_bytes == 2 || tpr >= 512 ? 4 : 3) || (vpt == 4 && tpr >= 256 && full && elem_bytes == 2) ? 2 : 1;
+}
 
 // Where a thread's slice of gamma~/s~ and beta~/s~ stays in registers for the whole kernel instead of being read from
 // shared memory for every pair of rows: two chunks per thread at most (32 registers) in groups of at least 128 threads,
@@ -78,11 +87,7 @@ __device__ __forceinline__ uint32_t push_pair_u8(int e0, int e1, uint32_t c) {
   return d;
 }
 
-// Sum over the TPR threads of a group, for kRows values at once.  Inside a warp: xor shuffles (two rows travel as one
-// packed pair per add; integers take the warp-wide reduction instruction).  Across the warps of a group: lane 0 of
-// every warp leaves its partial sums in shared memory, and after the barrier the first TPR / 32 lanes of every warp pick
-// up one warp's partials each and finish with log2(TPR / 32) more shuffle steps (instead of every thread adding up all
-// partials itself).
+// Reductions inside a warp are xor shuffles (integers of a whole warp take the warp-wide reduction instruction).
 // Barrier of one thread group: the whole block where a group is the block, else a named barrier of the group's own (the
 // groups of a block then no longer wait for one another).
 template <int TPR>
@@ -92,72 +97,28 @@ __device__ __forceinline__ void group_sync(int group_first_warp) {
 }
 
 template <int TPR, int kRows>
-__device__ __forceinline__ void group_reduce(float (&v)[kRows], float* red, int group_first_warp) {
-  constexpr int kShfl = TPR < 32 ? TPR : 32;
+__device__ __forceinline__ void warp_reduce(float (&v)[kRows]) {
   const bool odd = threadIdx.x & 1;
-  if constexpr (kRows == 2 && kShfl >= 4) {
+  if constexpr (kRows == 2 && TPR >= 4) {
     // neighbouring lanes split the two rows between them (one shuffle for both rows), every further step then moves one
-    // value per lane, and a last exchange hands each lane the other row's total: kShfl's log + 1 shuffles instead of
+    // value per lane, and a last exchange hands each lane the other row's total: log(TPR) + 1 shuffles instead of
     // twice the log.  All lanes of a parity add the same pairs at every step, so they end with the same bits.
     float t = (odd ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, odd ? v[0] : v[1], 1);
 #pragma unroll
-    for (int o = kShfl / 2; o > 1; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if constexpr (TPR <= 32) {
-      const float u = __shfl_xor_sync(0xffffffffu, t, 1);
-      v[0] = odd ? u : t;
-      v[1] = odd ? t : u;
-    } else {
-      v[0] = t;      // even lanes: row 0, odd lanes: row 1 (lanes 0 and 1 leave them in shared memory)
-    }
-  } else if constexpr (kRows == 2) {
-    f32x2 p = pack2(v[0], v[1]);
-#pragma unroll
-    for (int o = kShfl / 2; o > 0; o >>= 1) {
-      float a, b;
-      unpack2(p, a, b);
-      p = add2(p, pack2(__shfl_xor_sync(0xffffffffu, a, o), __shfl_xor_sync(0xffffffffu, b, o)));
-    }
-    unpack2(p, v[0], v[1]);
+    for (int o = TPR / 2; o > 1; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    const float u = __shfl_xor_sync(0xffffffffu, t, 1);
+    v[0] = odd ? u : t;
+    v[1] = odd ? t : u;
   } else {
 #pragma unroll
-    for (int o = kShfl / 2; o > 0; o >>= 1)
+    for (int o = TPR / 2; o > 0; o >>= 1)
 #pragma unroll
       for (int r = 0; r < kRows; ++r) v[r] += __shfl_xor_sync(0xffffffffu, v[r], o);
   }
-  if constexpr (TPR > 32) {
-    constexpr int kWarps = TPR / 32;
-    const int lane = threadIdx.x & 31;
-    if constexpr (kRows == 2) {
-      // lanes 0 and 1 hold the warp's sums of rows 0 and 1.  After the barrier lane l takes row (l mod 2) of warp
-      // (l / 2 mod kWarps): xor steps over the warp index, then one exchange between neighbours.
-      if (lane < 2) red[(threadIdx.x >> 5) * 2 + lane] = v[0];
-      group_sync<TPR>(group_first_warp);
-      float t = red[(group_first_warp + ((lane >> 1) & (kWarps - 1))) * 2 + (lane & 1)];
-#pragma unroll
-      for (int o = kWarps; o > 1; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      const float u = __shfl_xor_sync(0xffffffffu, t, 1);
-      v[0] = odd ? u : t;
-      v[1] = odd ? t : u;
-    } else {
-      if (lane == 0)
-#pragma unroll
-        for (int r = 0; r < kRows; ++r) red[(threadIdx.x >> 5) * kRows + r] = v[r];
-      group_sync<TPR>(group_first_warp);
-      // lane l < kWarps takes the partials of warp l of its group; the other lanes repeat them (l mod kWarps), so that
-      // the xor steps below leave the full sum in every lane
-      const float* src = red + (group_first_warp + (lane & (kWarps - 1))) * kRows;
-#pragma unroll
-      for (int r = 0; r < kRows; ++r) v[r] = src[r];
-#pragma unroll
-      for (int o = kWarps / 2; o > 0; o >>= 1)
-#pragma unroll
-        for (int r = 0; r < kRows; ++r) v[r] += __shfl_xor_sync(0xffffffffu, v[r], o);
-    }
-  }
 }
 template <int TPR, int kRows>
-__device__ __forceinline__ void group_reduce(int (&v)[kRows], int* red, int group_first_warp) {
-  if constexpr (TPR >= 32) {
+__device__ __forceinline__ void group_sum(int (&v)[kRows]) {
+  if constexpr (TPR == 32) {
 #pragma unroll
     for (int r = 0; r < kRows; ++r) v[r] = __reduce_add_sync(0xffffffffu, v[r]);
   } else {
@@ -166,43 +127,30 @@ __device__ __forceinline__ void group_reduce(int (&v)[kRows], int* red, int grou
 #pragma unroll
       for (int r = 0; r < kRows; ++r) v[r] += __shfl_xor_sync(0xffffffffu, v[r], o);
   }
-  if constexpr (TPR > 32) {
-    constexpr int kWarps = TPR / 32;
-    const int lane = threadIdx.x & 31;
-    if (lane == 0)
-#pragma unroll
-      for (int r = 0; r < kRows; ++r) red[(threadIdx.x >> 5) * kRows + r] = v[r];
-    group_sync<TPR>(group_first_warp);
-    const int* src = red + (group_first_warp + (lane & (kWarps - 1))) * kRows;
-#pragma unroll
-    for (int r = 0; r < kRows; ++r) {
-      // every group of kWarps consecutive lanes holds all partials: the warp-wide sum counts each 32 / kWarps times
-      v[r] = __reduce_add_sync(0xffffffffu, src[r]) / (32 / kWarps);
-    }
-  }
 }
 
 template <typename T, int TPR, int kVPT, bool kPack4, bool kFull>
 __global__ void __launch_bounds__((TPR > 256 ? TPR : 256),
-                                  (kVPT <= 2 && TPR == 256 ? (factors_in_registers(kVPT, TPR, sizeof(T)) ? 2 : 3) : 0))
+                                  (kVPT <= 2 && TPR == 256 ? (factors_in_registers(kVPT, TPR, sizeof(T)) ? 2 : 3) : sizeof(T) == 4 && TPR == 32 && (kVPT == 3 || kVPT == 4) ? 2 : 0))
 ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
                 const float* __restrict__ gamma_t, const float* __restrict__ beta_t, float eps, int rms,
                 float inv_s, int z, int qmax, uint8_t* __restrict__ codes, int64_t ldc,
                 int32_t* __restrict__ row_sum, int32_t* __restrict__ clear, int64_t n_clear) {
-  constexpr int kRows = rows_in_flight(kVPT, TPR);
+  constexpr int kRows = rows_in_flight(kVPT, TPR, kFull, sizeof(T));
   constexpr int kBlock = TPR > 256 ? TPR : 256;
   constexpr int kGroups = kBlock / TPR;
   constexpr int kRowsPerBlock = kGroups * kRows;
   constexpr bool kRegFactors = factors_in_registers(kVPT, TPR, sizeof(T));
   extern __shared__ __align__(16) float s_gb[];          // g[D] then b[D]: gamma~/s~ and beta~/s~ (unless in registers)
-  // One array per reduction of a row.  A slot may be overwritten only after every thread of the block has passed
-  // a barrier that follows its reads of the slot.  With two or three reductions per iteration the barrier of the
-  // next reduction is that barrier; the mean-free form without row sums has the variance reduction alone (one
-  // barrier per iteration), so red_b alternates between two halves by iteration parity: the write of iteration
-  // k + 2 follows the barrier of iteration k + 1, which every thread reaches after its reads of iteration k.
-  __shared__ __align__(8) float red_a[kBlock / 32 * kRows];
-  __shared__ __align__(8) float red_b[2][kBlock / 32 * kRows];
-  __shared__ __align__(8) int red_c[kBlock / 32 * kRows];
+  // Rows of several warps: one barrier per iteration.  A warp reduces its own slice twice (sum, then squares centred on the
+  // slice's own mean) and leaves both in `red`; behind the barrier every warp merges the slices' means and squares
+  // (M2 = sum M2_w + n_w (mean_w - mean)^2).  Code sums wait in `red_c` for the next iteration's barrier.  Both alternate by
+  // iteration parity: a slot written in iteration k is read before the barrier of k + 1 (`red`) or of k + 2 (`red_c`), and
+  // written again in k + 2, behind the barrier of k + 1 or, for `red_c`, behind that of k + 2.
+  constexpr bool kWide = TPR > 32;
+  constexpr int kWarps = kWide ? TPR / 32 : 1;             // warps of a row
+  __shared__ float2 red[kWide ? 2 : 1][kBlock / 32 * kRows];
+  __shared__ int red_c[kWide ? 2 : 1][kBlock / 32 * kRows];
 
   float* s_g = s_gb;
   float* s_b = s_gb + D;
@@ -281,6 +229,22 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
   const int64_t stride = int64_t(gridDim.x) * kRowsPerBlock;
   fetch(int64_t(blockIdx.x) * kRowsPerBlock + group * kRows);
 
+  // the warp's slice of a row, and the slice its lane merges
+  const int lane_w = threadIdx.x & 31;
+  const int slice_of_lane = (lane_w / kRows) & (kWarps - 1);
+  constexpr bool kConst = kFull && sizeof(T) == 2;         // (float rows: known sizes cost registers instead, 146 against 108)
+  auto slice_size = [&](int w) {                           // elements of a row that warp w of its group holds
+    if constexpr (kConst) return float(32 * kVPT * kChunk);
+    int n = 0;
+#pragma unroll
+    for (int i = 0; i < kVPT; ++i) n += max(0, min(32, nchunks - (w * 32 + i * TPR)));
+    return float(n * kChunk);
+  };
+  auto inverse = [](float n) { return kConst ? 1.f / float(32 * kVPT * kChunk) : n > 0.f ? 1.f / n : 0.f; };
+  const float n_slice_of_lane = kWide ? slice_size(slice_of_lane) : 0.f, inv_slice_of_lane = inverse(n_slice_of_lane);
+  const float inv_slice = kWide ? inverse(slice_size((threadIdx.x >> 5) - group_first_warp)) : 0.f;
+  bool parity_seen = false;
+  int64_t last_row0 = 0;
   int parity = 0;
   for (int64_t base = int64_t(blockIdx.x) * kRowsPerBlock; base < rows; base += stride, parity ^= 1) {
     const int64_t row0 = base + group * kRows;
@@ -304,19 +268,26 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
       sum[r] = lo + hi;
     }
 
-    float mu[kRows];
-    if (!rms) {
-      group_reduce<TPR, kRows>(sum, red_a, group_first_warp);
+    float mu[kRows], var[kRows];
+    if constexpr (!kWide) {
+      if (!rms) {
+        warp_reduce<TPR, kRows>(sum);
 #pragma unroll
-      for (int r = 0; r < kRows; ++r) mu[r] = sum[r] * inv_d;
+        for (int r = 0; r < kRows; ++r) mu[r] = sum[r] * inv_d;
+      } else {
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) mu[r] = 0.f;
+      }
     } else {
+      if (!rms) warp_reduce<32, kRows>(sum);
 #pragma unroll
-      for (int r = 0; r < kRows; ++r) mu[r] = 0.f;
+      for (int r = 0; r < kRows; ++r) mu[r] = rms ? 0.f : sum[r] * inv_slice;       // mean of the warp's slice
     }
 
-    float ss[kRows];
+    float ss[kRows], slice_mean[kRows];
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
+      slice_mean[r] = mu[r];
       const f32x2 neg_mu = splat2(-mu[r]);
       f32x2 acc = 0ull;
 #pragma unroll
@@ -333,10 +304,58 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
       unpack2(acc, lo, hi);
       ss[r] = lo + hi;
     }
-    group_reduce<TPR, kRows>(ss, red_b[parity], group_first_warp);
-    f32x2 rstd[kRows];
+    if constexpr (!kWide) {
+      warp_reduce<TPR, kRows>(ss);
 #pragma unroll
-    for (int r = 0; r < kRows; ++r) rstd[r] = splat2(rsqrtf(ss[r] * inv_d + eps));
+      for (int r = 0; r < kRows; ++r) var[r] = ss[r] * inv_d;
+    } else {
+      warp_reduce<32, kRows>(ss);
+      const int lane = threadIdx.x & 31;
+      if (lane < kRows) red[parity][(threadIdx.x >> 5) * kRows + lane] = make_float2(lane ? sum[kRows - 1] : sum[0], lane ? ss[kRows - 1] : ss[0]);
+      group_sync<TPR>(group_first_warp);
+      // the code sums of the iteration before
+      if (row_sum != nullptr && parity_seen && tig < kRows) {
+        int t = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) t += red_c[parity ^ 1][(group_first_warp + w) * kRows + tig];
+        const int64_t row = row0 - stride + tig;
+        if (row < rows) row_sum[row] = t;
+      }
+      parity_seen = true;
+      // lane l merges slice (l / kRows mod kWarps) of row (l mod kRows): xor steps over the slice index
+      const float2 p = red[parity][(group_first_warp + slice_of_lane) * kRows + (lane & (kRows - 1))];
+      float total = p.x;
+#pragma unroll
+      for (int o = kWarps * kRows / 2; o >= kRows; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+      const float mean = rms ? 0.f : total * inv_d;
+      const float off = rms ? 0.f : p.x * inv_slice_of_lane - mean;
+      float m2 = fmaf(n_slice_of_lane * off, off, p.y);
+#pragma unroll
+      for (int o = kWarps * kRows / 2; o >= kRows; o >>= 1) m2 += __shfl_xor_sync(0xffffffffu, m2, o);
+      if constexpr (kRows == 2) {
+        const float mean1 = __shfl_xor_sync(0xffffffffu, mean, 1), m21 = __shfl_xor_sync(0xffffffffu, m2, 1);
+        const bool odd = lane & 1;
+        mu[0] = odd ? mean1 : mean;
+        mu[1] = odd ? mean : mean1;
+        var[0] = (odd ? m21 : m2) * inv_d;
+        var[1] = (odd ? m2 : m21) * inv_d;
+      } else {
+        mu[0] = mean;
+        var[0] = m2 * inv_d;
+      }
+    }
+    // rows of several warps: v is centred on the slice's mean, the rest of the way to the row's mean is one more product
+    f32x2 rstd[kRows], rest[kRows];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      const float rs = rsqrtf(var[r] + eps);
+      rstd[r] = splat2(rs);
+      if constexpr (kWide) rest[r] = splat2((slice_mean[r] - mu[r]) * rs);
+    }
+    auto normalised = [&](f32x2 x, int r) {
+      if constexpr (kWide) return fma2(x, rstd[r], rest[r]);
+      else return mul2(x, rstd[r]);
+    };
 
     int csum[kRows];
     bool live[kRows];
@@ -372,14 +391,14 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
 #pragma unroll
             for (int e = 0; e < kChunk / 2; ++e) {
               float u0, u1;
-              unpack2(add2(fma2(mul2(v[r][i][e], rstd[r]), g[e], b[e]), magic2), u0, u1);
+              unpack2(add2(fma2(normalised(v[r][i][e], r), g[e], b[e]), magic2), u0, u1);
               q[2 * e] = __float_as_int(u0) + z_less_magic;
               q[2 * e + 1] = __float_as_int(u1) + z_less_magic;
             }
           } else {
             float t[kChunk];
 #pragma unroll
-            for (int e = 0; e < kChunk / 2; ++e) unpack2(fma2(mul2(v[r][i][e], rstd[r]), g[e], b[e]), t[2 * e], t[2 * e + 1]);
+            for (int e = 0; e < kChunk / 2; ++e) unpack2(fma2(normalised(v[r][i][e], r), g[e], b[e]), t[2 * e], t[2 * e + 1]);
 #pragma unroll
             for (int e = 0; e < kChunk; ++e) q[e] = __float2int_rn(fminf(fmaxf(t[e], -1.0e9f), 1.0e9f)) + z;
           }
@@ -403,11 +422,31 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
       }
     }
     if (row_sum != nullptr) {
-      group_reduce<TPR, kRows>(csum, red_c, group_first_warp);
-      if (tig == 0) {
+      if constexpr (!kWide) {
+        group_sum<TPR, kRows>(csum);
+        if (tig == 0) {
 #pragma unroll
-        for (int r = 0; r < kRows; ++r)
-          if (row0 + r < rows) row_sum[row0 + r] = csum[r];
+          for (int r = 0; r < kRows; ++r)
+            if (row0 + r < rows) row_sum[row0 + r] = csum[r];
+        }
+      } else {
+        group_sum<32, kRows>(csum);
+        if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+          for (int r = 0; r < kRows; ++r) red_c[parity][(threadIdx.x >> 5) * kRows + r] = csum[r];
+        }
+        last_row0 = row0;
+      }
+    }
+  }
+  if constexpr (kWide) {
+    if (row_sum != nullptr && parity_seen) {
+      group_sync<TPR>(group_first_warp);
+      if (tig < kRows) {
+        int t = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) t += red_c[parity ^ 1][(group_first_warp + w) * kRows + tig];
+        if (last_row0 + tig < rows) row_sum[last_row0 + tig] = t;
       }
     }
   }
@@ -418,16 +457,16 @@ repq_status launch(const T* x, int64_t rows, int D, int64_t ldx, const float* g,
                    int rms, float s_t, int z, int bits, uint8_t* codes, int64_t ldc, int32_t* row_sum,
                    ClearWords clear, cudaStream_t st) {
   constexpr int kBlock = TPR > 256 ? TPR : 256;
-  constexpr int kRowsPerBlock = kBlock / TPR * rows_in_flight(kVPT, TPR);
-  const int64_t need = (rows + kRowsPerBlock - 1) / kRowsPerBlock;
+  const bool full = D == TPR * kVPT * kChunk;   // the row fills the group exactly: no chunk is predicated
+  const int rows_per_block = kBlock / TPR * rows_in_flight(kVPT, TPR, full, sizeof(T));
+  const int64_t need = (rows + rows_per_block - 1) / rows_per_block;
   const float inv_s = 1.f / s_t;
   const int qmax = code_max(bits);
   const size_t smem = factors_in_registers(kVPT, TPR, sizeof(T)) ? 0 : size_t(D) * 2 * sizeof(float);
-  const bool full = D == TPR * kVPT * kChunk;   // the row fills the group exactly: no chunk is predicated
   const bool pack = packed4(bits);
   auto kern = pack ? (full ? ln_quant_kernel<T, TPR, kVPT, true, true> : ln_quant_kernel<T, TPR, kVPT, true, false>)
                    : (full ? ln_quant_kernel<T, TPR, kVPT, false, true> : ln_quant_kernel<T, TPR, kVPT, false, false>);
-  if (smem > 48 * 1024) REPQ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+  if (smem > 40 * 1024) REPQ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
   static Residency memo[2][2];
   // persistent grid: exactly the blocks that are resident at once, so that every block keeps its load pipeline
   // running over all of its rows
@@ -448,7 +487,9 @@ repq_status launch_vpt(int vpt, const T* x, int64_t rows, int D, int64_t ldx, co
     case 1: return launch<T, TPR, 1>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
     case 2: return launch<T, TPR, 2>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
     case 3: return launch<T, TPR, 3>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
-    default: return launch<T, TPR, 4>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
+    case 4: return launch<T, TPR, 4>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
+    case 5: return launch<T, TPR, (TPR >= 32 && TPR <= 128 ? 5 : 4)>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
+    default: return launch<T, TPR, (TPR >= 32 && TPR <= 128 ? 6 : 4)>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
   }
 }
 
@@ -457,17 +498,18 @@ repq_status dispatch(const T* x, int64_t rows, int D, int64_t ldx, const float* 
                      int rms, float s_t, int z, int bits, uint8_t* codes, int64_t ldc, int32_t* row_sum,
                      ClearWords clear, cudaStream_t st) {
   const int nchunks = D / kChunk;
-  // a row that would take four chunks per thread in a group of 128 goes to a whole block with two (measured:
-  // D = 4096 runs 9 % faster as 256 x 2 with three resident blocks than as 128 x 4 with one)
-#define REPQ_LN_CASE(TPR) \
-  if (nchunks <= TPR * (TPR == 128 ? 3 : kMaxVPT)) return launch_vpt<T, TPR>((nchunks + TPR - 1) / TPR, x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
-  REPQ_LN_CASE(8)
-  REPQ_LN_CASE(16)
-  REPQ_LN_CASE(32)
-  REPQ_LN_CASE(64)
-  REPQ_LN_CASE(128)
-  REPQ_LN_CASE(256)
-  REPQ_LN_CASE(512)
+  // The fewest warps whose threads hold the row in at most six chunks: a row of one warp has no barrier, and what a row costs
+  // beside its elements (shuffles, merges, barrier) is paid per thread (measured, 1536 elements: 45 us with one warp, 59 with
+  // two; 3072: 49 and 61).  Eight chunks leave too few warps on the SM (2048 float elements: 56 against 48).
+#define REPQ_LN_CASE(TPR, MOST) \
+  if (nchunks <= TPR * MOST) return launch_vpt<T, TPR>((nchunks + TPR - 1) / TPR, x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
+  REPQ_LN_CASE(8, 4)
+  REPQ_LN_CASE(16, 4)
+  REPQ_LN_CASE(32, 6)
+  REPQ_LN_CASE(64, 6)
+  REPQ_LN_CASE(128, 6)
+  REPQ_LN_CASE(256, 4)
+  REPQ_LN_CASE(512, 4)
 #undef REPQ_LN_CASE
   return fail(REPQ_UNSUPPORTED, "ln_quant: D = %d exceeds 16384", D);
 }

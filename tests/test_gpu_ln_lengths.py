@@ -1,0 +1,21 @@
+"""LayerNorm + quantization at the row lengths where the thread group or the chunks per thread change, both input types, and with
+more rows than one grid takes (the code sums of a row leave in the iteration after it)."""
+import pytest
+
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("bf16", [True, False])
+@pytest.mark.parametrize("D", [1024, 1032, 1280, 1536, 1544, 2048, 2056, 2560, 3072, 3080, 4096, 5120, 6144, 6152, 8192, 8200, 16384])
+def test_ln_quant_row_lengths(D, bf16):
+    rep = parity.check_ln_quant(37, D, 4, bf16, seed=D)
+    assert rep["bad"] == 0, rep
+
+
+@pytest.mark.parametrize("rows,D,bits,bf16,rms", [(3001, 2048, 4, True, False), (1500, 4096, 8, True, True), (2500, 1536, 6, False, False),
+                                                  (1203, 8192, 4, False, False), (1300, 8192, 4, True, False)])
+def test_ln_quant_many_rows(rows, D, bits, bf16, rms):
+    rep = parity.check_ln_quant(rows, D, bits, bf16, seed=rows, rms=rms)
+    assert rep["bad"] == 0, rep
