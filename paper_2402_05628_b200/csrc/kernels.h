@@ -43,7 +43,7 @@ size_t qgemm_workspace_least(const repq_gemm_desc& d);
 // Integer GEMM for few tokens (weights on the M side of the tensor-core instruction): plain products, byte codes, both
 // row sums given; `preferred` says whether it takes the problem and is the faster one.
 bool qgemm_skinny_preferred(const repq_gemm_desc& d);
-repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, cudaStream_t st);
+repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, bool weights_ready, cudaStream_t st);
 
 // P.V (Eqs. 16-17): kernel parameters shared by the two implementations, storage widths already resolved
 // (bits_v is 4 for packed codes, 8 for byte codes).

@@ -318,7 +318,7 @@ extern "C" repq_status repq_qgemm(const repq_gemm_desc* d, void* workspace, size
     d = &as_bytes;
   }
   const EpilogueParams ep = make_epilogue(*d);
-  if (qgemm_skinny_preferred(*d)) return qgemm_skinny(*d, ep, st);
+  if (qgemm_skinny_preferred(*d)) return qgemm_skinny(*d, ep, d != &as_bytes, st);
   if (qgemm_tc_supported(*d)) {
     const size_t need = qgemm_tc_workspace(*d);
     REPQ_REQUIRE(workspace_bytes >= need && (need == 0 || workspace), REPQ_WORKSPACE_TOO_SMALL,

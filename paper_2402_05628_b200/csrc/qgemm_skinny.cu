@@ -8,8 +8,8 @@
 //    distributed shared memory, every CTA finishing an equal share of the tile's tokens (integer sums: the result does
 //    not depend on the split);
 //  - two CTAs per SM where the ring of operand stages allows it, at least 64 KB of weights in flight per CTA;
-//  - while the kernel before it in the stream still runs, every CTA asks for its weights to be brought into L2
-//    (prefetches only: nothing is read before the dependency is resolved).
+//  - while the kernel before it in the stream still runs, every CTA asks for its first weights
+//    (activations and outputs are touched only behind the dependency).
 // The epilogue has one output channel per thread (the channel's terms live in registers), tokens along the accumulator
 // columns; for one token the 32 lanes of a warp are 32 neighbouring outputs, so loads and stores are coalesced without
 // staging.  The arithmetic is epilogue.cuh's, element by element.
@@ -50,6 +50,7 @@ struct SkinnyParams {
   int M, N, K;
   int mt;                      // tokens per tile (multiple of 16)
   int stages, kblocks, split;
+  int weights_ready;           // the weights do not come from the kernel ahead in the stream
   uint32_t stage_bytes, a_bytes;
   uint32_t tmem_cols;
   const int32_t* asum;
@@ -206,13 +207,24 @@ qgemm_skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(P.tmem_cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  if (warp == kEpiWarps && blockIdx.y == 0)                // weights into L2 while the kernel before this one finishes
-    if (lane < kPrefetch && kb0 + lane < kb1) tma_prefetch_2d(&map_w, (kb0 + lane) * kBK, n0);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = s_tmem;
   volatile int* abort = &s_abort;
+  // Ahead of the dependency wait, while the kernel before this one finishes (weights are parameters, unless that kernel has just
+  // expanded them): all of the CTA's weights where the ring holds them (ViT-S block of one image 33.0 -> 32.0 us), else the first
+  // k-blocks into L2 (copies into the ring cost a 7B-shaped block of 48 tokens 1 us there).
+  const int early = P.weights_ready && kb1 - kb0 <= stages ? kb1 - kb0 : 0;
+  if (warp == kEpiWarps) {
+    if (early == 0 && P.weights_ready && blockIdx.y == 0 && lane < kPrefetch && kb0 + lane < kb1) tma_prefetch_2d(&map_w, (kb0 + lane) * kBK, n0);
+    if (lane == 0) {
+      for (int s = 0; s < early; ++s) {
+        mbar_expect_tx(smem_u32(&s_full[s]), kWBytes + P.a_bytes);
+        tma_load_2d(smem_u32(ring) + s * P.stage_bytes, &map_w, smem_u32(&s_full[s]), (kb0 + s) * kBK, n0);
+      }
+    }
+  }
   grid_dependency_wait();
   grid_dependency_trigger();
 
@@ -233,8 +245,10 @@ qgemm_skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
         if (!mbar_wait(smem_u32(&s_empty[stage]), phase ^ 1, abort, 61, P.status)) break;
         const uint32_t bar = smem_u32(&s_full[stage]);
         const uint32_t base = smem_u32(ring) + stage * P.stage_bytes;
-        mbar_expect_tx(bar, kWBytes + P.a_bytes);
-        tma_load_2d(base, &map_w, bar, kb * kBK, n0);
+        if (early == 0) {
+          mbar_expect_tx(bar, kWBytes + P.a_bytes);
+          tma_load_2d(base, &map_w, bar, kb * kBK, n0);
+        }
         tma_load_2d(base + kWBytes, &map_a, bar, kb * kBK, m0);
         ++issued;
         if (++stage == uint32_t(stages)) { stage = 0; phase ^= 1; }
@@ -413,11 +427,12 @@ bool qgemm_skinny_preferred(const repq_gemm_desc& d) {
   return plan.us * 1.1f < other + 4.5f || (d.M <= 64 && plan.us < other + 4.5f);
 }
 
-repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, cudaStream_t st) {
+repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, bool weights_ready, cudaStream_t st) {
   SkinnyParams P{};
   P.M = d.M; P.N = d.N; P.K = d.K;
   P.asum = d.a_row_sum; P.wsum = d.w_row_sum;
   P.ep = ep;
+  P.weights_ready = weights_ready;
   P.status = device_status_word();
   REPQ_REQUIRE(P.status != nullptr, REPQ_CUDA_ERROR, "qgemm: device status word unavailable");
   const Plan plan = plan_of(d.M, d.N, d.K, sm_count());
