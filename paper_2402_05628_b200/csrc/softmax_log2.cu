@@ -19,8 +19,14 @@ namespace repq {
 namespace {
 
 constexpr int kChunk = 8;
-constexpr int kMaxVPT = 4;   // chunks per thread: 1..4, chosen per row length
-constexpr uint32_t kMagicBits = 0x4B400000u;   // 1.5 * 2^23
+// Chunks per thread: 1..5, chosen per row length; up to 6 (float32) or 8 (bf16) under a causal mask.  Few threads with many
+// chunks each: a row's reductions and per-row work are then shared out over fewer lanes (two to four rows of a warp go through
+// them at once), and fewer lanes idle in the last, ragged slot (577 keys: 73 of 80 slots with 16 threads, 73 of 96 with 32).
+// Five instead of four took 73856 x 577 from 33.0 to 31.4 us (float32, 4-bit codes; 6.1 TB/s) and from 30.9 to 25.4 us (bf16).
+constexpr int kMaxVPT = 5;
+// A row under a causal mask: the many registers of 6..8 chunks in blocks of 128 threads (30000 x 1500: 42.0 -> 33.0 us,
+// bf16 50000 x 2048: 75.8 -> 62.3); without a mask, or with float32 rows of 8 chunks, the wider group stayed faster.
+constexpr int block_of(int tpr, int vpt) { return tpr > 256 ? tpr : vpt > kMaxVPT ? 128 : 256; }
 
 __device__ __forceinline__ float ex2(float x) {
   float y;
@@ -83,6 +89,34 @@ __device__ __forceinline__ uint32_t push_pair_u8(int e0, int e1, uint32_t c) {
   return d;
 }
 
+// Eq. 15 for the 8 scores of a chunk: clip(round(t), 0, qmax) with t = k1 (S - m) + k0.  t 2^-149 is a denormal float whose
+// bits are t rounded half to even, so one packed multiply makes two integers; both clips are the saturation of the pack
+// (negative t, possible for s < 1 only, has the sign bit: a negative integer; t = +inf for keys past the row and underflowed
+// probabilities stays a large positive one).
+template <bool kPack4>
+__device__ __forceinline__ void store_codes(const f32x2 (&v)[kChunk / 2], f32x2 k1, f32x2 k0, uint32_t qmax4, bool live, uint8_t* out, int ch) {
+  const f32x2 tiny2 = splat2(__uint_as_float(1u));
+  int q[kChunk];
+#pragma unroll
+  for (int e = 0; e < kChunk / 2; ++e) {
+    float r0, r1;
+    unpack2(mul2(fma2(v[e], k1, k0), tiny2), r0, r1);
+    q[2 * e] = __float_as_int(r0);
+    q[2 * e + 1] = __float_as_int(r1);
+  }
+  if constexpr (kPack4) {
+    uint32_t w = 0;
+#pragma unroll
+    for (int e = kChunk - 2; e >= 0; e -= 2) w = push_pair_u4(q[e], q[e + 1], w);
+    if (live) reinterpret_cast<uint32_t*>(out)[ch] = w;
+  } else {
+    uint2 w;
+    w.x = __vminu4(push_pair_u8(q[0], q[1], push_pair_u8(q[2], q[3], 0u)), qmax4);   // 6-bit codes in bytes
+    w.y = __vminu4(push_pair_u8(q[4], q[5], push_pair_u8(q[6], q[7], 0u)), qmax4);
+    if (live) reinterpret_cast<uint2*>(out)[ch] = w;
+  }
+}
+
 template <int TPR, bool kMax>
 __device__ __forceinline__ float group_reduce(float v, float* red, int group_first_warp) {
   constexpr int kShfl = TPR < 32 ? TPR : 32;
@@ -105,11 +139,11 @@ __device__ __forceinline__ float group_reduce(float v, float* red, int group_fir
 }
 
 template <typename T, int TPR, int kVPT, bool kPack4>
-__global__ void __launch_bounds__((TPR > 256 ? TPR : 256))
+__global__ void __launch_bounds__(block_of(TPR, kVPT))
 softmax_log2_kernel(const T* __restrict__ scores, int64_t rows, int L, int64_t ld, bool vec_ok, float c,
                     int causal_period, int causal_offset, float log2_s, int qmax,
                     uint8_t* __restrict__ codes, int64_t ldc) {
-  constexpr int kBlock = TPR > 256 ? TPR : 256;
+  constexpr int kBlock = block_of(TPR, kVPT);
   constexpr int kRowsPerBlock = kBlock / TPR;
   __shared__ float red_a[kBlock / 32];
   __shared__ float red_b[kBlock / 32];
@@ -118,7 +152,7 @@ softmax_log2_kernel(const T* __restrict__ scores, int64_t rows, int L, int64_t l
   const int group = threadIdx.x / TPR;
   const int group_first_warp = (group * TPR) >> 5;
   const int nchunks = (L + kChunk - 1) / kChunk;
-  const float fq = float(qmax);
+  const uint32_t qmax4 = uint32_t(qmax) * 0x01010101u;
 
   // keys a row may see (0 for rows past the end)
   auto visible = [&](int64_t row) {
@@ -203,7 +237,6 @@ softmax_log2_kernel(const T* __restrict__ scores, int64_t rows, int L, int64_t l
     z = group_reduce<TPR, false>(z, red_b, group_first_warp);
     const f32x2 k0 = splat2(2.f * (log2f(z) + log2_s));
     const f32x2 k1 = splat2(-2.f * c);
-    const f32x2 magic2 = splat2(__uint_as_float(kMagicBits));
 
     if (live) {
       uint8_t* out = codes + row * ldc;
@@ -216,31 +249,7 @@ softmax_log2_kernel(const T* __restrict__ scores, int64_t rows, int L, int64_t l
           if constexpr (kPack4) reinterpret_cast<uint32_t*>(out)[ch] = top;
           else reinterpret_cast<uint2*>(out)[ch] = make_uint2(top, top);
         } else if (ch < nchunks) {
-          // Eq. 15: clip(round(t), 0, qmax).  The upper clip is a float min (t = +inf for masked keys and
-          // underflowed probabilities lands on the top code); rounding half to even is one packed float add of
-          // 1.5 * 2^23, which leaves the code in the low mantissa bits; negative t (possible for s < 1 only) would
-          // leave a negative integer there, which the saturating pack turns into code 0.
-          int q[kChunk];
-#pragma unroll
-          for (int e = 0; e < kChunk / 2; ++e) {
-            float t0, t1;
-            unpack2(fma2(v[i][e], k1, k0), t0, t1);
-            float r0, r1;
-            unpack2(add2(pack2(fminf(t0, fq), fminf(t1, fq)), magic2), r0, r1);
-            q[2 * e] = __float_as_int(r0) - int(kMagicBits);
-            q[2 * e + 1] = __float_as_int(r1) - int(kMagicBits);
-          }
-          if constexpr (kPack4) {
-            uint32_t w = 0;
-#pragma unroll
-            for (int e = kChunk - 2; e >= 0; e -= 2) w = push_pair_u4(q[e], q[e + 1], w);
-            reinterpret_cast<uint32_t*>(out)[ch] = w;
-          } else {
-            uint2 w;
-            w.x = push_pair_u8(q[0], q[1], push_pair_u8(q[2], q[3], 0u));
-            w.y = push_pair_u8(q[4], q[5], push_pair_u8(q[6], q[7], 0u));
-            reinterpret_cast<uint2*>(out)[ch] = w;
-          }
+          store_codes<kPack4>(v[i], k1, k0, qmax4, true, out, ch);
         }
       }
     }
@@ -255,7 +264,7 @@ softmax_log2_kernel(const T* __restrict__ scores, int64_t rows, int L, int64_t l
 // kWhole: the number of whole chunk slots when it is kVPT or kVPT - 1 (known at compile time, so that those slots
 // carry no test at all), -1 otherwise (taken from L at run time).
 template <typename T, int TPR, int kVPT, bool kPack4, int kWhole>
-__global__ void __launch_bounds__((TPR > 256 ? TPR : 256), (TPR <= 32 ? 3 : 0))
+__global__ void __launch_bounds__((TPR > 256 ? TPR : 256), (TPR <= 32 ? (kVPT <= 4 ? 3 : 2) : 0))
 softmax_log2_plain_kernel(const T* __restrict__ scores, int64_t rows, int L, int64_t ld, bool tail_half, float c,
                           float log2_s, int qmax, uint8_t* __restrict__ codes, int64_t ldc) {
   constexpr int kBlock = TPR > 256 ? TPR : 256;
@@ -290,7 +299,6 @@ softmax_log2_plain_kernel(const T* __restrict__ scores, int64_t rows, int L, int
 
   const f32x2 c2 = splat2(c);
   const f32x2 k1 = splat2(-2.f * c);
-  const f32x2 magic2 = splat2(__uint_as_float(kMagicBits));
   for (int64_t base = int64_t(blockIdx.x) * kRowsPerBlock; base < rows; base += stride) {
     const int64_t row = base + group;
     const bool live = row < rows;
@@ -341,60 +349,44 @@ softmax_log2_plain_kernel(const T* __restrict__ scores, int64_t rows, int L, int
     uint8_t* out = codes + row * ldc;
 #pragma unroll
     for (int i = 0; i < kVPT; ++i) {
-      const int ch = tig + i * TPR;
-      if (i < n_full || cnt[i] > 0) {
-        // Eq. 15: clip(round(t), 0, qmax); rounding half to even is one packed float add of 1.5 * 2^23, which
-        // leaves the code in the low mantissa bits; both clips are the saturation of the pack (negative t,
-        // possible for s < 1 only, leaves a negative integer; t = +inf for keys past the row and underflowed
-        // probabilities leaves a large positive one)
-        int q[kChunk];
-#pragma unroll
-        for (int e = 0; e < kChunk / 2; ++e) {
-          float r0, r1;
-          unpack2(add2(fma2(v[i][e], k1, k0), magic2), r0, r1);
-          q[2 * e] = __float_as_int(r0) - int(kMagicBits);
-          q[2 * e + 1] = __float_as_int(r1) - int(kMagicBits);
-        }
-        if constexpr (kPack4) {
-          uint32_t w = 0;
-#pragma unroll
-          for (int e = kChunk - 2; e >= 0; e -= 2) w = push_pair_u4(q[e], q[e + 1], w);
-          if (live) reinterpret_cast<uint32_t*>(out)[ch] = w;
-        } else {
-          uint2 w;
-          w.x = __vminu4(push_pair_u8(q[0], q[1], push_pair_u8(q[2], q[3], 0u)), qmax4);   // 6-bit codes in bytes
-          w.y = __vminu4(push_pair_u8(q[4], q[5], push_pair_u8(q[6], q[7], 0u)), qmax4);
-          if (live) reinterpret_cast<uint2*>(out)[ch] = w;
-        }
-      }
+      if (i < n_full || cnt[i] > 0) store_codes<kPack4>(v[i], k1, k0, qmax4, live, out, tig + i * TPR);
     }
   }
+}
+
+// Whether the predicate-free kernel takes the call; tail_half: see there.
+struct PlainRows { bool ok, tail_half; };
+PlainRows plain_rows(int L, int64_t ld, size_t elem, bool vec_ok, int period) {
+  const int64_t chunks8 = (int64_t(L) + kChunk - 1) / kChunk * kChunk;
+  const bool tail_half = chunks8 > ld && elem == 4 && L % kChunk >= 1 && L % kChunk <= 4 && chunks8 - 4 <= ld;
+  return PlainRows{vec_ok && period <= 0 && (chunks8 <= ld || tail_half), tail_half};
 }
 
 template <typename T, int TPR, int kVPT>
 repq_status launch(const T* scores, int64_t rows, int L, int64_t ld, bool vec_ok, float c, int period,
                    int offset, float log2_s, int bits, uint8_t* codes, int64_t ldc, cudaStream_t st) {
-  constexpr int kBlock = TPR > 256 ? TPR : 256;
+  constexpr int kBlock = block_of(TPR, kVPT);
   constexpr int kRowsPerBlock = kBlock / TPR;
   const int64_t need = (rows + kRowsPerBlock - 1) / kRowsPerBlock;
   const int qmax = code_max(bits);
-  const int64_t chunks8 = (int64_t(L) + kChunk - 1) / kChunk * kChunk;
-  const bool tail_half = chunks8 > ld && sizeof(T) == 4 && L % kChunk >= 1 && L % kChunk <= 4 && chunks8 - 4 <= ld;
-  if (vec_ok && period <= 0 && (chunks8 <= ld || tail_half)) {
-    const int whole = (L / kChunk) / TPR;
-    auto plain = packed4(bits) ? softmax_log2_plain_kernel<T, TPR, kVPT, true, -1> : softmax_log2_plain_kernel<T, TPR, kVPT, false, -1>;
-    if constexpr (TPR <= 64) {     // (measured: the compile-time count gains 2-5 % on short rows and loses 4 % with 256 threads per row)
-      if (whole == kVPT) plain = packed4(bits) ? softmax_log2_plain_kernel<T, TPR, kVPT, true, kVPT> : softmax_log2_plain_kernel<T, TPR, kVPT, false, kVPT>;
-      if (whole == kVPT - 1) plain = packed4(bits) ? softmax_log2_plain_kernel<T, TPR, kVPT, true, kVPT - 1> : softmax_log2_plain_kernel<T, TPR, kVPT, false, kVPT - 1>;
+  if constexpr (kVPT <= kMaxVPT) {
+    const PlainRows plain_call = plain_rows(L, ld, sizeof(T), vec_ok, period);
+    if (plain_call.ok) {
+      const int whole = (L / kChunk) / TPR;
+      auto plain = packed4(bits) ? softmax_log2_plain_kernel<T, TPR, kVPT, true, -1> : softmax_log2_plain_kernel<T, TPR, kVPT, false, -1>;
+      if constexpr (TPR <= 64) {     // (measured: the compile-time count gains 2-5 % on short rows and loses 4 % with 256 threads per row)
+        if (whole == kVPT) plain = packed4(bits) ? softmax_log2_plain_kernel<T, TPR, kVPT, true, kVPT> : softmax_log2_plain_kernel<T, TPR, kVPT, false, kVPT>;
+        if (whole == kVPT - 1) plain = packed4(bits) ? softmax_log2_plain_kernel<T, TPR, kVPT, true, kVPT - 1> : softmax_log2_plain_kernel<T, TPR, kVPT, false, kVPT - 1>;
+      }
+      int fit = 0;
+      static Residency memo[2][3];
+      REPQ_TRY(resident_blocks(memo[packed4(bits)][TPR > 64 ? 0 : whole == kVPT ? 1 : whole == kVPT - 1 ? 2 : 0], plain, kBlock, 0, &fit));
+      const int64_t most = int64_t(sm_count()) * fit;
+      plain<<<int(need < most ? need : most), kBlock, 0, st>>>(scores, rows, L, ld, plain_call.tail_half, c, log2_s, qmax, codes, ldc);
+      REPQ_CUDA(cudaGetLastError());
+      note_launch();
+      return REPQ_OK;
     }
-    int fit = 0;
-    static Residency memo[2][3];
-    REPQ_TRY(resident_blocks(memo[packed4(bits)][TPR > 64 ? 0 : whole == kVPT ? 1 : whole == kVPT - 1 ? 2 : 0], plain, kBlock, 0, &fit));
-    const int64_t most = int64_t(sm_count()) * fit;
-    plain<<<int(need < most ? need : most), kBlock, 0, st>>>(scores, rows, L, ld, tail_half, c, log2_s, qmax, codes, ldc);
-    REPQ_CUDA(cudaGetLastError());
-    note_launch();
-    return REPQ_OK;
   }
   auto kern = packed4(bits) ? softmax_log2_kernel<T, TPR, kVPT, true> : softmax_log2_kernel<T, TPR, kVPT, false>;
   // persistent grid: exactly the blocks that are resident at once (every block keeps its load pipeline running)
@@ -416,7 +408,8 @@ repq_status launch_vpt(int vpt, const T* scores, int64_t rows, int L, int64_t ld
     case 1: return launch<T, TPR, 1>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
     case 2: return launch<T, TPR, 2>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
     case 3: return launch<T, TPR, 3>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
-    default: return launch<T, TPR, 4>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
+    case 4: return launch<T, TPR, 4>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
+    default: return launch<T, TPR, 5>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
   }
 }
 
@@ -424,6 +417,15 @@ template <typename T>
 repq_status dispatch(const T* scores, int64_t rows, int L, int64_t ld, bool vec_ok, float c, int period,
                      int offset, float log2_s, int bits, uint8_t* codes, int64_t ldc, cudaStream_t st) {
   const int nchunks = (L + kChunk - 1) / kChunk;
+  if (vec_ok && !plain_rows(L, ld, sizeof(T), vec_ok, period).ok) {
+    constexpr int kMost = sizeof(T) == 2 ? 8 : 6;
+#define REPQ_SM_CASE(TPR) \
+  if (nchunks > TPR * kMaxVPT && nchunks <= TPR * kMost) return launch<T, TPR, kMost>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
+    REPQ_SM_CASE(8)
+    REPQ_SM_CASE(16)
+    REPQ_SM_CASE(32)
+#undef REPQ_SM_CASE
+  }
 #define REPQ_SM_CASE(TPR) \
   if (nchunks <= TPR * kMaxVPT) return launch_vpt<T, TPR>((nchunks + TPR - 1) / TPR, scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
   REPQ_SM_CASE(8)
