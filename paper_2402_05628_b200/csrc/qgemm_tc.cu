@@ -183,6 +183,7 @@ struct ChunkQuant {
   int zo;
   float inv_qs, qs, csat;   // byte codes of at most 7 bits: 1 / 2^bits, 2^bits, (z_o - magic) / 2^bits
   int qs_shift;             //   bits
+  float z_tiny;             // (z_o - magic) 2^-149
 };
 
 __device__ __forceinline__ ChunkQuant chunk_quant(const EpilogueParams& ep, const TcParams& P, int col0) {
@@ -202,6 +203,7 @@ __device__ __forceinline__ ChunkQuant chunk_quant(const EpilogueParams& ep, cons
   q.qs_shift = 32 - __clz(ep.qmax);                      // qmax = 2^bits - 1
   q.qs = __uint_as_float(uint32_t(127 + q.qs_shift) << 23);         // 2^bits
   q.inv_qs = __uint_as_float(uint32_t(127 - q.qs_shift) << 23);     // 2^-bits
+  q.z_tiny = (float(zo) - __uint_as_float(kMagicBits)) * __uint_as_float(1u);
   q.csat = (float(zo) - __uint_as_float(kMagicBits)) * q.inv_qs;    // exact: an integer below 2^24 times a power of two
   return q;
 }
@@ -232,6 +234,12 @@ __device__ __forceinline__ uint32_t box_slot(uint32_t buf, int lane, int j) {
 }
 __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+// Two codes pushed into the low byte of a word with saturation to [0, 15]: c << 8 | sat(e1) << 4 | sat(e0).
+__device__ __forceinline__ uint32_t push_pair_u4(int e0, int e1, uint32_t c) {
+  uint32_t d;
+  asm("cvt.pack.sat.u4.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(e1), "r"(e0), "r"(c));
+  return d;
 }
 __device__ __forceinline__ float fma_sat(float a, float b, float c) {       // fma clamped to [0, 1]
   float d;
@@ -272,6 +280,36 @@ __device__ __forceinline__ void emit_chunk(const CUtensorMap* map_out, uint32_t 
   } else {
     const float magic = __uint_as_float(kMagicBits);
     uint32_t u[kChunk];
+    if (OUT == kOutC8 && q.qs_shift == 4) {
+      // Byte codes of 4 bits: r = magic + round_half_even(t) as below; (r - magic + z_o) 2^-149 is exact, and a denormal float
+      // whose bits are that integer (the sign bit makes a negative one of it).  The pack instruction clips eight of them to a
+      // word of nibbles, which two masks and two byte permutes spread: 38 instructions for 16 codes instead of 60.
+      const f32x2 magic2 = splat2(magic), mult2 = splat2(q.mult), tiny2 = splat2(__uint_as_float(1u)), z2 = splat2(q.z_tiny);
+      uint32_t w[4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        int k[8];
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) {
+          const f32x2 v2 = pack2(v[8 * h + e], v[8 * h + e + 1]);
+          float u0, u1;
+          unpack2(fma2(direct ? add2(v2, magic2) : fma2(v2, mult2, magic2), tiny2, z2), u0, u1);
+          k[e] = __float_as_int(u0);
+          k[e + 1] = __float_as_int(u1);
+        }
+        uint32_t p = 0;
+#pragma unroll
+        for (int e = 6; e >= 0; e -= 2) p = push_pair_u4(k[e], k[e + 1], p);
+        const uint32_t lo = p & 0x0F0F0F0Fu, hi = (p >> 4) & 0x0F0F0F0Fu;
+        code_sum = int(__dp4a(lo, 0x01010101u, __dp4a(hi, 0x01010101u, uint32_t(code_sum))));
+        w[2 * h] = __byte_perm(lo, hi, 0x5140);
+        w[2 * h + 1] = __byte_perm(lo, hi, 0x7362);
+      }
+      if ((c & 1) == 0) box_begin(lane);
+      sts128(box_slot(buf, lane, c & 1), w[0], w[1], w[2], w[3]);
+      if (c & 1) box_end(map_out, buf, lane, col0 - kChunk, row0);
+      return;
+    }
     if (OUT == kOutC8 && sat) {
       // Byte codes of at most 7 bits, no comparisons: r = magic + round_half_even(t) by the float adder (one fma
       // from the value when the scale is still to be applied), w = clamp((r - magic + z_o) / 2^bits, 0, 1) by a
