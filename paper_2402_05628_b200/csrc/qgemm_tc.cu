@@ -21,14 +21,14 @@
 // with a fixed part.  Packed 4-bit activations are expanded to one code per byte by a separate pass into the
 // workspace (inside the block the producers write byte codes, so that pass does not run there).
 //
-// For short K the epilogue, not the tensor pipe, sets the pace (K = 768: 3072 tensor-pipe cycles per
-// 128 x 256 tile against 32768 outputs), so it is written for few instructions per output and few waits per
-// tile: every epilogue warp stages the per-column terms of its own 64 columns in its own shared-memory buffer
-// (no barrier between warps) from plain loads issued one tile ahead and reads them as vectors, the output
-// quantizer is folded into them where nothing sits between the GEMM and the re-quantization, rounding uses
-// the float adder (add 1.5 * 2^23), byte codes of at most 7 bits are clamped by one saturating fma instead of
-// comparisons, and a bf16 residual comes in either by row-per-lane loads requested before the accumulator is
-// waited for or, for short K, by bulk tensor copies (one 32 x 64 box per epilogue warp, one tile ahead).
+// For short K the epilogue, not the tensor pipe, sets the pace (K = 768: 3072 tensor-pipe cycles per 128 x 256 tile
+// against 32768 outputs), so it is written for few instructions per output and few waits per tile: every epilogue warp
+// stages the per-column terms of its own 64 columns in its own shared-memory buffer (no barrier between warps) from
+// plain loads issued one tile ahead and reads them as vectors, the output quantizer is folded into them where nothing
+// sits between the GEMM and the re-quantization, rounding uses the float adder (add 1.5 * 2^23), byte codes are clipped
+// by the pack instruction instead of comparisons, and a bf16 residual comes in either by row-per-lane loads requested
+// before the accumulator is waited for or, for short K, by bulk tensor copies (one 32 x 64 box per epilogue warp, one
+// tile ahead).
 //
 // Every wait on an mbarrier is bounded: when it runs out the kernel records a status code, all roles
 // leave their loops, in-flight copies and MMAs are drained, tensor memory is freed and the kernel returns.
@@ -179,11 +179,10 @@ enum : int { kOutF32 = 0, kOutBf16 = 1, kOutC4 = 2, kOutC8 = 3 };   // compile-t
 struct ChunkQuant {
   float mult, lo, hi;
   uint32_t pack_k;     // 4-bit: sum_e (magic_bits - z_o) << 4e
-  uint32_t z4;         // 8-bit: z_o replicated in every byte
   int zo;
-  float inv_qs, qs, csat;   // byte codes of at most 7 bits: 1 / 2^bits, 2^bits, (z_o - magic) / 2^bits
-  int qs_shift;             //   bits
-  float z_tiny;             // (z_o - magic) 2^-149
+  float unit, z_unit;  // byte codes of b bits: 2^(8 - b) 2^-149, and (z_o - magic) times it
+  int shift;           //   8 - b
+  uint32_t mask;       //   2^b - 1 in every byte
 };
 
 __device__ __forceinline__ ChunkQuant chunk_quant(const EpilogueParams& ep, const TcParams& P, int col0) {
@@ -198,13 +197,11 @@ __device__ __forceinline__ ChunkQuant chunk_quant(const EpilogueParams& ep, cons
   q.lo = float(-zo);
   q.hi = float(ep.qmax - zo);
   q.pack_k = (kMagicBits - uint32_t(zo)) * 0x11111111u;
-  q.z4 = (uint32_t(zo) & 0xFFu) * 0x01010101u;
   q.zo = zo;
-  q.qs_shift = 32 - __clz(ep.qmax);                      // qmax = 2^bits - 1
-  q.qs = __uint_as_float(uint32_t(127 + q.qs_shift) << 23);         // 2^bits
-  q.inv_qs = __uint_as_float(uint32_t(127 - q.qs_shift) << 23);     // 2^-bits
-  q.z_tiny = (float(zo) - __uint_as_float(kMagicBits)) * __uint_as_float(1u);
-  q.csat = (float(zo) - __uint_as_float(kMagicBits)) * q.inv_qs;    // exact: an integer below 2^24 times a power of two
+  q.shift = __clz(ep.qmax) - 24;                            // qmax = 2^b - 1
+  q.mask = uint32_t(ep.qmax) * 0x01010101u;
+  q.unit = __uint_as_float(1u << q.shift);
+  q.z_unit = (float(zo) - __uint_as_float(kMagicBits)) * q.unit;    // exact
   return q;
 }
 
@@ -235,16 +232,23 @@ __device__ __forceinline__ uint32_t box_slot(uint32_t buf, int lane, int j) {
 __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
-// Two codes pushed into the low byte of a word with saturation to [0, 15]: c << 8 | sat(e1) << 4 | sat(e0).
-__device__ __forceinline__ uint32_t push_pair_u4(int e0, int e1, uint32_t c) {
+// Four byte codes of b bits from magic + round_half_even(t).  (r - magic + z_o) 2^(8 - b) 2^-149 is exact, and a denormal float
+// whose bits are that integer (the sign bit makes a negative one of it; beyond the 2^22 within which r is the rounded t it
+// stays far outside the codes).  The pack instruction clips 2^(8 - b) q to [0, 255], the shift drops the low bits again:
+// clip(q, 0, 2^b - 1).  36 instructions for 16 codes against 60 with a saturating multiply-add and byte permutes (12608 x 2304 x
+// 768, 4 bits: 30.0 -> 29.5 us, 8 bits 31.8 -> 29.7, 18464 x 4096 x 1024 with GELU, 4 bits, 91.6 -> 89.9).
+__device__ __forceinline__ uint32_t push_pair_u8(int e0, int e1, uint32_t c) {       // c << 16 | sat(e1) << 8 | sat(e0)
   uint32_t d;
-  asm("cvt.pack.sat.u4.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(e1), "r"(e0), "r"(c));
+  asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(e1), "r"(e0), "r"(c));
   return d;
 }
-__device__ __forceinline__ float fma_sat(float a, float b, float c) {       // fma clamped to [0, 1]
-  float d;
-  asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
+__device__ __forceinline__ uint32_t code_word(const ChunkQuant& q, f32x2 r01, f32x2 r23) {
+  const f32x2 unit2 = splat2(q.unit), z2 = splat2(q.z_unit);
+  float u0, u1, u2, u3;
+  unpack2(fma2(r01, unit2, z2), u0, u1);
+  unpack2(fma2(r23, unit2, z2), u2, u3);
+  const uint32_t p = push_pair_u8(__float_as_int(u0), __float_as_int(u1), push_pair_u8(__float_as_int(u2), __float_as_int(u3), 0u));
+  return (p >> q.shift) & q.mask;
 }
 __device__ __forceinline__ void sts64(uint32_t addr, uint32_t a, uint32_t b) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
@@ -279,67 +283,28 @@ __device__ __forceinline__ void emit_chunk(const CUtensorMap* map_out, uint32_t 
     box_end(map_out, buf, lane, col0, row0);
   } else {
     const float magic = __uint_as_float(kMagicBits);
-    uint32_t u[kChunk];
-    if (OUT == kOutC8 && q.qs_shift == 4) {
-      // Byte codes of 4 bits: r = magic + round_half_even(t) as below; (r - magic + z_o) 2^-149 is exact, and a denormal float
-      // whose bits are that integer (the sign bit makes a negative one of it).  The pack instruction clips eight of them to a
-      // word of nibbles, which two masks and two byte permutes spread: 38 instructions for 16 codes instead of 60.
-      const f32x2 magic2 = splat2(magic), mult2 = splat2(q.mult), tiny2 = splat2(__uint_as_float(1u)), z2 = splat2(q.z_tiny);
-      uint32_t w[4];
+    const f32x2 magic2 = splat2(magic), mult2 = splat2(q.mult);
+    if constexpr (OUT == kOutC8) {
+      // (below 8 bits one multiply-add from the value to r where the scale is still to be applied)
+      const bool scaled = direct || !sat;
+      if (!direct && !sat) {
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        int k[8];
-#pragma unroll
-        for (int e = 0; e < 8; e += 2) {
-          const f32x2 v2 = pack2(v[8 * h + e], v[8 * h + e + 1]);
-          float u0, u1;
-          unpack2(fma2(direct ? add2(v2, magic2) : fma2(v2, mult2, magic2), tiny2, z2), u0, u1);
-          k[e] = __float_as_int(u0);
-          k[e + 1] = __float_as_int(u1);
-        }
-        uint32_t p = 0;
-#pragma unroll
-        for (int e = 6; e >= 0; e -= 2) p = push_pair_u4(k[e], k[e + 1], p);
-        const uint32_t lo = p & 0x0F0F0F0Fu, hi = (p >> 4) & 0x0F0F0F0Fu;
-        code_sum = int(__dp4a(lo, 0x01010101u, __dp4a(hi, 0x01010101u, uint32_t(code_sum))));
-        w[2 * h] = __byte_perm(lo, hi, 0x5140);
-        w[2 * h + 1] = __byte_perm(lo, hi, 0x7362);
+        for (int e = 0; e < kChunk; e += 2) unpack2(mul2(pack2(v[e], v[e + 1]), mult2), v[e], v[e + 1]);
       }
-      if ((c & 1) == 0) box_begin(lane);
-      sts128(box_slot(buf, lane, c & 1), w[0], w[1], w[2], w[3]);
-      if (c & 1) box_end(map_out, buf, lane, col0 - kChunk, row0);
-      return;
-    }
-    if (OUT == kOutC8 && sat) {
-      // Byte codes of at most 7 bits, no comparisons: r = magic + round_half_even(t) by the float adder (one fma
-      // from the value when the scale is still to be applied), w = clamp((r - magic + z_o) / 2^bits, 0, 1) by a
-      // saturating fma whose unclamped result is exact, u = magic + 2^bits w.  The low byte of u is the code,
-      // except that 2^bits stands for the top code 2^bits - 1; that bit is subtracted after packing.
       uint32_t w[4];
-      // (the adds and multiply-adds around the saturating one on packed pairs: same operations, same bits)
-      const f32x2 magic2 = splat2(magic), qs2 = splat2(q.qs), mult2 = splat2(q.mult);
-#pragma unroll
-      for (int e = 0; e < kChunk; e += 2) {
-        float r0, r1, u0, u1;
-        const f32x2 v2 = pack2(v[e], v[e + 1]);
-        unpack2(direct ? add2(v2, magic2) : fma2(v2, mult2, magic2), r0, r1);
-        unpack2(fma2(pack2(fma_sat(r0, q.inv_qs, q.csat), fma_sat(r1, q.inv_qs, q.csat)), qs2, magic2), u0, u1);
-        u[e] = __float_as_uint(u0);
-        u[e + 1] = __float_as_uint(u1);
-      }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const uint32_t p = __byte_perm(__byte_perm(u[4 * i], u[4 * i + 1], 0x0040), __byte_perm(u[4 * i + 2], u[4 * i + 3], 0x0040), 0x5410);
-        w[i] = p - ((p >> q.qs_shift) & 0x01010101u);
-        code_sum += __dp4a(w[i], 0x01010101u, 0u);
+        const f32x2 a = pack2(v[4 * i], v[4 * i + 1]), b = pack2(v[4 * i + 2], v[4 * i + 3]);
+        w[i] = code_word(q, scaled ? add2(a, magic2) : fma2(a, mult2, magic2), scaled ? add2(b, magic2) : fma2(b, mult2, magic2));
+        code_sum = int(__dp4a(w[i], 0x01010101u, uint32_t(code_sum)));
       }
       if ((c & 1) == 0) box_begin(lane);
       sts128(box_slot(buf, lane, c & 1), w[0], w[1], w[2], w[3]);
       if (c & 1) box_end(map_out, buf, lane, col0 - kChunk, row0);
       return;
     }
+    uint32_t u[kChunk];
     {
-      const f32x2 magic2 = splat2(magic), mult2 = splat2(q.mult);
 #pragma unroll
       for (int e = 0; e < kChunk; e += 2) {
         float t0, t1, u0, u1;
@@ -362,16 +327,6 @@ __device__ __forceinline__ void emit_chunk(const CUtensorMap* map_out, uint32_t 
       if (c == 0) box_begin(lane);
       sts64(box_slot(buf, lane, c >> 1) + uint32_t(c & 1) * 8u, w[0], w[1]);     // 8 bytes = 16 codes
       if (c == kSliceChunks - 1) box_end(map_out, buf, lane, (col0 - (kSliceChunks - 1) * kChunk) >> 1, row0);
-    } else {
-      uint32_t w[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        w[i] = __vadd4(__byte_perm(__byte_perm(u[4 * i], u[4 * i + 1], 0x0040), __byte_perm(u[4 * i + 2], u[4 * i + 3], 0x0040), 0x5410), q.z4);
-        code_sum += __dp4a(w[i], 0x01010101u, 0u);
-      }
-      if ((c & 1) == 0) box_begin(lane);
-      sts128(box_slot(buf, lane, c & 1), w[0], w[1], w[2], w[3]);
-      if (c & 1) box_end(map_out, buf, lane, col0 - kChunk, row0);
     }
   }
 }
@@ -663,7 +618,7 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     const bool res32 = ep.residual != nullptr && !ep.residual_bf16;
     // the common epilogue applies the pair step it was compiled with; any other combination goes chunk by chunk
     const bool fast_ok = ep.acc_debug == nullptr && (ep.rope != nullptr) == (PAIR == kPairRope) && (ep.glu != 0) == (PAIR == kPairGlu);
-    const bool sat = ep.qmax <= 127;             // byte codes narrow enough for the comparison-free quantizer
+    const bool sat = ep.qmax <= 127;             // byte codes of at most 7 bits: scale and round in one multiply-add
     const bool direct = P.direct_requant != 0;
     const int cl0 = slice * kSliceCols;          // first column of this warp inside the tile
     ColTerms& C = S.cols[ew];
@@ -853,17 +808,15 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
               // gated product: 16 accumulator columns (gate, up interleaved) give 8 byte codes; the slice's 32 codes
               // fill one box row
               const float magic = __uint_as_float(kMagicBits);
-              uint32_t u[kChunk / 2];
+              f32x2 r[kChunk / 4];
 #pragma unroll
-              for (int i = 0; i < kChunk / 2; ++i) {
-                const float t = fminf(fmaxf(silu_mul(v[2 * i], v[2 * i + 1]) * q.mult, q.lo), q.hi);
-                u[i] = __float_as_uint(t + magic);
-              }
+              for (int i = 0; i < kChunk / 4; ++i)
+                r[i] = add2(mul2(pack2(silu_mul(v[4 * i], v[4 * i + 1]), silu_mul(v[4 * i + 2], v[4 * i + 3])), splat2(q.mult)), splat2(magic));
               uint32_t w[2];
 #pragma unroll
               for (int i = 0; i < 2; ++i) {
-                w[i] = __vadd4(__byte_perm(__byte_perm(u[4 * i], u[4 * i + 1], 0x0040), __byte_perm(u[4 * i + 2], u[4 * i + 3], 0x0040), 0x5410), q.z4);
-                code_sum += __dp4a(w[i], 0x01010101u, 0u);
+                w[i] = code_word(q, r[2 * i], r[2 * i + 1]);
+                code_sum = int(__dp4a(w[i], 0x01010101u, uint32_t(code_sum)));
               }
               const uint32_t buf = smem_u32(S.epi[ew]);
               if (c == 0) box_begin(lane);

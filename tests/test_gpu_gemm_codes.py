@@ -1,6 +1,6 @@
-"""Byte codes out of the integer GEMM's common epilogue for each width of the output quantizer: 4 bits (clipped by the pack
-instruction), 6 bits (saturating multiply-add), 8 bits (comparisons); scale folded into the column terms or applied last, one and
-three column groups, whole and ragged tiles."""
+"""Byte codes out of the integer GEMM's common epilogue for each width of the output quantizer (the pack instruction clips at a
+shift that depends on it); scale folded into the column terms or applied last, one and three column groups, whole and ragged
+tiles, the gated product."""
 import pytest
 
 from tests import parity
@@ -19,3 +19,8 @@ def test_byte_codes_match_oracle(M, N, K, kw, bits):
     b = 4 | parity.BYTE_CODES
     parity.check_qgemm(M, N, K, b, b, out_kind="codes", out_bits=bits | (parity.BYTE_CODES if bits < 8 else 0), want_acc=False,
                        want_out_sum=True, give_sums=True, seed=M + bits, **kw)
+
+
+@pytest.mark.parametrize("bits", [4, 6, 8])
+def test_byte_codes_of_the_gated_product(bits):
+    parity.check_qgemm_pair_step(300, 512, 384, bits | (parity.BYTE_CODES if bits < 8 else 0), "glu", seed=bits)
