@@ -14,7 +14,8 @@
  *    The device entry points allocate no device memory: scratch comes from the `workspace` argument,
  *    sized by the matching *_workspace_bytes() call.
  *  - Device work is enqueued on `stream` (a cudaStream_t passed as void*; NULL = default stream) and
- *    the call returns without synchronising.
+ *    the call returns without synchronising.  It is ordered behind everything already on `stream`, parameters
+ *    included: weights, factors and tables may be written by work queued just ahead of the call.
  *  - Codes are unsigned integers in [0, 2^b - 1] exactly as Eq. 4 produces them.  4-bit codes are
  *    packed two per byte (even index in the low nibble); 6- and 8-bit codes take one byte each.
  *    Every `bits` argument or field may carry the flag REPQ_BYTE_CODES (e.g. 4 | REPQ_BYTE_CODES): the

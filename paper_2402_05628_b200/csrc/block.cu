@@ -149,8 +149,10 @@ static repq_status block_forward_impl(const repq_block_desc* dp, const repq_bloc
   REPQ_MARK();
 
   // ---- X_bar = MSA(LN(X)) + X
+  // (the first kernel waits for whatever precedes the block in the stream, its parameters' writers included, before it lets
+  // the next one start: from the second kernel on parameters are settled)
   REPQ_TRY(launch_ln_quant(x, d.act_dtype, M, D, D, p.ln1_gamma_t, p.ln1_beta_t, d.eps, d.norm_kind, p.ln1_s, p.ln1_z,
-                           ab, ln_c, L.ld_a, asum, clear, st));
+                           ab, ln_c, L.ld_a, asum, clear, Params::streamed, st));
   REPQ_MARK();
   {
     repq_gemm_desc g = linear_desc(d, M, 3 * D, D, ln_c, L.ld_a, p.ln1_s, p.ln1_z, asum, p.qkv);
@@ -161,7 +163,7 @@ static repq_status block_forward_impl(const repq_block_desc* dp, const repq_bloc
     if (d.rope) {                       // Q and K ranges rotated ahead of their quantizers, V left alone
       g.rope_cos_sin = p.rope_cos_sin; g.rope_period = S; g.rope_dim = dh; g.rope_groups = 2;
     }
-    REPQ_TRY(repq_qgemm(&g, gws, gws_bytes, stream));
+    REPQ_TRY(run_qgemm(g, gws, gws_bytes, Params::settled, st));
   }
   REPQ_MARK();
   if (!d.staged_attention) {
@@ -225,12 +227,12 @@ static repq_status block_forward_impl(const repq_block_desc* dp, const repq_bloc
     g.residual = x; g.residual_dtype = d.act_dtype; g.ld_residual = D;
     g.out_kind = d.act_dtype == REPQ_F32 ? REPQ_OUT_F32 : REPQ_OUT_BF16;
     g.out = xbar; g.ldo = D;
-    REPQ_TRY(repq_qgemm(&g, gws, gws_bytes, stream));
+    REPQ_TRY(run_qgemm(g, gws, gws_bytes, Params::settled, st));
   }
   REPQ_MARK();
   // ---- Y = MLP(LN(X_bar)) + X_bar
-  REPQ_TRY(repq_ln_quant(xbar, d.act_dtype, M, D, D, p.ln2_gamma_t, p.ln2_beta_t, d.eps, d.norm_kind, p.ln2_s, p.ln2_z,
-                         ab, ln_c, L.ld_a, asum, stream));
+  REPQ_TRY(launch_ln_quant(xbar, d.act_dtype, M, D, D, p.ln2_gamma_t, p.ln2_beta_t, d.eps, d.norm_kind, p.ln2_s, p.ln2_z,
+                           ab, ln_c, L.ld_a, asum, ClearWords{}, Params::settled, st));
   REPQ_MARK();
   {
     const bool swiglu = d.mlp_kind == REPQ_MLP_SWIGLU;
@@ -240,7 +242,7 @@ static repq_status block_forward_impl(const repq_block_desc* dp, const repq_bloc
     g.out_kind = REPQ_OUT_CODES; g.out_bits = ab; g.out_groups = 1;
     g.out_scale[0] = p.s_hidden; g.out_zero[0] = p.z_hidden;
     g.out = hid_c; g.ldo = L.ld_h; g.out_row_sum = asum_h;
-    REPQ_TRY(repq_qgemm(&g, gws, gws_bytes, stream));
+    REPQ_TRY(run_qgemm(g, gws, gws_bytes, Params::settled, st));
   }
   REPQ_MARK();
   {
@@ -248,7 +250,7 @@ static repq_status block_forward_impl(const repq_block_desc* dp, const repq_bloc
     g.residual = xbar; g.residual_dtype = d.act_dtype; g.ld_residual = D;
     g.out_kind = d.out_dtype == REPQ_F32 ? REPQ_OUT_F32 : REPQ_OUT_BF16;
     g.out = y; g.ldo = D;
-    REPQ_TRY(repq_qgemm(&g, gws, gws_bytes, stream));
+    REPQ_TRY(run_qgemm(g, gws, gws_bytes, Params::settled, st));
   }
   REPQ_MARK();
   return REPQ_OK;

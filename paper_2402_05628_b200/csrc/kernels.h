@@ -5,12 +5,21 @@
 
 namespace repq {
 
+// Whether a kernel may read its parameters (weight codes, normalisation factors) ahead of the dependency wait.  `streamed`:
+// no, like every other operand they may be the work of the kernel just ahead in the stream (the entry points of the library
+// promise stream order).  `settled`: a kernel of the same chain that waited for everything before the chain has started
+// already, so whatever wrote the parameters has completed (the kernels of a block behind its first one).
+enum class Params { streamed, settled };
+
 // LayerNorm + quantization (repq_ln_quant), which can also set a run of words to zero: row-sum accumulators that later
 // kernels of a chain add into, without a launch of their own.
 struct ClearWords { int32_t* at = nullptr; int64_t n = 0; };
 repq_status launch_ln_quant(const void* x, int x_dtype, int64_t rows, int D, int64_t ldx, const float* gamma_t,
                             const float* beta_t, float eps, int norm_kind, float s_t, int z_t, int bits, uint8_t* codes,
-                            int64_t ld_codes_bytes, int32_t* row_sum, ClearWords clear, cudaStream_t st);
+                            int64_t ld_codes_bytes, int32_t* row_sum, ClearWords clear, Params params, cudaStream_t st);
+
+// repq_qgemm, with the caller's word on the weights.
+repq_status run_qgemm(const repq_gemm_desc& d, void* workspace, size_t workspace_bytes, Params params, cudaStream_t st);
 
 // Row sums of a code matrix: out[r] = sum_c codes[r, c] (zero-point correction terms).
 repq_status launch_row_sum(const uint8_t* codes, int bits, int64_t rows, int64_t n, int64_t ld_bytes,
@@ -43,7 +52,7 @@ size_t qgemm_workspace_least(const repq_gemm_desc& d);
 // Integer GEMM for few tokens (weights on the M side of the tensor-core instruction): plain products, byte codes, both
 // row sums given; `preferred` says whether it takes the problem and is the faster one.
 bool qgemm_skinny_preferred(const repq_gemm_desc& d);
-repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, bool weights_ready, cudaStream_t st);
+repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, Params params, cudaStream_t st);
 
 // P.V (Eqs. 16-17): kernel parameters shared by the two implementations, storage widths already resolved
 // (bits_v is 4 for packed codes, 8 for byte codes).

@@ -131,11 +131,11 @@ __device__ __forceinline__ void group_sum(int (&v)[kRows]) {
 
 template <typename T, int TPR, int kVPT, bool kPack4, bool kFull>
 __global__ void __launch_bounds__((TPR > 256 ? TPR : 256),
-                                  (kVPT <= 2 && TPR == 256 ? (factors_in_registers(kVPT, TPR, sizeof(T)) ? 2 : 3) : sizeof(T) == 4 && TPR == 32 && (kVPT == 3 || kVPT == 4) ? 2 : 0))
+                                  (kVPT <= 2 && TPR == 256 ? (factors_in_registers(kVPT, TPR, sizeof(T)) ? 2 : 3) : TPR == 256 ? 2 : sizeof(T) == 4 && TPR == 32 && (kVPT == 3 || kVPT == 4) ? 2 : 0))
 ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
                 const float* __restrict__ gamma_t, const float* __restrict__ beta_t, float eps, int rms,
                 float inv_s, int z, int qmax, uint8_t* __restrict__ codes, int64_t ldc,
-                int32_t* __restrict__ row_sum, int32_t* __restrict__ clear, int64_t n_clear) {
+                int32_t* __restrict__ row_sum, int32_t* __restrict__ clear, int64_t n_clear, bool settled) {
   constexpr int kRows = rows_in_flight(kVPT, TPR, kFull, sizeof(T));
   constexpr int kBlock = TPR > 256 ? TPR : 256;
   constexpr int kGroups = kBlock / TPR;
@@ -152,62 +152,10 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
   __shared__ float2 red[kWide ? 2 : 1][kBlock / 32 * kRows];
   __shared__ int red_c[kWide ? 2 : 1][kBlock / 32 * kRows];
 
-  float* s_g = s_gb;
-  float* s_b = s_gb + D;
-  // |t| <= sqrt(D) |gamma~/s~| + |beta~/s~|.  While that bound stays below 2^22 the round operation is one packed
-  // float add of 1.5 * 2^23 (round half to even by the adder, rint(t) left in the low mantissa bits); otherwise t
-  // is clamped and converted, so that adding z cannot wrap (a whole-kernel decision, taken here once).
-  const float root_d = sqrtf(float(D));
-  bool wide = false;
-  f32x2 g_reg[kRegFactors ? kVPT : 1][kChunk / 2], b_reg[kRegFactors ? kVPT : 1][kChunk / 2];
-  if constexpr (kRegFactors) {
-    // every thread works on the same columns of every row: its factors are loaded once
-#pragma unroll
-    for (int i = 0; i < kVPT; ++i) {
-      const int c = threadIdx.x % TPR + i * TPR;
-      const bool on = kFull || c < D / kChunk;
-      float gi[kChunk], bi[kChunk];
-#pragma unroll
-      for (int e = 0; e < kChunk; ++e) {
-        gi[e] = on ? __ldg(gamma_t + c * kChunk + e) * inv_s : 0.f;
-        bi[e] = on ? __ldg(beta_t + c * kChunk + e) * inv_s : 0.f;
-      }
-#pragma unroll
-      for (int e = 0; e < kChunk; ++e) wide = wide || !(fabsf(gi[e]) * root_d + fabsf(bi[e]) < 4.0e6f);
-#pragma unroll
-      for (int e = 0; e < kChunk / 2; ++e) {
-        g_reg[i][e] = pack2(gi[2 * e], gi[2 * e + 1]);
-        b_reg[i][e] = pack2(bi[2 * e], bi[2 * e + 1]);
-      }
-    }
-  } else {
-    // layout: the first halves (4 floats) of all chunks, then the second halves, so that the 16-byte reads of
-    // neighbouring lanes are neighbours in shared memory (chunk by chunk they would sit 32 bytes apart: two-way
-    // bank conflicts)
-    const int half_stride = D / 2;
-    for (int i = threadIdx.x; i < D; i += kBlock) {
-      const float gi = __ldg(gamma_t + i) * inv_s, bi = __ldg(beta_t + i) * inv_s;
-      const int at = ((i >> 2) & 1) * half_stride + (i >> 3) * 4 + (i & 3);
-      s_g[at] = gi;
-      s_b[at] = bi;
-      wide = wide || !(fabsf(gi) * root_d + fabsf(bi) < 4.0e6f);
-    }
-  }
-  const bool guard = __syncthreads_or(wide) != 0;
-  // gamma~ and beta~ are parameters; x and the outputs belong to the chain of kernels
-  grid_dependency_wait();
-  grid_dependency_trigger();
-  for (int64_t i = int64_t(blockIdx.x) * kBlock + threadIdx.x; i < n_clear; i += int64_t(gridDim.x) * kBlock) clear[i] = 0;
-
   const int tig = threadIdx.x % TPR;             // thread in group
   const int group = threadIdx.x / TPR;
   const int group_first_warp = (group * TPR) >> 5;
   const int nchunks = D / kChunk;
-  const float inv_d = 1.f / float(D);
-  const uint32_t qmax4 = uint32_t(qmax) * 0x01010101u;
-  constexpr uint32_t kMagicBits = 0x4B400000u;   // 1.5 * 2^23
-  const f32x2 magic2 = splat2(__uint_as_float(kMagicBits));
-  const int z_less_magic = z - int(kMagicBits);
 
   // The rows of the next iteration are requested while those of the current one are processed, so that loads
   // stay in flight through the reductions and the packing.
@@ -226,8 +174,91 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
       }
     }
   };
+  const int64_t first_rows = int64_t(blockIdx.x) * kRowsPerBlock + group * kRows;
+  // Factors that the kernel ahead in the stream may have written are read behind the wait, settled ones while that kernel
+  // finishes.  (Loads past L1: what that kernel wrote must not meet an older line.)
+  // The next kernel's start is allowed as soon as everything ahead has completed, so that its prologue runs beside the staging.
+  if (!settled) {
+    grid_dependency_wait();
+    grid_dependency_trigger();
+  }
+
+  float* s_g = s_gb;
+  float* s_b = s_gb + D;
+  // |t| <= sqrt(D) |gamma~/s~| + |beta~/s~|.  While that bound stays below 2^22 the round operation is one packed
+  // float add of 1.5 * 2^23 (round half to even by the adder, rint(t) left in the low mantissa bits); otherwise t
+  // is clamped and converted, so that adding z cannot wrap (a whole-kernel decision, taken here once).
+  const float root_d = sqrtf(float(D));
+  bool wide = false;
+  f32x2 g_reg[kRegFactors ? kVPT : 1][kChunk / 2], b_reg[kRegFactors ? kVPT : 1][kChunk / 2];
+  if constexpr (kRegFactors) {
+    if (!settled) fetch(first_rows);
+    // every thread works on the same columns of every row: its factors are loaded once
+#pragma unroll
+    for (int i = 0; i < kVPT; ++i) {
+      const int c = threadIdx.x % TPR + i * TPR;
+      const bool on = kFull || c < D / kChunk;
+      float gi[kChunk], bi[kChunk];
+#pragma unroll
+      for (int e = 0; e < kChunk; ++e) {
+        gi[e] = on ? __ldcg(gamma_t + c * kChunk + e) * inv_s : 0.f;
+        bi[e] = on ? __ldcg(beta_t + c * kChunk + e) * inv_s : 0.f;
+      }
+#pragma unroll
+      for (int e = 0; e < kChunk; ++e) wide = wide || !(fabsf(gi[e]) * root_d + fabsf(bi[e]) < 4.0e6f);
+#pragma unroll
+      for (int e = 0; e < kChunk / 2; ++e) {
+        g_reg[i][e] = pack2(gi[2 * e], gi[2 * e + 1]);
+        b_reg[i][e] = pack2(bi[2 * e], bi[2 * e + 1]);
+      }
+    }
+  } else {
+    // layout: the first halves (4 floats) of all chunks, then the second halves, so that the 16-byte reads of
+    // neighbouring lanes are neighbours in shared memory (chunk by chunk they would sit 32 bytes apart: two-way
+    // bank conflicts)
+    const int half_stride = D / 2;
+    // Several factors of a thread in flight at a time, and the first rows asked for behind the first of them, so that rows and
+    // factors arrive together.  (What reading behind the wait costs a block pass of 64 x 197 tokens x 768: 1.2 us of 209, with
+    // the rows first and the factors one by one 2.1; one image through a ViT-S block 0.5 of 32.)
+    constexpr int kInFlight = 8;
+    for (int base = 0; base < D; base += kInFlight * kBlock) {
+      float gi[kInFlight], bi[kInFlight];
+#pragma unroll
+      for (int k = 0; k < kInFlight; ++k) {
+        const int i = base + k * kBlock + threadIdx.x;
+        gi[k] = i < D ? __ldcg(gamma_t + i) : 0.f;
+        bi[k] = i < D ? __ldcg(beta_t + i) : 0.f;
+      }
+      if (!settled && base == 0) fetch(first_rows);
+#pragma unroll
+      for (int k = 0; k < kInFlight; ++k) {
+        const int i = base + k * kBlock + threadIdx.x;
+        if (i >= D) break;
+        gi[k] *= inv_s;
+        bi[k] *= inv_s;
+        const int at = ((i >> 2) & 1) * half_stride + (i >> 3) * 4 + (i & 3);
+        s_g[at] = gi[k];
+        s_b[at] = bi[k];
+        wide = wide || !(fabsf(gi[k]) * root_d + fabsf(bi[k]) < 4.0e6f);
+      }
+    }
+  }
+  const bool guard = __syncthreads_or(wide) != 0;
+  // x and the outputs belong to the chain of kernels
+  if (settled) {
+    grid_dependency_wait();
+    grid_dependency_trigger();
+    fetch(first_rows);
+  }
+  for (int64_t i = int64_t(blockIdx.x) * kBlock + threadIdx.x; i < n_clear; i += int64_t(gridDim.x) * kBlock) clear[i] = 0;
+
+  const float inv_d = 1.f / float(D);
+  const uint32_t qmax4 = uint32_t(qmax) * 0x01010101u;
+  constexpr uint32_t kMagicBits = 0x4B400000u;   // 1.5 * 2^23
+  const f32x2 magic2 = splat2(__uint_as_float(kMagicBits));
+  const int z_less_magic = z - int(kMagicBits);
+
   const int64_t stride = int64_t(gridDim.x) * kRowsPerBlock;
-  fetch(int64_t(blockIdx.x) * kRowsPerBlock + group * kRows);
 
   // the warp's slice of a row, and the slice its lane merges
   const int lane_w = threadIdx.x & 31;
@@ -455,7 +486,7 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
 template <typename T, int TPR, int kVPT>
 repq_status launch(const T* x, int64_t rows, int D, int64_t ldx, const float* g, const float* b, float eps,
                    int rms, float s_t, int z, int bits, uint8_t* codes, int64_t ldc, int32_t* row_sum,
-                   ClearWords clear, cudaStream_t st) {
+                   ClearWords clear, Params params, cudaStream_t st) {
   constexpr int kBlock = TPR > 256 ? TPR : 256;
   const bool full = D == TPR * kVPT * kChunk;   // the row fills the group exactly: no chunk is predicated
   const int rows_per_block = kBlock / TPR * rows_in_flight(kVPT, TPR, full, sizeof(T));
@@ -474,7 +505,7 @@ repq_status launch(const T* x, int64_t rows, int D, int64_t ldx, const float* g,
   REPQ_TRY(resident_blocks(memo[pack][full], kern, kBlock, smem, &resident));
   const int64_t cap = int64_t(sm_count()) * resident;
   const int grid = int(need < cap ? need : cap);
-  REPQ_CUDA(launch_chained(kern, dim3(grid), dim3(kBlock), smem, st, x, rows, D, ldx, g, b, eps, rms, inv_s, z, qmax, codes, ldc, row_sum, clear.at, clear.n));
+  REPQ_CUDA(launch_chained(kern, dim3(grid), dim3(kBlock), smem, st, x, rows, D, ldx, g, b, eps, rms, inv_s, z, qmax, codes, ldc, row_sum, clear.at, clear.n, params == Params::settled));
   note_launch();
   return REPQ_OK;
 }
@@ -482,27 +513,27 @@ repq_status launch(const T* x, int64_t rows, int D, int64_t ldx, const float* g,
 template <typename T, int TPR>
 repq_status launch_vpt(int vpt, const T* x, int64_t rows, int D, int64_t ldx, const float* g, const float* b, float eps,
                        int rms, float s_t, int z, int bits, uint8_t* codes, int64_t ldc, int32_t* row_sum,
-                       ClearWords clear, cudaStream_t st) {
+                       ClearWords clear, Params params, cudaStream_t st) {
   switch (vpt) {
-    case 1: return launch<T, TPR, 1>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
-    case 2: return launch<T, TPR, 2>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
-    case 3: return launch<T, TPR, 3>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
-    case 4: return launch<T, TPR, 4>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
-    case 5: return launch<T, TPR, (TPR >= 32 && TPR <= 128 ? 5 : 4)>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
-    default: return launch<T, TPR, (TPR >= 32 && TPR <= 128 ? 6 : 4)>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
+    case 1: return launch<T, TPR, 1>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, params, st);
+    case 2: return launch<T, TPR, 2>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, params, st);
+    case 3: return launch<T, TPR, 3>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, params, st);
+    case 4: return launch<T, TPR, 4>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, params, st);
+    case 5: return launch<T, TPR, (TPR >= 32 && TPR <= 128 ? 5 : 4)>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, params, st);
+    default: return launch<T, TPR, (TPR >= 32 && TPR <= 128 ? 6 : 4)>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, params, st);
   }
 }
 
 template <typename T>
 repq_status dispatch(const T* x, int64_t rows, int D, int64_t ldx, const float* g, const float* b, float eps,
                      int rms, float s_t, int z, int bits, uint8_t* codes, int64_t ldc, int32_t* row_sum,
-                     ClearWords clear, cudaStream_t st) {
+                     ClearWords clear, Params params, cudaStream_t st) {
   const int nchunks = D / kChunk;
   // The fewest warps whose threads hold the row in at most six chunks: a row of one warp has no barrier, and what a row costs
   // beside its elements (shuffles, merges, barrier) is paid per thread (measured, 1536 elements: 45 us with one warp, 59 with
   // two; 3072: 49 and 61).  Eight chunks leave too few warps on the SM (2048 float elements: 56 against 48).
 #define REPQ_LN_CASE(TPR, MOST) \
-  if (nchunks <= TPR * MOST) return launch_vpt<T, TPR>((nchunks + TPR - 1) / TPR, x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, st);
+  if (nchunks <= TPR * MOST) return launch_vpt<T, TPR>((nchunks + TPR - 1) / TPR, x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, params, st);
   REPQ_LN_CASE(8, 4)
   REPQ_LN_CASE(16, 4)
   REPQ_LN_CASE(32, 6)
@@ -518,7 +549,7 @@ repq_status dispatch(const T* x, int64_t rows, int D, int64_t ldx, const float* 
 
 repq_status launch_ln_quant(const void* x, int x_dtype, int64_t rows, int D, int64_t ldx, const float* gamma_t,
                             const float* beta_t, float eps, int norm_kind, float s_t, int z_t, int bits, uint8_t* codes,
-                            int64_t ld_codes_bytes, int32_t* row_sum, ClearWords clear, cudaStream_t st) {
+                            int64_t ld_codes_bytes, int32_t* row_sum, ClearWords clear, Params params, cudaStream_t st) {
   REPQ_REQUIRE(rows >= 0 && D > 0, REPQ_INVALID_ARG, "ln_quant: rows must be >= 0 and D > 0");
   if (rows == 0) return REPQ_OK;
   REPQ_REQUIRE(x && gamma_t && beta_t && codes, REPQ_INVALID_ARG, "ln_quant: NULL pointer");
@@ -538,8 +569,8 @@ repq_status launch_ln_quant(const void* x, int x_dtype, int64_t rows, int D, int
                "ln_quant: codes rows must be %d-byte aligned", int(unit));
   const int rms = norm_kind == REPQ_NORM_RMS;
   if (x_dtype == REPQ_F32)
-    return dispatch(static_cast<const float*>(x), rows, D, ldx, gamma_t, beta_t, eps, rms, s_t, z_t, bits, codes, ld_codes_bytes, row_sum, clear, st);
-  return dispatch(static_cast<const __nv_bfloat16*>(x), rows, D, ldx, gamma_t, beta_t, eps, rms, s_t, z_t, bits, codes, ld_codes_bytes, row_sum, clear, st);
+    return dispatch(static_cast<const float*>(x), rows, D, ldx, gamma_t, beta_t, eps, rms, s_t, z_t, bits, codes, ld_codes_bytes, row_sum, clear, params, st);
+  return dispatch(static_cast<const __nv_bfloat16*>(x), rows, D, ldx, gamma_t, beta_t, eps, rms, s_t, z_t, bits, codes, ld_codes_bytes, row_sum, clear, params, st);
 }
 
 }  // namespace repq
@@ -549,5 +580,5 @@ extern "C" repq_status repq_ln_quant(const void* x, int x_dtype, int64_t rows, i
                                      float s_t, int z_t, int bits, uint8_t* codes, int64_t ld_codes_bytes,
                                      int32_t* row_sum, void* stream) {
   return repq::launch_ln_quant(x, x_dtype, rows, D, ldx, gamma_t, beta_t, eps, norm_kind, s_t, z_t, bits, codes, ld_codes_bytes,
-                               row_sum, repq::ClearWords{}, static_cast<cudaStream_t>(stream));
+                               row_sum, repq::ClearWords{}, repq::Params::streamed, static_cast<cudaStream_t>(stream));
 }

@@ -88,8 +88,8 @@ __global__ void expand4_kernel(const uint8_t* __restrict__ src, int64_t rows, in
   }
 }
 
-// Packed weight codes -> one byte per code, 64 codes (32 or 48 bytes) per thread and step.  The packed bytes are requested
-// before the kernel ahead in the stream has finished (weights are parameters), the scratch is written after it.
+// Packed weight codes -> one byte per code, 64 codes (32 or 48 bytes) per thread and step.  Settled weights are requested
+// before the kernel ahead in the stream has finished; the scratch is written after it in any case.
 template <int kBits>
 __device__ __forceinline__ void expand_words(const uint32_t (&w)[2 * kBits], uint32_t (&o)[16]) {
   if constexpr (kBits == 4) {
@@ -115,11 +115,12 @@ __device__ __forceinline__ void expand_words(const uint32_t (&w)[2 * kBits], uin
 }
 template <int kBits>
 __global__ void __launch_bounds__(256) expand_weights_kernel(const uint8_t* __restrict__ src, int rows, int groups, int64_t ld_src,
-                                                             uint8_t* __restrict__ dst, int64_t ld_dst) {
+                                                             uint8_t* __restrict__ dst, int64_t ld_dst, bool settled) {
   constexpr int kIn = 8 * kBits;                           // packed bytes of 64 codes
   const int64_t total = int64_t(rows) * groups, stride = int64_t(gridDim.x) * blockDim.x;
   grid_dependency_trigger();
-  bool waited = false;
+  if (!settled) grid_dependency_wait();
+  bool waited = !settled;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < total; i += stride) {
     const int64_t r = i / groups;
     const int g = int(i - r * groups);
@@ -127,7 +128,7 @@ __global__ void __launch_bounds__(256) expand_weights_kernel(const uint8_t* __re
 #pragma unroll
     for (int q = 0; q < kIn / 16; ++q) {                   // (a row ends on a 16-byte boundary)
       uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (int64_t(g) * kIn + 16 * q < ld_src) v = __ldg(reinterpret_cast<const uint4*>(src + r * ld_src + int64_t(g) * kIn) + q);
+      if (int64_t(g) * kIn + 16 * q < ld_src) v = __ldcg(reinterpret_cast<const uint4*>(src + r * ld_src + int64_t(g) * kIn) + q);
       w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
     }
     expand_words<kBits>(w, o);
@@ -160,11 +161,11 @@ bool byte_weights(const repq_gemm_desc& d, repq_gemm_desc* as_bytes, ByteWeights
   return true;
 }
 
-repq_status launch_expand_weights(const repq_gemm_desc& d, uint8_t* dst, int64_t ld, cudaStream_t st) {
+repq_status launch_expand_weights(const repq_gemm_desc& d, uint8_t* dst, int64_t ld, Params params, cudaStream_t st) {
   const int groups = int((int64_t(d.K) + 63) / 64);
   const int64_t blocks = (int64_t(d.N) * groups + 255) / 256, most = int64_t(sm_count()) * 8;
   auto kern = packed4(d.bits_w) ? expand_weights_kernel<4> : expand_weights_kernel<6>;
-  REPQ_CUDA(launch_chained(kern, dim3(unsigned(blocks < most ? blocks : most)), dim3(256), 0, st, d.w_codes, d.N, groups, d.ldw_bytes, dst, ld));
+  REPQ_CUDA(launch_chained(kern, dim3(unsigned(blocks < most ? blocks : most)), dim3(256), 0, st, d.w_codes, d.N, groups, d.ldw_bytes, dst, ld, params == Params::settled));
   note_launch();
   return REPQ_OK;
 }
@@ -303,22 +304,22 @@ extern "C" repq_status repq_qgemm_workspace_bytes(const repq_gemm_desc* d, size_
   return REPQ_OK;
 }
 
-extern "C" repq_status repq_qgemm(const repq_gemm_desc* d, void* workspace, size_t workspace_bytes, void* stream) {
-  REPQ_REQUIRE(d, REPQ_INVALID_ARG, "qgemm: NULL descriptor");
+repq_status repq::run_qgemm(const repq_gemm_desc& given, void* workspace, size_t workspace_bytes, Params params, cudaStream_t st) {
+  const repq_gemm_desc* d = &given;
   REPQ_TRY(validate(*d));
   if (d->M == 0) return REPQ_OK;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (scores_supported(*d)) return scores_tc_supported(*d) ? launch_scores_tc(*d, st) : launch_scores(*d, st);
   repq_gemm_desc as_bytes;
   ByteWeights B;
   if (byte_weights(*d, &as_bytes, &B) && workspace && workspace_bytes >= B.total && aligned(workspace, 256)) {
     uint8_t* w = static_cast<uint8_t*>(workspace) + B.offset;
-    REPQ_TRY(launch_expand_weights(*d, w, B.ld, st));
+    REPQ_TRY(launch_expand_weights(*d, w, B.ld, params, st));
     as_bytes.w_codes = w;
     d = &as_bytes;
+    params = Params::streamed;                             // (the expansion is the kernel just ahead now)
   }
   const EpilogueParams ep = make_epilogue(*d);
-  if (qgemm_skinny_preferred(*d)) return qgemm_skinny(*d, ep, d != &as_bytes, st);
+  if (qgemm_skinny_preferred(*d)) return qgemm_skinny(*d, ep, params, st);
   if (qgemm_tc_supported(*d)) {
     const size_t need = qgemm_tc_workspace(*d);
     REPQ_REQUIRE(workspace_bytes >= need && (need == 0 || workspace), REPQ_WORKSPACE_TOO_SMALL,
@@ -326,4 +327,9 @@ extern "C" repq_status repq_qgemm(const repq_gemm_desc* d, void* workspace, size
     return qgemm_tc(*d, ep, workspace, workspace_bytes, st);
   }
   return qgemm_mma(*d, ep, st);
+}
+
+extern "C" repq_status repq_qgemm(const repq_gemm_desc* d, void* workspace, size_t workspace_bytes, void* stream) {
+  REPQ_REQUIRE(d, REPQ_INVALID_ARG, "qgemm: NULL descriptor");
+  return run_qgemm(*d, workspace, workspace_bytes, Params::streamed, static_cast<cudaStream_t>(stream));
 }

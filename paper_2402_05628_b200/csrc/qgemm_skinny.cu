@@ -8,8 +8,8 @@
 //    distributed shared memory, every CTA finishing an equal share of the tile's tokens (integer sums: the result does
 //    not depend on the split);
 //  - two CTAs per SM where the ring of operand stages allows it, at least 64 KB of weights in flight per CTA;
-//  - while the kernel before it in the stream still runs, every CTA asks for its first weights
-//    (activations and outputs are touched only behind the dependency).
+//  - inside a block, while the kernel before it in the stream still runs, every CTA asks for its first weights
+//    (activations and outputs, and weights that the kernel before may have written, are touched only behind the dependency).
 // The epilogue has one output channel per thread (the channel's terms live in registers), tokens along the accumulator
 // columns; for one token the 32 lanes of a warp are 32 neighbouring outputs, so loads and stores are coalesced without
 // staging.  The arithmetic is epilogue.cuh's, element by element.
@@ -50,7 +50,7 @@ struct SkinnyParams {
   int M, N, K;
   int mt;                      // tokens per tile (multiple of 16)
   int stages, kblocks, split;
-  int weights_ready;           // the weights do not come from the kernel ahead in the stream
+  int weights_settled;         // the weights may be read ahead of the dependency wait
   uint32_t stage_bytes, a_bytes;
   uint32_t tmem_cols;
   const int32_t* asum;
@@ -212,12 +212,12 @@ qgemm_skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
   tc_fence_after();
   const uint32_t tmem = s_tmem;
   volatile int* abort = &s_abort;
-  // Ahead of the dependency wait, while the kernel before this one finishes (weights are parameters, unless that kernel has just
-  // expanded them): all of the CTA's weights where the ring holds them (ViT-S block of one image 33.0 -> 32.0 us), else the first
+  // Ahead of the dependency wait, while the kernel before this one finishes (inside a block, unless that kernel has just expanded
+  // them): all of the CTA's weights where the ring holds them (ViT-S block of one image 33.0 -> 32.0 us), else the first
   // k-blocks into L2 (copies into the ring cost a 7B-shaped block of 48 tokens 1 us there).
-  const int early = P.weights_ready && kb1 - kb0 <= stages ? kb1 - kb0 : 0;
+  const int early = P.weights_settled && kb1 - kb0 <= stages ? kb1 - kb0 : 0;
   if (warp == kEpiWarps) {
-    if (early == 0 && P.weights_ready && blockIdx.y == 0 && lane < kPrefetch && kb0 + lane < kb1) tma_prefetch_2d(&map_w, (kb0 + lane) * kBK, n0);
+    if (early == 0 && P.weights_settled && blockIdx.y == 0 && lane < kPrefetch && kb0 + lane < kb1) tma_prefetch_2d(&map_w, (kb0 + lane) * kBK, n0);
     if (lane == 0) {
       for (int s = 0; s < early; ++s) {
         mbar_expect_tx(smem_u32(&s_full[s]), kWBytes + P.a_bytes);
@@ -427,12 +427,12 @@ bool qgemm_skinny_preferred(const repq_gemm_desc& d) {
   return plan.us * 1.1f < other + 4.5f || (d.M <= 64 && plan.us < other + 4.5f);
 }
 
-repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, bool weights_ready, cudaStream_t st) {
+repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, Params params, cudaStream_t st) {
   SkinnyParams P{};
   P.M = d.M; P.N = d.N; P.K = d.K;
   P.asum = d.a_row_sum; P.wsum = d.w_row_sum;
   P.ep = ep;
-  P.weights_ready = weights_ready;
+  P.weights_settled = params == Params::settled;
   P.status = device_status_word();
   REPQ_REQUIRE(P.status != nullptr, REPQ_CUDA_ERROR, "qgemm: device status word unavailable");
   const Plan plan = plan_of(d.M, d.N, d.K, sm_count());
