@@ -448,7 +448,8 @@ repq_status repq_device_status(int32_t* status, int reset);
  * drain and return instead of hanging; the paper has no counterpart.)  Launches, on `stream`, a one-thread
  * kernel whose barrier is never completed and whose wait uses the same routine with a limit of
  * limit_cycles SM clock cycles (1 .. 2e9): the kernel returns after that long, repq_device_status then
- * reports REPQ_TIMEOUT with code 77 until it is reset, and the context stays usable. */
+ * reports REPQ_TIMEOUT with code 77 until it is reset, and the context stays usable.  A bulk copy of the kernel that is in
+ * flight when the wait runs out is drained before it returns, as in the tensor-core kernels (code 78 if it did not end). */
 repq_status repq_bounded_wait_selftest(int64_t limit_cycles, void* stream);
 
 #ifdef __cplusplus

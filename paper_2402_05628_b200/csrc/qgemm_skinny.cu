@@ -215,12 +215,12 @@ qgemm_skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
   // Ahead of the dependency wait, while the kernel before this one finishes (inside a block, unless that kernel has just expanded
   // them): all of the CTA's weights where the ring holds them (ViT-S block of one image 33.0 -> 32.0 us), else the first
   // k-blocks into L2 (copies into the ring cost a 7B-shaped block of 48 tokens 1 us there).
-  const int early = P.weights_settled && kb1 - kb0 <= stages ? kb1 - kb0 : 0;
+  const int early = P.weights_settled && kb1 - kb0 <= stages && !*abort ? kb1 - kb0 : 0;
   if (warp == kEpiWarps) {
     if (early == 0 && P.weights_settled && blockIdx.y == 0 && lane < kPrefetch && kb0 + lane < kb1) tma_prefetch_2d(&map_w, (kb0 + lane) * kBK, n0);
     if (lane == 0) {
       for (int s = 0; s < early; ++s) {
-        mbar_expect_tx(smem_u32(&s_full[s]), kWBytes + P.a_bytes);
+        mbar_expect_only(smem_u32(&s_full[s]), kWBytes);   // (the activations of the stage bring the arrival)
         tma_load_2d(smem_u32(ring) + s * P.stage_bytes, &map_w, smem_u32(&s_full[s]), (kb0 + s) * kBK, n0);
       }
     }
@@ -245,10 +245,8 @@ qgemm_skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
         if (!mbar_wait(smem_u32(&s_empty[stage]), phase ^ 1, abort, 61, P.status)) break;
         const uint32_t bar = smem_u32(&s_full[stage]);
         const uint32_t base = smem_u32(ring) + stage * P.stage_bytes;
-        if (early == 0) {
-          mbar_expect_tx(bar, kWBytes + P.a_bytes);
-          tma_load_2d(base, &map_w, bar, kb * kBK, n0);
-        }
+        mbar_expect_tx(bar, early ? P.a_bytes : kWBytes + P.a_bytes);
+        if (early == 0) tma_load_2d(base, &map_w, bar, kb * kBK, n0);
         tma_load_2d(base + kWBytes, &map_a, bar, kb * kBK, m0);
         ++issued;
         if (++stage == uint32_t(stages)) { stage = 0; phase ^= 1; }
@@ -258,6 +256,8 @@ qgemm_skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
         if (stage == 0) { stage = uint32_t(stages) - 1; phase ^= 1; } else { --stage; }
         mbar_drain(smem_u32(&s_full[stage]), phase);
       }
+      // weights asked for early whose activations were given up on
+      for (int s = issued; s < early; ++s) mbar_drain_unjoined(smem_u32(&s_full[s]), 0);
     }
   } else if (warp == kEpiWarps + 1) {
     // ---------------------------------------------------------------- MMA issue: D = s32, A = B = unsigned bytes, K-major

@@ -1073,15 +1073,24 @@ repq_status launch_tc(const CUtensorMap& map_a, const CUtensorMap& map_b, const 
 
 // A wait that nothing ends: one thread sets up an mbarrier that never receives its arrival and waits on it through the
 // same bounded-wait routine as the tensor-core kernels, with the caller's limit.  The wait runs out, the status word
-// takes the code, the kernel returns.
+// takes the code, the kernel drains a copy that was asked for ahead and never joined (as the few-token GEMM's weights are), and
+// returns; a copy that does not end replaces the code by the next one.
+constexpr uint32_t kSelftestBytes = 1024;
+__device__ alignas(16) uint8_t g_selftest_src[kSelftestBytes];
 __global__ void wait_selftest_kernel(long long limit_cycles, int code) {
-  __shared__ alignas(8) uint64_t bar;
+  __shared__ alignas(8) uint64_t bar, copied;
+  __shared__ alignas(16) uint8_t buf[kSelftestBytes];
   __shared__ volatile int abort_flag;
   if (threadIdx.x == 0) {
     abort_flag = 0;
     mbar_init(smem_u32(&bar), 1);
+    mbar_init(smem_u32(&copied), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    mbar_expect_only(smem_u32(&copied), kSelftestBytes);
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(smem_u32(buf)), "l"(g_selftest_src), "r"(kSelftestBytes), "r"(smem_u32(&copied)) : "memory");
     tc::mbar_wait(smem_u32(&bar), 0, &abort_flag, code, &g_status_word, limit_cycles);
+    if (!mbar_drain_unjoined(smem_u32(&copied), 0)) atomicExch(&g_status_word, code + 1);
   }
 }
 

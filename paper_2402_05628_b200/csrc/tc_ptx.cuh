@@ -21,6 +21,10 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
+// (bytes to wait for without the arrival: the phase stays open until an arrival joins them)
+__device__ __forceinline__ void mbar_expect_only(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -75,9 +79,16 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 }
 
 // Wait without side effects, for draining copies or MMAs that are still in flight before the CTA exits.
-__device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity) {
   const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity) && clock64() - t0 < kWaitCycles) {}
+  bool done;
+  while (!(done = mbar_try_wait(bar, parity)) && clock64() - t0 < kWaitCycles) {}
+  return done;
+}
+// The same where copies were asked for (mbar_expect_only) and the arrival that joins them will not come any more.
+__device__ __forceinline__ bool mbar_drain_unjoined(uint32_t bar, uint32_t parity) {
+  mbar_arrive(bar);
+  return mbar_drain(bar, parity);
 }
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y) {

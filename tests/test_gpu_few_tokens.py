@@ -51,3 +51,14 @@ def test_few_tokens_same_bits_as_the_warp_mma_kernel(M, N, K, mode):
         got.append((out, rs))
     assert B.repq_device_status() == 0
     assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("limit", [1, 100_000])
+def test_copies_asked_for_early_are_drained_when_a_wait_runs_out(limit):
+    """A stage whose weights were asked for ahead and whose activations never are: the copy is waited for all the same before
+    the kernel returns (code 77, the wait that ran out; 78 would be a copy that did not end), also where it is still in flight."""
+    from paper_2402_05628_b200 import binding as B
+    B.repq_bounded_wait_selftest(limit)
+    assert B.repq_device_status(reset=True) == 77
+    parity.check_qgemm(16, 384, 384, 4 | parity.BYTE_CODES, 4 | parity.BYTE_CODES, out_kind="f32", want_acc=False, give_sums=True)
+    assert B.repq_device_status() == 0
