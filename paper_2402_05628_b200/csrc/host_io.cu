@@ -23,6 +23,8 @@ constexpr size_t kPieceBytes = size_t(4) << 20;
 constexpr int kPieceBatches = 4;
 
 struct Pipeline {                 // per device, created on first use, kept for the life of the process
+  std::mutex queueing;            // held while a call queues its work: a wait on an event means its last record, and calls of
+                                  // several threads record the same events
   bool ready = false;
   cudaStream_t in = nullptr, out = nullptr;
   cudaEvent_t start = nullptr;
@@ -79,6 +81,7 @@ extern "C" repq_status repq_block_forward_host(const repq_block_desc* d, const r
   const size_t x_bytes = elems * dtype_size(d->act_dtype), y_bytes = elems * dtype_size(d->out_dtype);
   Pipeline* P = nullptr;
   REPQ_TRY(pipeline(&P));
+  std::lock_guard<std::mutex> queueing(P->queueing);
   cudaStream_t main = static_cast<cudaStream_t>(stream);
 
   // the helper streams start after everything already queued on the caller's stream

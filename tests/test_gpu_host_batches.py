@@ -1,0 +1,47 @@
+"""Batches in host memory: calls of several threads at once, and sequences of any length against the block on the device."""
+import threading
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _block(batch, seed):
+    import torch
+    from paper_2402_05628_b200.engine import QuantBlock
+    from workloads import make_block_inputs
+    blk = QuantBlock(make_block_inputs("c1_vit_s", batch=2))
+    rows, D = batch * blk.cfg["L"], blk.cfg["D"]
+    rng = np.random.default_rng(seed)
+    xs = [torch.from_numpy(rng.standard_normal((rows, D), dtype=np.float32)).to(blk.act_dtype).pin_memory() for _ in range(3)]
+    expect = [blk.forward(x.to(blk.device)).cpu() for x in xs]
+    return blk, xs, expect
+
+
+def test_calls_of_two_threads_do_not_take_each_others_events():
+    """Each thread has a block, a stream and buffers of its own; only the helper streams and events are the library's."""
+    import torch
+    work = [_block(batch, seed) for batch, seed in ((24, 1), (40, 2))]
+    wrong = []
+
+    def loop(blk, xs, expect):
+        try:
+            stream = torch.cuda.Stream()
+            for i in range(25):
+                n = 1 + i % 7
+                ys = [torch.empty(x.shape, dtype=blk.out_dtype).pin_memory() for x in (xs * 3)[:n]]
+                with torch.cuda.stream(stream):
+                    blk.forward_host((xs * 3)[:n], ys)
+                stream.synchronize()
+                if not all(torch.equal(y, e) for y, e in zip(ys, (expect * 3)[:n])):
+                    wrong.append(i)
+        except Exception as e:                                  # noqa: BLE001  (reported by the main thread)
+            wrong.append(e)
+
+    threads = [threading.Thread(target=loop, args=w) for w in work]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
