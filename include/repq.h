@@ -411,7 +411,7 @@ repq_status repq_block_forward_static(const repq_block_desc* d, const repq_block
  * memory: batch i is read from x_host[i] and its result written to y_host[i] (each (batch*seq) x dim, dense,
  * act_dtype / out_dtype).  The library copies through the caller's device staging buffers and overlaps the
  * copies with the block's kernels: batch i + 1 is copied in and batch i - 1 copied out while batch i is
- * computed, and the batches of a short sequence also pass through in pieces of whole items (two helper streams per device, created on first use and kept).  The same x_host or y_host pointer
+ * computed, and batches of several megabytes also pass through in pieces of whole items where that is worth the further copies (two helper streams per device, created on first use and kept).  The same x_host or y_host pointer
  * may be given for several batches.  (Plumbing around Eqs. 1-3 of the block; the paper has no counterpart.)
  *
  *  - x_dev[2], y_dev[2] [device]: staging buffers of one batch each; workspace as for repq_block_forward

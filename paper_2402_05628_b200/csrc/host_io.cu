@@ -2,13 +2,10 @@
 // memory.  The copies and the block's kernels overlap through two device staging buffers per direction and two helper
 // streams.  (Plumbing around the block; the block itself is repq_block_forward.)
 //
-// What bounds it is the host link, one direction each for inputs and outputs; beside that, the first copy in and the last
-// copy out, which nothing overlaps.  The items of a batch are independent, so a batch passes through the pipeline in up to
-// kMaxPieces pieces of whole items: piece c is computed while piece c + 1 is copied in and piece c - 1 copied out, and what
-// nothing overlaps is a piece instead of a batch.  A piece is at least kPieceBytes of input (below, the launches of the
-// block and the small copies take longer than the link does).  Long sequences of batches stay whole: there the ends weigh
-// little and smaller blocks and copies run at lower rates.  64 DeiT-B items per batch: one batch 950 -> 650 us, two
-// 1350 -> 1120, four 2240 -> 2150 (sixteen in pieces would be 7.8 -> 8.4 ms).
+// What bounds it is the host link: 53 GB/s in one direction, 44 GB/s in each when both are busy.  With whole batches the outputs
+// run one batch behind the inputs, which costs a batch's time on the link and the block's own time at the end.  The items of a
+// batch are independent, so a batch passes through the pipeline in pieces of whole items: piece c is computed while piece
+// c + 1 is copied in and piece c - 1 copied out, and the outputs run one piece behind.  See `pieces_of` for when.
 #include <mutex>
 
 #include "kernels.h"
@@ -19,8 +16,26 @@ namespace {
 constexpr int kMaxDevices = 64;
 constexpr int kSlots = 2;
 constexpr int kMaxPieces = 8;
-constexpr size_t kPieceBytes = size_t(4) << 20;
-constexpr int kPieceBatches = 4;
+constexpr size_t kPieceBytes = size_t(2400) << 10;        // 2.4 MB: some 50 us of the link, what queueing a piece takes the host
+constexpr size_t kGapBytes = size_t(448) << 10;          // what the link would move between two copies of a stream (10 us)
+
+// Pieces per batch: as many as are at least kPieceBytes of input each, unless what they save (the link time of a batch: the
+// outputs no longer run a batch behind) is less than the gaps they add (one per piece and batch).
+// Measured, us (DeiT-B, 64 images of 19.4 MB, 7 pieces | ViT-L, 32 images of 37.8 MB, 8 pieces; whole -> pieces): one batch
+// 934 -> 602 | 1841 -> 1029, two 1336 -> 1078 | 2577 -> 1860, four 2235 -> 2048 | 4237 -> 3530, five 2700 -> 2511 | 5065 -> 4362,
+// eight 4051 -> 3957 (whole by the rule) | 7541 -> 6943, sixteen 7664 -> 7769 (whole) | 14157 -> 13644 (whole).  64 ViT-S images
+// (9.7 MB, 3 pieces): one 488 -> 340, five 1462 -> 1456, eight 2219 -> 2259 (whole), sixteen 4247 -> 4477 (whole).  16 DeiT-B
+// images (4.8 MB) in two pieces: one batch 278 -> 240, but four 605 -> 633.
+// Three to five pieces of the two larger batches are slower than the counts on either side of them (four DeiT-B batches: 2372,
+// 2252 and 2218 us against 2219 with two and 2083 with six); the cause was not found.  Pieces for the first and the last batch
+// only gain nothing beyond two batches: the outputs then fall a batch behind in between.
+int pieces_of(size_t x_bytes, int batch, int n_batches) {
+  const size_t fit = x_bytes / kPieceBytes;
+  int pieces = int(fit < size_t(kMaxPieces) ? fit : size_t(kMaxPieces));
+  if (pieces > batch) pieces = batch;
+  if (pieces < 2) return 1;
+  return size_t(n_batches) * size_t(pieces) * kGapBytes <= x_bytes ? pieces : 1;
+}
 
 struct Pipeline {                 // per device, created on first use, kept for the life of the process
   std::mutex queueing;            // held while a call queues its work: a wait on an event means its last record, and calls of
@@ -88,9 +103,7 @@ extern "C" repq_status repq_block_forward_host(const repq_block_desc* d, const r
   REPQ_CUDA(cudaEventRecord(P->start, main));
   REPQ_CUDA(cudaStreamWaitEvent(P->in, P->start, 0));
   REPQ_CUDA(cudaStreamWaitEvent(P->out, P->start, 0));
-  int64_t fit = int64_t(x_bytes / kPieceBytes);
-  fit = fit < 1 ? 1 : fit > kMaxPieces ? kMaxPieces : fit;
-  const int pieces = n_batches > kPieceBatches ? 1 : int(fit < d->batch ? fit : d->batch);
+  const int pieces = pieces_of(x_bytes, d->batch, n_batches);
   const size_t x_item = x_bytes / size_t(d->batch), y_item = y_bytes / size_t(d->batch);
   repq_block_desc piece = *d;
   for (int i = 0; i < n_batches; ++i) {

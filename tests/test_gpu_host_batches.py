@@ -45,3 +45,27 @@ def test_calls_of_two_threads_do_not_take_each_others_events():
     for t in threads:
         t.join()
     assert not wrong
+
+
+@pytest.mark.parametrize("batch", [1, 5, 24, 65])               # (whole batches, two to eight pieces, ragged ones)
+def test_sequences_of_any_length(batch):
+    import torch
+    from paper_2402_05628_b200 import binding as B
+    blk, xs, expect = _block(batch, batch)
+    blk.forward(xs[0].to(blk.device))
+    torch.cuda.synchronize()
+    before = B.repq_launch_count()
+    blk.forward(xs[0].to(blk.device))
+    per_block = B.repq_launch_count() - before
+    bytes_in, per_batch = xs[0].numel() * xs[0].element_size(), {}
+    for n in (1, 2, 4, 5, 9, 40):
+        ys = [torch.zeros(x.shape, dtype=blk.out_dtype).pin_memory() for x in (xs * 14)[:n]]
+        before = B.repq_launch_count()
+        blk.forward_host((xs * 14)[:n], ys)
+        torch.cuda.synchronize()
+        per_batch[n] = (B.repq_launch_count() - before) / n / per_block
+        assert all(torch.equal(y, e) for y, e in zip(ys, (expect * 14)[:n]))
+    # pieces by the bytes they save against the gaps they add, at four batches as at five
+    most = min(8, bytes_in // 2457600, batch)
+    for n, pieces in per_batch.items():
+        assert pieces == (most if most > 1 and n * most * (448 << 10) <= bytes_in else 1)
