@@ -8,6 +8,7 @@ between numpy, torch and the C ABI.
 from __future__ import annotations
 
 import dataclasses
+import operator
 from typing import Dict, List, Optional
 
 import numpy as np
@@ -16,18 +17,18 @@ import torch
 from . import binding as B
 
 
-class _Tracked:
-    """Counts assignments to public attributes of any instance, so that what was derived from them can be kept."""
-    changes = 0
-
-    def __setattr__(self, name, value):
-        object.__setattr__(self, name, value)
-        if not name.startswith("_"):
-            _Tracked.changes += 1
+# what the parameters of a pass are made from, read anew for every pass
+_TENSORS = ["ln1_g", "ln1_b", "ln2_g", "ln2_b"] + [
+    layer + "." + t for layer in ("qkv", "proj", "fc1", "fc2") for t in ("codes", "s_w", "z_w", "w_row_sum", "bias")]
+_tensors_of = operator.attrgetter(*_TENSORS)
+_codes_of = operator.itemgetter(*(i for i, t in enumerate(_TENSORS) if t.endswith(".codes")))
+_values_of = operator.attrgetter("ln1_s", "ln1_z", "ln2_s", "ln2_z", "softmax_s", "bits_w", "llama", "act_dtype", "out_dtype",
+                                 "staged_attention")
+_address, _strides = torch.Tensor.data_ptr, torch.Tensor.stride
 
 
 @dataclasses.dataclass
-class PreparedLinear(_Tracked):
+class PreparedLinear:
     codes: torch.Tensor
     s_w: torch.Tensor
     z_w: torch.Tensor
@@ -48,8 +49,9 @@ def _pack_linear(W: np.ndarray, bias: np.ndarray, bits_w: int, dev) -> PreparedL
     return PreparedLinear(t(codes), t(s_w), t(z_w), t(wsum), t(np.asarray(bias, dtype=np.float32)))
 
 
-class QuantBlock(_Tracked):
-    """Device-resident parameters of one block plus its workspace; `forward` runs the hot path."""
+class QuantBlock:
+    """Device-resident parameters of one block plus its workspace; `forward` runs the hot path.  Passes of one block share the
+    workspace: queue them on one stream (or one after the other)."""
 
     def __init__(self, w, device="cuda:0", out_dtype: Optional[torch.dtype] = None, staged_attention: bool = False,
                  weight_storage: str = "bytes"):
@@ -105,7 +107,6 @@ class QuantBlock(_Tracked):
         self.softmax_s = float(w.softmax_scale)
         self._ws: Optional[torch.Tensor] = None
         self._staging = None
-        self._batch = None
         self._call = (None, None, None, None)
 
     def desc(self, batch: int) -> B.BlockDesc:
@@ -138,22 +139,26 @@ class QuantBlock(_Tracked):
         return p
 
     def workspace(self, batch: int) -> torch.Tensor:
-        if self._ws is None or self._batch != batch:
-            n = B.repq_block_workspace_bytes(self.desc(batch))
-            self._ws = torch.empty(n + 256, dtype=torch.uint8, device=self.device)
-            off = (-self._ws.data_ptr()) % 256
-            self._ws = self._ws[off:off + n]
-            self._batch = batch
-        return self._ws
+        n = B.repq_block_workspace_bytes(self.desc(batch))
+        ws = self._ws
+        if ws is None or ws.numel() != n:
+            ws = torch.empty(n + 256, dtype=torch.uint8, device=self.device)
+            off = (-ws.data_ptr()) % 256
+            ws = ws[off:off + n]
+            self._ws = ws
+        return ws
 
     def _prepared(self, batch: int):
-        """Descriptor, parameters and workspace of a pass over `batch` items, kept from the pass before while nothing they
-        were made from has changed (building them takes longer than a small block runs)."""
-        # (attributes of blocks and layers by their assignments; the quantizer dict and the config may be edited in place)
-        key = (batch, _Tracked.changes, tuple(self.act_q.values()), tuple(self.cfg.values()))
-        if self._call[0] != key:
-            self._call = (key, self.desc(batch), self.params(), self.workspace(batch))
-        return self._call[1:]
+        """Descriptor, parameters and workspace of a pass over `batch` items, kept from the pass before while everything they
+        were made from reads the same, addresses included (4 us of host time; building them takes 8)."""
+        tensors = _tensors_of(self)
+        key = (batch, list(map(_address, tensors)), list(map(_strides, _codes_of(tensors))), _values_of(self),
+               None if self.rope is None else self.rope.data_ptr(), list(self.act_q.values()), list(self.cfg.values()))
+        call = self._call
+        if call[0] != key:
+            call = (key, self.desc(batch), self.params(), self.workspace(batch))
+            self._call = call
+        return call[1:]                                  # (of this call's own: another thread may have replaced the kept one)
 
     def forward(self, x: torch.Tensor, y: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
         """x: [batch * seq, dim] on the device, dtype = activation dtype of the config."""
