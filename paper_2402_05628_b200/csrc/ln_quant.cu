@@ -13,14 +13,15 @@
 // slots 59 % busy).  Measured against three barriers per iteration: 32768 bf16 rows of 4096 78 -> 73 us, 65536 of 1536 53 -> 45,
 // 32768 float rows of 2048 83 -> 48, 16384 of 4096 76 -> 49.
 // The per-channel factors gamma~/s~ and beta~/s~ are staged once per CTA in shared memory (halves of the 8-element
-// chunks apart, so that a warp's 16-byte reads are free of bank conflicts), or, for rows of 3080 to 4096 bf16 elements,
-// kept in the registers of the thread that owns their columns.
+// chunks apart, so that a warp's 16-byte reads are free of bank conflicts).
 //
 // The float work runs on packed pairs (two elements per add / mul / fma issue slot).  Rounding is done by the
 // float adder: t + 1.5 * 2^23 leaves rint(t) (half to even, on t itself, as Eq. 4 has it) in the low mantissa
 // bits while |t| < 2^22; inputs that cannot guarantee that bound are clamped and converted with cvt.rni
 // instead.  z is added as an integer and the clip of Eq. 4 is the saturation of the packing instruction.
 #include <cuda_bf16.h>
+
+#include <type_traits>
 
 #include "f32x2.cuh"
 #include "kernels.h"
@@ -29,7 +30,6 @@ namespace repq {
 namespace {
 
 constexpr int kChunk = 8;   // elements per 128-bit bf16 load
-constexpr int kMaxVPT = 4;  // chunks per thread: 1..4, chosen per row length
 
 // Rows a thread group works on at a time (the loads of the next ones are always in flight as well): two, except where the
 // chunks per thread leave the registers for one (measured: bf16 rows of 2048 / 4096 elements, 64 x 4 / 128 x 4 threads x
@@ -37,14 +37,6 @@ constexpr int kMaxVPT = 4;  // chunks per thread: 1..4, chosen per row length
 // 28).
 __host__ __device__ constexpr int rows_in_flight(int vpt, int tpr, bool full, int elem_bytes) {
   return vpt < (elem_bytes == 2 || tpr >= 512 ? 4 : 3) || (vpt == 4 && tpr >= 256 && full && elem_bytes == 2) ? 2 : 1;
-}
-
-// Where a thread's slice of gamma~/s~ and beta~/s~ stays in registers for the whole kernel instead of being read from
-// shared memory for every pair of rows: two chunks per thread at most (32 registers) in groups of at least 128 threads,
-// bf16 input (two resident blocks of 256 threads at 108 registers; measured at D = 4096: 670 -> 595 us for 262144 rows,
-// three blocks with spills or one row at a time were slower).
-__host__ __device__ constexpr bool factors_in_registers(int vpt, int tpr, int elem_bytes) {
-  return vpt <= 2 && tpr >= 128 && elem_bytes == 2;
 }
 
 // A chunk of 8 elements as it is loaded (kept in this form while the rows before it are processed), and
@@ -131,7 +123,7 @@ __device__ __forceinline__ void group_sum(int (&v)[kRows]) {
 
 template <typename T, int TPR, int kVPT, bool kPack4, bool kFull>
 __global__ void __launch_bounds__((TPR > 256 ? TPR : 256),
-                                  (kVPT <= 2 && TPR == 256 ? (factors_in_registers(kVPT, TPR, sizeof(T)) ? 2 : 3) : TPR == 256 ? 2 : sizeof(T) == 4 && TPR == 32 && (kVPT == 3 || kVPT == 4) ? 2 : 0))
+                                  (TPR == 256 ? 2 : sizeof(T) == 4 && TPR == 32 && (kVPT == 3 || kVPT == 4) ? 2 : 0))
 ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
                 const float* __restrict__ gamma_t, const float* __restrict__ beta_t, float eps, int rms,
                 float inv_s, int z, int qmax, uint8_t* __restrict__ codes, int64_t ldc,
@@ -140,8 +132,7 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
   constexpr int kBlock = TPR > 256 ? TPR : 256;
   constexpr int kGroups = kBlock / TPR;
   constexpr int kRowsPerBlock = kGroups * kRows;
-  constexpr bool kRegFactors = factors_in_registers(kVPT, TPR, sizeof(T));
-  extern __shared__ __align__(16) float s_gb[];          // g[D] then b[D]: gamma~/s~ and beta~/s~ (unless in registers)
+  extern __shared__ __align__(16) float s_gb[];          // g[D] then b[D]: gamma~/s~ and beta~/s~
   // Rows of several warps: one barrier per iteration.  A warp reduces its own slice twice (sum, then squares centred on the
   // slice's own mean) and leaves both in `red`; behind the barrier every warp merges the slices' means and squares
   // (M2 = sum M2_w + n_w (mean_w - mean)^2).  Code sums wait in `red_c` for the next iteration's barrier.  Both alternate by
@@ -190,57 +181,33 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
   // is clamped and converted, so that adding z cannot wrap (a whole-kernel decision, taken here once).
   const float root_d = sqrtf(float(D));
   bool wide = false;
-  f32x2 g_reg[kRegFactors ? kVPT : 1][kChunk / 2], b_reg[kRegFactors ? kVPT : 1][kChunk / 2];
-  if constexpr (kRegFactors) {
-    if (!settled) fetch(first_rows);
-    // every thread works on the same columns of every row: its factors are loaded once
+  // layout: the first halves (4 floats) of all chunks, then the second halves, so that the 16-byte reads of
+  // neighbouring lanes are neighbours in shared memory (chunk by chunk they would sit 32 bytes apart: two-way
+  // bank conflicts)
+  const int half_stride = D / 2;
+  // Several factors of a thread in flight at a time, and the first rows asked for behind the first of them, so that rows and
+  // factors arrive together.  (What reading behind the wait costs a block pass of 64 x 197 tokens x 768: 1.2 us of 209, with
+  // the rows first and the factors one by one 2.1; one image through a ViT-S block 0.5 of 32.)
+  constexpr int kInFlight = 8;
+  for (int base = 0; base < D; base += kInFlight * kBlock) {
+    float gi[kInFlight], bi[kInFlight];
 #pragma unroll
-    for (int i = 0; i < kVPT; ++i) {
-      const int c = threadIdx.x % TPR + i * TPR;
-      const bool on = kFull || c < D / kChunk;
-      float gi[kChunk], bi[kChunk];
-#pragma unroll
-      for (int e = 0; e < kChunk; ++e) {
-        gi[e] = on ? __ldcg(gamma_t + c * kChunk + e) * inv_s : 0.f;
-        bi[e] = on ? __ldcg(beta_t + c * kChunk + e) * inv_s : 0.f;
-      }
-#pragma unroll
-      for (int e = 0; e < kChunk; ++e) wide = wide || !(fabsf(gi[e]) * root_d + fabsf(bi[e]) < 4.0e6f);
-#pragma unroll
-      for (int e = 0; e < kChunk / 2; ++e) {
-        g_reg[i][e] = pack2(gi[2 * e], gi[2 * e + 1]);
-        b_reg[i][e] = pack2(bi[2 * e], bi[2 * e + 1]);
-      }
+    for (int k = 0; k < kInFlight; ++k) {
+      const int i = base + k * kBlock + threadIdx.x;
+      gi[k] = i < D ? __ldcg(gamma_t + i) : 0.f;
+      bi[k] = i < D ? __ldcg(beta_t + i) : 0.f;
     }
-  } else {
-    // layout: the first halves (4 floats) of all chunks, then the second halves, so that the 16-byte reads of
-    // neighbouring lanes are neighbours in shared memory (chunk by chunk they would sit 32 bytes apart: two-way
-    // bank conflicts)
-    const int half_stride = D / 2;
-    // Several factors of a thread in flight at a time, and the first rows asked for behind the first of them, so that rows and
-    // factors arrive together.  (What reading behind the wait costs a block pass of 64 x 197 tokens x 768: 1.2 us of 209, with
-    // the rows first and the factors one by one 2.1; one image through a ViT-S block 0.5 of 32.)
-    constexpr int kInFlight = 8;
-    for (int base = 0; base < D; base += kInFlight * kBlock) {
-      float gi[kInFlight], bi[kInFlight];
+    if (!settled && base == 0) fetch(first_rows);
 #pragma unroll
-      for (int k = 0; k < kInFlight; ++k) {
-        const int i = base + k * kBlock + threadIdx.x;
-        gi[k] = i < D ? __ldcg(gamma_t + i) : 0.f;
-        bi[k] = i < D ? __ldcg(beta_t + i) : 0.f;
-      }
-      if (!settled && base == 0) fetch(first_rows);
-#pragma unroll
-      for (int k = 0; k < kInFlight; ++k) {
-        const int i = base + k * kBlock + threadIdx.x;
-        if (i >= D) break;
-        gi[k] *= inv_s;
-        bi[k] *= inv_s;
-        const int at = ((i >> 2) & 1) * half_stride + (i >> 3) * 4 + (i & 3);
-        s_g[at] = gi[k];
-        s_b[at] = bi[k];
-        wide = wide || !(fabsf(gi[k]) * root_d + fabsf(bi[k]) < 4.0e6f);
-      }
+    for (int k = 0; k < kInFlight; ++k) {
+      const int i = base + k * kBlock + threadIdx.x;
+      if (i >= D) break;
+      gi[k] *= inv_s;
+      bi[k] *= inv_s;
+      const int at = ((i >> 2) & 1) * half_stride + (i >> 3) * 4 + (i & 3);
+      s_g[at] = gi[k];
+      s_b[at] = bi[k];
+      wide = wide || !(fabsf(gi[k]) * root_d + fabsf(bi[k]) < 4.0e6f);
     }
   }
   const bool guard = __syncthreads_or(wide) != 0;
@@ -402,17 +369,12 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
       const int c = tig + i * TPR;
       if (kFull || c < nchunks) {
         f32x2 g[kChunk / 2], b[kChunk / 2];
-        if constexpr (kRegFactors) {
-#pragma unroll
-          for (int e = 0; e < kChunk / 2; ++e) { g[e] = g_reg[i][e]; b[e] = b_reg[i][e]; }
-        } else {
-          const float4 g0 = *reinterpret_cast<const float4*>(s_g + c * 4);
-          const float4 g1 = *reinterpret_cast<const float4*>(s_g + D / 2 + c * 4);
-          const float4 b0 = *reinterpret_cast<const float4*>(s_b + c * 4);
-          const float4 b1 = *reinterpret_cast<const float4*>(s_b + D / 2 + c * 4);
-          g[0] = pack2(g0.x, g0.y); g[1] = pack2(g0.z, g0.w); g[2] = pack2(g1.x, g1.y); g[3] = pack2(g1.z, g1.w);
-          b[0] = pack2(b0.x, b0.y); b[1] = pack2(b0.z, b0.w); b[2] = pack2(b1.x, b1.y); b[3] = pack2(b1.z, b1.w);
-        }
+        const float4 g0 = *reinterpret_cast<const float4*>(s_g + c * 4);
+        const float4 g1 = *reinterpret_cast<const float4*>(s_g + D / 2 + c * 4);
+        const float4 b0 = *reinterpret_cast<const float4*>(s_b + c * 4);
+        const float4 b1 = *reinterpret_cast<const float4*>(s_b + D / 2 + c * 4);
+        g[0] = pack2(g0.x, g0.y); g[1] = pack2(g0.z, g0.w); g[2] = pack2(g1.x, g1.y); g[3] = pack2(g1.z, g1.w);
+        b[0] = pack2(b0.x, b0.y); b[1] = pack2(b0.z, b0.w); b[2] = pack2(b1.x, b1.y); b[3] = pack2(b1.z, b1.w);
 #pragma unroll
         for (int r = 0; r < kRows; ++r) {
           // Eq. 4: clip(round(t) + z, 0, qmax): round half to even by the float -> int conversion, then the
@@ -483,66 +445,71 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
   }
 }
 
-template <typename T, int TPR, int kVPT>
-repq_status launch(const T* x, int64_t rows, int D, int64_t ldx, const float* g, const float* b, float eps,
-                   int rms, float s_t, int z, int bits, uint8_t* codes, int64_t ldc, int32_t* row_sum,
-                   ClearWords clear, Params params, cudaStream_t st) {
+template <typename T>
+struct Call {
+  const T* x;
+  int64_t rows;
+  int D;
+  int64_t ldx;
+  const float *gamma_t, *beta_t;
+  float eps;
+  int rms;
+  float s_t;
+  int z, bits;
+  uint8_t* codes;
+  int64_t ldc;
+  int32_t* row_sum;
+  ClearWords clear;
+  bool settled;
+};
+
+template <typename T, int TPR, int kVPT, bool kPack4, bool kFull>
+repq_status launch(const Call<T>& c, cudaStream_t st) {
   constexpr int kBlock = TPR > 256 ? TPR : 256;
-  const bool full = D == TPR * kVPT * kChunk;   // the row fills the group exactly: no chunk is predicated
-  const int rows_per_block = kBlock / TPR * rows_in_flight(kVPT, TPR, full, sizeof(T));
-  const int64_t need = (rows + rows_per_block - 1) / rows_per_block;
-  const float inv_s = 1.f / s_t;
-  const int qmax = code_max(bits);
-  const size_t smem = factors_in_registers(kVPT, TPR, sizeof(T)) ? 0 : size_t(D) * 2 * sizeof(float);
-  const bool pack = packed4(bits);
-  auto kern = pack ? (full ? ln_quant_kernel<T, TPR, kVPT, true, true> : ln_quant_kernel<T, TPR, kVPT, true, false>)
-                   : (full ? ln_quant_kernel<T, TPR, kVPT, false, true> : ln_quant_kernel<T, TPR, kVPT, false, false>);
-  if (smem > 40 * 1024) REPQ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-  static Residency memo[2][2];
+  constexpr int kRowsPerBlock = kBlock / TPR * rows_in_flight(kVPT, TPR, kFull, sizeof(T));
+  constexpr int kMostSmem = TPR * kVPT * kChunk * 2 * int(sizeof(float));
+  auto kern = ln_quant_kernel<T, TPR, kVPT, kPack4, kFull>;
+  const int64_t need = (c.rows + kRowsPerBlock - 1) / kRowsPerBlock;
+  const size_t smem = size_t(c.D) * 2 * sizeof(float);
+  if constexpr (kMostSmem > 40 * 1024) REPQ_TRY((allow_smem<ln_quant_kernel<T, TPR, kVPT, kPack4, kFull>>(kMostSmem)));
+  static Residency memo;
   // persistent grid: exactly the blocks that are resident at once, so that every block keeps its load pipeline
   // running over all of its rows
   int resident = 0;
-  REPQ_TRY(resident_blocks(memo[pack][full], kern, kBlock, smem, &resident));
+  REPQ_TRY(resident_blocks(memo, kern, kBlock, smem, &resident));
   const int64_t cap = int64_t(sm_count()) * resident;
   const int grid = int(need < cap ? need : cap);
-  REPQ_CUDA(launch_chained(kern, dim3(grid), dim3(kBlock), smem, st, x, rows, D, ldx, g, b, eps, rms, inv_s, z, qmax, codes, ldc, row_sum, clear.at, clear.n, params == Params::settled));
+  REPQ_CUDA(launch_chained(kern, dim3(grid), dim3(kBlock), smem, st, c.x, c.rows, c.D, c.ldx, c.gamma_t, c.beta_t, c.eps, c.rms, 1.f / c.s_t,
+                           c.z, code_max(c.bits), c.codes, c.ldc, c.row_sum, c.clear.at, c.clear.n, c.settled));
   note_launch();
   return REPQ_OK;
 }
 
-template <typename T, int TPR>
-repq_status launch_vpt(int vpt, const T* x, int64_t rows, int D, int64_t ldx, const float* g, const float* b, float eps,
-                       int rms, float s_t, int z, int bits, uint8_t* codes, int64_t ldc, int32_t* row_sum,
-                       ClearWords clear, Params params, cudaStream_t st) {
-  switch (vpt) {
-    case 1: return launch<T, TPR, 1>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, params, st);
-    case 2: return launch<T, TPR, 2>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, params, st);
-    case 3: return launch<T, TPR, 3>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, params, st);
-    case 4: return launch<T, TPR, 4>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, params, st);
-    case 5: return launch<T, TPR, (TPR >= 32 && TPR <= 128 ? 5 : 4)>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, params, st);
-    default: return launch<T, TPR, (TPR >= 32 && TPR <= 128 ? 6 : 4)>(x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, params, st);
+// Chunks per thread kVPT .. kMost, the row lengths that narrower groups leave to groups of TPR threads.
+template <typename T, int TPR, int kVPT, int kMost>
+repq_status launch_group(const Call<T>& c, cudaStream_t st) {
+  if constexpr (kVPT < kMost) {
+    if (c.D > TPR * kVPT * kChunk) return launch_group<T, TPR, kVPT + 1, kMost>(c, st);
   }
+  const bool full = c.D == TPR * kVPT * kChunk;   // the row fills the group exactly: no chunk is predicated
+  if (packed4(c.bits)) return full ? launch<T, TPR, kVPT, true, true>(c, st) : launch<T, TPR, kVPT, true, false>(c, st);
+  return full ? launch<T, TPR, kVPT, false, true>(c, st) : launch<T, TPR, kVPT, false, false>(c, st);
 }
 
 template <typename T>
-repq_status dispatch(const T* x, int64_t rows, int D, int64_t ldx, const float* g, const float* b, float eps,
-                     int rms, float s_t, int z, int bits, uint8_t* codes, int64_t ldc, int32_t* row_sum,
-                     ClearWords clear, Params params, cudaStream_t st) {
-  const int nchunks = D / kChunk;
+repq_status dispatch(const Call<T>& c, cudaStream_t st) {
+  const int nchunks = c.D / kChunk;
   // The fewest warps whose threads hold the row in at most six chunks: a row of one warp has no barrier, and what a row costs
   // beside its elements (shuffles, merges, barrier) is paid per thread (measured, 1536 elements: 45 us with one warp, 59 with
   // two; 3072: 49 and 61).  Eight chunks leave too few warps on the SM (2048 float elements: 56 against 48).
-#define REPQ_LN_CASE(TPR, MOST) \
-  if (nchunks <= TPR * MOST) return launch_vpt<T, TPR>((nchunks + TPR - 1) / TPR, x, rows, D, ldx, g, b, eps, rms, s_t, z, bits, codes, ldc, row_sum, clear, params, st);
-  REPQ_LN_CASE(8, 4)
-  REPQ_LN_CASE(16, 4)
-  REPQ_LN_CASE(32, 6)
-  REPQ_LN_CASE(64, 6)
-  REPQ_LN_CASE(128, 6)
-  REPQ_LN_CASE(256, 4)
-  REPQ_LN_CASE(512, 4)
-#undef REPQ_LN_CASE
-  return fail(REPQ_UNSUPPORTED, "ln_quant: D = %d exceeds 16384", D);
+  if (nchunks <= 8 * 4) return launch_group<T, 8, 1, 4>(c, st);
+  if (nchunks <= 16 * 4) return launch_group<T, 16, 3, 4>(c, st);
+  if (nchunks <= 32 * 6) return launch_group<T, 32, 3, 6>(c, st);
+  if (nchunks <= 64 * 6) return launch_group<T, 64, 4, 6>(c, st);
+  if (nchunks <= 128 * 6) return launch_group<T, 128, 4, 6>(c, st);
+  if (nchunks <= 256 * 4) return launch_group<T, 256, 4, 4>(c, st);
+  if (nchunks <= 512 * 4) return launch_group<T, 512, 3, 4>(c, st);
+  return fail(REPQ_UNSUPPORTED, "ln_quant: D = %d exceeds 16384", c.D);
 }
 
 }  // namespace
@@ -567,10 +534,12 @@ repq_status launch_ln_quant(const void* x, int x_dtype, int64_t rows, int D, int
   REPQ_REQUIRE(ld_codes_bytes >= code_row_bytes(D, bits), REPQ_INVALID_ARG, "ln_quant: ld_codes_bytes shorter than a row");
   REPQ_REQUIRE(aligned(codes, unit) && ld_codes_bytes % unit == 0, REPQ_ALIGNMENT,
                "ln_quant: codes rows must be %d-byte aligned", int(unit));
-  const int rms = norm_kind == REPQ_NORM_RMS;
-  if (x_dtype == REPQ_F32)
-    return dispatch(static_cast<const float*>(x), rows, D, ldx, gamma_t, beta_t, eps, rms, s_t, z_t, bits, codes, ld_codes_bytes, row_sum, clear, params, st);
-  return dispatch(static_cast<const __nv_bfloat16*>(x), rows, D, ldx, gamma_t, beta_t, eps, rms, s_t, z_t, bits, codes, ld_codes_bytes, row_sum, clear, params, st);
+  auto run = [&](auto* typed) {
+    return dispatch(Call<std::remove_const_t<std::remove_pointer_t<decltype(typed)>>>{
+        typed, rows, D, ldx, gamma_t, beta_t, eps, norm_kind == REPQ_NORM_RMS, s_t, z_t, bits, codes, ld_codes_bytes, row_sum, clear,
+        params == Params::settled}, st);
+  };
+  return x_dtype == REPQ_F32 ? run(static_cast<const float*>(x)) : run(static_cast<const __nv_bfloat16*>(x));
 }
 
 }  // namespace repq

@@ -401,16 +401,14 @@ repq_status launch(const T* scores, int64_t rows, int L, int64_t ld, bool vec_ok
   return REPQ_OK;
 }
 
-template <typename T, int TPR>
-repq_status launch_vpt(int vpt, const T* scores, int64_t rows, int L, int64_t ld, bool vec_ok, float c, int period,
-                       int offset, float log2_s, int bits, uint8_t* codes, int64_t ldc, cudaStream_t st) {
-  switch (vpt) {
-    case 1: return launch<T, TPR, 1>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
-    case 2: return launch<T, TPR, 2>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
-    case 3: return launch<T, TPR, 3>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
-    case 4: return launch<T, TPR, 4>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
-    default: return launch<T, TPR, 5>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
+// Chunks per thread kVPT .. kMost, the row lengths that narrower groups leave to groups of TPR threads.
+template <typename T, int TPR, int kVPT, int kMost>
+repq_status launch_group(const T* scores, int64_t rows, int L, int64_t ld, bool vec_ok, float c, int period,
+                         int offset, float log2_s, int bits, uint8_t* codes, int64_t ldc, cudaStream_t st) {
+  if constexpr (kVPT < kMost) {
+    if (L > TPR * kVPT * kChunk) return launch_group<T, TPR, kVPT + 1, kMost>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
   }
+  return launch<T, TPR, kVPT>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
 }
 
 template <typename T>
@@ -426,16 +424,16 @@ repq_status dispatch(const T* scores, int64_t rows, int L, int64_t ld, bool vec_
     REPQ_SM_CASE(32)
 #undef REPQ_SM_CASE
   }
-#define REPQ_SM_CASE(TPR) \
-  if (nchunks <= TPR * kMaxVPT) return launch_vpt<T, TPR>((nchunks + TPR - 1) / TPR, scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
-  REPQ_SM_CASE(8)
-  REPQ_SM_CASE(16)
-  REPQ_SM_CASE(32)
-  REPQ_SM_CASE(64)
-  REPQ_SM_CASE(128)
-  REPQ_SM_CASE(256)
-  REPQ_SM_CASE(512)
+#define REPQ_SM_CASE(TPR, FEWEST) \
+  if (nchunks <= TPR * kMaxVPT) return launch_group<T, TPR, FEWEST, kMaxVPT>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
+  REPQ_SM_CASE(8, 1)
+  REPQ_SM_CASE(16, 3)
+  REPQ_SM_CASE(32, 3)
+  REPQ_SM_CASE(64, 3)
+  REPQ_SM_CASE(128, 3)
+  REPQ_SM_CASE(256, 3)
 #undef REPQ_SM_CASE
+  if (nchunks <= 512 * 4) return launch_group<T, 512, 3, 4>(scores, rows, L, ld, vec_ok, c, period, offset, log2_s, bits, codes, ldc, st);
   return fail(REPQ_UNSUPPORTED, "softmax_log2: L = %d exceeds 16384", L);
 }
 
