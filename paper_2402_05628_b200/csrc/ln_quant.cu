@@ -32,12 +32,20 @@ namespace {
 constexpr int kChunk = 8;   // elements per 128-bit bf16 load
 
 // Rows a thread group works on at a time (the loads of the next ones are always in flight as well): two, except where the
-// chunks per thread leave the registers for one (measured: bf16 rows of 2048 / 4096 elements, 64 x 4 / 128 x 4 threads x
-// chunks, 69 / 73 us with one row, 97 / 101 with two; whole bf16 rows of 256 x 4 74 and 69; float rows of 768, 32 x 3, 21 and
-// 28).
-__host__ __device__ constexpr int rows_in_flight(int vpt, int tpr, bool full, int elem_bytes) {
-  return vpt < (elem_bytes == 2 || tpr >= 512 ? 4 : 3) || (vpt == 4 && tpr >= 256 && full && elem_bytes == 2) ? 2 : 1;
+// chunks per thread leave the registers for one.  bf16: from four chunks on in groups that share an SM with others (2048 / 4096
+// elements, 64 x 4 / 128 x 4 threads x chunks, 69 / 73 us with one row, 97 / 101 with two); groups of 256 and 512 threads have no
+// more than two blocks on an SM either way and hide a row's latencies behind the second (268 MB of rows, one -> two: 6152
+// elements 122 -> 116 us, 8192 93 -> 85, 12296 130 -> 118, 16384 103 -> 95).  float: from three chunks on (768, 32 x 3, 21 and 28),
+// from four in groups of 512 (8200, 512 x 3, 88 with one, 83 with two; 12296, 512 x 4, 78 and 107).
+__host__ __device__ constexpr int rows_in_flight(int vpt, int tpr, int elem_bytes) {
+  if (elem_bytes == 2) return vpt < 4 || tpr >= 256 ? 2 : 1;
+  return vpt < (tpr >= 512 ? 4 : 3) ? 2 : 1;
 }
+
+// Blocks per SM that the register budget is cut for (0: left to the compiler): two where the compiler would take a few registers
+// too many for the second.  float rows of one warp or less: up to five chunks per thread (268 MB of rows, without -> with: 512
+// elements 85 -> 65 us, 1024 83 -> 63, 1280 78 -> 66); six (1536 elements) would spill, 69 -> 77.
+constexpr int min_blocks(int vpt, int tpr, int elem_bytes) { return tpr == 256 || (elem_bytes == 4 && tpr <= 32 && vpt <= 5) ? 2 : 0; }
 
 // A chunk of 8 elements as it is loaded (kept in this form while the rows before it are processed), and
 // its expansion into 4 packed float pairs.
@@ -122,13 +130,12 @@ __device__ __forceinline__ void group_sum(int (&v)[kRows]) {
 }
 
 template <typename T, int TPR, int kVPT, bool kPack4, bool kFull>
-__global__ void __launch_bounds__((TPR > 256 ? TPR : 256),
-                                  (TPR == 256 ? 2 : sizeof(T) == 4 && TPR == 32 && (kVPT == 3 || kVPT == 4) ? 2 : 0))
+__global__ void __launch_bounds__((TPR > 256 ? TPR : 256), min_blocks(kVPT, TPR, sizeof(T)))
 ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
                 const float* __restrict__ gamma_t, const float* __restrict__ beta_t, float eps, int rms,
                 float inv_s, int z, int qmax, uint8_t* __restrict__ codes, int64_t ldc,
                 int32_t* __restrict__ row_sum, int32_t* __restrict__ clear, int64_t n_clear, bool settled) {
-  constexpr int kRows = rows_in_flight(kVPT, TPR, kFull, sizeof(T));
+  constexpr int kRows = rows_in_flight(kVPT, TPR, sizeof(T));
   constexpr int kBlock = TPR > 256 ? TPR : 256;
   constexpr int kGroups = kBlock / TPR;
   constexpr int kRowsPerBlock = kGroups * kRows;
@@ -466,7 +473,7 @@ struct Call {
 template <typename T, int TPR, int kVPT, bool kPack4, bool kFull>
 repq_status launch(const Call<T>& c, cudaStream_t st) {
   constexpr int kBlock = TPR > 256 ? TPR : 256;
-  constexpr int kRowsPerBlock = kBlock / TPR * rows_in_flight(kVPT, TPR, kFull, sizeof(T));
+  constexpr int kRowsPerBlock = kBlock / TPR * rows_in_flight(kVPT, TPR, sizeof(T));
   constexpr int kMostSmem = TPR * kVPT * kChunk * 2 * int(sizeof(float));
   auto kern = ln_quant_kernel<T, TPR, kVPT, kPack4, kFull>;
   const int64_t need = (c.rows + kRowsPerBlock - 1) / kRowsPerBlock;

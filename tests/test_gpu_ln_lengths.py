@@ -19,3 +19,12 @@ def test_ln_quant_row_lengths(D, bf16):
 def test_ln_quant_many_rows(rows, D, bits, bf16, rms):
     rep = parity.check_ln_quant(rows, D, bits, bf16, seed=rows, rms=rms)
     assert rep["bad"] == 0, rep
+
+
+@pytest.mark.parametrize("rows,D,bf16", [(700, 6152, True), (601, 7168, True), (450, 12296, True), (333, 16376, True), (400, 8200, False),
+                                         (3001, 512, False), (2500, 1280, False), (4001, 200, False)])
+def test_ln_quant_row_forms(rows, D, bf16):
+    """Two rows per group where the row does not fill it, and the float forms under a register bound; odd numbers of rows, more than
+    one grid takes at a time."""
+    rep = parity.check_ln_quant(rows, D, 4, bf16, seed=rows + D)
+    assert rep["bad"] == 0, rep
