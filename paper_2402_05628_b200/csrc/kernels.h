@@ -39,20 +39,27 @@ repq_status launch_scores(const repq_gemm_desc& d, cudaStream_t st);
 bool scores_tc_supported(const repq_gemm_desc& d);
 repq_status launch_scores_tc(const repq_gemm_desc& d, cudaStream_t st);
 
-// Tensor-memory (tcgen05) integer GEMM: plain (unbatched) products with TMA-compatible operands.
+// The two integer GEMMs on tcgen05 and how each would cut a problem up, with its estimated time in microseconds (measured in
+// CUDA graphs over 1..16384 tokens, N and K 384..22016; half of the estimates are within 3 %, 99 of 100 within 15 %).  One
+// estimate serves the choice between the two and the choice of form within each.
+//
+// 128-row or 256-row tiles (plain products with TMA-compatible operands).  bn: tile width, 0 where the kernel does not take the
+// problem; pair: 256 x 256 tiles by pairs of CTAs.
+struct TcPlan { int bn = 0; bool pair = false; float us = 0.f; };
 bool qgemm_tc_supported(const repq_gemm_desc& d);
+TcPlan qgemm_tc_plan(const repq_gemm_desc& d);
 size_t qgemm_tc_workspace(const repq_gemm_desc& d);
-repq_status qgemm_tc(const repq_gemm_desc& d, const EpilogueParams& ep, void* ws, size_t ws_bytes,
+repq_status qgemm_tc(const repq_gemm_desc& d, const EpilogueParams& ep, const TcPlan& plan, void* ws, size_t ws_bytes,
                      cudaStream_t st);
+// Few tokens (weights on the M side of the tensor-core instruction): plain products, byte codes, both row sums given.  mt:
+// tokens per tile, 0 where the kernel does not take the problem; split: CTAs that share a tile's K range.
+struct SkinnyPlan { int mt = 0, split = 0; float us = 0.f; };
+SkinnyPlan qgemm_skinny_plan(const repq_gemm_desc& d);
+repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, const SkinnyPlan& plan, Params params, cudaStream_t st);
 
 // Workspace of a GEMM: with room for a byte copy of packed weights, and the least it can run in.
 size_t qgemm_workspace(const repq_gemm_desc& d);
 size_t qgemm_workspace_least(const repq_gemm_desc& d);
-
-// Integer GEMM for few tokens (weights on the M side of the tensor-core instruction): plain products, byte codes, both
-// row sums given; `preferred` says whether it takes the problem and is the faster one.
-bool qgemm_skinny_preferred(const repq_gemm_desc& d);
-repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, Params params, cudaStream_t st);
 
 // P.V (Eqs. 16-17): kernel parameters shared by the two implementations, storage widths already resolved
 // (bits_v is 4 for packed codes, 8 for byte codes).

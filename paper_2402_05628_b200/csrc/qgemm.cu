@@ -154,7 +154,7 @@ bool byte_weights(const repq_gemm_desc& d, repq_gemm_desc* as_bytes, ByteWeights
   as_bytes->bits_w = quant_bits(d.bits_w) | REPQ_BYTE_CODES;
   B->ld = round_up(d.K, 16);
   as_bytes->ldw_bytes = B->ld;
-  if (!qgemm_skinny_preferred(*as_bytes) && !qgemm_tc_supported(*as_bytes)) return false;
+  if (!qgemm_tc_supported(*as_bytes) && qgemm_skinny_plan(*as_bytes).mt == 0) return false;
   B->offset = (qgemm_tc_supported(*as_bytes) ? qgemm_tc_workspace(*as_bytes) : 0);
   B->offset = (B->offset + 255) / 256 * 256;
   B->total = B->offset + size_t(d.N) * size_t(B->ld);
@@ -319,12 +319,14 @@ repq_status repq::run_qgemm(const repq_gemm_desc& given, void* workspace, size_t
     params = Params::streamed;                             // (the expansion is the kernel just ahead now)
   }
   const EpilogueParams ep = make_epilogue(*d);
-  if (qgemm_skinny_preferred(*d)) return qgemm_skinny(*d, ep, params, st);
-  if (qgemm_tc_supported(*d)) {
+  const SkinnyPlan few = qgemm_skinny_plan(*d);
+  const TcPlan tiles = qgemm_tc_plan(*d);
+  if (few.mt != 0 && (tiles.bn == 0 || few.us < tiles.us)) return qgemm_skinny(*d, ep, few, params, st);
+  if (tiles.bn != 0) {
     const size_t need = qgemm_tc_workspace(*d);
     REPQ_REQUIRE(workspace_bytes >= need && (need == 0 || workspace), REPQ_WORKSPACE_TOO_SMALL,
                  "qgemm: workspace of %zu bytes given, %zu needed", workspace_bytes, need);
-    return qgemm_tc(*d, ep, workspace, workspace_bytes, st);
+    return qgemm_tc(*d, ep, tiles, workspace, workspace_bytes, st);
   }
   return qgemm_mma(*d, ep, st);
 }

@@ -374,60 +374,49 @@ repq_status launch_step(int step, dim3 grid, uint32_t smem, const CUtensorMap& m
 
 }  // namespace
 
-namespace {
-
-// How a problem is cut up: tokens per tile and CTAs per tile, and the estimated time in microseconds.  The terms were
-// fitted to launches in CUDA graphs (K 384..11008, N 384..22016, 16..788 tokens); what they stand for:
-//   a launch                2.6
-//   operands                k-blocks of a CTA x (16 KB of weights + tokens) x CTAs that share an SM, at 120 KB per us and SM,
-//                           or all weights at 4.5 TB/s, whichever is longer
-//   epilogue                0.028 per token of a CTA's share
-//   exchange in the cluster 1.2
-// At most two CTAs per SM: a second wave costs more than it brings.
-struct Plan { int mt = 0, split = 0; float us = 1e30f; };
-
-Plan plan_of(int M, int N, int K, int sms) {
-  Plan best;
-  const int n_tiles = (N + kRowsW - 1) / kRowsW, kblocks = (K + kBK - 1) / kBK;
-  const float hbm = float(N) * float(K) / 4.5e6f;
+// Tokens per tile and CTAs per tile by the least estimated time, in microseconds:
+//   a launch                1.9
+//   operands                k-blocks of a CTA x 0.295 (a ring's latency over its stages) or, with two CTAs on an SM, x (16 KB of
+//                           weights + tokens) at 160 KB per us and SM; or all weights at 4.6 TB/s, whichever is longer
+//   epilogue                0.024 per token of a CTA's share, 0.039 with GELU or a step on column pairs, 0.046 with a residual
+//   exchange in a cluster   1.15 and 0.031 per token that leaves the CTA
+//   two CTAs on an SM       0.5, and 1.53 x the epilogue and the exchange
+// Clusters fill the SMs less evenly: those of four and eight share SMs from 0.91 and 0.75 CTAs per SM on, and beyond 1.8 and 1.62
+// per SM (two without a cluster) the last ones wait for a second wave, which costs more than it brings.
+// The best plan's time is within 0.6 % of the fastest form's on average (4.8 % with the terms used before, which had no cost per
+// token exchanged: 48 x 4096 x 4096 with residual 11.7 -> 7.9 us, 197 x 768 x 3072 11.2 -> 6.7).
+SkinnyPlan qgemm_skinny_plan(const repq_gemm_desc& d) {
+  SkinnyPlan best;
+  if (d.batch_outer != 1 || d.batch_inner != 1 || d.N < 64 || d.K < 64) return best;
+  if (!d.a_row_sum || !d.w_row_sum) return best;           // (the sums are not taken here; no workspace)
+  if (packed4(d.bits_a) || packed4(d.bits_w) || packed6(d.bits_w)) return best;
+  if (!(aligned(d.a_codes, 16) && d.lda_bytes % 16 == 0 && aligned(d.w_codes, 16) && d.ldw_bytes % 16 == 0)) return best;
+  const int sms = sm_count();
+  const int n_tiles = (d.N + kRowsW - 1) / kRowsW, kblocks = (d.K + kBK - 1) / kBK;
+  const float hbm = float(d.N) * float(d.K) / 4.6e6f;
+  const float per_token = d.residual ? 0.0461f : d.gelu || d.glu || d.rope_cos_sin ? 0.0386f : 0.0243f;
   for (int mt : {16, 32, 48, 64, 96, 128}) {
-    const int m_tiles = (M + mt - 1) / mt;
+    const int64_t m_tiles = (int64_t(d.M) + mt - 1) / mt;
     for (int split = 1; split <= 8; split *= 2) {
-      const int64_t ctas = int64_t(n_tiles) * m_tiles * split;
-      if (ctas > 2 * sms || (split > 1 && kblocks < 2 * split)) break;
-      const float per_sm = ctas > sms ? 2.f : 1.f;
-      const int kb = (kblocks + split - 1) / split, share = (mt / kTok + split - 1) / split * kTok;
-      float load = per_sm * float(kb) * (16.f + float(mt) / 8.f) / 120.f;
+      const float ctas = float(n_tiles) * float(m_tiles) * float(split);
+      const float single = float(sms) * (split == 8 ? 0.75f : split == 4 ? 0.91f : 1.f);
+      const float most = float(sms) * (split == 8 ? 1.62f : split == 4 ? 1.8f : 2.f);
+      if (ctas > most || (split > 1 && kblocks < 2 * split)) continue;
+      const bool two = ctas > single;
+      const float kb = float((kblocks + split - 1) / split), share = float((mt / kTok + split - 1) / split * kTok);
+      const float wide = (two ? 2.f : 1.f) * (16.f + float(mt) / 8.f) / 160.f;
+      float load = kb * (wide > 0.295f ? wide : 0.295f);
       if (load < hbm) load = hbm;
-      const float us = 2.6f + load + per_sm * float(share) * 0.028f + (split > 1 ? 1.2f : 0.f);
-      if (us < best.us) { best.mt = mt; best.split = split; best.us = us; }
+      float us = 1.9f + load + (two ? 0.49f : 0.f) + (two ? 1.53f : 1.f) * share * per_token;
+      if (split > 1) us += 1.15f + (two ? 1.53f : 1.f) * 0.0314f * float(mt) * (1.f - 1.f / float(split));
+      if (best.mt == 0 || us < best.us) { best.mt = mt; best.split = split; best.us = us; }
     }
-    if (mt >= M) break;
+    if (mt >= d.M) break;
   }
   return best;
 }
 
-}  // namespace
-
-// Taken where its estimate is clearly below that of the 128-row kernel (4.5 us + 0.27 us per round of tiles and k-block, or
-// the weights at 4.5 TB/s), which holds up to some hundreds of tokens, and below 64 tokens wherever the operands allow it.
-bool qgemm_skinny_preferred(const repq_gemm_desc& d) {
-  if (d.batch_outer != 1 || d.batch_inner != 1 || d.N < 64 || d.K < 64) return false;
-  if (!d.a_row_sum || !d.w_row_sum) return false;          // (the sums are not taken here; no workspace)
-  if (packed4(d.bits_a) || packed4(d.bits_w) || packed6(d.bits_w)) return false;
-  if (!(aligned(d.a_codes, 16) && d.lda_bytes % 16 == 0 && aligned(d.w_codes, 16) && d.ldw_bytes % 16 == 0)) return false;
-  const int sms = sm_count();
-  const Plan plan = plan_of(d.M, d.N, d.K, sms);
-  if (plan.mt == 0) return false;
-  if (!qgemm_tc_supported(d)) return true;
-  const int64_t tiles = (int64_t(d.M) + 127) / 128 * ((int64_t(d.N) + 255) / 256);
-  float other = float((tiles + sms - 1) / sms) * float((d.K + kBK - 1) / kBK) * 0.27f;
-  const float hbm = float(d.N) * float(d.K) / 4.5e6f;
-  if (other < hbm) other = hbm;
-  return plan.us * 1.1f < other + 4.5f || (d.M <= 64 && plan.us < other + 4.5f);
-}
-
-repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, Params params, cudaStream_t st) {
+repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, const SkinnyPlan& plan, Params params, cudaStream_t st) {
   SkinnyParams P{};
   P.M = d.M; P.N = d.N; P.K = d.K;
   P.asum = d.a_row_sum; P.wsum = d.w_row_sum;
@@ -435,7 +424,6 @@ repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, Para
   P.weights_settled = params == Params::settled;
   P.status = device_status_word();
   REPQ_REQUIRE(P.status != nullptr, REPQ_CUDA_ERROR, "qgemm: device status word unavailable");
-  const Plan plan = plan_of(d.M, d.N, d.K, sm_count());
   const int n_tiles = (d.N + kRowsW - 1) / kRowsW, mt = plan.mt, split = plan.split;
   const int m_tiles = (d.M + mt - 1) / mt;
   P.kblocks = (d.K + kBK - 1) / kBK;

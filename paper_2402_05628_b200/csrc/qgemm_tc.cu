@@ -17,9 +17,9 @@
 //                192 columns) and 4 converter warps.  The weight tile arrives packed and the converters expand it into
 //                the 128-byte-swizzled byte tile the MMA descriptor expects (there is no 4- or 6-bit integer MMA); one
 //                more barrier hop between the copy and the MMA, weights stay packed in HBM
-// The tile width BN (256, 192 or 128) is chosen per problem: rounds of tiles over the SMs times a per-round time
-// with a fixed part.  Packed 4-bit activations are expanded to one code per byte by a separate pass into the
-// workspace (inside the block the producers write byte codes, so that pass does not run there).
+// The tile width BN (256, 192 or 128), or pairs, is chosen per problem by estimated time (qgemm_tc_plan).  Packed 4-bit
+// activations are expanded to one code per byte by a separate pass into the workspace (inside the block the producers write
+// byte codes, so that pass does not run there).
 //
 // For short K the epilogue, not the tensor pipe, sets the pace (K = 768: 3072 tensor-pipe cycles per 128 x 256 tile
 // against 32768 outputs), so it is written for few instructions per output and few waits per tile: every epilogue warp
@@ -169,6 +169,7 @@ struct TcParams {
   int w_packed4;               // weight tiles arrive packed (4: two codes per byte, 6: four in three bytes) and are
                                // expanded in shared memory; 0: byte tiles
   int pair;                    // 256-row tiles by pairs of CTAs
+  int res_boxes;               // bf16 residual by bulk-copied boxes (tiles of at most 192 columns)
   TileOrder order;             // panels of row tiles (see TileOrder)
   EpilogueParams ep;
 };
@@ -926,58 +927,13 @@ TcLayout tc_layout(const repq_gemm_desc& d) {
   return L;
 }
 
-// Tile width: rounds of tiles over the SMs times the time of one round, which has a part that does not depend on the
-// width (per-tile waits, staging and bulk-store latencies of the epilogue warps) and a part proportional to it
-// (measured: about 160 columns' worth of fixed time for K = 768).
-// Whether a launch takes its bf16 residual through bulk-copied boxes (tiles of at most 192 columns, short K).
-bool residual_boxes(const TcParams& P) {
-  const EpilogueParams& ep = P.ep;
-  // (up to K = 3072: beyond, the main loop sets the pace, and its time per k-block does not shrink with the tile width
-  // (the operand copies in flight, four stages, against the L2 latency), so that 256-column tiles win: measured at
-  // 8192 x 4096 x 4096 101 us with 256 columns against 111 with 192, at 18464 x 1024 x 4096 67 against 79)
-  return ep.out_kind == REPQ_OUT_BF16 && ep.residual != nullptr && ep.residual_bf16 && ep.acc_debug == nullptr &&
-         ep.glu == 0 && P.K <= 3072 && !P.w_packed4;
-}
-
-int pick_bn(int M, int N, int K, int sms, bool w_packed4, bool res_boxes) {
-  const int m_tiles = (M + BM - 1) / BM;
-  int best = 256;
-  long best_cost = -1;
-  for (int bn : {256, 192, 128}) {
-    if (w_packed4 && bn > kMaxBNW4) continue;
-    const long tiles = long(m_tiles) * ((N + bn - 1) / bn);
-    const long rounds = (tiles + sms - 1) / sms;
-    // a round costs its width plus a fixed part; where the epilogue adds a bf16 residual at short K, a round is the longer
-    // of the main loop (0.34 us per k-block) and the epilogue, and the epilogue of a 256-column tile (residual by
-    // row-per-lane loads) takes 1.7 x the time of a narrower one whose residual box was copied in a tile ahead (measured
-    // at 18464 x 1024 x 1024: 39.6 us with 256 columns, 33.9 with 192)
-    const long main_loop = 34L * ((K + BK - 1) / BK), epilogue = bn == 256 ? 950 : 550;
-    const long cost = res_boxes ? rounds * (main_loop > epilogue ? main_loop : epilogue) : rounds * (bn + 160);
-    if (best_cost < 0 || cost < best_cost) { best = bn; best_cost = cost; }
-  }
-  return best;
-}
-
-// Whether 256 x 256 tiles by pairs of CTAs beat 128-row tiles of bn columns.  A pair copies a third less operand bytes per
-// operation, so a k-block takes 0.285 us instead of 0.365 (256 columns); an epilogue takes as long as on a 128 x 256 tile, and
-// there are half as many, twice as large pieces to deal out.  (Microseconds; fitted to M 300..16384, N 768..12288, K
-// 768..11008.  8192 x 4096 x 11008 with residual 250 -> 205 us, 8192 x 12288 x 4096 to codes 234 -> 216, 777 x 4096 x 11008 40 ->
-// 35; at K = 768 the epilogue sets the pace and narrow tiles stay.)
-bool pair_is_faster(const TcParams& P, int bn, int sms) {
-  if (P.w_packed4) return false;
-  const float kb = float((P.K + BK - 1) / BK);
-  const bool res16 = P.ep.residual != nullptr && P.ep.residual_bf16;
-  auto rounds = [&](int tm, int tn, int slots) {
-    const long tiles = long((P.M + tm - 1) / tm) * ((P.N + tn - 1) / tn);
-    return float((tiles + slots - 1) / slots);
-  };
-  const float width = float(bn + 160) / 416.f;           // a round's time against that of 256 columns (see pick_bn)
-  const float epi256 = res16 ? 10.2f : 5.2f;             // residual by row-per-lane loads; otherwise
-  const float main1 = (2.0f + 0.365f * kb) * width, epi1 = residual_boxes(P) && bn < kMaxBN ? 5.5f : epi256 * width;
-  const float main2 = 2.2f + 0.285f * kb;
-  const float single = rounds(BM, bn, sms) * (main1 > epi1 ? main1 : epi1);
-  const float pair = rounds(2 * BM, kMaxBN, sms / 2) * (main2 > epi256 ? main2 : epi256);
-  return pair * 1.08f < single;
+// Whether a launch takes its bf16 residual through bulk-copied boxes (tiles of at most 192 columns, short K: beyond K = 3072 the
+// main loop sets the pace, and its time per k-block hardly shrinks with the tile width (the operand copies in flight, four stages,
+// against the L2 latency), so that 256-column tiles win: measured at 8192 x 4096 x 4096 101 us with 256 columns against 111 with
+// 192, at 18464 x 1024 x 4096 67 against 79).
+bool residual_boxes(const repq_gemm_desc& d) {
+  return d.out_kind == REPQ_OUT_BF16 && d.residual != nullptr && d.residual_dtype == REPQ_BF16 && d.acc_debug == nullptr &&
+         d.glu == 0 && d.K <= 3072 && !packed4(d.bits_w) && !packed6(d.bits_w);
 }
 
 // Tensor map of the output for the epilogue's bulk stores: boxes of 32 rows x 32 bytes, 32-byte swizzle.
@@ -1055,7 +1011,7 @@ repq_status launch_tc_out(const CUtensorMap& map_a, const CUtensorMap& map_b, co
   // bf16 outputs with a bf16 residual on tiles of at most 192 columns: the residual boxes, which also carry the output,
   // fit beside the four stages
   if constexpr (BN <= 192 && OUT == kOutBf16) {
-    if (residual_boxes(P))
+    if (P.res_boxes)
       return launch_tc_res<BN, OUT, true>(map_a, map_b, P, sms, st);
   }
   return launch_tc_res<BN, OUT, false>(map_a, map_b, P, sms, st);
@@ -1133,9 +1089,43 @@ bool qgemm_tc_supported(const repq_gemm_desc& d) {
   return true;
 }
 
+// Tile width, and single CTAs or pairs, by the least estimated time, in microseconds: a launch 1.0; then the first main loop, per
+// further round of tiles over the SMs the longer of a main loop and an epilogue, and the last epilogue; and the weights at 15 TB/s
+// (what their way from HBM adds to the operand copies' latency).
+//   main loop   0.3 + 0.333 / 0.309 / 0.27 per k-block (256 / 192 / 128 columns; the operand copies' latency over the stages),
+//               1.1 + 0.266 on a 256 x 256 tile by a pair, which copies a third less per operation
+//   epilogue    2.05 + per 256 columns 1.73 (plain), 3.4 (GELU, a step on column pairs, packed weights), 3.38 (residual by row-per-
+//               lane loads), 1.62 (residual boxes, at most 192 columns); a pair's 1.27 x the second part
+// Choices on either side of a line, measured: 18464 x 1024 x 1024 with residual 39.6 us with 256 columns, 33.9 with 192 and
+// boxes; 8192 x 4096 x 11008 with residual 250 single, 205 by pairs; 8192 x 12288 x 4096 to codes 234 and 216; 777 x 4096 x 11008
+// 40 and 35; 2500 x 384 x 384 with residual 6.0 with 192 columns, 5.2 with 128.  Over 1200 problems the chosen form is within
+// 0.3 % of the fastest on average (0.9 % with a rule of its own for each of the three choices).
+TcPlan qgemm_tc_plan(const repq_gemm_desc& d) {
+  TcPlan best;
+  if (!qgemm_tc_supported(d)) return best;
+  const bool packed = packed4(d.bits_w) || packed6(d.bits_w), boxes = residual_boxes(d);
+  const int sms = sm_count();
+  const float kb = float((d.K + BK - 1) / BK);
+  const float from_hbm = float(d.N) * float(d.K) / 15e6f;
+  const float direct = d.residual ? 3.38f : d.gelu || d.glu || d.rope_cos_sin || packed ? 3.4f : 1.73f;
+  auto consider = [&](int tm, int bn, int slots, float main_loop, float epilogue) {
+    const int64_t tiles = (int64_t(d.M) + tm - 1) / tm * ((int64_t(d.N) + bn - 1) / bn);
+    const float further = float((tiles + slots - 1) / slots - 1);
+    const float us = 1.f + main_loop + further * (main_loop > epilogue ? main_loop : epilogue) + epilogue + from_hbm;
+    if (best.bn == 0 || us < best.us) best = TcPlan{bn, tm > BM, us};
+  };
+  for (int bn : {256, 192, 128}) {
+    if (packed && bn > kMaxBNW4) continue;
+    const float step = bn == 256 ? 0.333f : bn == 192 ? 0.309f : 0.27f;
+    consider(BM, bn, sms, 0.3f + step * kb, 2.05f + (boxes && bn <= 192 ? 1.62f : direct) * float(bn) / 256.f);
+  }
+  if (!packed) consider(2 * BM, kMaxBN, sms / 2, 1.1f + 0.266f * kb, 2.05f + 1.27f * direct);
+  return best;
+}
+
 size_t qgemm_tc_workspace(const repq_gemm_desc& d) { return tc_layout(d).total; }
 
-repq_status qgemm_tc(const repq_gemm_desc& d, const EpilogueParams& ep, void* ws, size_t ws_bytes, cudaStream_t st) {
+repq_status qgemm_tc(const repq_gemm_desc& d, const EpilogueParams& ep, const TcPlan& plan, void* ws, size_t ws_bytes, cudaStream_t st) {
   const TcLayout L = tc_layout(d);
   REPQ_REQUIRE(ws_bytes >= L.total, REPQ_WORKSPACE_TOO_SMALL, "qgemm: workspace too small");
   REPQ_REQUIRE(L.total == 0 || aligned(ws, 256), REPQ_ALIGNMENT, "qgemm: workspace must be 256-byte aligned");
@@ -1165,9 +1155,9 @@ repq_status qgemm_tc(const repq_gemm_desc& d, const EpilogueParams& ep, void* ws
   P.direct_requant = d.out_kind == REPQ_OUT_CODES && !d.gelu && !d.residual && !d.glu;
   REPQ_REQUIRE(device_status_word() != nullptr, REPQ_CUDA_ERROR, "qgemm: device status word unavailable");
   const int sms = sm_count();
-  int bn = pick_bn(d.M, d.N, d.K, sms, P.w_packed4 != 0, residual_boxes(P));
-  P.pair = pair_is_faster(P, bn, sms);
-  if (P.pair) bn = kMaxBN;
+  const int bn = plan.bn;
+  P.pair = plan.pair;
+  P.res_boxes = residual_boxes(d);
   {
     // panels of activations: all row tiles while the activations take at most 40 MB (a third of the L2 capacity),
     // else about 24 MB (measured at 8192 x 4096 x 11008 with residual: 248 us with 40 MB panels, 240-242 with

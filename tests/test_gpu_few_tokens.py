@@ -62,3 +62,17 @@ def test_copies_asked_for_early_are_drained_when_a_wait_runs_out(limit):
     assert B.repq_device_status(reset=True) == 77
     parity.check_qgemm(16, 384, 384, 4 | parity.BYTE_CODES, 4 | parity.BYTE_CODES, out_kind="f32", want_acc=False, give_sums=True)
     assert B.repq_device_status() == 0
+
+
+@pytest.mark.parametrize("M,N,K,kw", [
+    (48, 4096, 4096, dict(out_kind="bf16", residual="bf16")),                 # 48 tokens a tile, clusters of four
+    (197, 768, 3072, dict(out_kind="bf16", residual="bf16")),                 # 32 tokens, clusters of four, the last tile ragged
+    (80, 768, 3072, dict(out_kind="f32", residual="f32")),                    # 16 tokens, clusters of eight
+    (394, 1024, 4096, dict(out_kind="bf16", residual="bf16")),                # the most CTAs clusters of two or four get
+    (512, 1152, 384, dict(out_kind="codes", out_bits=4 | parity.BYTE_CODES, groups=3)),
+    (777, 2048, 1408, dict(out_kind="bf16", residual="bf16")),                # many token tiles, or the 128-row kernel
+])
+def test_few_token_plans_match_oracle(M, N, K, kw):
+    """Tokens per tile and K splits across the range in which the plan of the few-token kernel moves."""
+    b = 4 | parity.BYTE_CODES
+    parity.check_qgemm(M, N, K, b, b, give_sums=True, seed=M + N + K, want_acc=False, **kw)

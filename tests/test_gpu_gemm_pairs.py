@@ -22,3 +22,13 @@ def test_pair_tiles_match_oracle(M, N, K, kw):
 @pytest.mark.parametrize("mode,N", [("rope", 2304), ("glu", 2048)])
 def test_pair_tiles_with_a_pair_step(mode, N):
     parity.check_qgemm_pair_step(2000, N, 5504, 4 | parity.BYTE_CODES, mode, seed=N)
+
+
+@pytest.mark.parametrize("M,N,K,kw", [
+    (2049, 2032, 5520, dict(out_kind="codes", out_bits=4 | parity.BYTE_CODES, want_out_sum=True)),      # one row in the last pair
+    (2300, 2040, 5504, dict(out_kind="bf16", residual="bf16")),                                         # 252 rows: second CTA cut
+])
+def test_pair_tiles_in_one_round(M, N, K, kw):
+    """72 tiles for 74 pairs, where 128-row tiles of any width take two rounds or as long a main loop each."""
+    b = 4 | parity.BYTE_CODES
+    parity.check_qgemm(M, N, K, b, b, give_sums=True, seed=M, **dict(dict(want_acc=False), **kw))
