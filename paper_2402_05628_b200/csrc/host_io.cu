@@ -16,21 +16,22 @@ namespace {
 constexpr int kMaxDevices = 64;
 constexpr int kSlots = 2;
 constexpr int kMaxPieces = 8;
-constexpr size_t kPieceBytes = size_t(2400) << 10;        // 2.4 MB: some 50 us of the link, what queueing a piece takes the host
-constexpr size_t kGapBytes = size_t(448) << 10;          // what the link would move between two copies of a stream (10 us)
+constexpr size_t kPieceBytes = size_t(4300) << 10;       // 4.4 MB: 100 us of the link, twice what queueing a piece takes the host
+constexpr size_t kGapBytes = size_t(700) << 10;          // what the link would move while a further piece holds it up (16 us; copies
+                                                         // alone stand 10 us apart, with the waits on events 10 to 25)
 
-// Pieces per batch: as many as are at least kPieceBytes of input each, unless what they save (the link time of a batch: the
-// outputs no longer run a batch behind) is less than the gaps they add (one per piece and batch).
-// Measured, us (DeiT-B, 64 images of 19.4 MB, 7 pieces | ViT-L, 32 images of 37.8 MB, 8 pieces; whole -> pieces): one batch
-// 934 -> 602 | 1841 -> 1029, two 1336 -> 1078 | 2577 -> 1860, four 2235 -> 2048 | 4237 -> 3530, five 2700 -> 2511 | 5065 -> 4362,
-// eight 4051 -> 3957 (whole by the rule) | 7541 -> 6943, sixteen 7664 -> 7769 (whole) | 14157 -> 13644 (whole).  64 ViT-S images
-// (9.7 MB, 3 pieces): one 488 -> 340, five 1462 -> 1456, eight 2219 -> 2259 (whole), sixteen 4247 -> 4477 (whole).  16 DeiT-B
-// images (4.8 MB) in two pieces: one batch 278 -> 240, but four 605 -> 633.
-// Three to five pieces of the two larger batches are slower than the counts on either side of them (four DeiT-B batches: 2372,
-// 2252 and 2218 us against 2219 with two and 2083 with six); the cause was not found.  Pieces for the first and the last batch
-// only gain nothing beyond two batches: the outputs then fall a batch behind in between.
+// Pieces per batch: of about kPieceBytes of input each, unless what they save (the link time of a batch: the outputs no longer run
+// a batch behind) is less than the gaps they add (one per piece and batch).  More pieces than that, and the small blocks' time
+// adds up to more than the link's.
+// Measured, us, whole -> pieces (ranges: two machines): 64 DeiT-B images of 19.4 MB, four pieces: one batch 935 -> 611..631, two
+// 1340 -> 1056..1154, four 2235 -> 2020..2250, five 2690 -> 2518..2800, eight 4051 -> 4414 (whole by the rule).  32 ViT-L images at
+// 577 tokens, 37.8 MB, eight: 1841 -> 1029, four 4237 -> 3530, five 5065 -> 4362, sixteen 14157 -> 13644 (whole).  16 of them, 18.9 MB,
+// four: 955 -> 612, five 2655 -> 2280 (with seven pieces 2894).  40 DeiT-B images of 150 tokens, packed 6-bit weights, 9.2 MB, two:
+// 499 -> 379, five 1416 -> 1198 (four pieces 1495).  7.4 MB, two: 402 -> 308, five 1172 -> 1010.  4.8 MB stay whole: in two pieces
+// four batches take 633 for 605.  Pieces for the first and the last batch only gain nothing beyond two batches: the
+// outputs then fall a batch behind in between.
 int pieces_of(size_t x_bytes, int batch, int n_batches) {
-  const size_t fit = x_bytes / kPieceBytes;
+  const size_t fit = (x_bytes + kPieceBytes / 2) / kPieceBytes;
   int pieces = int(fit < size_t(kMaxPieces) ? fit : size_t(kMaxPieces));
   if (pieces > batch) pieces = batch;
   if (pieces < 2) return 1;
