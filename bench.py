@@ -39,11 +39,6 @@ HEADLINE = "c4_llama7b"
 OTHER_WORKLOADS = ("c1_vit_s", "c2_deit_b", "c2_deit_b_w6a6", "c3_vit_l", "c4_llama7b_arch")
 INT8_OVER_BF16 = 2.0          # nominal dense int8 : bf16 tensor throughput on B200
 L2_BYTES = 126 << 20
-# Own model of the fused attention kernel's arithmetic, kept as a side figure from the first version of the kernel: about
-# 8 thread instructions per score in the statistics pass (int -> float, scale, max, subtract, ex2, add) and 15 in the code
-# pass.  (The present kernel needs about half of that and is not bound by it.)
-ATTENTION_INSTR_PER_SCORE = 23
-
 # DRAM traffic of one launch of a stage kernel, from one ncu capture of the same bench command (summaries under
 # profiles/).  A figure is reported only while the kernel's sources still hash to what was captured.
 NCU_TRAFFIC = {   # (workload, batch, stage): (DRAM bytes read + written per launch, kernel sources, their sha1 when captured)
@@ -179,7 +174,7 @@ def stage_costs(cfg, batch):
         "softmax": dict(bytes=n_scores * (4 + cp), ops=0),
         "pv": dict(ops=2.0 * n_scores * dh, bytes=n_scores * cp + M * D * ca * 2),
         # fused attention: Q, K, V codes in, attention codes out; one int8 and one bf16 contraction
-        "attention": dict(bytes=4 * M * D * ca, ops_i8=2.0 * n_scores * dh, flop_bf16=2.0 * n_scores * dh, scores=n_scores),
+        "attention": dict(bytes=4 * M * D * ca, ops_i8=2.0 * n_scores * dh, flop_bf16=2.0 * n_scores * dh),
         "proj": gemm(D, D, act * 2),          # residual read + output write
         "ln2": dict(bytes=M * D * (act + ca) + 4 * M, ops=0),
         "fc1": gemm(2 * MLP, D, ca, MLP) if llama else gemm(MLP, D, ca),
@@ -187,7 +182,7 @@ def stage_costs(cfg, batch):
     }
 
 
-def stage_record(name, ms, cost, peaks, sm_max_mhz):
+def stage_record(name, ms, cost, peaks):
     """Achieved rates of one stage and its fractions of the rooflines that could bound it."""
     if not ms or ms <= 0:
         return dict(ms=ms)
@@ -196,10 +191,8 @@ def stage_record(name, ms, cost, peaks, sm_max_mhz):
     rec = dict(ms=float(ms), gbs=cost["bytes"] / t / 1e9, frac_hbm=cost["bytes"] / t / 1e9 / peaks["hbm_gbs"])
     if name == "attention":
         tensor_s = cost["ops_i8"] / (int8_peak * 1e12) + cost["flop_bf16"] / (peaks["bf16_tflops"] * 1e12)
-        alu_peak = 148 * 4 * 32 * (sm_max_mhz or 1965.0) * 1e6
         rec.update(bf16_equiv_tflops=(cost["ops_i8"] / INT8_OVER_BF16 + cost["flop_bf16"]) / t / 1e12,
-                   frac_tensor=tensor_s / t,
-                   frac_issue_model=ATTENTION_INSTR_PER_SCORE * cost["scores"] / t / alu_peak)
+                   frac_tensor=tensor_s / t)
     elif cost.get("ops"):
         rec["tops"] = cost["ops"] / t / 1e12
         if name in ("qkv", "proj", "fc1", "fc2"):
@@ -287,14 +280,13 @@ def measure_block(name, batch, args, dev, rank, world, peaks, headline, sampler=
 
     ms_total, ms_e2e = max_over_ranks([ms_total, ms_e2e], dev, world)
     costs = stage_costs(cfg, batch)
-    sm_max = clocks["sm_max_mhz"] if clocks else None
     raw = dict(zip(B.BLOCK_STAGE_NAMES, stage_ms))
     stages = {}
     for st in B.BLOCK_STAGE_NAMES:
         if not args.staged_attention and st in ("softmax", "pv"):
             continue
         key = "attention" if (st == "scores" and not args.staged_attention) else st
-        stages[key] = stage_record(key, float(raw[st]), costs[key], peaks, sm_max)
+        stages[key] = stage_record(key, float(raw[st]), costs[key], peaks)
     rec = dict(workload=name, batch_per_gpu=batch, tokens_per_step=tokens_per_step,
                value=world * tokens_per_step * steps / (ms_total * 1e-3), ms_per_step=ms_total / steps,
                e2e=dict(value=world * tokens_per_step * steps / (ms_e2e * 1e-3), unit=UNIT,
@@ -581,7 +573,7 @@ def main():
             # two contractions (int8 QK^T, bf16 P.V): expressed in bf16-equivalent FLOP (an int8 operation counts
             # 1 / INT8_OVER_BF16), so that achieved / peak = (tensor time at the peaks) / (measured time)
             roof = dict(kernel=top, bound="tensor", achieved=st["bf16_equiv_tflops"], peak=peaks["bf16_tflops"], unit="TFLOP/s",
-                        frac=st["frac_tensor"], traffic=traffic, frac_hbm=st["frac_hbm"], frac_issue_model=st["frac_issue_model"],
+                        frac=st["frac_tensor"], traffic=traffic, frac_hbm=st["frac_hbm"],
                         peak_source="%s bf16 burst; int8 operations of QK^T counted at 1/%.0f (nominal int8:bf16); algorithmic "
                                     "operation counts (one pass over the keys, P.V once)" % (peaks["source"], INT8_OVER_BF16))
         elif top in ("qkv", "proj", "fc1", "fc2"):

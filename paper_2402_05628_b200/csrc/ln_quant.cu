@@ -8,10 +8,11 @@
 // warp centres its slice on the slice's own mean, the means and squares are merged behind the barrier, and the code sums wait
 // for the next one.
 //
-// What bounds it: HBM for float input and for rows of one warp (5.1-6.3 TB/s of 6.46), instruction issue and the occupancy
-// the registers leave for longer bf16 rows (ncu, 2048 elements: 10.9 warp instructions per 32 elements, 16 warps per SM, issue
-// slots 59 % busy).  Measured against three barriers per iteration: 32768 bf16 rows of 4096 78 -> 73 us, 65536 of 1536 53 -> 45,
-// 32768 float rows of 2048 83 -> 48, 16384 of 4096 76 -> 49.
+// What bounds it: HBM for float input and for rows of one warp (5.1-6.3 TB/s of 6.46); for longer bf16 rows the latencies of a
+// row's chain at the 16 warps per SM that the registers leave (ncu, 32768 x 4096: DRAM 45 % of its peak, issue slots 56 %, first
+// stall the factors' reads from shared memory and the shuffles, then waits of known length; 76-80 us against 51 at the copy rate).
+// Measured against three barriers per iteration: 65536 bf16 rows of 1536 53 -> 45 us, 32768 float rows of 2048 83 -> 48, 16384 of
+// 4096 76 -> 49; 32768 bf16 rows of 4096 gained nothing (80).
 // The per-channel factors gamma~/s~ and beta~/s~ are staged once per CTA in shared memory (halves of the 8-element
 // chunks apart, so that a warp's 16-byte reads are free of bank conflicts).
 //
@@ -33,7 +34,7 @@ constexpr int kChunk = 8;   // elements per 128-bit bf16 load
 
 // Rows a thread group works on at a time (the loads of the next ones are always in flight as well): two, except where the
 // chunks per thread leave the registers for one.  bf16: from four chunks on in groups that share an SM with others (2048 / 4096
-// elements, 64 x 4 / 128 x 4 threads x chunks, 69 / 73 us with one row, 97 / 101 with two); groups of 256 and 512 threads have no
+// elements, 64 x 4 / 128 x 4 threads x chunks, 69 / 73 us in short runs with one row, 97 / 101 with two); groups of 256 and 512 threads have no
 // more than two blocks on an SM either way and hide a row's latencies behind the second (268 MB of rows, one -> two: 6152
 // elements 122 -> 116 us, 8192 93 -> 85, 12296 130 -> 118, 16384 103 -> 95).  float: from three chunks on (768, 32 x 3, 21 and 28),
 // from four in groups of 512 (8200, 512 x 3, 88 with one, 83 with two; 12296, 512 x 4, 78 and 107).

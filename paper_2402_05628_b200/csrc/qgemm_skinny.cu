@@ -14,8 +14,8 @@
 // columns; for one token the 32 lanes of a warp are 32 neighbouring outputs, so loads and stores are coalesced without
 // staging.  The arithmetic is epilogue.cuh's, element by element.
 //
-// Measured (block passes, 7B-shaped decoder layer of 48 tokens, one byte per weight code): 1860 -> 84 us against the warp-MMA
-// kernel (3.2 TB/s of weights over the whole pass, all seven kernels included); one image through a ViT-S block 52 -> 40 us
+// Measured (block passes, 7B-shaped decoder layer of 48 tokens, one byte per weight code): 1860 -> 75 us against the warp-MMA
+// kernel (2.7 TB/s of weights over the whole pass, all seven kernels included); one image through a ViT-S block 52 -> 32 us
 // against 128-row tiles, of which so small a layer fills only a handful of SMs.
 //
 // Every wait on an mbarrier is bounded as in the other tensor-core kernels; all threads reach the two cluster barriers
