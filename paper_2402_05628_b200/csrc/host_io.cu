@@ -6,6 +6,7 @@
 // run one batch behind the inputs, which costs a batch's time on the link and the block's own time at the end.  The items of a
 // batch are independent, so a batch passes through the pipeline in pieces of whole items: piece c is computed while piece
 // c + 1 is copied in and piece c - 1 copied out, and the outputs run one piece behind.  See `pieces_of` for when.
+#include <algorithm>
 #include <mutex>
 
 #include "kernels.h"
@@ -16,26 +17,30 @@ namespace {
 constexpr int kMaxDevices = 64;
 constexpr int kSlots = 2;
 constexpr int kMaxPieces = 8;
-constexpr size_t kPieceBytes = size_t(4300) << 10;       // 4.4 MB: 100 us of the link, twice what queueing a piece takes the host
-constexpr size_t kGapBytes = size_t(700) << 10;          // what the link would move while a further piece holds it up (16 us; copies
+constexpr size_t kPieceBytes = size_t(2685) << 10;       // 2.75 MB: 60 us of the link, a little more than queueing a piece takes the host
+constexpr int64_t kPieceTokens = 2048;                   // (2765 with packed weights, whose expansion every piece repeats)
+constexpr size_t kGapBytes = size_t(585) << 10;          // what the link would move while a further piece holds it up (14 us; copies
                                                          // alone stand 10 us apart, with the waits on events 10 to 25)
 
-// Pieces per batch: of about kPieceBytes of input each, unless what they save (the link time of a batch: the outputs no longer run
-// a batch behind) is less than the gaps they add (one per piece and batch).  More pieces than that, and the small blocks' time
-// adds up to more than the link's.
-// Measured, us, whole -> pieces (ranges: two machines): 64 DeiT-B images of 19.4 MB, four pieces: one batch 935 -> 611..631, two
-// 1340 -> 1056..1154, four 2235 -> 2020..2250, five 2690 -> 2518..2800, eight 4051 -> 4414 (whole by the rule).  32 ViT-L images at
-// 577 tokens, 37.8 MB, eight: 1841 -> 1029, four 4237 -> 3530, five 5065 -> 4362, sixteen 14157 -> 13644 (whole).  16 of them, 18.9 MB,
-// four: 955 -> 612, five 2655 -> 2280 (with seven pieces 2894).  40 DeiT-B images of 150 tokens, packed 6-bit weights, 9.2 MB, two:
-// 499 -> 379, five 1416 -> 1198 (four pieces 1495).  7.4 MB, two: 402 -> 308, five 1172 -> 1010.  4.8 MB stay whole: in two pieces
-// four batches take 633 for 605.  Pieces for the first and the last batch only gain nothing beyond two batches: the
-// outputs then fall a batch behind in between.
-int pieces_of(size_t x_bytes, int batch, int n_batches) {
-  const size_t fit = (x_bytes + kPieceBytes / 2) / kPieceBytes;
-  int pieces = int(fit < size_t(kMaxPieces) ? fit : size_t(kMaxPieces));
-  if (pieces > batch) pieces = batch;
+// Pieces per batch: as many as have kPieceBytes of input and kPieceTokens tokens each (below, the host, or the blocks of the pieces
+// together, take longer than the link), unless what they save (the link time of a batch: the outputs no longer run a batch behind)
+// is less than the gaps they add (one per piece and batch).
+// Measured, us, whole -> pieces (ranges: different machines).  64 DeiT-B images of 19.4 MB, six pieces: one batch 935 -> 580, two
+// 1340 -> 1092..1106, four 2240 -> 2083, five 2690 -> 2614..2638, eight 4051 -> 4194 (whole by the rule); four pieces: four 2250, five
+// 2518..2833.  32 ViT-L images of 577 tokens, 37.8 MB, eight: 1841 -> 1029, four 4237 -> 3530, five 5065 -> 4362, sixteen 14157 -> 13644
+// (whole).  16 of them, 18.9 MB, four: 955 -> 612, five 2655 -> 2280 (seven pieces, 1300 tokens each: 2894).  28 x 371 tokens of
+// DeiT-B, 16 MB, five: two 1143 -> 922, five 2266 -> 2086.  64 x 133 with packed weights, 13.1 MB, three: 667 -> 467, five 1905 -> 1655
+// (four pieces 1846).  100 x 50, 7.7 MB, two: 412 -> 316, five 1214 -> 1064.  4 x 2048 LLaMA tokens, 67 MB, four: five 9036..9373 ->
+// 7841..7950, twenty 30340..32116 -> 31095..32195.  Batches of 4.8 MB stay whole: in two pieces four take 633 for 605.
+// Pieces for the first and the last batch only gain nothing beyond two batches: the outputs then fall a batch behind in between.
+int pieces_of(size_t x_bytes, const repq_block_desc& d, int n_batches) {
+  const bool packed = packed4(d.bits_w) || packed6(d.bits_w);
+  int64_t pieces = kMaxPieces;
+  pieces = std::min(pieces, int64_t(x_bytes / kPieceBytes));
+  pieces = std::min(pieces, int64_t(d.batch) * d.seq / (packed ? kPieceTokens * 27 / 20 : kPieceTokens));
+  pieces = std::min(pieces, int64_t(d.batch));
   if (pieces < 2) return 1;
-  return size_t(n_batches) * size_t(pieces) * kGapBytes <= x_bytes ? pieces : 1;
+  return size_t(n_batches) * size_t(pieces) * kGapBytes <= x_bytes ? int(pieces) : 1;
 }
 
 struct Pipeline {                 // per device, created on first use, kept for the life of the process
@@ -104,7 +109,7 @@ extern "C" repq_status repq_block_forward_host(const repq_block_desc* d, const r
   REPQ_CUDA(cudaEventRecord(P->start, main));
   REPQ_CUDA(cudaStreamWaitEvent(P->in, P->start, 0));
   REPQ_CUDA(cudaStreamWaitEvent(P->out, P->start, 0));
-  const int pieces = pieces_of(x_bytes, d->batch, n_batches);
+  const int pieces = pieces_of(x_bytes, *d, n_batches);
   const size_t x_item = x_bytes / size_t(d->batch), y_item = y_bytes / size_t(d->batch);
   repq_block_desc piece = *d;
   for (int i = 0; i < n_batches; ++i) {

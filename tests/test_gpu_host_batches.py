@@ -66,7 +66,7 @@ def test_sequences_of_any_length(batch):
         per_batch[n] = (B.repq_launch_count() - before) / n / per_block
         assert all(torch.equal(y, e) for y, e in zip(ys, (expect * 14)[:n]))
     # pieces by the bytes they save against the gaps they add, at four batches as at five
-    piece, gap = 4300 << 10, 700 << 10
-    most = min(8, (bytes_in + piece // 2) // piece, batch)
+    gap = 585 << 10
+    most = min(8, bytes_in // (2685 << 10), xs[0].shape[0] // 2048, batch)
     for n, pieces in per_batch.items():
         assert pieces == (most if most > 1 and n * most * gap <= bytes_in else 1)
