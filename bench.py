@@ -39,17 +39,16 @@ HEADLINE = "c4_llama7b"
 OTHER_WORKLOADS = ("c1_vit_s", "c2_deit_b", "c2_deit_b_w6a6", "c3_vit_l", "c4_llama7b_arch")
 INT8_OVER_BF16 = 2.0          # nominal dense int8 : bf16 tensor throughput on B200
 L2_BYTES = 126 << 20
-# DRAM traffic of one launch of a stage kernel, from one ncu capture of the same bench command (summaries under
-# profiles/).  A figure is reported only while the kernel's sources still hash to what was captured.
+# DRAM traffic of one launch of a stage kernel, from an ncu capture of the same block shape (the `block_llama7b_4x2048` case of
+# perf/cases.py).  A figure is reported only while the kernel's sources still hash to what was captured.
 NCU_TRAFFIC = {   # (workload, batch, stage): (DRAM bytes read + written per launch, kernel sources, their sha1 when captured)
-    ("c4_llama7b", 4, "attention"): (138199296, ["attention_tc.cu", "tc_ptx.cuh"], "47dd87935b26"),
-    ("c4_llama7b", 4, "qkv"): (166124032, ["qgemm_tc.cu", "tc_ptx.cuh", "epilogue.cuh"], "f76285585384"),
-    ("c4_llama7b", 4, "proj"): (201283840, ["qgemm_tc.cu", "tc_ptx.cuh", "epilogue.cuh"], "f76285585384"),
-    ("c4_llama7b", 4, "fc1"): (148836608, ["qgemm_tc.cu", "tc_ptx.cuh", "epilogue.cuh"], "f76285585384"),
-    ("c4_llama7b", 4, "fc2"): (517648896, ["qgemm_tc.cu", "tc_ptx.cuh", "epilogue.cuh"], "f76285585384"),
-    ("c4_llama7b", 4, "ln1"): (71826432, ["ln_quant.cu", "f32x2.cuh"], "1eacf83c9513"),
-    ("c4_llama7b", 4, "ln2"): (71635712, ["ln_quant.cu", "f32x2.cuh"], "1eacf83c9513"),
-    ("c2_deit_b", 64, "attention"): (29160192, ["attention_tc.cu", "tc_ptx.cuh"], "47dd87935b26"),
+    ("c4_llama7b", 4, "ln1"): (71432192, ["ln_quant.cu", "f32x2.cuh"], "30540a1f857f"),
+    ("c4_llama7b", 4, "qkv"): (166772992, ["qgemm_tc.cu", "tc_ptx.cuh", "epilogue.cuh"], "f5634ba14147"),
+    ("c4_llama7b", 4, "attention"): (135463936, ["attention_pipe.cu", "attention_common.cuh", "tc_ptx.cuh"], "f3f737b3cd0c"),
+    ("c4_llama7b", 4, "proj"): (195583232, ["qgemm_tc.cu", "tc_ptx.cuh", "epilogue.cuh"], "f5634ba14147"),
+    ("c4_llama7b", 4, "ln2"): (69735680, ["ln_quant.cu", "f32x2.cuh"], "30540a1f857f"),
+    ("c4_llama7b", 4, "fc1"): (149176576, ["qgemm_tc.cu", "tc_ptx.cuh", "epilogue.cuh"], "f5634ba14147"),
+    ("c4_llama7b", 4, "fc2"): (508679168, ["qgemm_tc.cu", "tc_ptx.cuh", "epilogue.cuh"], "f5634ba14147"),
 }
 
 

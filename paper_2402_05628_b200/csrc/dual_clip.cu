@@ -18,7 +18,7 @@
 // square root, divisions (ncu, 6304 x 384: float64 pipe 34 % busy, conversions to double 23 % of theirs, first stall the barrier
 // around the reduction and the update).  Hence the quotient by a reciprocal taken once per step, the round operation by adding
 // 1.5 * 2^52 (its integer, in the low word, also decides the clip, on the integer pipe), and several CTAs per SM, so that one
-// channel's chain runs under the others' passes.  6304 x 384: 4850 -> 320-360 us (more where more values are clipped),
+// channel's chain runs under the others' passes.  6304 x 384: 4850 -> 290-360 us (more where more values are clipped),
 // 16384 x 4096: 63 -> 4.6 ms; before, 48 CTAs re-read their slab from L2 in every step and divided.  Arithmetic is float64
 // throughout (the decisions of the two round operations steer the gradient).
 // No scratch memory, no atomics, no inter-CTA traffic.

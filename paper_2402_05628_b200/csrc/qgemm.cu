@@ -144,8 +144,8 @@ __global__ void __launch_bounds__(256) expand_weights_kernel(const uint8_t* __re
 // The byte form of packed weights in the caller's workspace, where it has the room (repq_qgemm_workspace_bytes asks for it): one
 // pass over the weights, after which every GEMM kernel takes them.  The GEMM that expands the tiles it copies (bound by its
 // converters' shared-memory traffic, once per row tile) remains for smaller workspaces.  Measured (packed against that form):
-// 3152 tokens through a DeiT-B block with 6-bit weights 125 -> 98 us (bytes: 86), a 7B-shaped decoder block of 48 tokens with
-// 4-bit weights 1860 -> 143 us (bytes: 78).
+// 3152 tokens through a DeiT-B block with 6-bit weights 125 -> 96 us (bytes: 84), a 7B-shaped decoder block of 48 tokens with
+// 4-bit weights 1860 -> 139 us (bytes: 75).
 struct ByteWeights { size_t offset = 0, total = 0; int64_t ld = 0; };
 bool byte_weights(const repq_gemm_desc& d, repq_gemm_desc* as_bytes, ByteWeights* B) {
   if (!(packed4(d.bits_w) || packed6(d.bits_w)) || d.batch_outer != 1 || d.batch_inner != 1) return false;

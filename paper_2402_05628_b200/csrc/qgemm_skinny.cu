@@ -1,5 +1,5 @@
 // Integer GEMM for few tokens (decoding, short prompts, single images): the weights are the M = 128 operand of the
-// tensor-core instruction and the tokens its N operand, so that a tile is 128 output channels x 16..256 tokens and no
+// tensor-core instruction and the tokens its N operand, so that a tile is 128 output channels x 16..128 tokens and no
 // tensor-core row is spent on padding of the token side.
 //
 // What bounds it: with few tokens a layer is one pass over its weights, i.e. the HBM (or, for weights that fit, L2) copy
