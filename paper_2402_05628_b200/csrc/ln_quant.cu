@@ -173,14 +173,39 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
       }
     }
   };
-  const int64_t first_rows = int64_t(blockIdx.x) * kRowsPerBlock + group * kRows;
-  // Factors that the kernel ahead in the stream may have written are read behind the wait, settled ones while that kernel
-  // finishes.  (Loads past L1: what that kernel wrote must not meet an older line.)
-  // The next kernel's start is allowed as soon as everything ahead has completed, so that its prologue runs beside the staging.
+  // Factors that the kernel ahead in the stream may have written are read behind the wait, together with the first rows; settled
+  // ones while that kernel finishes.  (Loads past L1: what that kernel wrote must not meet an older line.)  The next kernel's start
+  // is allowed as soon as everything ahead has completed, so that its prologue runs beside the staging.
+  // Pieces of 4 factors, all of a thread's in flight at once; a block starts at a piece of its own, since all blocks read the same
+  // 8 D bytes at the same moment and would queue for the same lines of L2.
+  // What reading behind the wait costs, back to back against a settled start: 0.3-1.3 us per launch up to 4096 elements (32768 x 4096
+  // 76.0 -> 76.4, 4239 x 4096 11.8 -> 12.9), 2-3 at 8192 (9950 rows 47.5 -> 50.4); in a block pass 0.2-1.3 (one ViT-S image 31.9 -> 32.1,
+  // 64 DeiT-B images 208.6 -> 209.9).  With factors one by one behind the first rows 1-3.
+  constexpr int kPieces = (TPR * kVPT * kChunk / 4 + kBlock - 1) / kBlock;
+  const int n4 = D / 4, rot = int(blockIdx.x * 32u % uint32_t(n4));
+  const bool vec = ((reinterpret_cast<uintptr_t>(gamma_t) | reinterpret_cast<uintptr_t>(beta_t)) & 15) == 0;
+  auto load4 = [&](const float* p) {
+    return vec ? __ldcg(reinterpret_cast<const float4*>(p)) : make_float4(__ldcg(p), __ldcg(p + 1), __ldcg(p + 2), __ldcg(p + 3));
+  };
+  auto piece = [&](int k) {
+    const int q = k * kBlock + int(threadIdx.x) + rot;
+    return q < n4 ? q : q - n4;
+  };
   if (!settled) {
     grid_dependency_wait();
     grid_dependency_trigger();
   }
+  float4 g4[kPieces], b4[kPieces];
+#pragma unroll
+  for (int k = 0; k < kPieces; ++k) {
+    g4[k] = b4[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (k * kBlock + int(threadIdx.x) < n4) {
+      g4[k] = load4(gamma_t + 4 * piece(k));
+      b4[k] = load4(beta_t + 4 * piece(k));
+    }
+  }
+  const int64_t first_rows = int64_t(blockIdx.x) * kRowsPerBlock + group * kRows;
+  if (!settled) fetch(first_rows);
 
   float* s_g = s_gb;
   float* s_b = s_gb + D;
@@ -192,30 +217,16 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
   // layout: the first halves (4 floats) of all chunks, then the second halves, so that the 16-byte reads of
   // neighbouring lanes are neighbours in shared memory (chunk by chunk they would sit 32 bytes apart: two-way
   // bank conflicts)
-  const int half_stride = D / 2;
-  // Several factors of a thread in flight at a time, and the first rows asked for behind the first of them, so that rows and
-  // factors arrive together.  (What reading behind the wait costs a block pass of 64 x 197 tokens x 768: 1.2 us of 209, with
-  // the rows first and the factors one by one 2.1; one image through a ViT-S block 0.5 of 32.)
-  constexpr int kInFlight = 8;
-  for (int base = 0; base < D; base += kInFlight * kBlock) {
-    float gi[kInFlight], bi[kInFlight];
 #pragma unroll
-    for (int k = 0; k < kInFlight; ++k) {
-      const int i = base + k * kBlock + threadIdx.x;
-      gi[k] = i < D ? __ldcg(gamma_t + i) : 0.f;
-      bi[k] = i < D ? __ldcg(beta_t + i) : 0.f;
-    }
-    if (!settled && base == 0) fetch(first_rows);
+  for (int k = 0; k < kPieces; ++k) {
+    if (k * kBlock + int(threadIdx.x) < n4) {
+      const int q = piece(k), at = (q & 1) * (D / 2) + (q >> 1) * 4;
+      const float gi[4] = {g4[k].x * inv_s, g4[k].y * inv_s, g4[k].z * inv_s, g4[k].w * inv_s};
+      const float bi[4] = {b4[k].x * inv_s, b4[k].y * inv_s, b4[k].z * inv_s, b4[k].w * inv_s};
+      *reinterpret_cast<float4*>(s_g + at) = make_float4(gi[0], gi[1], gi[2], gi[3]);
+      *reinterpret_cast<float4*>(s_b + at) = make_float4(bi[0], bi[1], bi[2], bi[3]);
 #pragma unroll
-    for (int k = 0; k < kInFlight; ++k) {
-      const int i = base + k * kBlock + threadIdx.x;
-      if (i >= D) break;
-      gi[k] *= inv_s;
-      bi[k] *= inv_s;
-      const int at = ((i >> 2) & 1) * half_stride + (i >> 3) * 4 + (i & 3);
-      s_g[at] = gi[k];
-      s_b[at] = bi[k];
-      wide = wide || !(fabsf(gi[k]) * root_d + fabsf(bi[k]) < 4.0e6f);
+      for (int e = 0; e < 4; ++e) wide = wide || !(fabsf(gi[e]) * root_d + fabsf(bi[e]) < 4.0e6f);
     }
   }
   const bool guard = __syncthreads_or(wide) != 0;
