@@ -57,6 +57,7 @@ __global__ void row_sum_kernel(const uint8_t* __restrict__ codes, int bits, int6
 // Each thread expands 8 source bytes (16 codes) into 16 destination bytes.
 __global__ void expand4_kernel(const uint8_t* __restrict__ src, int64_t rows, int64_t n, int64_t ld_src,
                                uint8_t* __restrict__ dst, int64_t ld_dst, int64_t n_pad) {
+  grid_dependency_wait();            // (no early trigger: a GEMM's persistent blocks would take this grid's later ones' places)
   const int64_t groups_per_row = n_pad / 16;
   const int64_t total = rows * groups_per_row;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < total;
@@ -119,7 +120,12 @@ __global__ void __launch_bounds__(256) expand_weights_kernel(const uint8_t* __re
   constexpr int kIn = 8 * kBits;                           // packed bytes of 64 codes
   const int64_t total = int64_t(rows) * groups, stride = int64_t(gridDim.x) * blockDim.x;
   grid_dependency_trigger();
-  if (!settled) grid_dependency_wait();
+  if (!settled) {
+    // what the kernel ahead may still write comes into L2 at least (where its writes end up as well)
+    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (i < total) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + (i / groups) * ld_src + (i % groups) * kIn));
+    grid_dependency_wait();
+  }
   bool waited = !settled;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < total; i += stride) {
     const int64_t r = i / groups;
@@ -287,8 +293,7 @@ repq_status launch_expand4(const uint8_t* src, int64_t rows, int64_t n, int64_t 
   const int64_t total = rows * (n_pad / 16);
   const int64_t blocks = (total + 255) / 256;
   const int grid = int(blocks < 8192 ? blocks : 8192);
-  expand4_kernel<<<grid, 256, 0, st>>>(src, rows, n, ld_src, dst, ld_dst, n_pad);
-  REPQ_CUDA(cudaGetLastError());
+  REPQ_CUDA(launch_chained(expand4_kernel, dim3(grid), dim3(256), 0, st, src, rows, n, ld_src, dst, ld_dst, n_pad));
   note_launch();
   return REPQ_OK;
 }
