@@ -42,13 +42,13 @@ L2_BYTES = 126 << 20
 # DRAM traffic of one launch of a stage kernel, from an ncu capture of the same block shape (the `block_llama7b_4x2048` case of
 # perf/cases.py).  A figure is reported only while the kernel's sources still hash to what was captured.
 NCU_TRAFFIC = {   # (workload, batch, stage): (DRAM bytes read + written per launch, kernel sources, their sha1 when captured)
-    ("c4_llama7b", 4, "ln1"): (71432192, ["ln_quant.cu", "f32x2.cuh"], "30540a1f857f"),
-    ("c4_llama7b", 4, "qkv"): (166772992, ["qgemm_tc.cu", "tc_ptx.cuh", "epilogue.cuh"], "f5634ba14147"),
-    ("c4_llama7b", 4, "attention"): (135463936, ["attention_pipe.cu", "attention_common.cuh", "tc_ptx.cuh"], "f3f737b3cd0c"),
-    ("c4_llama7b", 4, "proj"): (195583232, ["qgemm_tc.cu", "tc_ptx.cuh", "epilogue.cuh"], "f5634ba14147"),
-    ("c4_llama7b", 4, "ln2"): (69735680, ["ln_quant.cu", "f32x2.cuh"], "30540a1f857f"),
-    ("c4_llama7b", 4, "fc1"): (149176576, ["qgemm_tc.cu", "tc_ptx.cuh", "epilogue.cuh"], "f5634ba14147"),
-    ("c4_llama7b", 4, "fc2"): (508679168, ["qgemm_tc.cu", "tc_ptx.cuh", "epilogue.cuh"], "f5634ba14147"),
+    ("c4_llama7b", 4, "ln1"): (71619840, ["ln_quant.cu", "f32x2.cuh"], "b78cdda96848"),
+    ("c4_llama7b", 4, "qkv"): (166109696, ["qgemm_tc.cu", "tc_ptx.cuh", "epilogue.cuh"], "acc91ee82804"),
+    ("c4_llama7b", 4, "attention"): (137083904, ["attention_pipe.cu", "attention_common.cuh", "tc_ptx.cuh"], "f3f737b3cd0c"),
+    ("c4_llama7b", 4, "proj"): (198752512, ["qgemm_tc.cu", "tc_ptx.cuh", "epilogue.cuh"], "acc91ee82804"),
+    ("c4_llama7b", 4, "ln2"): (69334016, ["ln_quant.cu", "f32x2.cuh"], "b78cdda96848"),
+    ("c4_llama7b", 4, "fc1"): (148743424, ["qgemm_tc.cu", "tc_ptx.cuh", "epilogue.cuh"], "acc91ee82804"),
+    ("c4_llama7b", 4, "fc2"): (511341056, ["qgemm_tc.cu", "tc_ptx.cuh", "epilogue.cuh"], "acc91ee82804"),
 }
 
 

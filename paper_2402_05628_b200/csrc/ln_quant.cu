@@ -9,7 +9,7 @@
 // for the next one.
 //
 // What bounds it: HBM for float input and for rows of one warp (5.1-6.3 TB/s of 6.46); for longer bf16 rows the latencies of a
-// row's chain at the 16 warps per SM that the registers leave (ncu, 32768 x 4096: DRAM 45 % of its peak, issue slots 56 %, first
+// row's chain at the 16 warps per SM that the registers leave (ncu, 32768 x 4096: DRAM 43 % of its peak, issue slots 56 %, first
 // stall the factors' reads from shared memory and the shuffles, then waits of known length; 76-80 us against 51 at the copy rate).
 // Measured against three barriers per iteration: 65536 bf16 rows of 1536 53 -> 45 us, 32768 float rows of 2048 83 -> 48, 16384 of
 // 4096 76 -> 49; 32768 bf16 rows of 4096 gained nothing (80).

@@ -28,3 +28,22 @@ def test_ln_quant_row_forms(rows, D, bf16):
     one grid takes at a time."""
     rep = parity.check_ln_quant(rows, D, 4, bf16, seed=rows + D)
     assert rep["bad"] == 0, rep
+
+
+@pytest.mark.parametrize("D", [200, 4096])
+def test_factors_off_the_16_byte_boundary(D):
+    """gamma~ and beta~ are plain float arrays: the same codes and sums wherever they start."""
+    import torch
+    from paper_2402_05628_b200 import binding as B
+    dev, g = "cuda:0", torch.Generator(device="cuda:0").manual_seed(D)
+    x = torch.randn(301, D, device=dev, generator=g).to(torch.bfloat16)
+    gamma, beta = torch.randn(D + 4, device=dev, generator=g), torch.randn(D + 4, device=dev, generator=g)
+    got = []
+    for shift_g, shift_b in ((0, 0), (1, 0), (0, 2), (3, 1)):
+        gm, bt = torch.empty(D + 4, device=dev), torch.empty(D + 4, device=dev)
+        gm, bt = gm[shift_g:shift_g + D].copy_(gamma[:D]), bt[shift_b:shift_b + D].copy_(beta[:D])
+        codes, sums = torch.zeros(301, D, device=dev, dtype=torch.uint8), torch.zeros(301, device=dev, dtype=torch.int32)
+        B.repq_ln_quant(x, gm, bt, 1e-6, 0.3, 8, 4 | B.REPQ_BYTE_CODES, codes, sums)
+        torch.cuda.synchronize()
+        got.append((codes, sums))
+    assert all(torch.equal(c, got[0][0]) and torch.equal(s, got[0][1]) for c, s in got[1:])
