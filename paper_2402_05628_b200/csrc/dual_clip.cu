@@ -13,20 +13,28 @@
 // over the values clipped at either end, and the objective is s^2 sum d^2.
 //
 // Channels are independent, so the whole optimisation of a channel stays inside one CTA (1 to 16 warps), which holds the
-// channel's values in shared memory from the first pass to the last.  What bounds it is the float64 pipe (64 lanes per cycle
-// and SM: five operations per value and step) and, for few values per channel, the chain of one step: reduction, exp,
-// square root, divisions (ncu, 6304 x 384: float64 pipe 34 % busy, conversions to double 23 % of theirs, first stall the barrier
-// around the reduction and the update).  Hence the quotient by a reciprocal taken once per step, the round operation by adding
-// 1.5 * 2^52 (its integer, in the low word, also decides the clip, on the integer pipe), and several CTAs per SM, so that one
-// channel's chain runs under the others' passes.  6304 x 384: 4850 -> 290-360 us (more where more values are clipped),
-// 16384 x 4096: 63 -> 4.6 ms; before, 48 CTAs re-read their slab from L2 in every step and divided.  Arithmetic is float64
-// throughout (the decisions of the two round operations steer the gradient).
-// No scratch memory, no atomics, no inter-CTA traffic.
+// channel's values in shared memory from the first pass to the last.  Two forms:
+//  - passes over the values in every step.  What bounds them is the float64 pipe (64 lanes per cycle and SM: five operations per
+//    value and step) and, for few values per channel, the chain of one step: reduction, exp, square root, divisions (ncu, 6304 x
+//    384: float64 pipe 34 % busy, conversions to double 23 % of theirs, first stall the barrier around the reduction and the
+//    update).  Hence the quotient by a reciprocal taken once per step, the round operation by adding 1.5 * 2^52 (its integer,
+//    in the low word, also decides the clip, on the integer pipe), and several CTAs per SM, so that one channel's chain runs
+//    under the others' passes.
+//  - values sorted once, a step's sums from prefix sums at the edges between the 16 codes of a 4-bit quantizer.  What bounds it is the
+//    chain of a step alone (1.3 us: 16 cycles per float64 operation, 90 to 220 for a square root, a division, the sigmoid), one warp per
+//    channel without a barrier.  100 steps: 6304 x 384 321 -> 164 us, 12608 x 192 369 -> 200, 591 x 4096 436 -> 254, 500 x 384
+//    139 -> 133; the learned bounds are the same floats, the objective within 1e-9 (float64 in both).  A full merge sort took 85 us of
+//    6304 x 384 against 25 for buckets and ranks.
+// Arithmetic is float64 throughout (the decisions of the two round operations steer the gradient).
+// No scratch memory, no inter-CTA traffic, no atomics outside the counting of the sort (whose result does not depend on their order).
 // Channels of more values than shared memory holds take the kernel that re-reads them: a CTA owns 8 neighbouring channels
 // (one 32-byte sector per token row) and 32 token lanes, every step is one pass over the CTA's slab.
 #include <cuda_bf16.h>
+#include <math_constants.h>
 
+#include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "common.h"
 
@@ -44,6 +52,16 @@ struct ClipParams {
 };
 
 constexpr int kMaxResident = 50 * 1024;        // values of a channel that fit the shared memory of one CTA
+
+
+// Sorted form: most values of a channel (its 10 bytes per value fill shared memory), values of a bucket above which the channel
+// counts as crowded (ranks cost a bucket's square), buckets of n values, shared memory.
+constexpr int kMaxSorted = 22 * 1024, kCrowd = 48;
+__host__ __device__ constexpr int sorted_buckets(int n, int shift) { return (n >> shift) + 8; }
+constexpr size_t sorted_bytes(int64_t n, int shift) {
+  const int64_t n8 = (n + 7) / 8 * 8;
+  return size_t(2 * n8 + 4 + sorted_buckets(int(n), shift) + 1) * 4;
+}
 
 __device__ __forceinline__ double sigmoid(double a) { return 1.0 / (1.0 + exp(-a)); }
 
@@ -348,6 +366,325 @@ repq_status launch_resident(const ClipParams& P, cudaStream_t st) {
   return REPQ_OK;
 }
 
+// ---- sorted form
+
+__device__ __forceinline__ void order(float& a, float& b) {
+  const float t = fminf(a, b);
+  b = fmaxf(a, b);
+  a = t;
+}
+
+// Ascending sort of the n values (n8 with the infinities that fill the last group of eight).  Every merge of two sorted runs starts by
+// comparing mirrored positions, so that each comparison leaves the smaller value at the lower index and positions past n8 act
+// as infinities that never move: any n is sorted in place.  A thread takes eight values through up to three steps at a time.
+template <int T>
+__device__ __forceinline__ void sort_channel(float* val, int n8, int tid) {
+  auto sync = [] { if (T > 32) __syncthreads(); else __syncwarp(); };
+  auto load8 = [&](int i, float (&v)[8]) {
+    const float4 a = *reinterpret_cast<const float4*>(val + i), b = *reinterpret_cast<const float4*>(val + i + 4);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+  };
+  auto store8 = [&](int i, const float (&v)[8]) {
+    *reinterpret_cast<float4*>(val + i) = make_float4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<float4*>(val + i + 4) = make_float4(v[4], v[5], v[6], v[7]);
+  };
+  auto steps = [](float (&v)[8], int first) {            // distances 4, 2, 1 from `first` on
+    if (first >= 4) { order(v[0], v[4]); order(v[1], v[5]); order(v[2], v[6]); order(v[3], v[7]); }
+    if (first >= 2) { order(v[0], v[2]); order(v[1], v[3]); order(v[4], v[6]); order(v[5], v[7]); }
+    order(v[0], v[1]); order(v[2], v[3]); order(v[4], v[5]); order(v[6], v[7]);
+  };
+  const int groups = n8 >> 3;
+  for (int t = tid; t < groups; t += T) {                // runs of eight
+    float v[8];
+    load8(8 * t, v);
+    order(v[0], v[1]); order(v[2], v[3]); order(v[4], v[5]); order(v[6], v[7]);
+    order(v[0], v[3]); order(v[1], v[2]); order(v[4], v[7]); order(v[5], v[6]);
+    order(v[0], v[1]); order(v[2], v[3]); order(v[4], v[5]); order(v[6], v[7]);
+    order(v[0], v[7]); order(v[1], v[6]); order(v[2], v[5]); order(v[3], v[4]);
+    steps(v, 2);
+    store8(8 * t, v);
+  }
+  for (int k = 4; (8 << (k - 4)) < n8; ++k) {            // runs of 2^k out of runs of 2^(k-1)
+    sync();
+    {
+      // mirrored step and distances 2^(k-2), 2^(k-3): the upper four of a thread's values come from the mirrored offset
+      const int lh = k - 3, h = 1 << lh;
+      for (int t = tid; t < ((n8 + (1 << k) - 1) >> k) << lh; t += T) {
+        const int base = (t >> lh) << k, o = t & (h - 1);
+        float v[8];
+        int i[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          i[j] = base + j * h + (j < 4 ? o : h - 1 - o);
+          v[j] = i[j] < n8 ? val[i[j]] : INFINITY;
+        }
+        order(v[0], v[7]); order(v[1], v[6]); order(v[2], v[5]); order(v[3], v[4]);
+        steps(v, 2);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (i[j] < n8) val[i[j]] = v[j];
+      }
+    }
+    int lt = k - 4;                                      // log2 of the next distance
+    for (; lt >= 3; lt -= 3) {
+      sync();
+      const int lh = lt - 2, h = 1 << lh;
+      for (int t = tid; t < ((n8 + (8 << lh) - 1) >> (lh + 3)) << lh; t += T) {
+        const int base = ((t >> lh) << (lh + 3)) + (t & (h - 1));
+        float v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = base + j * h < n8 ? val[base + j * h] : INFINITY;
+        steps(v, 4);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (base + j * h < n8) val[base + j * h] = v[j];
+      }
+    }
+    if (lt >= 0) {
+      sync();
+      for (int t = tid; t < groups; t += T) {
+        float v[8];
+        load8(8 * t, v);
+        steps(v, 1 << lt);
+        store8(8 * t, v);
+      }
+    }
+  }
+  sync();
+}
+
+// Bucket of a value: equal parts of the channel's range, monotone in x (every operation rounds once).
+struct Buckets {
+  float low, scale;
+  int last;
+  __device__ __forceinline__ int of(float x) const { return max(0, min(last, __float2int_rz(__fmul_rn(__fsub_rn(x, low), scale)))); }
+};
+
+// One channel per CTA of kWarps warps.  All of them load the channel's values, sort them (by bucket, then by rank inside
+// the bucket; a channel whose values crowd in few buckets is sorted by merging) and form prefix sums of every fourth; the first
+// warp then runs the optimisation alone, since a step no longer passes over the values: those of code q lie between two edges of
+// the sorted order, and with y = x - pivot, kappa_q = q - z - pivot/s,
+//     sum over a code of (q - z - x/s)^2 = n kappa^2 - 2 (kappa/s) sum y + (1/s^2) sum y^2
+// from counts and prefix sums at the edges (the pivot, the channel's median, keeps |kappa| below twice the number of codes and small
+// where most values are: the terms cancel to no more than about Q^2 2^-53).  An edge is the smallest float whose rounded quotient reaches the next
+// code, so every value has the code that its own quotient rounds to.
+template <int kWarps>
+__global__ void __launch_bounds__(32 * kWarps, kWarps == 16 ? 2 : 28 / kWarps) dual_clip_sorted_kernel(ClipParams P, int bucket_shift) {
+  constexpr int T = 32 * kWarps;
+  extern __shared__ __align__(16) float smem[];
+  __shared__ float ext[2][kWarps];
+  __shared__ int part_n[kWarps];
+  __shared__ double2 part[kWarps];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int d = blockIdx.x, n = int(P.n), n8 = (n + 7) & ~7;
+  // values (raw, then sorted), values by bucket (later the prefix sums, 16 bytes per four values), starts of the buckets
+  float* val = smem;
+  float* by_bucket = smem + n8;
+  double2* pre = reinterpret_cast<double2*>(by_bucket);
+  int* start = reinterpret_cast<int*>(by_bucket + n8 + 4);
+  const int nb = sorted_buckets(n, bucket_shift), blocks = (n >> 2) + 1;
+  const float* col = P.x + d;
+  auto sync = [] { if (kWarps > 1) __syncthreads(); else __syncwarp(); };
+
+  float mxf = -INFINITY, mnf = INFINITY;
+  bool odd_value = false;                                // an infinity or a NaN: no order, and no finite sums either
+#pragma unroll 8
+  for (int t = tid; t < n; t += T) {
+    const float v = __ldg(col + int64_t(t) * P.ldx);
+    val[t] = v;
+    mxf = fmaxf(mxf, v);
+    mnf = fminf(mnf, v);
+    odd_value = odd_value || !(fabsf(v) < INFINITY);
+  }
+  if (tid < n8 - n) val[n + tid] = INFINITY;
+  for (int i = tid; i <= nb; i += T) start[i] = 0;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    mxf = fmaxf(mxf, __shfl_xor_sync(0xffffffffu, mxf, o));
+    mnf = fminf(mnf, __shfl_xor_sync(0xffffffffu, mnf, o));
+  }
+  if (lane == 0) { ext[0][warp] = mxf; ext[1][warp] = mnf; }
+  const bool finite = __syncthreads_or(odd_value) == 0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) { mxf = fmaxf(mxf, ext[0][w]); mnf = fminf(mnf, ext[1][w]); }
+  Buckets B{mnf, float(nb) / (mxf - mnf), nb - 1};
+  if (!(B.scale < INFINITY)) B.scale = 0.f;              // one value, or a range below the normal numbers: a single bucket
+
+  double pivot = 0.0;
+  if (finite) {
+    for (int t = tid; t < n; t += T) atomicAdd(&start[B.of(val[t])], 1);
+    sync();
+    // inclusive scan of the counts, a run of buckets per thread
+    bool crowded = false;
+    {
+      const int run = (nb + T - 1) / T, first = min(nb, tid * run), last = min(nb, first + run);
+      int own = 0;
+      for (int b = first; b < last; ++b) { own += start[b]; crowded = crowded || start[b] > kCrowd; }
+      int sum = own;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, sum, o);
+        if (lane >= o) sum += t;
+      }
+      if (lane == 31) part_n[warp] = sum;
+      crowded = __syncthreads_or(crowded) != 0;
+      int at = sum - own;
+      for (int w = 0; w < warp; ++w) at += part_n[w];
+      for (int b = first; b < last; ++b) start[b] = at += start[b];
+      if (tid == 0) start[nb] = n;
+    }
+    sync();
+    for (int t = tid; t < n; t += T) {                   // leaves every bucket's start behind
+      const float v = val[t];
+      const int at = atomicSub(&start[B.of(v)], 1) - 1;
+      by_bucket[at] = v;
+    }
+    sync();
+    if (crowded) {
+      sort_channel<T>(val, n8, tid);
+    } else {
+      for (int t = tid; t < n; t += T) {
+        const float v = by_bucket[t];
+        const int b = B.of(v), first = start[b], last = start[b + 1];
+        int rank = first;
+        for (int i = first; i < last; ++i) {
+          const float w = by_bucket[i];
+          rank += (w < v || (w == v && i < t)) ? 1 : 0;
+        }
+        val[rank] = v;
+      }
+      sync();
+    }
+    pivot = double(val[n >> 1]);
+    // prefix sums: a run of blocks of four values per thread, summed twice (total, then block by block behind the threads before)
+    const int run = (blocks + T - 1) / T, first = min(blocks, tid * run), last = min(blocks, first + run);
+    auto add_block = [&](int b, double2& t) {
+      for (int i = 4 * b; i < min(n, 4 * b + 4); ++i) {
+        const double y = double(val[i]) - pivot;
+        t.x += y;
+        t.y = fma(y, y, t.y);
+      }
+    };
+    double2 own = make_double2(0.0, 0.0);
+    for (int b = first; b < last; ++b) add_block(b, own);
+    double2 sum = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double sx = __shfl_up_sync(0xffffffffu, sum.x, o), sy = __shfl_up_sync(0xffffffffu, sum.y, o);
+      if (lane >= o) { sum.x += sx; sum.y += sy; }
+    }
+    if (lane == 31) part[warp] = sum;
+    sync();
+    double2 at = make_double2(__shfl_up_sync(0xffffffffu, sum.x, 1), __shfl_up_sync(0xffffffffu, sum.y, 1));
+    if (lane == 0) at = make_double2(0.0, 0.0);
+    for (int w = 0; w < warp; ++w) { at.x += part[w].x; at.y += part[w].y; }
+    for (int b = first; b < last; ++b) {
+      pre[b] = at;
+      add_block(b, at);
+    }
+    sync();
+  }
+  if (warp != 0) return;
+
+  // ---- the optimisation: even lanes carry the upper factor, odd lanes the lower one (every pair of lanes holds the same numbers)
+  const int top_lane = int(P.Q) + 1;                     // a lane per edge: below code 0, between the codes, above code Q
+  struct Below { double c, y, yy; };                     // number of the values below an edge, sums of y and y^2
+  auto sums_below = [&](int c) {
+    const double2 t = pre[c >> 2];
+    const float4 q = *reinterpret_cast<const float4*>(val + min(c & ~3, n8 - 4));
+    const int r = c & 3;
+    const double y0 = r > 0 ? double(q.x) - pivot : 0.0, y1 = r > 1 ? double(q.y) - pivot : 0.0, y2 = r > 2 ? double(q.z) - pivot : 0.0;
+    return Below{double(c), t.x + ((y0 + y1) + y2), t.y + (fma(y0, y0, y1 * y1) + y2 * y2)};
+  };
+  Below all{0.0, 0.0, 0.0};
+  if (finite) all = sums_below(n);
+
+  const bool upper = (lane & 1) == 0;
+  const double mine = upper ? double(mxf) : double(mnf), inv_q = 1.0 / P.Q;
+  double bound = 0.0, other = 0.0, a = P.alpha0, m = 0.0, v = 0.0, b1t = 1.0, b2t = 1.0, c1s = 0.0, c2s = 0.0, loss_first = 0.0;
+  for (int it = 0; it <= P.iters; ++it) {
+    // the channel's quantizer for this step (Eq. 6 on the bounds of Eqs. 18-19)
+    const double sg = sigmoid(a);
+    bound = mine * sg;
+    other = __shfl_xor_sync(0xffffffffu, bound, 1);
+    if (it == P.iters && P.loss == nullptr) break;       // the pass after the last update serves the objective alone
+    if ((it & 31) == 0) {                                // Adam's bias corrections of the next 32 steps, one per lane
+      double p1 = 1.0, p2 = 1.0;
+#pragma unroll 1
+      for (int i = 0; i < 32; ++i) {
+        b1t *= P.beta1;
+        b2t *= P.beta2;
+        if (i == lane) { p1 = b1t; p2 = b2t; }
+      }
+      c1s = P.lr / (1.0 - p1);
+      c2s = 1.0 / (1.0 - p2);
+    }
+    const double up = upper ? bound : other, low = upper ? other : bound;
+    const double s = (up - low) * inv_q, inv = 1.0 / s, zc = -low * inv, z = rint(zc), lo = -z;
+    // a channel whose bounds coincide (a constant channel, or extremes of 0) has no quantizer to learn: its sums stay
+    // 0, its factors keep their starting value and the contracted extremes are returned as they are
+    const bool live = s > 0.0;
+    double in2 = 0.0, sum_low = 0.0, sum_high = 0.0, out2 = 0.0;
+    if (live && finite) {
+      const double shift_p = pivot * inv, k_lo = lo - shift_p, k_hi = (P.Q - z) - shift_p;
+      const double k = lo + double(lane);                // first code at or above the lane's edge
+      float edge = float((k - 0.5) * s);
+      const int bucket = B.of(edge);                     // (no value of a later bucket is below the next float either)
+      int first = start[bucket], last = start[bucket + 1];
+      if (rint(double(edge) * inv) < k) edge = nextafterf(edge, INFINITY);
+      while (first < last) {
+        const int mid = (first + last) >> 1;
+        if (val[mid] < edge) first = mid + 1; else last = mid;
+      }
+      const Below t = sums_below(first);
+      // the code between the lane's edge and the one before; its squares without those of y, which add up over the codes
+      const double kappa = k_lo + double(lane - 1), inv2 = inv * inv;
+      const double dc = t.c - __shfl_up_sync(0xffffffffu, t.c, 1), dy = t.y - __shfl_up_sync(0xffffffffu, t.y, 1);
+      if (lane > 0 && lane <= top_lane) in2 = kappa * (kappa * dc - 2.0 * inv * dy);
+      // what is clipped, beyond the first and the last edge
+      const bool top = lane == top_lane;
+      const double c = top ? all.c - t.c : t.c, y = top ? all.y - t.y : t.y, yy = top ? all.yy - t.yy : t.yy, end = top ? k_hi : k_lo;
+      const double linear = end * c - inv * y;
+      if (top) in2 = fma(inv2, t.yy, in2);
+      if (lane == 0) in2 = -inv2 * t.yy;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) in2 += __shfl_xor_sync(0xffffffffu, in2, o);
+      sum_low = __shfl_sync(0xffffffffu, linear, 0);
+      sum_high = __shfl_sync(0xffffffffu, linear, top_lane);
+      if (it == 0 || it == P.iters) {
+        const double square = fma(end, linear - inv * y, inv2 * yy);
+        out2 = __shfl_sync(0xffffffffu, square, 0) + __shfl_sync(0xffffffffu, square, top_lane);
+      }
+    } else if (live) {
+      in2 = sum_low = sum_high = out2 = CUDART_NAN;
+    }
+    const double loss = live ? s * s * (in2 + out2) : 0.0;
+    if (it == 0) loss_first = loss;
+    if (it == P.iters) {
+      if (lane == 0) { P.loss[d] = loss_first; P.loss[P.D + d] = loss; }
+    } else {
+      const double dL_ds = live ? 2.0 * s * (in2 + (zc - z) * sum_low + (P.Q - z + zc) * sum_high) : 0.0;
+      const double dL_dl = live ? 2.0 * s * (sum_low + sum_high) : 0.0;
+      const double g = (upper ? dL_ds * inv_q : dL_dl - dL_ds * inv_q) * (mine * sg * (1.0 - sg));
+      m = P.beta1 * m + (1.0 - P.beta1) * g;
+      v = P.beta2 * v + (1.0 - P.beta2) * g * g;
+      const double c1 = __shfl_sync(0xffffffffu, c1s, it & 31), c2 = __shfl_sync(0xffffffffu, c2s, it & 31);
+      a -= c1 * m / (sqrt(c2 * v) + P.eps);
+    }
+  }
+  if (lane == 0) {
+    P.x_up[d] = float(bound);
+    P.x_low[d] = float(other);
+  }
+}
+
+template <int kWarps>
+repq_status launch_sorted(const ClipParams& P, int shift, cudaStream_t st) {
+  REPQ_TRY((allow_smem<dual_clip_sorted_kernel<kWarps>>(int(sorted_bytes(kMaxSorted, 1)))));
+  dual_clip_sorted_kernel<kWarps><<<P.D, 32 * kWarps, sorted_bytes(P.n, shift), st>>>(P, shift);
+  REPQ_CUDA(cudaGetLastError());
+  return REPQ_OK;
+}
 // Full-precision normalisation of the calibration batch (Eq. 9; mean-free variant for RMS): the activations the
 // clipping factors are learned on.  One CTA per row at a time, mean and centred variance in float32 with a
 // float64 block reduction, float32 output.  Calibration-time only: the inference path never forms X'.
@@ -431,17 +768,29 @@ extern "C" repq_status repq_dual_clip(const float* x, int64_t n, int D, int64_t 
   P.x_low = x_low; P.x_up = x_up; P.loss = loss;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (n <= kMaxResident) {
+    const int sms = sm_count();
+    const int share = (D + sms - 1) / sms;                                  // channels of an SM
+    // channels that an SM holds at a time, at so many bytes each, and its turns
+    auto held = [&](size_t bytes) { return std::max(1, int(228 * 1024 / int64_t(bytes + 1536))); };
+    auto turns = [&](int shift) { return (share + held(sorted_bytes(n, shift)) - 1) / held(sorted_bytes(n, shift)); };
+    // Sorted form: 16 codes (a lane per edge; 64 and 256 codes were slower than passes over the values, 1182 x 2048 430 against 389
+    // and 6304 x 384 1360 against 346), enough steps to pay for the sort (500 x 384, 16 steps: 31 against 28) and no long queue of
+    // channels behind one another (16384 x 4096, 28 turns: 4600 against 4566; 20000 x 1024, 7 turns: 1335 against 1662).
+    const bool sorted = bits == 4 && iters >= 32 && n <= kMaxSorted && turns(3) <= 16;
+    int shift = 3;                                          // as many buckets as do not cost a further turn
+    while (shift > 1 && turns(shift - 1) <= turns(3)) --shift;
     // warps per channel: about 28 warps on every SM over all channels, and as many where shared memory limits the
     // channels an SM holds at a time
-    const int sms = sm_count();
-    const int held = int(int64_t(kMaxResident) * 4 / (n * 4 + 1024));       // channels an SM can hold
-    const int want_d = 28 * sms / D, want_n = 24 / (held > 0 ? held : 1);
-    const int want = want_d > want_n ? want_d : want_n;
-    if (want >= 16) REPQ_TRY(launch_resident<16>(P, st));
-    else if (want >= 8) REPQ_TRY(launch_resident<8>(P, st));
-    else if (want >= 4) REPQ_TRY(launch_resident<4>(P, st));
-    else if (want >= 2) REPQ_TRY(launch_resident<2>(P, st));
-    else REPQ_TRY(launch_resident<1>(P, st));
+    const int want = std::max(28 * sms / D, 24 / held(sorted ? sorted_bytes(n, shift) : size_t(n) * 4));
+    auto launch = [&](auto warps) {
+      constexpr int kWarps = decltype(warps)::value;
+      return sorted ? launch_sorted<kWarps>(P, shift, st) : launch_resident<kWarps>(P, st);
+    };
+    if (want >= 16) REPQ_TRY(launch(std::integral_constant<int, 16>()));
+    else if (want >= 8) REPQ_TRY(launch(std::integral_constant<int, 8>()));
+    else if (want >= 4) REPQ_TRY(launch(std::integral_constant<int, 4>()));
+    else if (want >= 2) REPQ_TRY(launch(std::integral_constant<int, 2>()));
+    else REPQ_TRY(launch(std::integral_constant<int, 1>()));
   } else {
     const int grid = (D + kCh - 1) / kCh;
     dual_clip_kernel<<<grid, kThreads, 0, st>>>(P);
