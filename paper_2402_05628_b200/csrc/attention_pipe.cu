@@ -1,7 +1,7 @@
 // Fused attention on integer codes, persistent form (quantizers of at most 7 bits): scores (Eq. 3 with quantized Q and K),
 // Softmax, log-sqrt2 codes (Eq. 15) and P.V with the reparameterized log2 de-quantization (Eqs. 16-17) in one kernel.
 // Scores and codes never leave the SM.  The code of a score depends on the row's final Softmax sum, so the keys are walked
-// twice, a visit being 64 keys (heads of up to 64 channels) or 128 keys (wider heads):
+// twice, a visit being 64 keys (heads of up to 64 channels and more tiles than SMs) or 128 keys (wider heads, few tiles):
 //   pass 1   S = Q K^T per visit (tcgen05.mma on 8-bit operands into one of two slots of tensor memory), running row
 //            maximum m and sum Z = sum 2^(c (S - m))
 //   pass 2   S again, t = 2 (log2 Z + log2 s) - 2 c (S - m), code p = clip(round(t), 0, 2^b - 1), operand values
@@ -396,7 +396,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     // ---- V tile of a visit.  8-bit floats: a thread has one key and 16 channels, z_v - v in sign and magnitude (byte * 2^-9).
     // bf16: a thread keeps its group of 8 channels and moves down the keys, 32 per step.
     using VRaw = typename std::conditional<kLut, uint2, uint4>::type;
-    constexpr int kVItems = kLut ? kKeys / 32 : 1, kVChan = kLut ? 8 : 16, kVGroups = 64 * NB / kVChan;
+    constexpr int kVItems = kLut ? kKeys / 32 : 1, kVChan = kLut ? 8 : 16, kVGroups = (kLut ? 64 * NB : 64) / kVChan;
     const int v_g = tid % kVGroups, v_key0 = tid / kVGroups;
     const bool v_live = v_g * kVChan < P.dh;
     const uint32_t v_off = kLut ? uint32_t(v_g >> 3) * Shared::kVBlockBytes + tile_offset(v_key0, v_g & 7) : tile_offset(v_key0, v_g);
@@ -713,13 +713,21 @@ repq_status launch_kernel(const AttnParams& P, int64_t pairs, cudaStream_t st) {
 
 template <bool kF8>
 repq_status launch_form(const AttnParams& P, int64_t pairs, bool small_v, cudaStream_t st) {
-  if (P.dh <= 64) {
+  // Heads of up to 64 channels: two CTAs per SM with visits of 64 keys, except where every tile has an SM to itself; then the
+  // tile's chain of visits is all there is, and half as many visits of 128 keys (16 worker warps) shorten it.  A pass of a
+  // W4A4 block: one image of 577 tokens and 16 heads 62.8 -> 53.9 us, 8 of 197 and 6 heads 46.9 -> 43.7, one 34.6 -> 33.6 (W6A6,
+  // 2 of 197 and 12 heads 49.2 -> 45.7).  Up to 64 keys there is a single visit either way (100 keys 30.7 -> 30.3, 64 keys 28.0
+  // against 29.2).
+  const int64_t tiles = int64_t((P.Lq + kRows - 1) / kRows) * pairs;
+  const bool f8_pv = P.dh <= 64 && P.qmax_p <= 15 && small_v && P.log2_s >= 0.f;
+  if (P.dh <= 64 && (P.Lk <= 64 || tiles > sm_count())) {
     // 4-bit codes of 4-bit values: P.V in 8-bit floats (V rows by 16-byte loads; s >= 1 keeps t >= 0)
     if (P.qmax_p <= 15)
-      return small_v && P.log2_s >= 0.f ? launch_kernel<1, 0, kF8>(P, pairs, st) : launch_kernel<1, 4, kF8>(P, pairs, st);
+      return f8_pv ? launch_kernel<1, 0, kF8>(P, pairs, st) : launch_kernel<1, 4, kF8>(P, pairs, st);
     if (P.qmax_p <= 63) return launch_kernel<1, 6, kF8>(P, pairs, st);
     return launch_kernel<1, 8, kF8>(P, pairs, st);
   }
+  if (f8_pv) return launch_kernel<2, 0, kF8>(P, pairs, st);
   if (P.qmax_p <= 15) return launch_kernel<2, 4, kF8>(P, pairs, st);
   if (P.qmax_p <= 63) return launch_kernel<2, 6, kF8>(P, pairs, st);
   return launch_kernel<2, 8, kF8>(P, pairs, st);
