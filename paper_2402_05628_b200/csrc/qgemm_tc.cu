@@ -13,6 +13,10 @@
 //                the main loop of tile i + 1
 //   warps 2..17  epilogue: warp w reads TMEM lanes 32 (w mod 4) .. +31 (one output row per thread) and a
 //                64-column slice of the accumulator columns
+//   warp 18      the column and row terms of the epilogue (zero-point corrections, scales, biases, output quantizers, row sums),
+//                one tile ahead, in one of two shared-memory buffers.  (The register file is dealt out per four warps, so this
+//                warp costs the others nothing.)  12608 x 2304 x 768 to codes 29.6 -> 25.6 us, 18464 x 4096 x 1024 with GELU 89.4 ->
+//                79.2, 3152 x 3072 x 768 17.3 -> 16.0 against every epilogue warp preparing its own 64 columns
 //   packed weights (4-bit, two codes per byte; 6-bit, four codes in three bytes): 12 epilogue warps (tiles of at most
 //                192 columns) and 4 converter warps.  The weight tile arrives packed and the converters expand it into
 //                the 128-byte-swizzled byte tile the MMA descriptor expects (there is no 4- or 6-bit integer MMA); one
@@ -22,9 +26,8 @@
 // byte codes, so that pass does not run there).
 //
 // For short K the epilogue, not the tensor pipe, sets the pace (K = 768: 3072 tensor-pipe cycles per 128 x 256 tile
-// against 32768 outputs), so it is written for few instructions per output and few waits per tile: every epilogue warp
-// stages the per-column terms of its own 64 columns in its own shared-memory buffer (no barrier between warps) from
-// plain loads issued one tile ahead and reads them as vectors, the output quantizer is folded into them where nothing
+// against 32768 outputs), so it is written for few instructions per output and few waits per tile: the per-column terms are
+// prepared by a warp of their own and read as vectors, the output quantizer is folded into them where nothing
 // sits between the GEMM and the re-quantization, rounding uses the float adder (add 1.5 * 2^23), byte codes are clipped
 // by the pack instruction instead of comparisons, and a bf16 residual comes in either by row-per-lane loads requested
 // before the accumulator is waited for or, for short K, by bulk tensor copies (one 32 x 64 box per epilogue warp, one
@@ -47,7 +50,8 @@ constexpr int BM = 128, BK = 128;                   // BK in bytes (= codes); BN
 constexpr int kMaxBN = 256;
 constexpr int kChunk = 16;                           // accumulator columns per tcgen05.ld / per store
 constexpr int kEpiWarps = 16;
-constexpr int kThreads = 32 * (2 + kEpiWarps);
+constexpr int kTermsWarp = 2 + kEpiWarps;            // prepares the tiles' column and row terms
+constexpr int kThreads = 32 * (3 + kEpiWarps);
 constexpr int kTmemCols = 512;
 constexpr int kAccStride = 256;                      // TMEM columns between the two accumulator buffers
 constexpr int kSliceCols = 64;                       // accumulator columns per epilogue warp
@@ -61,11 +65,28 @@ constexpr uint32_t kMagicBits = 0x4B400000u;         // 1.5 * 2^23
 
 __device__ int32_t g_status_word = 0;
 
-struct alignas(16) ColTerms {                          // per output column of a warp's slice, staged once per tile
-  int32_t nzw[kSliceCols];  // -z_w[j]
-  int32_t kw[kSliceCols];   // -z_a * wsum[j]
-  float sc[kSliceCols];     // alpha s_a s_w[j]   (times 1/s_o in direct re-quantization mode)
-  float bi[kSliceCols];     // bias[j]            (times 1/s_o in direct re-quantization mode)
+// Output quantizer of one 16-column chunk (Eq. 4 with the chunk's column group).
+struct alignas(16) ChunkQuant {
+  float mult;
+  float unit, z_unit;  // byte codes of b bits: 2^(8 - b) 2^-149, and (z_o - magic) times it
+  int shift;           //   8 - b
+  uint32_t mask;       //   2^b - 1 in every byte
+  float lo, hi;
+  uint32_t pack_k;     // 4-bit: sum_e (magic_bits - z_o) << 4e
+  int zo;
+};
+
+// What the epilogue needs beside the accumulators of a tile, prepared one tile ahead by a warp of its own (by every epilogue warp
+// for its own 64 columns the same work took 2000-2200 of 7300 cycles per tile at K = 768).
+struct alignas(16) TileTerms {
+  int32_t nzw[kMaxBN];  // -z_w[j]
+  int32_t kw[kMaxBN];   // -z_a * wsum[j]
+  float sc[kMaxBN];     // alpha s_a s_w[j]   (times 1/s_o in direct re-quantization mode)
+  float bi[kMaxBN];     // bias[j]            (times 1/s_o in direct re-quantization mode)
+  int32_t asum[BM];     // row sum - K z_a
+  int32_t pos[BM];      // rotary embedding: the row's position
+  ChunkQuant quant[kMaxBN / kChunk];
+  int32_t m0, n0;       // first row (of this CTA) and column
 };
 
 constexpr uint32_t kResBytes = 32 * 128;            // bf16 residual of one warp and tile: 32 rows x 64 columns
@@ -90,12 +111,13 @@ struct SharedStorage {
   alignas(1024) uint8_t res[RES ? (BN / kSliceCols) * 4 * kResBytes : 1024];   // one box per active epilogue warp
   uint64_t res_full[kEpiWarps];
   alignas(1024) uint8_t epi[RES ? 1 : kEpi][1024]; // per-warp staging box of the epilogue's bulk stores (RES: the residual box itself)
-  ColTerms cols[kEpi];                            // each epilogue warp stages the terms of its own slice: no barrier
+  TileTerms terms[2];
   alignas(128) uint8_t bp[W4 ? kStages : 1][W4 ? BN * kPackedRow : 128];   // packed weight tiles: unswizzled rows
   alignas(8) uint64_t full[kStages];
   uint64_t empty[kStages];
   uint64_t ready[kStagesB];                         // packed variant: byte weight tile written by the converters
   uint64_t bfree[kStagesB];                         //                 ... and read by the MMAs
+  uint64_t terms_full[2], terms_empty[2];
   uint64_t tmem_full[2];
   uint64_t tmem_empty[2];
   uint64_t done;
@@ -175,16 +197,6 @@ struct TcParams {
 };
 
 enum : int { kOutF32 = 0, kOutBf16 = 1, kOutC4 = 2, kOutC8 = 3 };   // compile-time output kinds of the fast path
-
-// Output quantizer of one 16-column chunk (Eq. 4 with the chunk's column group).
-struct ChunkQuant {
-  float mult, lo, hi;
-  uint32_t pack_k;     // 4-bit: sum_e (magic_bits - z_o) << 4e
-  int zo;
-  float unit, z_unit;  // byte codes of b bits: 2^(8 - b) 2^-149, and (z_o - magic) times it
-  int shift;           //   8 - b
-  uint32_t mask;       //   2^b - 1 in every byte
-};
 
 __device__ __forceinline__ ChunkQuant chunk_quant(const EpilogueParams& ep, const TcParams& P, int col0) {
   const int gw = ep.group_width;
@@ -334,7 +346,7 @@ __device__ __forceinline__ void emit_chunk(const CUtensorMap* map_out, uint32_t 
 
 // General path for one chunk of one thread (ragged rows / columns, float32 residual, accumulator dump):
 // element by element, kept out of line so that the common path stays small.
-__device__ __noinline__ void slow_chunk(const EpilogueParams& ep, const TcParams& P, const ColTerms& C, const uint32_t* r,
+__device__ __noinline__ void slow_chunk(const EpilogueParams& ep, const TcParams& P, const TileTerms& C, const uint32_t* r,
                                         int cl, int64_t m, int col0, int32_t asum_c, int* code_sum) {
   const ChunkQuant q = chunk_quant(ep, P, col0);
   const float magic = __uint_as_float(kMagicBits);
@@ -432,6 +444,7 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     }
     for (int s = 0; s < Storage::kStagesB; ++s) { mbar_init(smem_u32(&S.ready[s]), kConvWarps); mbar_init(smem_u32(&S.bfree[s]), 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(smem_u32(&S.tmem_full[a]), 1); mbar_init(smem_u32(&S.tmem_empty[a]), TWO ? 2 * EW : EW); }
+    for (int a = 0; a < 2; ++a) { mbar_init(smem_u32(&S.terms_full[a]), 1); mbar_init(smem_u32(&S.terms_empty[a]), EW); }
     for (int w = 0; w < kEpiWarps; ++w) mbar_init(smem_u32(&S.res_full[w]), 1);
     mbar_init(smem_u32(&S.done), 1);
     S.abort = 0;
@@ -538,6 +551,61 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       const long long t0 = clock64();
       while (!mbar_try_wait(smem_u32(&S.done), 0) && clock64() - t0 < kWaitCycles) {}
     }
+  } else if (warp == kTermsWarp) {
+    // ---------------------------------------------------------------- column and row terms of the tiles, one tile ahead
+    const EpilogueParams& ep = P.ep;
+    const int kza = P.K * ep.z_a;
+    const bool direct = P.direct_requant != 0;
+    constexpr int kPer = BN / 32;                          // columns of a lane
+    int it = 0;
+    for (int tile = tile0; tile < tiles && !*abort; tile += tile_step, ++it) {
+      const TileOrigin o = tile_origin(tile, P.order, kTileM, BN);
+      const int m0 = o.m0 + rank * BM, n0 = o.n0;
+      TileTerms& C = S.terms[it & 1];
+      // loads from clamped indices, all in flight before the buffer is waited for
+      int zw[kPer], ws[kPer], rows[BM / 32];
+      float sw[kPer], bs[kPer];
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        const int j = min(n0 + lane + 32 * i, P.N - 1);
+        zw[i] = ep.z_w ? __ldg(ep.z_w + j) : ep.z_w_scalar;
+        ws[i] = __ldg(P.wsum + j);
+        sw[i] = ep.s_w ? __ldg(ep.s_w + j) : ep.s_w_scalar;
+        bs[i] = ep.bias ? __ldg(ep.bias + j) : 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < BM / 32; ++i) rows[i] = __ldg(P.asum + min(m0 + lane + 32 * i, P.M - 1));
+      if (!mbar_wait(smem_u32(&S.terms_empty[it & 1]), ((it >> 1) & 1) ^ 1, abort, 11)) break;
+#pragma unroll
+      for (int i = 0; i < BM / 32; ++i) {
+        const int r = lane + 32 * i, a = m0 + r < P.M ? rows[i] - kza : 0;
+        C.asum[r] = a;
+        if (PAIR == kPairRope || ep.rope != nullptr) C.pos[r] = (m0 + r) % ep.rope_period;
+      }
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        const int cs = lane + 32 * i, j = n0 + cs;
+        const bool in = j < P.N;                             // columns outside the matrix: all terms 0
+        float sc = in ? ep.scale_a * sw[i] : 0.f, bi = in ? bs[i] : 0.f;
+        if (direct) {
+          const int gw = ep.group_width;
+          const int gi = (j >= gw) + (j >= 2 * gw) + (j >= 3 * gw);
+          const float inv = gi == 0 ? ep.inv_out_scale[0] : gi == 1 ? ep.inv_out_scale[1] : gi == 2 ? ep.inv_out_scale[2] : ep.inv_out_scale[3];
+          sc *= inv;
+          bi *= inv;
+        }
+        C.nzw[cs] = in ? -zw[i] : 0;
+        C.kw[cs] = in ? -ep.z_a * ws[i] : 0;
+        C.sc[cs] = sc;
+        C.bi[cs] = bi;
+      }
+      if (OUT == kOutC4 || OUT == kOutC8) {
+        if (lane < BN / kChunk) C.quant[lane] = chunk_quant(ep, P, n0 + lane * kChunk);
+      }
+      if (lane == 0) { C.m0 = m0; C.n0 = n0; }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&S.terms_full[it & 1]));
+    }
   } else if (W4 && warp >= 2 + EW) {
     // ---------------------------------------------------------------- converters (packed 4-bit weights)
     // A packed tile holds BN rows of 64 bytes (128 codes, even index in the low nibble).  Thread ct takes 16-byte
@@ -614,7 +682,6 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     const int slice = ew >> 2;                   // which 64 accumulator columns
     const bool slice_on = slice * kSliceCols < BN;
     const EpilogueParams& ep = P.ep;
-    const int kza = P.K * ep.z_a;
     const bool res16 = ep.residual != nullptr && ep.residual_bf16;
     const bool res32 = ep.residual != nullptr && !ep.residual_bf16;
     // the common epilogue applies the pair step it was compiled with; any other combination goes chunk by chunk
@@ -622,29 +689,6 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     const bool sat = ep.qmax <= 127;             // byte codes of at most 7 bits: scale and round in one multiply-add
     const bool direct = P.direct_requant != 0;
     const int cl0 = slice * kSliceCols;          // first column of this warp inside the tile
-    ColTerms& C = S.cols[ew];
-    // Raw per-column inputs of the warp's slice (lane: columns lane and lane + 32 of the slice) and the row's code
-    // sum, fetched one tile ahead; nothing is computed from them before the next tile starts, so the loads stay in
-    // flight behind this tile's epilogue.
-    int nx_zw[2] = {0, 0}, nx_ws[2] = {0, 0}, nx_asum = 0;
-    float nx_sw[2] = {0.f, 0.f}, nx_bs[2] = {0.f, 0.f};
-    auto fetch_terms = [&](int t) {
-      if (t >= tiles || !slice_on) return;
-      const TileOrigin o = tile_origin(t, P.order, kTileM, BN);
-      const int tm0 = o.m0 + rank * BM, tn0 = o.n0;
-      // plain loads from clamped indices: nothing here may consume a loaded value (a select on it would hold the
-      // warp until the load returns); rows and columns outside the matrix are dealt with where the values are used
-      const int64_t tm = min(int64_t(tm0) + quarter * 32 + lane, int64_t(P.M) - 1);
-      nx_asum = __ldg(P.asum + tm);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int j = min(tn0 + cl0 + lane + 32 * h, P.N - 1);
-        if (ep.z_w) nx_zw[h] = __ldg(ep.z_w + j);
-        nx_ws[h] = __ldg(P.wsum + j);
-        if (ep.s_w) nx_sw[h] = __ldg(ep.s_w + j);
-        if (ep.bias) nx_bs[h] = __ldg(ep.bias + j);
-      }
-    };
     // bulk copy of the residual box of tile t (rows and columns outside the matrix are zero-filled)
     const uint32_t res_buf = smem_u32(S.res) + uint32_t(RES ? ew : 0) * kResBytes;
     const uint32_t res_bar = smem_u32(&S.res_full[ew]);
@@ -662,12 +706,12 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       res_pending = true;
     };
     fetch_residual(tile0);
-    fetch_terms(tile0);
     int it = 0;
     for (int tile = tile0; tile < tiles && !*abort; tile += tile_step, ++it) {
       const uint32_t acc = it & 1, acc_phase = (it >> 1) & 1;
-      const TileOrigin o = tile_origin(tile, P.order, kTileM, BN);
-      const int m0 = o.m0 + rank * BM, n0 = o.n0;
+      if (!mbar_wait(smem_u32(&S.terms_full[acc]), acc_phase, abort, 10)) break;
+      const TileTerms& C = S.terms[acc];
+      const int m0 = C.m0, n0 = C.n0;
       const int64_t m = int64_t(m0) + quarter * 32 + lane;
       const bool row_ok = m < P.M;
       // warp-uniform: whole 64-column slice inside the matrix, common epilogue (rows beyond M are clipped by
@@ -689,37 +733,14 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 #pragma unroll
         for (int i = 0; i < kPairPieces; ++i) res[i] = __ldg(res_ptr + i);
       }
-      // corr = acc - z_w (asum - K z_a) - z_a wsum; this tile's inputs were fetched during the previous tile
-      const int32_t asum_c = row_ok ? nx_asum - kza : 0;
-      // stage the per-column terms of the warp's slice in the warp's own buffer (read by this warp alone)
-      if (slice_on) {
-        __syncwarp();                                          // the previous tile's reads of the buffer are done
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int cs = lane + 32 * h, j = n0 + cl0 + cs;
-          const bool in = j < P.N;                             // columns outside the matrix: all terms 0
-          float sc = in ? ep.scale_a * (ep.s_w ? nx_sw[h] : ep.s_w_scalar) : 0.f, bi = in && ep.bias ? nx_bs[h] : 0.f;
-          if (direct) {
-            const int gw = ep.group_width;
-            const int gi = (j >= gw) + (j >= 2 * gw) + (j >= 3 * gw);
-            const float inv = gi == 0 ? ep.inv_out_scale[0] : gi == 1 ? ep.inv_out_scale[1] : gi == 2 ? ep.inv_out_scale[2] : ep.inv_out_scale[3];
-            sc *= inv;
-            bi *= inv;
-          }
-          C.nzw[cs] = in ? -(ep.z_w ? nx_zw[h] : ep.z_w_scalar) : 0;
-          C.kw[cs] = in ? -ep.z_a * nx_ws[h] : 0;
-          C.sc[cs] = sc;
-          C.bi[cs] = bi;
-        }
-        __syncwarp();
-      }
-      fetch_terms(tile + tile_step);                    // next tile's inputs: in flight during this epilogue
+      // corr = acc - z_w (asum - K z_a) - z_a wsum
+      const int32_t asum_c = C.asum[quarter * 32 + lane];
       int code_sum = 0;
       // rotary embedding: this row's line of the (cos, sin) table and the slice's first column inside its head
       const float2* rope_row = nullptr;
       int rope_hb = 0;
       if (PAIR == kPairRope && n0 + cl0 < ep.rope_cols) {
-        rope_row = ep.rope + int64_t(m % ep.rope_period) * (ep.rope_dim >> 1);
+        rope_row = ep.rope + int64_t(C.pos[quarter * 32 + lane]) * (ep.rope_dim >> 1);
         rope_hb = (n0 + cl0) % ep.rope_dim;
       }
 
@@ -746,10 +767,10 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           float v[kChunk];
 #pragma unroll
           for (int q4 = 0; q4 < kChunk / 4; ++q4) {
-            const int4 nz = *reinterpret_cast<const int4*>(&C.nzw[c * kChunk + 4 * q4]);
-            const int4 kw = *reinterpret_cast<const int4*>(&C.kw[c * kChunk + 4 * q4]);
-            const float4 sc = *reinterpret_cast<const float4*>(&C.sc[c * kChunk + 4 * q4]);
-            const float4 bi = *reinterpret_cast<const float4*>(&C.bi[c * kChunk + 4 * q4]);
+            const float4 sc = *reinterpret_cast<const float4*>(&C.sc[cl + 4 * q4]);
+            const float4 bi = *reinterpret_cast<const float4*>(&C.bi[cl + 4 * q4]);
+            const int4 nz = *reinterpret_cast<const int4*>(&C.nzw[cl + 4 * q4]);
+            const int4 kw = *reinterpret_cast<const int4*>(&C.kw[cl + 4 * q4]);
             const float f0 = float(int32_t(r[4 * q4 + 0]) + nz.x * asum_c + kw.x), f1 = float(int32_t(r[4 * q4 + 1]) + nz.y * asum_c + kw.y);
             const float f2 = float(int32_t(r[4 * q4 + 2]) + nz.z * asum_c + kw.z), f3 = float(int32_t(r[4 * q4 + 3]) + nz.w * asum_c + kw.w);
             unpack2(fma2(pack2(sc.x, sc.y), pack2(f0, f1), pack2(bi.x, bi.y)), v[4 * q4 + 0], v[4 * q4 + 1]);
@@ -802,8 +823,7 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
               rope_rotate(make_float2(t4.z, t4.w), v[4 * i + 2], v[4 * i + 3]);
             }
           }
-          ChunkQuant q{};
-          if constexpr (OUT == kOutC4 || OUT == kOutC8) q = chunk_quant(ep, P, col0);
+          const ChunkQuant& q = C.quant[cl / kChunk];
           if constexpr (OUT == kOutC8 && PAIR == kPairGlu) {
             {
               // gated product: 16 accumulator columns (gate, up interleaved) give 8 byte codes; the slice's 32 codes
@@ -861,13 +881,14 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           __syncwarp();
           tmem_ld16(taddr0 + c * kChunk, r);
           tmem_ld_wait();
-          if (row_ok && n0 + cl < P.N) slow_chunk(ep, P, C, r, c * kChunk, m, n0 + cl, asum_c, &code_sum);
+          if (row_ok && n0 + cl < P.N) slow_chunk(ep, P, C, r, cl, m, n0 + cl, asum_c, &code_sum);
         }
       }
-      // accumulator buffer free again
+      // accumulator buffer and terms free again
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
+        mbar_arrive(smem_u32(&S.terms_empty[acc]));
         if constexpr (TWO) mbar_arrive_cluster(map_to_rank(smem_u32(&S.tmem_empty[acc]), 0));
         else mbar_arrive(smem_u32(&S.tmem_empty[acc]));
       }
