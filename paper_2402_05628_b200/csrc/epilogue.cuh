@@ -69,14 +69,21 @@ __device__ __forceinline__ ColumnTerms column_terms(const EpilogueParams& p, int
   return c;
 }
 
-// erf-form GELU, v * Phi(v), without branches.  With t = |v| / sqrt2 clamped to 4 (erfc(4) < 2e-8),
+// erf-form GELU, v * Phi(v), without branches.  With |v| clamped to 4 sqrt2 (erfc(4) < 2e-8; beyond, v Phi(v) is 0 or v to within
+// 5e-8, infinities included) and t = |v| / sqrt2,
 //     erfc(t) = 2^(-t q(t)),   Phi(v) = h for v < 0,   1 - h otherwise,   h = erfc(t) / 2 = 2^(-t q(t) - 1),
 // so v Phi(v) = max(v, 0) - |v| h, one multiply-add (a select between h and 1 - h, then a product: 12608 x 3072 x 768 42.7 us, 41.5 so),
 // and q, which is smooth (q(0) = 2 / (sqrt(pi) ln 2), q(t) ~ t / ln 2), is a degree-6 polynomial fitted so that
 // the error of erf stays below 1e-7.  The negative tail keeps its relative accuracy (no 1 + erf cancellation).
 // Against the float64 erf form the float32 result is within 1.4e-7 |v| (about one ulp).
+constexpr float kGeluLow = -5.65685424949238f;                               // -4 sqrt2
+__device__ __forceinline__ float max_nan(float a, float b) {                 // (fmaxf drops a NaN)
+  float d;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
 __device__ __forceinline__ float gelu_erf(float v) {
-  const float t = fminf(fabsf(v) * 0.70710678118654752f, 4.f);
+  const float n = fmaxf(fminf(v, -v), kGeluLow), t = n * -0.70710678118654752f;
   float q = -1.002269491e-04f;
   q = fmaf(q, t, 4.616116930e-04f);
   q = fmaf(q, t, 2.302142326e-03f);
@@ -86,16 +93,14 @@ __device__ __forceinline__ float gelu_erf(float v) {
   q = fmaf(q, t, 1.627913713e+00f);
   float h;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(h) : "f"(fmaf(-t, q, -1.f)));
-  return fmaf(fminf(v, -v), h, fmaxf(v, 0.f));
+  return fmaf(n, h, max_nan(v, 0.f));
 }
 
 // The same on two values at once (packed float pairs where the operation exists in that form): every lane goes through
 // the operations of gelu_erf in the same order, so the results are the same bits.
 __device__ __forceinline__ void gelu_erf_pair(float& v0, float& v1) {
-  const f32x2 n = pack2(fminf(v0, -v0), fminf(v1, -v1));                     // -|v|
-  float a0, a1;
-  unpack2(mul2(n, splat2(-0.70710678118654752f)), a0, a1);
-  const f32x2 t = pack2(fminf(a0, 4.f), fminf(a1, 4.f));
+  const f32x2 n = pack2(fmaxf(fminf(v0, -v0), kGeluLow), fmaxf(fminf(v1, -v1), kGeluLow));
+  const f32x2 t = mul2(n, splat2(-0.70710678118654752f));
   f32x2 q = splat2(-1.002269491e-04f);
   q = fma2(q, t, splat2(4.616116930e-04f));
   q = fma2(q, t, splat2(2.302142326e-03f));
@@ -107,7 +112,7 @@ __device__ __forceinline__ void gelu_erf_pair(float& v0, float& v1) {
   unpack2(fma2(t, q, splat2(1.f)), e0, e1);                                  // fma(-t, q, -1) = -fma(t, q, 1)
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(h0) : "f"(-e0));
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(h1) : "f"(-e1));
-  unpack2(fma2(n, pack2(h0, h1), pack2(fmaxf(v0, 0.f), fmaxf(v1, 0.f))), v0, v1);
+  unpack2(fma2(n, pack2(h0, h1), pack2(max_nan(v0, 0.f), max_nan(v1, 0.f))), v0, v1);
 }
 
 // acc -> corrected integer -> float value before the output conversion.
