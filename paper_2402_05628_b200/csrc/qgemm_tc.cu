@@ -413,10 +413,10 @@ __device__ __noinline__ void slow_chunk(const EpilogueParams& ep, const TcParams
 enum : int { kPairNone = 0, kPairRope = 1, kPairGlu = 2 };
 
 // EPI: what stands between accumulator and output, fixed at compile time for the common cases: kEpiPlain (nothing; RES: the
-// residual), kEpiGelu (GELU, no residual), kEpiAny (as the parameters say).  Branches on the parameters in every 16-column chunk kept
+// residual), kEpiGelu (GELU, no residual), kEpiResidual (bf16 residual by row-per-lane loads), kEpiAny (as the parameters say).  Branches on the parameters in every 16-column chunk kept
 // the loads and chains of its steps apart: 12608 x 2304 x 768 to codes 25.6 -> 23.0 us, 12608 x 3072 x 768 with GELU 44.7 -> 42.7,
-// 18464 x 3072 x 1024 45.0 -> 41.6.
-enum : int { kEpiAny = 0, kEpiPlain = 1, kEpiGelu = 2 };
+// 18464 x 3072 x 1024 45.0 -> 41.6; bf16 residual, 18464 x 1024 x 4096 61.5 -> 59.1, 8192 x 4096 x 4096 97.7 -> 93.5.
+enum : int { kEpiAny = 0, kEpiPlain = 1, kEpiGelu = 2, kEpiResidual = 3 };
 
 template <int BN, int OUT, bool RES, int PAIR, int WP, bool TWO, int EPI>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -689,7 +689,7 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     const bool slice_on = slice * kSliceCols < BN;
     const EpilogueParams& ep = P.ep;
     const bool gelu = EPI == kEpiAny ? ep.gelu != 0 : EPI == kEpiGelu;
-    const bool res16 = EPI == kEpiAny ? ep.residual != nullptr && ep.residual_bf16 : RES;
+    const bool res16 = EPI == kEpiAny ? ep.residual != nullptr && ep.residual_bf16 : RES || EPI == kEpiResidual;
     const bool res32 = EPI == kEpiAny && ep.residual != nullptr && !ep.residual_bf16;
     // the common epilogue applies the pair step it was compiled with; any other combination goes chunk by chunk
     const bool fast_ok = ep.acc_debug == nullptr && (ep.rope != nullptr) == (PAIR == kPairRope) && (ep.glu != 0) == (PAIR == kPairGlu);
@@ -1028,6 +1028,9 @@ repq_status launch_tc_w(const CUtensorMap& map_a, const CUtensorMap& map_b, cons
   if constexpr (WP == 0 && OUT != kOutC4) {
     const bool residual = P.ep.residual != nullptr;
     if (!P.ep.gelu && (RES ? P.ep.residual_bf16 != 0 : !residual)) return launch_tc_e<BN, OUT, RES, PAIR, WP, TWO, kEpiPlain>(map_a, map_b, P, sms, st);
+    if constexpr (!RES && OUT == kOutBf16) {
+      if (!P.ep.gelu && P.ep.residual_bf16) return launch_tc_e<BN, OUT, RES, PAIR, WP, TWO, kEpiResidual>(map_a, map_b, P, sms, st);
+    }
     if constexpr (!RES && OUT == kOutC8 && PAIR == kPairNone) {
       if (P.ep.gelu && !residual) return launch_tc_e<BN, OUT, RES, PAIR, WP, TWO, kEpiGelu>(map_a, map_b, P, sms, st);
     }
