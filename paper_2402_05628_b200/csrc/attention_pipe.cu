@@ -58,7 +58,7 @@ template <int NB> struct Shape {
   static constexpr int kTmem = 256 * NB;                            // 2 S slots + 2 accumulators
 };
 
-template <int NB, int kLutBits>
+template <int NB, int kLutBits, bool kChains>
 struct PipeShared {
   using Sh = Shape<NB>;
   static constexpr uint32_t kKBytes = Sh::kKeys * 128;
@@ -68,6 +68,7 @@ struct PipeShared {
   static constexpr int kV = NB == 1 && kLutBits != 8 ? 3 : 2;       // V tiles (two where the table takes 33 KB of half an SM)
   alignas(1024) uint8_t v[kV][NB * kVBlockBytes];
   float stat_m[Sh::kParts][kRows], stat_z[Sh::kParts][kRows];
+  float visit_m[kChains ? 2 : 1][kChains ? 4 : 1][kRows], visit_z[kChains ? 2 : 1][kChains ? 2 : 1][kRows];  // kChains: what two parts tell each other
   static constexpr int kLutEntries = kLutBits ? (1 << kLutBits) + 1 : 1;
   uint32_t lut[kLutEntries][32];                  // [code][lane] = E value | O value << 16; the last entry repeats the top code
                                                   // (a clamp at 2^bits that rounds up lands there)
@@ -75,6 +76,7 @@ struct PipeShared {
   uint64_t k_empty[Sh::kK], v_empty[kV];
   uint64_t s_full[2], s_empty[2], s_spent[2], p_full[2];            // s_empty: read in pass 1; s_spent: P.V MMAs have read the operands
   uint64_t q_full, acc_full, acc_empty, done_s, done_pv, merged[4];   // merged: statistics of a lane quarter's rows are there
+  uint64_t visit[kChains ? 8 : 1];                // kChains: both parts of a chain and lane quarter have told
   uint32_t tmem_base;
   volatile int abort;
 };
@@ -176,11 +178,16 @@ __device__ __forceinline__ uint32_t zero_minus(uint32_t v, uint32_t shift4) {
 // kLutBits: width of the table of operand pairs (4, 6, 8; P.V in bf16), or 0: 4-bit codes of 4-bit values, P.V in 8-bit
 // floats.  kF8: 4-bit Q / K codes read as 8-bit floats (a byte below 16 is the e4m3 number byte * 2^-9; the accumulator holds
 // 2^-18 sum (q - z_q) k as a float, exactly); otherwise signed x unsigned bytes.
-template <int NB, int kLutBits, bool kF8>
+// kChains: heads of up to 64 channels in visits of 128 keys (few tiles).  An item's Softmax sums must not depend on how many items
+// share the call, so they are formed as in visits of 64 keys: two chains, the even and the odd blocks of 32 keys, each a running
+// maximum m and z <- z 2^(c (m' - m)) + sum of the block.  A chain's two blocks of a visit belong to two threads, which tell each other
+// their block's maximum before they sum (in shared memory, an mbarrier per pair of warps and visit); the second's sum joins a visit later.
+template <int NB, int kLutBits, bool kF8, bool kChains>
 __global__ void __launch_bounds__(Shape<NB>::kThreads, Shape<NB>::kCtas)
 attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ AttnParams P) {
+  static_assert(!kChains || NB == 2, "chains are those of two 64-key visits in one of 128");
   using Sh = Shape<NB>;
-  using Shared = PipeShared<NB, kLutBits>;
+  using Shared = PipeShared<NB, kLutBits, kChains>;
   constexpr int kKeys = Sh::kKeys, kWork = Sh::kWork, kParts = Sh::kParts, kT = Sh::kWorkThreads, kK = Sh::kK, kV = Shared::kV;
   constexpr bool kLut = kLutBits != 0;
   constexpr int kAccCol = 2 * kKeys;
@@ -202,6 +209,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     mbar_init(smem_u32(&S.q_full), kWork);
     mbar_init(smem_u32(&S.acc_full), 1);
     for (int s = 0; s < 4; ++s) mbar_init(smem_u32(&S.merged[s]), kParts);
+    for (int s = 0; s < (kChains ? 8 : 0); ++s) mbar_init(smem_u32(&S.visit[s]), 2);
     mbar_init(smem_u32(&S.acc_empty), kWork);
     mbar_init(smem_u32(&S.done_s), 1);
     mbar_init(smem_u32(&S.done_pv), 1);
@@ -435,38 +443,78 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
 
     float m = -CUDART_INF_F, z = 0.f;       // running maximum (in units of the score scale) and sum of this thread's columns
     const float sc = P.scale * c;           // exponent of 2 per unit
+    // Largest of `start` and the thread's scores, and sum of 2^(sc (sf - mn)) over them: of all columns, or of the columns e < seen.
+    auto max_all = [&](const float (&sf)[kCols], float start) {
+      float b0 = max3(sf[0], sf[1], sf[2]), b1 = max3(sf[3], sf[4], sf[5]);
+#pragma unroll
+      for (int e = 6; e + 3 < kCols; e += 4) { b0 = max3(b0, sf[e], sf[e + 1]); b1 = max3(b1, sf[e + 2], sf[e + 3]); }
+      return fmaxf(max3(start, b0, b1), fmaxf(sf[kCols - 2], sf[kCols - 1]));
+    };
+    auto sum_all = [&](const float (&sf)[kCols], float mn) {
+      const f32x2 sc2 = splat2(sc), nm2 = splat2(-(mn * sc));
+      f32x2 acc[2] = {0ull, 0ull};
+#pragma unroll
+      for (int e = 0; e < kCols; e += 2) {
+        float a0, a1;
+        unpack2(fma2(pack2(sf[e], sf[e + 1]), sc2, nm2), a0, a1);
+        acc[(e >> 1) & 1] = add2(acc[(e >> 1) & 1], pack2(ex2(a0), ex2(a1)));
+      }
+      float z0, z1;
+      unpack2(add2(acc[0], acc[1]), z0, z1);
+      return z0 + z1;
+    };
+    auto max_some = [&](const float (&sf)[kCols], int seen, float start) {
+      float bm = sf[0];
+#pragma unroll
+      for (int e = 1; e < kCols; ++e)
+        if (e < seen) bm = fmaxf(bm, sf[e]);
+      return fmaxf(start, bm);
+    };
+    auto sum_some = [&](const float (&sf)[kCols], int seen, float mn) {
+      const float nm = -(mn * sc);
+      float acc = 0.f;
+#pragma unroll
+      for (int e = 0; e < kCols; ++e)
+        if (e < seen) acc += ex2(fmaf(sf[e], sc, nm));
+      return acc;
+    };
     // `seen`: columns e < seen are keys the row sees
     auto stats = [&](const float (&sf)[kCols], int seen) {
       if (__builtin_expect(seen >= kCols, 1)) {
-        float b0 = max3(sf[0], sf[1], sf[2]), b1 = max3(sf[3], sf[4], sf[5]);
-#pragma unroll
-        for (int e = 6; e + 3 < kCols; e += 4) { b0 = max3(b0, sf[e], sf[e + 1]); b1 = max3(b1, sf[e + 2], sf[e + 3]); }
-        const float mn = fmaxf(max3(m, b0, b1), fmaxf(sf[kCols - 2], sf[kCols - 1]));
-        const f32x2 sc2 = splat2(sc), nm2 = splat2(-(mn * sc));
-        f32x2 acc[2] = {0ull, 0ull};
-#pragma unroll
-        for (int e = 0; e < kCols; e += 2) {
-          float a0, a1;
-          unpack2(fma2(pack2(sf[e], sf[e + 1]), sc2, nm2), a0, a1);
-          acc[(e >> 1) & 1] = add2(acc[(e >> 1) & 1], pack2(ex2(a0), ex2(a1)));
-        }
-        float z0, z1;
-        unpack2(add2(acc[0], acc[1]), z0, z1);
-        z = z * ex2((m - mn) * sc) + (z0 + z1);        // m = -inf at first: factor 0
+        const float mn = max_all(sf, m);
+        z = fmaf(z, ex2((m - mn) * sc), sum_all(sf, mn));               // m = -inf at first: factor 0
         m = mn;
       } else if (seen > 0) {
-        float bm = sf[0];
-#pragma unroll
-        for (int e = 1; e < kCols; ++e)
-          if (e < seen) bm = fmaxf(bm, sf[e]);
-        const float mn = fmaxf(m, bm), nm = -(mn * sc);
-        float acc = 0.f;
-#pragma unroll
-        for (int e = 0; e < kCols; ++e)
-          if (e < seen) acc += ex2(fmaf(sf[e], sc, nm));
-        z = z * ex2((m - mn) * sc) + acc;
+        const float mn = max_some(sf, seen, m);
+        z = fmaf(z, ex2((m - mn) * sc), sum_some(sf, seen, mn));
         m = mn;
       }
+    };
+    // kChains: m is the chain's maximum after the visit, `mid` between its two blocks; z and `mid` belong to the first part, the
+    // second's `block_z` waits for the next visit.  A block without keys is one of maximum -inf and sum 0: it changes no bit.
+    float mid = -CUDART_INF_F, block_z = 0.f;
+    int told = 0;                           // visits of pass 1, over all tiles
+    auto chain_stats = [&](const float (&sf)[kCols], int seen) -> bool {
+      auto sum = [&](float mn) { return seen >= kCols ? sum_all(sf, mn) : seen > 0 ? sum_some(sf, seen, mn) : 0.f; };
+      const int at = told & 1;
+      const float none = -CUDART_INF_F, own = seen >= kCols ? max_all(sf, none) : seen > 0 ? max_some(sf, seen, none) : none;
+      S.visit_m[at][part][r] = own;
+      if (part >= 2) S.visit_z[at][part & 1][r] = block_z;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&S.visit[warp & 7]));
+      if (!wait_for(smem_u32(&S.visit[warp & 7]), told & 1, abort, 51, P.status)) return false;
+      ++told;
+      const float other = S.visit_m[at][part ^ 2][r];
+      if (part < 2) {
+        if (m > -CUDART_INF_F) z = fmaf(z, ex2((mid - m) * sc), S.visit_z[at][part][r]);
+        mid = fmaxf(m, own);
+        if (mid > -CUDART_INF_F) z = fmaf(z, ex2((m - mid) * sc), sum(mid));
+        m = fmaxf(mid, other);
+      } else {
+        m = fmaxf(fmaxf(m, other), own);
+        block_z = sum(m);
+      }
+      return true;
     };
 
     float w1 = 0.f, w0 = 0.f;               // pass 2: value handed to the saturating fma is w1 (sf - m) + w0
@@ -591,8 +639,8 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
       if (more) {
         v_ptr = P.v + t.bo * P.v_so + t.bi * P.v_si + int64_t(v_key0) * P.ldv + v_g * kVChan;
         if (kDefer) fetch_v(0);
-        m = -CUDART_INF_F;
-        z = 0.f;
+        m = mid = -CUDART_INF_F;
+        z = block_z = 0.f;
         for (int b = 0; b < t.nb; ++b, ++g) {
           const int slot = g & 1, first = b * kKeys + part * kCols;
           if (!wait_for(smem_u32(&S.s_full[slot]), (g >> 1) & 1, abort, 44, P.status)) { ok = false; break; }
@@ -603,16 +651,21 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&S.s_empty[slot]));
-            stats(sf, valid - first);
-          } else if (lane == 0) {
-            mbar_arrive(smem_u32(&S.s_empty[slot]));
+            if constexpr (!kChains) stats(sf, valid - first);
+            else if (!chain_stats(sf, valid - first)) { ok = false; break; }
+          } else {
+            if (lane == 0) mbar_arrive(smem_u32(&S.s_empty[slot]));
+            if constexpr (kChains) {
+              const float none[kCols] = {};
+              if (!chain_stats(none, 0)) { ok = false; break; }
+            }
           }
         }
         if (!ok || *abort) break;
         if (!kDefer) fetch_v(0);
         // the column parts of a row are merged below
-        S.stat_m[part][r] = m;
-        S.stat_z[part][r] = z;
+        S.stat_m[part][r] = kChains && part < 2 ? mid : m;
+        S.stat_z[part][r] = kChains && part >= 2 ? block_z : z;
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&S.merged[quarter]));
       }
@@ -624,9 +677,14 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
 #pragma unroll
       for (int q = 0; q < kParts; ++q) m = fmaxf(m, S.stat_m[q][r]);
 #pragma unroll
-      for (int q = 0; q < kParts; ++q) {
-        const float mq = S.stat_m[q][r];
-        if (mq > -CUDART_INF_F) zt += S.stat_z[q][r] * ex2((mq - m) * sc);
+      for (int q = 0; q < (kChains ? 2 : kParts); ++q) {
+        float mq = S.stat_m[q][r], zq = S.stat_z[q][r];
+        if constexpr (kChains) {                            // the second part's last block
+          const float mid_q = mq;
+          mq = S.stat_m[q + 2][r];
+          zq = fmaf(zq, ex2((mid_q - mq) * sc), S.stat_z[q + 2][r]);
+        }
+        if (mq > -CUDART_INF_F) zt = fmaf(zq, ex2((mq - m) * sc), zt);
       }
       {
         const float k0 = 2.f * (log2f(zt) + P.log2_s);
@@ -692,12 +750,12 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
   }
 }
 
-template <int NB, int kLutBits, bool kF8>
+template <int NB, int kLutBits, bool kF8, bool kChains = false>
 repq_status launch_kernel(const AttnParams& P, int64_t pairs, cudaStream_t st) {
   using Sh = Shape<NB>;
-  constexpr size_t smem = sizeof(PipeShared<NB, kLutBits>);
+  constexpr size_t smem = sizeof(PipeShared<NB, kLutBits, kChains>);
   static_assert(smem <= (NB == 1 ? 113 : 227) * 1024, "shared storage exceeds a CTA's share");
-  REPQ_TRY((allow_smem<attention_pipe_kernel<NB, kLutBits, kF8>>(int(smem))));
+  REPQ_TRY((allow_smem<attention_pipe_kernel<NB, kLutBits, kF8, kChains>>(int(smem))));
   AttnParams Q = P;
   Q.pairs = int(pairs);
   Q.tiles = (P.Lq + kRows - 1) / kRows;
@@ -706,7 +764,7 @@ repq_status launch_kernel(const AttnParams& P, int64_t pairs, cudaStream_t st) {
   REPQ_TRY(make_k_map(&map_k, P, int(pairs / P.batch_inner), Sh::kKeys));
   const int64_t tiles = int64_t(Q.tiles) * pairs, slots = int64_t(sm_count()) * Sh::kCtas;
   const dim3 grid{unsigned(tiles < slots ? tiles : slots)};
-  REPQ_CUDA(launch_chained(attention_pipe_kernel<NB, kLutBits, kF8>, grid, dim3(Sh::kThreads), smem, st, map_k, Q));
+  REPQ_CUDA(launch_chained(attention_pipe_kernel<NB, kLutBits, kF8, kChains>, grid, dim3(Sh::kThreads), smem, st, map_k, Q));
   note_launch();
   return REPQ_OK;
 }
@@ -727,7 +785,11 @@ repq_status launch_form(const AttnParams& P, int64_t pairs, bool small_v, cudaSt
     if (P.qmax_p <= 63) return launch_kernel<1, 6, kF8>(P, pairs, st);
     return launch_kernel<1, 8, kF8>(P, pairs, st);
   }
-  if (f8_pv) return launch_kernel<2, 0, kF8>(P, pairs, st);
+  if (P.dh <= 64) {
+    if (P.qmax_p <= 15) return f8_pv ? launch_kernel<2, 0, kF8, true>(P, pairs, st) : launch_kernel<2, 4, kF8, true>(P, pairs, st);
+    if (P.qmax_p <= 63) return launch_kernel<2, 6, kF8, true>(P, pairs, st);
+    return launch_kernel<2, 8, kF8, true>(P, pairs, st);
+  }
   if (P.qmax_p <= 15) return launch_kernel<2, 4, kF8>(P, pairs, st);
   if (P.qmax_p <= 63) return launch_kernel<2, 6, kF8>(P, pairs, st);
   return launch_kernel<2, 8, kF8>(P, pairs, st);
