@@ -6,6 +6,13 @@
 // run one batch behind the inputs, which costs a batch's time on the link and the block's own time at the end.  The items of a
 // batch are independent, so a batch passes through the pipeline in pieces of whole items: piece c is computed while piece
 // c + 1 is copied in and piece c - 1 copied out, and the outputs run one piece behind.  See `pieces_of` for when.
+//
+// Copies of the two directions begin together: the copy out of a piece waits for the next piece's copy in, and so starts with the one
+// after it.  Where a copy begins while the other direction is under way the link stands for 10 us and more; with blocks shorter than
+// their copies every copy did that to the other direction (six pieces of 3.2 MB: 100 us a piece, 76 while the two ran in step), and
+// a faster block made a call slower.  Four batches of 64 DeiT-B images 2160 -> 1936 us, 20 of 40 ViT-S images, whole, 3790 -> 2860,
+// four of 65 ViT-S images in float32 2590 -> 2030; 28 x 371 DeiT-B tokens and batches of 4.8 MB as before.  A single batch has too
+// few copies to gain by it (64 DeiT-B images 580 us, 591 so): its pieces leave as their blocks end.
 #include <algorithm>
 #include <mutex>
 
@@ -25,7 +32,7 @@ constexpr size_t kGapBytes = size_t(585) << 10;          // what the link would 
 // Pieces per batch: as many as have kPieceBytes of input and kPieceTokens tokens each (below, the host, or the blocks of the pieces
 // together, take longer than the link), unless what they save (the link time of a batch: the outputs no longer run a batch behind)
 // is less than the gaps they add (one per piece and batch).
-// Measured, us, whole -> pieces (ranges: different machines).  64 DeiT-B images of 19.4 MB, six pieces: one batch 935 -> 580, two
+// Measured with every piece leaving as its block ended, us, whole -> pieces (ranges: different machines).  64 DeiT-B images of 19.4 MB, six pieces: one batch 935 -> 580, two
 // 1340 -> 1092..1106, four 2240 -> 2083, five 2690 -> 2614..2638, eight 4051 -> 4194 (whole by the rule); four pieces: four 2250, five
 // 2518..2833.  32 ViT-L images of 577 tokens, 37.8 MB, eight: 1841 -> 1029, four 4237 -> 3530, five 5065 -> 4362, sixteen 14157 -> 13644
 // (whole).  16 of them, 18.9 MB, four: 955 -> 612, five 2655 -> 2280 (seven pieces, 1300 tokens each: 2894).  28 x 371 tokens of
@@ -111,11 +118,23 @@ extern "C" repq_status repq_block_forward_host(const repq_block_desc* d, const r
   REPQ_CUDA(cudaStreamWaitEvent(P->out, P->start, 0));
   const int pieces = pieces_of(x_bytes, *d, n_batches);
   const size_t x_item = x_bytes / size_t(d->batch), y_item = y_bytes / size_t(d->batch);
+  auto first_item = [&](int c) { return size_t(int64_t(d->batch) * c / pieces); };
+  // copy out of piece c of batch i, behind the copy in that `with` marks
+  auto copy_out = [&](int i, int c, cudaEvent_t with) -> repq_status {
+    const size_t first = first_item(c), bytes = (first_item(c + 1) - first) * y_item;
+    const int k = i % kSlots;
+    REPQ_CUDA(cudaStreamWaitEvent(P->out, P->computed[k][c], 0));
+    if (with != nullptr && n_batches > 1) REPQ_CUDA(cudaStreamWaitEvent(P->out, with, 0));
+    REPQ_CUDA(cudaMemcpyAsync(static_cast<uint8_t*>(y_host[i]) + first * y_item, static_cast<const uint8_t*>(s->y_dev[k]) + first * y_item, bytes,
+                              cudaMemcpyDeviceToHost, P->out));
+    REPQ_CUDA(cudaEventRecord(P->copied_out[k][c], P->out));
+    return REPQ_OK;
+  };
   repq_block_desc piece = *d;
   for (int i = 0; i < n_batches; ++i) {
     const int k = i % kSlots;
     for (int c = 0; c < pieces; ++c) {
-      const size_t first = size_t(int64_t(d->batch) * c / pieces), end = size_t(int64_t(d->batch) * (c + 1) / pieces);
+      const size_t first = first_item(c), end = first_item(c + 1);
       piece.batch = int32_t(end - first);
       uint8_t* xd = static_cast<uint8_t*>(s->x_dev[k]) + first * x_item;
       uint8_t* yd = static_cast<uint8_t*>(s->y_dev[k]) + first * y_item;
@@ -128,12 +147,12 @@ extern "C" repq_status repq_block_forward_host(const repq_block_desc* d, const r
       if (i >= kSlots) REPQ_CUDA(cudaStreamWaitEvent(main, P->copied_out[k][c], 0));
       REPQ_TRY(repq_block_forward(&piece, p, xd, yd, s->workspace, s->workspace_bytes, stream));
       REPQ_CUDA(cudaEventRecord(P->computed[k][c], main));
-      // copy out
-      REPQ_CUDA(cudaStreamWaitEvent(P->out, P->computed[k][c], 0));
-      REPQ_CUDA(cudaMemcpyAsync(static_cast<uint8_t*>(y_host[i]) + first * y_item, yd, (end - first) * y_item, cudaMemcpyDeviceToHost, P->out));
-      REPQ_CUDA(cudaEventRecord(P->copied_out[k][c], P->out));
+      // the piece before this one leaves with the next copy in
+      if (c > 0) REPQ_TRY(copy_out(i, c - 1, P->copied_in[k][c]));
+      else if (i > 0) REPQ_TRY(copy_out(i - 1, pieces - 1, P->copied_in[k][c]));
     }
   }
+  REPQ_TRY(copy_out(n_batches - 1, pieces - 1, nullptr));
   // the caller's stream completes only after the last copy out (and hence, copies leaving in order, after every copy)
   REPQ_CUDA(cudaStreamWaitEvent(main, P->copied_out[(n_batches - 1) % kSlots][pieces - 1], 0));
   return REPQ_OK;
