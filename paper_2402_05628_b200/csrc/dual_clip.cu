@@ -23,7 +23,7 @@
 //  - values sorted once, a step's sums from prefix sums at the edges between the 16 codes of a 4-bit quantizer.  What bounds it is the
 //    chain of a step alone (1.3 us: 16 cycles per float64 operation, 90 to 220 for a square root, a division, the sigmoid), one warp per
 //    channel without a barrier.  100 steps: 6304 x 384 321 -> 164 us, 12608 x 192 369 -> 200, 591 x 4096 436 -> 254, 500 x 384
-//    139 -> 133; the learned bounds are the same floats, the objective within 1e-9 (float64 in both).  A full merge sort took 85 us of
+//    139 -> 133; the learned bounds are the same floats.  A full merge sort took 85 us of
 //    6304 x 384 against 25 for buckets and ranks.
 // Arithmetic is float64 throughout (the decisions of the two round operations steer the gradient).
 // No scratch memory, no inter-CTA traffic, no atomics outside the counting of the sort (whose result does not depend on their order).
@@ -465,18 +465,24 @@ struct Buckets {
 // warp then runs the optimisation alone, since a step no longer passes over the values: those of code q lie between two edges of
 // the sorted order, and with y = x - pivot, kappa_q = q - z - pivot/s,
 //     sum over a code of (q - z - x/s)^2 = n kappa^2 - 2 (kappa/s) sum y + (1/s^2) sum y^2
-// from counts and prefix sums at the edges (the pivot, the channel's median, keeps |kappa| below twice the number of codes and small
-// where most values are: the terms cancel to no more than about Q^2 2^-53).  An edge is the smallest float whose rounded quotient reaches the next
-// code, so every value has the code that its own quotient rounds to.
+// from counts and prefix sums at the edges.  The prefix sums run outwards from the pivot, the channel's median, in both directions, so
+// that the sums between two inner edges never contain a tail; what cancels is kappa^2 per value against at most 1/4.  |kappa| is at
+// most Q where the median lies inside the clip, and about Q (1 + 1 / sigmoid(alpha)) where it does not and any value does.  The three
+// sums that steer a step, float64 against 80-bit floats, 6304 values, alpha from 6 down to -3: 1e-13 of the sum of squares inside the clip
+// (one value at -3000 among normal ones 9e-14, normal values 2e-14; summed from the least value on 1e-11 and 3e-13; value by value 1e-16),
+// where the squares inside are a part of the gradient.  Only the float32 bounds, 6e-8 apart, leave the kernel with it.
+// An edge is the smallest float whose rounded quotient reaches the next code, so every value has the code that its own quotient
+// rounds to.
 template <int kWarps>
 __global__ void __launch_bounds__(32 * kWarps, kWarps == 16 ? 2 : 28 / kWarps) dual_clip_sorted_kernel(ClipParams P, int bucket_shift) {
   constexpr int T = 32 * kWarps;
   extern __shared__ __align__(16) float smem[];
   __shared__ float ext[2][kWarps];
   __shared__ int part_n[kWarps];
-  __shared__ double2 part[kWarps];
+  __shared__ double2 part[2][kWarps];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int d = blockIdx.x, n = int(P.n), n8 = (n + 7) & ~7;
+  const int middle = (n >> 1) & ~3;                      // the prefix sums start here
   // values (raw, then sorted), values by bucket (later the prefix sums, 16 bytes per four values), starts of the buckets
   float* val = smem;
   float* by_bucket = smem + n8;
@@ -556,8 +562,10 @@ __global__ void __launch_bounds__(32 * kWarps, kWarps == 16 ? 2 : 28 / kWarps) d
       sync();
     }
     pivot = double(val[n >> 1]);
-    // prefix sums: a run of blocks of four values per thread, summed twice (total, then block by block behind the threads before)
+    // prefix sums at every fourth value, those below `middle` negative: a run of blocks of four values per thread, summed twice
+    // (total, then block by block beyond the threads nearer to the middle)
     const int run = (blocks + T - 1) / T, first = min(blocks, tid * run), last = min(blocks, first + run);
+    const int up0 = max(first, middle >> 2), down1 = min(last, middle >> 2);
     auto add_block = [&](int b, double2& t) {
       for (int i = 4 * b; i < min(n, 4 * b + 4); ++i) {
         const double y = double(val[i]) - pivot;
@@ -565,22 +573,32 @@ __global__ void __launch_bounds__(32 * kWarps, kWarps == 16 ? 2 : 28 / kWarps) d
         t.y = fma(y, y, t.y);
       }
     };
-    double2 own = make_double2(0.0, 0.0);
-    for (int b = first; b < last; ++b) add_block(b, own);
-    double2 sum = own;
+    double2 up = make_double2(0.0, 0.0), down = up;
+    for (int b = up0; b < last; ++b) add_block(b, up);
+    for (int b = down1 - 1; b >= first; --b) add_block(b, down);
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const double sx = __shfl_up_sync(0xffffffffu, sum.x, o), sy = __shfl_up_sync(0xffffffffu, sum.y, o);
-      if (lane >= o) { sum.x += sx; sum.y += sy; }
+      const double ux = __shfl_up_sync(0xffffffffu, up.x, o), uy = __shfl_up_sync(0xffffffffu, up.y, o);
+      const double dx = __shfl_down_sync(0xffffffffu, down.x, o), dy = __shfl_down_sync(0xffffffffu, down.y, o);
+      if (lane >= o) { up.x += ux; up.y += uy; }
+      if (lane + o < 32) { down.x += dx; down.y += dy; }
     }
-    if (lane == 31) part[warp] = sum;
+    if (lane == 31) part[0][warp] = up;
+    if (lane == 0) part[1][warp] = down;
     sync();
-    double2 at = make_double2(__shfl_up_sync(0xffffffffu, sum.x, 1), __shfl_up_sync(0xffffffffu, sum.y, 1));
-    if (lane == 0) at = make_double2(0.0, 0.0);
-    for (int w = 0; w < warp; ++w) { at.x += part[w].x; at.y += part[w].y; }
-    for (int b = first; b < last; ++b) {
-      pre[b] = at;
-      add_block(b, at);
+    up = make_double2(__shfl_up_sync(0xffffffffu, up.x, 1), __shfl_up_sync(0xffffffffu, up.y, 1));
+    down = make_double2(__shfl_down_sync(0xffffffffu, down.x, 1), __shfl_down_sync(0xffffffffu, down.y, 1));
+    if (lane == 0) up = make_double2(0.0, 0.0);
+    if (lane == 31) down = make_double2(0.0, 0.0);
+    for (int w = 0; w < warp; ++w) { up.x += part[0][w].x; up.y += part[0][w].y; }
+    for (int w = kWarps - 1; w > warp; --w) { down.x += part[1][w].x; down.y += part[1][w].y; }
+    for (int b = up0; b < last; ++b) {
+      pre[b] = up;
+      add_block(b, up);
+    }
+    for (int b = down1 - 1; b >= first; --b) {
+      add_block(b, down);
+      pre[b] = make_double2(-down.x, -down.y);
     }
     sync();
   }
@@ -588,20 +606,24 @@ __global__ void __launch_bounds__(32 * kWarps, kWarps == 16 ? 2 : 28 / kWarps) d
 
   // ---- the optimisation: even lanes carry the upper factor, odd lanes the lower one (every pair of lanes holds the same numbers)
   const int top_lane = int(P.Q) + 1;                     // a lane per edge: below code 0, between the codes, above code Q
-  struct Below { double c, y, yy; };                     // number of the values below an edge, sums of y and y^2
-  auto sums_below = [&](int c) {
-    const double2 t = pre[c >> 2];
-    const float4 q = *reinterpret_cast<const float4*>(val + min(c & ~3, n8 - 4));
-    const int r = c & 3;
-    const double y0 = r > 0 ? double(q.x) - pivot : 0.0, y1 = r > 1 ? double(q.y) - pivot : 0.0, y2 = r > 2 ? double(q.z) - pivot : 0.0;
-    return Below{double(c), t.x + ((y0 + y1) + y2), t.y + (fma(y0, y0, y1 * y1) + y2 * y2)};
+  struct Below { double c, y, yy; };                     // number of the values below an edge, sums of y and y^2 from the middle to it
+  auto sums_to = [&](int c) {
+    // from the prefix sums on the middle's side of the edge, and up to three values more
+    const bool up = c >= middle;
+    const double2 t = pre[(up ? c : c + 3) >> 2];
+    const float4 q = *reinterpret_cast<const float4*>(val + max(0, min((up ? c : c - 1) & ~3, n8 - 4)));
+    const int r = (up ? c : -c) & 3;
+    const float f0 = up ? q.x : q.w, f1 = up ? q.y : q.z, f2 = up ? q.z : q.y;
+    const double y0 = r > 0 ? double(f0) - pivot : 0.0, y1 = r > 1 ? double(f1) - pivot : 0.0, y2 = r > 2 ? double(f2) - pivot : 0.0;
+    const double sign = up ? 1.0 : -1.0;
+    return Below{double(c), fma(sign, (y0 + y1) + y2, t.x), fma(sign, fma(y0, y0, y1 * y1) + y2 * y2, t.y)};
   };
-  Below all{0.0, 0.0, 0.0};
-  if (finite) all = sums_below(n);
+  Below none{0.0, 0.0, 0.0}, all = none;
+  if (finite) { none = sums_to(0); all = sums_to(n); }
 
   const bool upper = (lane & 1) == 0;
   const double mine = upper ? double(mxf) : double(mnf), inv_q = 1.0 / P.Q;
-  double bound = 0.0, other = 0.0, a = P.alpha0, m = 0.0, v = 0.0, b1t = 1.0, b2t = 1.0, c1s = 0.0, c2s = 0.0, loss_first = 0.0;
+  double bound = 0.0, other = 0.0, a = P.alpha0, m = 0.0, v = 0.0, b1t = 1.0, b2t = 1.0, c1s = 0.0, c2s = 0.0;
   for (int it = 0; it <= P.iters; ++it) {
     // the channel's quantizer for this step (Eq. 6 on the bounds of Eqs. 18-19)
     const double sg = sigmoid(a);
@@ -624,7 +646,7 @@ __global__ void __launch_bounds__(32 * kWarps, kWarps == 16 ? 2 : 28 / kWarps) d
     // a channel whose bounds coincide (a constant channel, or extremes of 0) has no quantizer to learn: its sums stay
     // 0, its factors keep their starting value and the contracted extremes are returned as they are
     const bool live = s > 0.0;
-    double in2 = 0.0, sum_low = 0.0, sum_high = 0.0, out2 = 0.0;
+    double in2 = 0.0, sum_low = 0.0, sum_high = 0.0;
     if (live && finite) {
       const double shift_p = pivot * inv, k_lo = lo - shift_p, k_hi = (P.Q - z) - shift_p;
       const double k = lo + double(lane);                // first code at or above the lane's edge
@@ -636,14 +658,14 @@ __global__ void __launch_bounds__(32 * kWarps, kWarps == 16 ? 2 : 28 / kWarps) d
         const int mid = (first + last) >> 1;
         if (val[mid] < edge) first = mid + 1; else last = mid;
       }
-      const Below t = sums_below(first);
+      const Below t = sums_to(first);
       // the code between the lane's edge and the one before; its squares without those of y, which add up over the codes
       const double kappa = k_lo + double(lane - 1), inv2 = inv * inv;
       const double dc = t.c - __shfl_up_sync(0xffffffffu, t.c, 1), dy = t.y - __shfl_up_sync(0xffffffffu, t.y, 1);
       if (lane > 0 && lane <= top_lane) in2 = kappa * (kappa * dc - 2.0 * inv * dy);
       // what is clipped, beyond the first and the last edge
       const bool top = lane == top_lane;
-      const double c = top ? all.c - t.c : t.c, y = top ? all.y - t.y : t.y, yy = top ? all.yy - t.yy : t.yy, end = top ? k_hi : k_lo;
+      const double c = top ? all.c - t.c : t.c, y = top ? all.y - t.y : t.y - none.y, end = top ? k_hi : k_lo;
       const double linear = end * c - inv * y;
       if (top) in2 = fma(inv2, t.yy, in2);
       if (lane == 0) in2 = -inv2 * t.yy;
@@ -651,18 +673,27 @@ __global__ void __launch_bounds__(32 * kWarps, kWarps == 16 ? 2 : 28 / kWarps) d
       for (int o = 16; o > 0; o >>= 1) in2 += __shfl_xor_sync(0xffffffffu, in2, o);
       sum_low = __shfl_sync(0xffffffffu, linear, 0);
       sum_high = __shfl_sync(0xffffffffu, linear, top_lane);
-      if (it == 0 || it == P.iters) {
-        const double square = fma(end, linear - inv * y, inv2 * yy);
-        out2 = __shfl_sync(0xffffffffu, square, 0) + __shfl_sync(0xffffffffu, square, top_lane);
-      }
     } else if (live) {
-      in2 = sum_low = sum_high = out2 = CUDART_NAN;
+      in2 = sum_low = sum_high = CUDART_NAN;
     }
-    const double loss = live ? s * s * (in2 + out2) : 0.0;
-    if (it == 0) loss_first = loss;
-    if (it == P.iters) {
-      if (lane == 0) { P.loss[d] = loss_first; P.loss[P.D + d] = loss; }
-    } else {
+    if (P.loss != nullptr && (it == 0 || it == P.iters)) {
+      // the objective goes to the caller in float64: value by value, as in the other forms (4 us each of the two times, 6304 values)
+      double sum[2] = {0.0, 0.0};
+#pragma unroll 4
+      for (int i = 2 * lane; i < n8; i += 64) {
+        const float2 x2 = *reinterpret_cast<const float2*>(val + i);
+        const double u0 = double(x2.x) * inv, u1 = double(x2.y) * inv;
+        const double d0 = fmin(fmax(rint(u0), lo), P.Q - z) - u0, d1 = fmin(fmax(rint(u1), lo), P.Q - z) - u1;
+        sum[0] = i < n ? fma(d0, d0, sum[0]) : sum[0];
+        sum[1] = i + 1 < n ? fma(d1, d1, sum[1]) : sum[1];
+      }
+      sum[0] += sum[1];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) sum[0] += __shfl_xor_sync(0xffffffffu, sum[0], o);
+      const double loss = !live ? 0.0 : finite ? s * s * sum[0] : CUDART_NAN;
+      if (lane == 0) P.loss[it == 0 ? d : P.D + d] = loss;
+    }
+    if (it < P.iters) {
       const double dL_ds = live ? 2.0 * s * (in2 + (zc - z) * sum_low + (P.Q - z + zc) * sum_high) : 0.0;
       const double dL_dl = live ? 2.0 * s * (sum_low + sum_high) : 0.0;
       const double g = (upper ? dL_ds * inv_q : dL_dl - dL_ds * inv_q) * (mine * sg * (1.0 - sg));

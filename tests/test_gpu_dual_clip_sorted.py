@@ -65,3 +65,37 @@ def test_dual_clip_of_channels_with_infinities(n):
             assert np.isnan(lo[d]) and np.isnan(hi[d])
         else:
             assert lo[d] == clean[0][d] and hi[d] == clean[1][d]
+
+
+def _objective(X, alpha0, Q=15.0):
+    """Objective at the starting bounds in 80-bit floats, and what float64 quotients x / s leave open: an error of a few ulp in each
+    quotient u, shared through s, moves (q - z - u)^2 by twice its distance."""
+    keep = 1.0 / (1.0 + np.exp(-alpha0))
+    up, low = X.max(axis=0).astype(np.float64) * keep, X.min(axis=0).astype(np.float64) * keep
+    s = (up - low) / Q
+    z = np.rint(-low / s)
+    u = X.astype(np.longdouble) / s.astype(np.longdouble)
+    d = np.clip(np.rint(u), -z, Q - z) - u
+    return (s * s * (d * d).sum(axis=0)).astype(np.float64), (2.0 ** -50 * s * s * (2.0 * np.abs(d * u) + d * d).sum(axis=0)).astype(np.float64)
+
+
+@pytest.mark.parametrize("alpha0", [6.0, 3.0, 2.0, 0.0, -3.0])
+def test_objective_is_as_exact_as_float64_values(alpha0):
+    """Far outliers on either side, values that lie beyond one of their bounds from the start, two clusters."""
+    rng = np.random.default_rng(5)
+    X = rng.standard_normal((20001, 9)).astype(np.float32)
+    X[7, 1], X[7, 2], X[7, 3], X[9, 4] = -3000.0, 3000.0, -60.0, -3e4
+    X[:, 5] = 10.0 - np.abs(X[:, 5]) ** 0.3
+    X[:, 6] = np.where(np.arange(len(X)) % 100 == 0, -8.0, 10.0) + 0.2 * X[:, 6]
+    X[:, 7] = -np.exp(3.0 * X[:, 7])
+    lo, hi, loss = _run(X, 4, iters=100, alpha0=alpha0)
+    exact, open_ = _objective(X, alpha0)
+    assert np.all(np.abs(loss[:9] - exact) <= open_), np.abs(loss[:9] - exact) / open_
+    # (a channel that lies beyond one of its bounds steps back and forth over the jumps of its zero point: the order of the sums alone
+    # then moves the bounds by per cent; such channels are told by the oracle's own answer to the rows in reverse)
+    from oracle import repq_oracle as orc
+    ref, again = (orc.dual_clip(x, 4, iters=100, lr=0.01, alpha0=alpha0) for x in (X, X[::-1]))
+    span = X.max(axis=0).astype(np.float64) - X.min(axis=0)
+    settled = np.maximum(np.abs(ref["x_low"] - again["x_low"]), np.abs(ref["x_up"] - again["x_up"])) <= 1e-9 * span
+    assert settled.sum() >= 8
+    assert np.all((np.abs(lo - ref["x_low"]) <= 1e-6 * span)[settled]) and np.all((np.abs(hi - ref["x_up"]) <= 1e-6 * span)[settled])
