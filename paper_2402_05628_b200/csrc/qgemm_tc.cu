@@ -1035,7 +1035,9 @@ repq_status launch_tc_w(const CUtensorMap& map_a, const CUtensorMap& map_b, cons
       if (P.ep.gelu && !residual) return launch_tc_e<BN, OUT, RES, PAIR, WP, TWO, kEpiGelu>(map_a, map_b, P, sms, st);
     }
   }
-  return launch_tc_e<BN, OUT, RES, PAIR, WP, TWO, kEpiAny>(map_a, map_b, P, sms, st);
+  // (a pair step on byte weights excludes GELU and residuals: it has returned above)
+  if constexpr (PAIR == kPairNone || WP != 0) return launch_tc_e<BN, OUT, RES, PAIR, WP, TWO, kEpiAny>(map_a, map_b, P, sms, st);
+  else return fail(REPQ_UNSUPPORTED, "qgemm: rope / glu are for plain products without gelu or residual");
 }
 
 template <int BN, int OUT, bool RES, int PAIR = kPairNone>
