@@ -12,3 +12,11 @@ pytestmark = pytest.mark.gpu
 ])
 def test_dual_clip_sizes_match_oracle(n, D, iters):
     parity.check_dual_clip(n, D, 4, seed=n + D, iters=iters)
+
+
+@pytest.mark.parametrize("n,D,iters,strided", [
+    (131, 200, 40, False), (131, 300, 40, True), (1003, 640, 40, True), (257, 1200, 40, False), (66, 2500, 40, True),
+])
+def test_sorted_values_match_oracle_at_every_number_of_warps(n, D, iters, strided):
+    """16, 8, 4, 2 and 1 warps per channel (28 per SM over all channels); 32 steps and more at 4 bits take the sorted values."""
+    parity.check_dual_clip(n, D, 4, seed=n + D, iters=iters, strided=strided)

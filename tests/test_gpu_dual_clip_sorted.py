@@ -31,13 +31,11 @@ def _channels(n, rng):
     return base
 
 
-@pytest.mark.parametrize("n,bits", [(1, 4), (5, 4), (9, 4), (64, 4), (1031, 4), (4098, 4), (22528, 4), (22529, 4), (513, 6)])
-def test_dual_clip_of_crowded_channels(n, bits):
+def _check_against_oracle(X, lo, hi, loss, bits):
     """Both sides are float64 with sums in another order (relative error below 2^-53 n Q^2): the tolerances of the other
     dual-clipping checks, 1e-6 of the range for the bounds, 1e-9 for the objective at the start."""
     from oracle import repq_oracle as orc
-    X = _channels(n, np.random.default_rng(n))
-    lo, hi, loss = _run(X, bits, iters=32, alpha0=6.0)
+    n, D = X.shape
     ref = orc.dual_clip(X, bits, iters=32, lr=0.01, alpha0=6.0)
     span = X.max(axis=0).astype(np.float64) - X.min(axis=0)
     same = span == 0.0                                       # nothing to learn: contracted extremes, no objective
@@ -47,10 +45,28 @@ def test_dual_clip_of_crowded_channels(n, bits):
     ref["loss0"], ref["loss"] = np.where(same, 0.0, ref["loss0"]), np.where(same, 0.0, ref["loss"])
     assert np.all(np.abs(lo - ref["x_low"]) <= 1e-6 * span + 1e-7 * np.abs(ref["x_low"]) + 1e-45)
     assert np.all(np.abs(hi - ref["x_up"]) <= 1e-6 * span + 1e-7 * np.abs(ref["x_up"]) + 1e-45)
-    D = X.shape[1]
     floor = 1e-12 * n * span ** 2
     assert np.all(np.abs(loss[:D] - ref["loss0"]) <= 1e-9 * ref["loss0"] + floor)
     assert np.all(np.abs(loss[D:] - ref["loss"]) <= 1e-5 * ref["loss"] + floor)
+
+
+@pytest.mark.parametrize("n,bits", [(1, 4), (5, 4), (9, 4), (64, 4), (1031, 4), (4098, 4), (22528, 4), (22529, 4), (513, 6)])
+def test_dual_clip_of_crowded_channels(n, bits):
+    X = _channels(n, np.random.default_rng(n))
+    _check_against_oracle(X, *_run(X, bits, iters=32, alpha0=6.0), bits)
+
+
+@pytest.mark.parametrize("D", [300, 640, 1200, 3108, 3256])
+def test_crowded_channels_at_every_number_of_warps(D):
+    """8, 4, 2, 1 and 1 warps per channel; 1031 values take buckets of two, and of four and eight where 21 or 22 channels share an SM (a
+    channel more with the larger buckets).  Equal channels have equal results wherever they stand."""
+    X = _channels(1031, np.random.default_rng(D))
+    at = np.arange(D) % X.shape[1]
+    lo, hi, loss = _run(np.ascontiguousarray(X[:, at]), 4, iters=32, alpha0=6.0)
+    for got in (lo, hi, loss[:D], loss[D:]):
+        assert np.array_equal(got, got[:X.shape[1]][at])
+    few = X.shape[1]
+    _check_against_oracle(X, lo[:few], hi[:few], np.concatenate([loss[:few], loss[D:D + few]]), 4)
 
 
 @pytest.mark.parametrize("n", [40, 3000])

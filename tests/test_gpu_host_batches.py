@@ -7,11 +7,11 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-def _block(batch, seed):
+def _block(batch, seed, **overrides):
     import torch
     from paper_2402_05628_b200.engine import QuantBlock
     from workloads import make_block_inputs
-    blk = QuantBlock(make_block_inputs("c1_vit_s", batch=2))
+    blk = QuantBlock(make_block_inputs("c1_vit_s", batch=2, **overrides))
     rows, D = batch * blk.cfg["L"], blk.cfg["D"]
     rng = np.random.default_rng(seed)
     xs = [torch.from_numpy(rng.standard_normal((rows, D), dtype=np.float32)).to(blk.act_dtype).pin_memory() for _ in range(3)]
@@ -70,3 +70,16 @@ def test_sequences_of_any_length(batch):
     most = min(8, bytes_in // (2685 << 10), xs[0].shape[0] // 2048, batch)
     for n, pieces in per_batch.items():
         assert pieces == (most if most > 1 and n * most * gap <= bytes_in else 1)
+
+
+def test_pieces_of_wider_codes_are_parts_of_the_whole():
+    """6-bit codes, and Softmax codes of 8 bits, which show a last bit of a Softmax sum soonest: pieces of 12 images have 144 attention
+    tiles, the whole batch of 24 has 288, on either side of the number of SMs."""
+    import torch
+    for bits in (dict(bits_a=6, bits_w=6, bits_p=6), dict(bits_p=8)):
+        blk, xs, expect = _block(24, 11, **bits)
+        for n in (1, 5):
+            ys = [torch.zeros(x.shape, dtype=blk.out_dtype).pin_memory() for x in (xs * 2)[:n]]
+            blk.forward_host((xs * 2)[:n], ys)
+            torch.cuda.synchronize()
+            assert all(torch.equal(y, e) for y, e in zip(ys, (expect * 2)[:n]))

@@ -6,11 +6,16 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("dim,ldx", [(64, 64), (384, 384), (384, 400), (768, 768), (1536, 1536)])
-def test_layernorm_of_many_rows_is_that_of_few(dim, ldx):
+# (a block of 256 threads takes 64 rows of up to 128 elements at a time, 32 of 256: more than three turns of 148 SMs with at most eight
+# blocks each are 227328 rows)
+@pytest.mark.parametrize("rows,dim,ldx", [
+    (227401, 64, 64), (227401, 128, 128), (227401, 256, 256),
+    (40009, 384, 384), (40009, 384, 400), (40009, 768, 768), (40009, 1536, 1536),
+])
+def test_layernorm_of_many_rows_is_that_of_few(rows, dim, ldx):
     import torch
     from paper_2402_05628_b200 import binding as B
-    rows, dev = 40009, "cuda:0"
+    dev = "cuda:0"
     g = torch.Generator(dev).manual_seed(dim)
     x = torch.randn(rows, ldx, device=dev, generator=g)[:, :dim]
     gamma, beta = 1.0 + 0.1 * torch.randn(dim, device=dev, generator=g), 0.1 * torch.randn(dim, device=dev, generator=g)
