@@ -957,8 +957,8 @@ TcLayout tc_layout(const repq_gemm_desc& d) {
 
 // Whether a launch takes its bf16 residual through bulk-copied boxes (tiles of at most 192 columns, short K: beyond K = 3072 the
 // main loop sets the pace, and its time per k-block hardly shrinks with the tile width (the operand copies in flight, four stages,
-// against the L2 latency), so that 256-column tiles win: measured at 8192 x 4096 x 4096 101 us with 256 columns against 111 with
-// 192, at 18464 x 1024 x 4096 67 against 79).
+// against the L2 latency), so that 256-column tiles win: measured at 8192 x 4096 x 4096 95 us with 256 columns against 111 with
+// 192 and boxes, at 18464 x 1024 x 4096 58 against 72).
 bool residual_boxes(const repq_gemm_desc& d) {
   return d.out_kind == REPQ_OUT_BF16 && d.residual != nullptr && d.residual_dtype == REPQ_BF16 && d.acc_debug == nullptr &&
          d.glu == 0 && d.K <= 3072 && !packed4(d.bits_w) && !packed6(d.bits_w);
@@ -1144,8 +1144,9 @@ bool qgemm_tc_supported(const repq_gemm_desc& d) {
 //               lane loads), 1.62 (residual boxes, at most 192 columns); a pair's 1.27 x the second part
 // Choices on either side of a line, measured: 18464 x 1024 x 1024 with residual 39.6 us with 256 columns, 33.9 with 192 and
 // boxes; 8192 x 4096 x 11008 with residual 250 single, 205 by pairs; 8192 x 12288 x 4096 to codes 234 and 216; 777 x 4096 x 11008
-// 40 and 35; 2500 x 384 x 384 with residual 6.0 with 192 columns, 5.2 with 128.  Over 1200 problems the chosen form is within
-// 0.3 % of the fastest on average (0.9 % with a rule of its own for each of the three choices).
+// 40 and 35; 2500 x 384 x 384 with residual 6.0 with 192 columns, 5.2 with 128.  The constants were fitted when every epilogue warp
+// prepared its own terms; with the present epilogue the estimates are off by 8 % in the median (too long), and over 208 problems the
+// chosen form is within 0.14 % of the fastest on average, 4 % at worst (6304 x 3072 x 768 with GELU 25.4 us, 24.4 with 192 columns).
 TcPlan qgemm_tc_plan(const repq_gemm_desc& d) {
   TcPlan best;
   if (!qgemm_tc_supported(d)) return best;
