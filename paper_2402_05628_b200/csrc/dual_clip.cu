@@ -55,8 +55,10 @@ constexpr int kMaxResident = 50 * 1024;        // values of a channel that fit t
 
 
 // Sorted form: most values of a channel (its 10 bytes per value fill shared memory), values of a bucket above which the channel
-// counts as crowded (ranks cost a bucket's square), buckets of n values, shared memory.
-constexpr int kMaxSorted = 22 * 1024, kCrowd = 48;
+// counts as crowded (ranks cost a bucket's square; the densest of a normal channel's buckets holds three times the average of
+// 1 << shift and its scatter), buckets of n values, shared memory.
+constexpr int kMaxSorted = 22 * 1024;
+__host__ __device__ constexpr int crowd(int shift) { return 16 + (4 << shift); }
 __host__ __device__ constexpr int sorted_buckets(int n, int shift) { return (n >> shift) + 8; }
 constexpr size_t sorted_bytes(int64_t n, int shift) {
   const int64_t n8 = (n + 7) / 8 * 8;
@@ -453,11 +455,20 @@ __device__ __forceinline__ void sort_channel(float* val, int n8, int tid) {
   sync();
 }
 
-// Bucket of a value: equal parts of the channel's range, monotone in x (every operation rounds once).
+// Bucket of a value, monotone in x (every operation rounds once): equal parts of the channel's range or, `spread`, of the range of
+// u / (1 + |u|), u = (x - low) scale, whose parts grow with the distance from `low` like the density of a long tail falls.
 struct Buckets {
   float low, scale;
   int last;
-  __device__ __forceinline__ int of(float x) const { return max(0, min(last, __float2int_rz(__fmul_rn(__fsub_rn(x, low), scale)))); }
+  bool spread;
+  __device__ __forceinline__ int of(float x) const {
+    float u = __fmul_rn(__fsub_rn(x, low), scale);
+    if (spread) {
+      const float half = 0.5f * float(last + 1);
+      u = __fmaf_rn(copysignf(__fsub_rn(1.f, __frcp_rn(__fadd_rn(1.f, fabsf(u)))), u), half, half);
+    }
+    return max(0, min(last, __float2int_rz(u)));
+  }
 };
 
 // One channel per CTA of kWarps warps.  All of them load the channel's values, sort them (by bucket, then by rank inside
@@ -515,19 +526,39 @@ __global__ void __launch_bounds__(32 * kWarps, kWarps == 16 ? 2 : 28 / kWarps) d
   const bool finite = __syncthreads_or(odd_value) == 0;
 #pragma unroll
   for (int w = 0; w < kWarps; ++w) { mxf = fmaxf(mxf, ext[0][w]); mnf = fminf(mnf, ext[1][w]); }
-  Buckets B{mnf, float(nb) / (mxf - mnf), nb - 1};
+  Buckets B{mnf, float(nb) / (mxf - mnf), nb - 1, false};
   if (!(B.scale < INFINITY)) B.scale = 0.f;              // one value, or a range below the normal numbers: a single bucket
 
   double pivot = 0.0;
   if (finite) {
-    for (int t = tid; t < n; t += T) atomicAdd(&start[B.of(val[t])], 1);
-    sync();
-    // inclusive scan of the counts, a run of buckets per thread
+    // counts of the buckets; where they are crowded, again in spread ones around the middle of 32 of the values
+    const int run_b = (nb + T - 1) / T, first_b = min(nb, tid * run_b), last_b = min(nb, first_b + run_b);
     bool crowded = false;
+    int own = 0;
+    for (;;) {
+      for (int t = tid; t < n; t += T) atomicAdd(&start[B.of(val[t])], 1);
+      sync();
+      own = 0;
+      crowded = false;
+      for (int b = first_b; b < last_b; ++b) { own += start[b]; crowded = crowded || start[b] > crowd(bucket_shift); }
+      crowded = __syncthreads_or(crowded) != 0;
+      if (!crowded || B.spread) break;
+      const float w = val[int(int64_t(n) * lane >> 5)];
+      int rank = 0;
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        const float o = __shfl_sync(0xffffffffu, w, i);
+        rank += o < w || (o == w && i < lane) ? 1 : 0;
+      }
+      auto ranked = [&](int r) { return __shfl_sync(0xffffffffu, w, __ffs(__ballot_sync(0xffffffffu, rank == r)) - 1); };
+      const float middle_w = ranked(16), scale = 2.f / (ranked(24) - ranked(8));
+      if (!(scale < INFINITY)) break;
+      B = Buckets{middle_w, scale, nb - 1, true};
+      for (int i = tid; i <= nb; i += T) start[i] = 0;
+      sync();
+    }
     {
-      const int run = (nb + T - 1) / T, first = min(nb, tid * run), last = min(nb, first + run);
-      int own = 0;
-      for (int b = first; b < last; ++b) { own += start[b]; crowded = crowded || start[b] > kCrowd; }
+      // inclusive scan of the counts, a run of buckets per thread
       int sum = own;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -535,10 +566,10 @@ __global__ void __launch_bounds__(32 * kWarps, kWarps == 16 ? 2 : 28 / kWarps) d
         if (lane >= o) sum += t;
       }
       if (lane == 31) part_n[warp] = sum;
-      crowded = __syncthreads_or(crowded) != 0;
+      sync();
       int at = sum - own;
       for (int w = 0; w < warp; ++w) at += part_n[w];
-      for (int b = first; b < last; ++b) start[b] = at += start[b];
+      for (int b = first_b; b < last_b; ++b) start[b] = at += start[b];
       if (tid == 0) start[nb] = n;
     }
     sync();

@@ -69,6 +69,22 @@ def test_crowded_channels_at_every_number_of_warps(D):
     _check_against_oracle(X, lo[:few], hi[:few], np.concatenate([loss[:few], loss[D:D + few]]), 4)
 
 
+@pytest.mark.parametrize("n", [33, 2000, 12000])
+def test_dual_clip_of_values_far_apart(n):
+    """Channels that linear buckets do not part: outliers of every size, two narrow clusters, quartiles that coincide, values that repeat
+    around a long tail, a tail on each side over 60 binary orders."""
+    rng = np.random.default_rng(n)
+    X = rng.standard_normal((n, 9)).astype(np.float32)
+    X[3, 0], X[5, 1], X[7, 2], X[9, 2] = 100.0, 1e6, -1e20, 1e25
+    X[:, 3] = np.where(np.arange(n) % 2 == 0, -5.0, 5.0) + 1e-4 * X[:, 3]
+    X[:, 4] = np.where(rng.random(n) < 0.7, 0.25, X[:, 4])
+    X[:, 5] = np.round(np.exp(2.0 * X[:, 5]))
+    X[:, 6] = np.exp(14.0 * X[:, 6]) * np.sign(X[:, 7])
+    X[:, 7] = np.sort(X[:, 7])
+    X[:, 8] = np.where(np.arange(n) < 3, 1e4, 1.0 + 1e-6 * X[:, 8])
+    _check_against_oracle(X, *_run(X, 4, iters=32, alpha0=6.0), 4)
+
+
 @pytest.mark.parametrize("n", [40, 3000])
 def test_dual_clip_of_channels_with_infinities(n):
     X = _channels(n, np.random.default_rng(n))
