@@ -773,12 +773,14 @@ template <bool kF8>
 repq_status launch_form(const AttnParams& P, int64_t pairs, bool small_v, cudaStream_t st) {
   // Heads of up to 64 channels: two CTAs per SM with visits of 64 keys, except where every tile has an SM to itself; then the
   // tile's chain of visits is all there is, and half as many visits of 128 keys (16 worker warps) shorten it.  A pass of a
-  // W4A4 block: one image of 577 tokens and 16 heads 62.8 -> 53.9 us, 8 of 197 and 6 heads 46.9 -> 43.7, one 34.6 -> 33.6 (W6A6,
-  // 2 of 197 and 12 heads 49.2 -> 45.7).  Up to 64 keys there is a single visit either way (100 keys 30.7 -> 30.3, 64 keys 28.0
-  // against 29.2).
+  // W4A4 block: one image of 577 tokens and 16 heads 62.5 -> 53.8 us, 8 of 197 and 6 heads 47.0 -> 41.4, one, float32 32.8 -> 32.2 (W6A6,
+  // 2 of 197 and 12 heads 49.3 -> 45.6; of these 0.6 to 1.7 go to forming the sums as the 64-key form does).  Up to 64 keys there
+  // is a single visit either way, and fewer than 32 tiles with up to 191 keys gain no whole visit of 128 (6 heads, 4-bit, one image of 129
+  // keys 31.4 against 31.7, of 160 31.4 and 31.9, 6-bit 32.1 and 32.8; two images of 128 33.2 and 31.8).
   const int64_t tiles = int64_t((P.Lq + kRows - 1) / kRows) * pairs;
   const bool f8_pv = P.dh <= 64 && P.qmax_p <= 15 && small_v && P.log2_s >= 0.f;
-  if (P.dh <= 64 && (P.Lk <= 64 || tiles > sm_count())) {
+  const bool short_keys = P.Lk <= 64 || (tiles < 32 && P.Lk < 192 && P.Lk != 128);
+  if (P.dh <= 64 && (short_keys || tiles > sm_count())) {
     // 4-bit codes of 4-bit values: P.V in 8-bit floats (V rows by 16-byte loads; s >= 1 keeps t >= 0)
     if (P.qmax_p <= 15)
       return f8_pv ? launch_kernel<1, 0, kF8>(P, pairs, st) : launch_kernel<1, 4, kF8>(P, pairs, st);

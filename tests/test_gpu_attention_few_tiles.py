@@ -12,6 +12,8 @@ pytestmark = pytest.mark.gpu
     (2, 2, 129, 129, 64, 4, 4, True, 1.0), (1, 2, 260, 257, 64, 6, 4, False, 1.0), (1, 2, 200, 255, 32, 6, 6, True, 1.0),
     (160, 1, 129, 129, 64, 4, 8, True, 1.0), (80, 2, 66, 100, 64, 4, 4, False, 0.7), (160, 1, 20, 130, 64, 6, 4, False, 1.0),
     (1, 2, 90, 190, 64, 4, 6, False, 0.7),
+    (31, 1, 9, 129, 64, 4, 4, False, 1.0), (32, 1, 9, 129, 64, 4, 4, False, 1.0), (2, 1, 140, 191, 64, 6, 6, True, 1.0),   # 31, 32 tiles
+    (2, 1, 140, 192, 64, 6, 6, True, 1.0),
 ])
 def test_attention_with_few_tiles_matches_oracle(Bn, H, Lq, Lk, dh, bits, bp, causal, s_p):
     parity.check_attention(Bn, H, Lq, Lk, dh, bits, bp, causal, seed=Lq + Lk + dh, s_p=s_p)
@@ -21,6 +23,7 @@ def test_attention_with_few_tiles_matches_oracle(Bn, H, Lq, Lk, dh, bits, bp, ca
     (5, 8, 640, 5000, 64, 4, 8, False, 1.0), (5, 8, 640, 5000, 64, 6, 6, False, 1.0), (5, 8, 640, 5000, 32, 4, 4, False, 3.0),
     (5, 8, 640, 3000, 64, 4, 8, True, 1.0), (7, 8, 333, 577, 64, 6, 6, False, 2.0), (40, 6, 130, 197, 64, 4, 4, False, 3.0),
     (30, 6, 60, 67, 48, 6, 8, True, 1.0), (30, 6, 129, 129, 64, 4, 8, False, 1.0),
+    (9, 32, 60, 67, 48, 6, 8, True, 1.0), (6, 16, 129, 129, 64, 4, 8, False, 1.0),
 ])
 def test_an_items_output_does_not_depend_on_the_number_of_items(Bn, H, Lq, Lk, dh, bits, bp, causal, spread):
     """Calls of more tiles than SMs and of fewer take different kernels: the same bits, down to the last bit of the Softmax sum.  (A
