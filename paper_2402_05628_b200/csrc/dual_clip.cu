@@ -862,15 +862,18 @@ extern "C" repq_status repq_dual_clip(const float* x, int64_t n, int D, int64_t 
     // channels that an SM holds at a time, at so many bytes each, and its turns
     auto held = [&](size_t bytes) { return std::max(1, int(228 * 1024 / int64_t(bytes + 1536))); };
     auto turns = [&](int shift) { return (share + held(sorted_bytes(n, shift)) - 1) / held(sorted_bytes(n, shift)); };
+    const int held_resident = int(int64_t(kMaxResident) * 4 / (n * 4 + 1024));
     // Sorted form: 16 codes (a lane per edge; 64 and 256 codes were slower than passes over the values, 1182 x 2048 430 against 389
-    // and 6304 x 384 1360 against 346), enough steps to pay for the sort (500 x 384, 16 steps: 31 against 28) and no long queue of
-    // channels behind one another (16384 x 4096, 28 turns: 4600 against 4566; 20000 x 1024, 7 turns: 1335 against 1662).
-    const bool sorted = bits == 4 && iters >= 32 && n <= kMaxSorted && turns(3) <= 16;
+    // and 6304 x 384 1360 against 346), no long queue of channels behind one another (16384 x 4096, 28 turns: 4600 against 4566) and
+    // enough steps to pay for the sort: a step of all channels that an SM holds at a time takes 1.1 us against 1.3 to 2.9, the sort 35
+    // to 70 us a turn (6304 x 384 46 against 11, and from the 20th step on, or the 28th with outliers, it is ahead); beyond one
+    // turn the passes of three times as many channels run side by side (12608 x 768 ahead from the 39th or 52nd step, 20000 x 1024 the 41st or 54th).
+    const bool sorted = bits == 4 && n <= kMaxSorted && turns(3) <= 16 && iters >= (turns(3) > 1 ? 72 : 32);
     int shift = 3;                                          // as many buckets as do not cost a further turn
     while (shift > 1 && turns(shift - 1) <= turns(3)) --shift;
     // warps per channel: about 28 warps on every SM over all channels, and as many where shared memory limits the
     // channels an SM holds at a time
-    const int want = std::max(28 * sms / D, 24 / held(sorted ? sorted_bytes(n, shift) : size_t(n) * 4));
+    const int want = std::max(28 * sms / D, 24 / std::max(1, sorted ? held(sorted_bytes(n, shift)) : held_resident));
     auto launch = [&](auto warps) {
       constexpr int kWarps = decltype(warps)::value;
       return sorted ? launch_sorted<kWarps>(P, shift, st) : launch_resident<kWarps>(P, st);
