@@ -21,10 +21,10 @@
 //    in the low word, also decides the clip, on the integer pipe), and several CTAs per SM, so that one channel's chain runs
 //    under the others' passes.
 //  - values sorted once, a step's sums from prefix sums at the edges between the 16 codes of a 4-bit quantizer.  What bounds it is the
-//    chain of a step alone (1.3 us: 16 cycles per float64 operation, 90 to 220 for a square root, a division, the sigmoid), one warp per
-//    channel without a barrier.  100 steps: 6304 x 384 321 -> 164 us, 12608 x 192 369 -> 200, 591 x 4096 436 -> 254, 500 x 384
-//    139 -> 133; the learned bounds are the same floats.  A full merge sort took 85 us of
-//    6304 x 384 against 25 for buckets and ranks.
+//    chain of a step alone (1.15 us: 16 cycles per float64 operation, 90 to 220 for a square root, a division, the sigmoid), one warp per
+//    channel without a barrier.  100 steps, passes -> this: 6304 x 384 294 -> 158 us, 12608 x 768 823 -> 557, 591 x 4096 398 -> 250,
+//    20000 x 1024 1754 -> 1219, 64 x 384 136 -> 125; the objective adds 2 to 45.  The learned bounds are the same floats.
+//    A full merge sort took 85 us of 6304 x 384 against 25 for buckets and ranks.
 // Arithmetic is float64 throughout (the decisions of the two round operations steer the gradient).
 // No scratch memory, no inter-CTA traffic, no atomics outside the counting of the sort (whose result does not depend on their order).
 // Channels of more values than shared memory holds take the kernel that re-reads them: a CTA owns 8 neighbouring channels
@@ -472,7 +472,8 @@ struct Buckets {
 };
 
 // One channel per CTA of kWarps warps.  All of them load the channel's values, sort them (by bucket, then by rank inside
-// the bucket; a channel whose values crowd in few buckets is sorted by merging) and form prefix sums of every fourth; the first
+// the bucket; where values crowd in few buckets, by buckets that widen with the distance from the middle, and where they crowd there too,
+// as values that repeat do, by merging) and form prefix sums of every fourth; the first
 // warp then runs the optimisation alone, since a step no longer passes over the values: those of code q lie between two edges of
 // the sorted order, and with y = x - pivot, kappa_q = q - z - pivot/s,
 //     sum over a code of (q - z - x/s)^2 = n kappa^2 - 2 (kappa/s) sum y + (1/s^2) sum y^2

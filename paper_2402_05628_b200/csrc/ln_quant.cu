@@ -207,8 +207,10 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
   const int64_t first_rows = int64_t(blockIdx.x) * kRowsPerBlock + group * kRows;
   const int64_t stride = int64_t(gridDim.x) * kRowsPerBlock;
   // Float rows of one warp without gaps between them: a block's rows of the iteration after the next one are brought into L2 by one
-  // bulk request (85000 x 768 57.8 -> 51.9 us, 131072 x 384 44.8 -> 40.2, 65536 x 1024 57.1 -> 54.6; rows of several warps gained
-  // nothing, 30000 x 2048 48.1 -> 50.4, and bf16 rows, which wait for instructions, lost 6 to 12 %).
+  // bulk request (inputs new from pass to pass, 400 MB of them: 80000 x 768 53.5 -> 48.4 us, 131072 x 384 45.4 -> 40.0, 80000 x 1024 68.7 ->
+  // 64.6, 262144 x 64 19.6 -> 15.8; rows of several warps gained nothing, 30000 x 2048 48.1 -> 50.4, and bf16 rows, which wait for
+  // instructions, lost 6 to 12 %).  Fewer rows ask for nothing; 20000 and 40000 rows of 64 elements take 0.3 to 0.4 us longer than without this
+  // code, of 128 and more 6 to 20 % less (other registers, another number of blocks).
   constexpr bool kToL2 = sizeof(T) == 4 && TPR <= 32;
   const bool deep = kToL2 && ldx == D && rows > 3 * stride;
   auto to_l2 = [&](int64_t first) {
