@@ -20,6 +20,20 @@ constexpr int kRows = 128;                        // query rows per tile (MMA M)
 constexpr uint32_t kQBytes = kRows * 128;         // Q tile: rows of 128 bytes (the head's codes, zero-padded)
 constexpr uint32_t kMagicBits = 0x4B400000u;      // float 1.5 * 2^23
 
+// Division by a number that is fixed per launch: q = (t + ((n - t) >> sh1)) >> sh2 with t = umulhi(n, mul), exact for every 32-bit n
+// (Granlund and Montgomery, Division by invariant integers using multiplication, 1994).  A division by a run-time number is some 20
+// instructions, and every role of a CTA takes two per tile.
+struct FixedDiv { uint32_t mul; int sh1, sh2; };
+inline FixedDiv fixed_div(uint32_t d) {
+  int l = 0;
+  while ((uint64_t(1) << l) < d) ++l;                     // ceil(log2 d)
+  return {uint32_t((((uint64_t(1) << l) - d) << 32) / d + 1), l < 1 ? l : 1, l > 1 ? l - 1 : 0};
+}
+__device__ __forceinline__ int div_by(int n, const FixedDiv& f) {
+  const uint32_t t = __umulhi(uint32_t(n), f.mul);
+  return int((t + ((uint32_t(n) - t) >> f.sh1)) >> f.sh2);
+}
+
 struct AttnParams {
   const uint8_t* q; const uint8_t* k; const uint8_t* v;
   int64_t ldq, ldk, ldv, q_so, q_si, k_so, k_si, v_so, v_si;
@@ -36,6 +50,7 @@ struct AttnParams {
   int32_t* out_row_sum;
   int n_pad, tmem_cols, vec_store;
   int no_f8;                                         // keep integer scores where the 8-bit float form would apply
+  FixedDiv by_pairs, by_inner;
   int pairs, tiles;                                  // (batch, head) pairs and query tiles of 128 rows: the grid is their product
   int32_t* status;
 };
@@ -69,7 +84,29 @@ __device__ __forceinline__ float ex2(float x) {
 }
 
 
-// Output conversion of 16 values of one row, channels c0 .. c0 + 15 (Eq. 4 or float).
+// Output conversion of 16 values of one row, channels c0 .. c0 + 15: byte codes (Eq. 4) by 16-byte stores ...
+__device__ __forceinline__ void store_codes(const AttnParams& P, const float (&v)[16], int64_t roff, int c0, int& code_sum) {
+  // t = v / s_o clamped, rounded half to even by the float adder (1.5 * 2^23), z_o added as an integer
+  const float zo_lo = float(-P.zo), zo_hi = float(P.qmax - P.zo);
+  const f32x2 inv2 = splat2(P.inv_so), magic2 = splat2(__uint_as_float(kMagicBits));
+  uint32_t w[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    uint32_t u[4];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      float t0, t1, u0, u1;
+      unpack2(mul2(pack2(v[4 * i + 2 * k], v[4 * i + 2 * k + 1]), inv2), t0, t1);
+      unpack2(add2(pack2(fminf(fmaxf(t0, zo_lo), zo_hi), fminf(fmaxf(t1, zo_lo), zo_hi)), magic2), u0, u1);
+      u[2 * k] = __float_as_uint(u0) + uint32_t(P.zo);
+      u[2 * k + 1] = __float_as_uint(u1) + uint32_t(P.zo);
+    }
+    w[i] = __byte_perm(__byte_perm(u[0], u[1], 0x0040), __byte_perm(u[2], u[3], 0x0040), 0x5410);
+    code_sum = int(__dp4a(w[i], 0x01010101u, uint32_t(code_sum)));
+  }
+  *reinterpret_cast<uint4*>(static_cast<uint8_t*>(P.out) + roff + c0) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+// ... and every form (float, packed codes, rows off the 16-byte grid).
 __device__ __forceinline__ void store_values(const AttnParams& P, const float (&v)[16], int64_t roff, int c0, int& code_sum) {
   if (P.out_kind == REPQ_OUT_F32) {
     float* o = static_cast<float*>(P.out) + roff + c0;
@@ -96,25 +133,7 @@ __device__ __forceinline__ void store_values(const AttnParams& P, const float (&
       for (int e = 0; e < 16; ++e) o[e] = __float2bfloat16_rn(v[e]);
     }
   } else if (!P.pack4 && P.vec_store) {
-    // t = v / s_o clamped, rounded half to even by the float adder (1.5 * 2^23), z_o added as an integer
-    const float zo_lo = float(-P.zo), zo_hi = float(P.qmax - P.zo);
-    const f32x2 inv2 = splat2(P.inv_so), magic2 = splat2(__uint_as_float(kMagicBits));
-    uint32_t w[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      uint32_t u[4];
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        float t0, t1, u0, u1;
-        unpack2(mul2(pack2(v[4 * i + 2 * k], v[4 * i + 2 * k + 1]), inv2), t0, t1);
-        unpack2(add2(pack2(fminf(fmaxf(t0, zo_lo), zo_hi), fminf(fmaxf(t1, zo_lo), zo_hi)), magic2), u0, u1);
-        u[2 * k] = __float_as_uint(u0) + uint32_t(P.zo);
-        u[2 * k + 1] = __float_as_uint(u1) + uint32_t(P.zo);
-      }
-      w[i] = __byte_perm(__byte_perm(u[0], u[1], 0x0040), __byte_perm(u[2], u[3], 0x0040), 0x5410);
-      code_sum = int(__dp4a(w[i], 0x01010101u, uint32_t(code_sum)));
-    }
-    *reinterpret_cast<uint4*>(static_cast<uint8_t*>(P.out) + roff + c0) = make_uint4(w[0], w[1], w[2], w[3]);
+    store_codes(P, v, roff, c0, code_sum);
   } else {
     const float zo_lo = float(-P.zo), zo_hi = float(P.qmax - P.zo);
     uint32_t q[16];

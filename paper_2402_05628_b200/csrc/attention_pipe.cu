@@ -125,8 +125,8 @@ template <int kKeys>
 __device__ __forceinline__ bool tile_at(const AttnParams& P, int it, int cta, int ctas, Tile& t) {
   const int pos = it * ctas + (P.causal && (it & 1) ? ctas - 1 - cta : cta);
   if (pos >= P.pairs * P.tiles) return false;
-  const int slot = pos / P.pairs, pair = pos - slot * P.pairs, tile = P.causal ? P.tiles - 1 - slot : slot;
-  t.bo = pair / P.batch_inner;
+  const int slot = div_by(pos, P.by_pairs), pair = pos - slot * P.pairs, tile = P.causal ? P.tiles - 1 - slot : slot;
+  t.bo = div_by(pair, P.by_inner);
   t.bi = pair - t.bo * P.batch_inner;
   t.q0 = tile * kRows;
   t.k_end = P.causal ? max(1, min(P.Lk, min(t.q0 + kRows, P.Lq) + P.Lk - P.Lq)) : P.Lk;
@@ -182,7 +182,9 @@ __device__ __forceinline__ uint32_t zero_minus(uint32_t v, uint32_t shift4) {
 // share the call, so they are formed as in visits of 64 keys: two chains, the even and the odd blocks of 32 keys, each a running
 // maximum m and z <- z 2^(c (m' - m)) + sum of the block.  A chain's two blocks of a visit belong to two threads, which tell each other
 // their block's maximum before they sum (in shared memory, an mbarrier per pair of warps and visit); the second's sum joins a visit later.
-template <int NB, int kLutBits, bool kF8, bool kChains>
+// kBytes: the output is byte codes by 16-byte stores, as in a block; the other output forms have kernels of their own, since their code
+// (10 of 50 KB) stood between what every tile runs: the warps wait for instructions (ncu, 64 x 197: two of three issues).
+template <int NB, int kLutBits, bool kF8, bool kChains, bool kBytes>
 __global__ void __launch_bounds__(Shape<NB>::kThreads, Shape<NB>::kCtas)
 attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ AttnParams P) {
   static_assert(!kChains || NB == 2, "chains are those of two 64-key visits in one of 128");
@@ -611,12 +613,15 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                 for (int e = 0; e < 16; e += 2)
                   unpack2(mul2(scale2, fma2(root2, pack2(__uint_as_float(ro[e]), __uint_as_float(ro[e + 1])),
                                             pack2(__uint_as_float(re[e]), __uint_as_float(re[e + 1])))), v[e], v[e + 1]);
-                if (roff >= 0) store_values(P, v, roff, c0, code_sum);
+                if (roff >= 0) {
+                  if constexpr (kBytes) store_codes(P, v, roff, c0, code_sum);
+                  else store_values(P, v, roff, c0, code_sum);
+                }
               }
               if (part * 16 >= P.dh) {                          // no chunk for this thread
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&S.acc_empty));
-              } else if (roff >= 0 && P.out_row_sum != nullptr && P.out_kind == REPQ_OUT_CODES) {
+              } else if (roff >= 0 && P.out_row_sum != nullptr && (kBytes || P.out_kind == REPQ_OUT_CODES)) {
                 atomicAdd(P.out_row_sum + sum_at, code_sum);
               }
       return true;
@@ -750,23 +755,31 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
   }
 }
 
-template <int NB, int kLutBits, bool kF8, bool kChains = false>
-repq_status launch_kernel(const AttnParams& P, int64_t pairs, cudaStream_t st) {
+template <int NB, int kLutBits, bool kF8, bool kChains, bool kBytes>
+repq_status launch_form_out(const AttnParams& P, int64_t pairs, cudaStream_t st) {
   using Sh = Shape<NB>;
   constexpr size_t smem = sizeof(PipeShared<NB, kLutBits, kChains>);
   static_assert(smem <= (NB == 1 ? 113 : 227) * 1024, "shared storage exceeds a CTA's share");
-  REPQ_TRY((allow_smem<attention_pipe_kernel<NB, kLutBits, kF8, kChains>>(int(smem))));
+  REPQ_TRY((allow_smem<attention_pipe_kernel<NB, kLutBits, kF8, kChains, kBytes>>(int(smem))));
   AttnParams Q = P;
   Q.pairs = int(pairs);
   Q.tiles = (P.Lq + kRows - 1) / kRows;
+  Q.by_pairs = fixed_div(uint32_t(pairs));
+  Q.by_inner = fixed_div(uint32_t(P.batch_inner));
   if (kF8) Q.scale = P.scale * 262144.f;                  // the accumulators hold 2^-18 sum (q - z_q) k
   CUtensorMap map_k;
   REPQ_TRY(make_k_map(&map_k, P, int(pairs / P.batch_inner), Sh::kKeys));
   const int64_t tiles = int64_t(Q.tiles) * pairs, slots = int64_t(sm_count()) * Sh::kCtas;
   const dim3 grid{unsigned(tiles < slots ? tiles : slots)};
-  REPQ_CUDA(launch_chained(attention_pipe_kernel<NB, kLutBits, kF8, kChains>, grid, dim3(Sh::kThreads), smem, st, map_k, Q));
+  REPQ_CUDA(launch_chained(attention_pipe_kernel<NB, kLutBits, kF8, kChains, kBytes>, grid, dim3(Sh::kThreads), smem, st, map_k, Q));
   note_launch();
   return REPQ_OK;
+}
+
+template <int NB, int kLutBits, bool kF8, bool kChains = false>
+repq_status launch_kernel(const AttnParams& P, int64_t pairs, cudaStream_t st) {
+  return P.out_kind == REPQ_OUT_CODES && !P.pack4 && P.vec_store ? launch_form_out<NB, kLutBits, kF8, kChains, true>(P, pairs, st)
+                                                                 : launch_form_out<NB, kLutBits, kF8, kChains, false>(P, pairs, st);
 }
 
 template <bool kF8>

@@ -59,23 +59,17 @@ template <bool kSuspend = true>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort, int code, int32_t* status,
                                           long long limit_cycles = kWaitCycles) {
   if (mbar_try_wait<kSuspend>(bar, parity)) return true;
-  // a short run of further tries (each may keep the warp suspended for kSuspendNs) before the clock is read at all:
-  // most waits end here
+  const uint32_t t0 = uint32_t(clock());
 #pragma unroll 1
-  for (int i = 0; i < 8; ++i)
-    if (mbar_try_wait<kSuspend>(bar, parity)) return true;
-  const long long t0 = clock64();
-  for (;;) {
+  do {
 #pragma unroll 1
     for (int i = 0; i < kTriesPerCheck; ++i)
       if (mbar_try_wait<kSuspend>(bar, parity)) return true;
     if (*abort) return false;
-    if (clock64() - t0 > limit_cycles) {
-      atomicCAS(status, 0, code);
-      *abort = 1;
-      return false;
-    }
-  }
+  } while (uint32_t(clock()) - t0 <= uint32_t(limit_cycles));
+  atomicCAS(status, 0, code);
+  *abort = 1;
+  return false;
 }
 
 // Wait without side effects, for draining copies or MMAs that are still in flight before the CTA exits.
