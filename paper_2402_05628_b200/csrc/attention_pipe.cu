@@ -30,7 +30,7 @@
 // Measured against one CTA per tile with two groups of warps on alternate visits: 64 x 12 heads of 64 channels with 197 keys,
 // 4-bit codes, 83 -> 64 us; 32 x 16 heads, 577 keys 240 -> 192; 4 x 32 heads of 128 channels, 2048 causal keys, 8-bit codes,
 // 400 -> 305.  A warp of its own for the V tiles was slower (one warp's chain of loads and conversions per visit).
-// Roles: worker warps, then a warp each (one lane) for the S MMAs, the P.V MMAs and the K copies.  Every mbarrier wait is
+// Roles: worker warps, then a warp each (one lane issues) for the S MMAs, the P.V MMAs and the K copies.  Every mbarrier wait is
 // bounded; when one runs out the kernel records a status code, all roles leave their loops, MMAs and copies in flight are
 // drained, tensor memory is freed and the kernel returns.
 #include <cuda.h>
@@ -245,8 +245,10 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
   Tile t;
   if (warp == kWork) {
     // ---------------------------------------------------------------- S MMAs
-    // (one lane issues; the loops are kept short, since a visit costs as many issue latencies as they have instructions)
-    if (lane == 0) {
+    // (the whole warp walks the loop, one lane issues: what every lane holds alike stays in uniform registers, from which these
+    // instructions take their operands; with the loop in one lane a visit of two MMAs and two commits took 350 cycles.  The loops are
+    // kept short, since a visit costs as many issue latencies as they have instructions)
+    const bool issues = elect_one();
     // D = s32 from signed x unsigned bytes, or D = f32 from e4m3 x e4m3; both K-major, M = 128, N = the visit's keys
     constexpr uint32_t idesc = (kF8 ? (1u << 4) : (2u << 4) | (1u << 7)) | (uint32_t(kKeys >> 3) << 17) | (uint32_t(kRows >> 4) << 24);
     const uint64_t dk0 = smem_desc_sw128(smem_u32(S.k[0]));
@@ -256,23 +258,24 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     uint32_t ks = 0, kp = 0;                              // K ring: slot and parity
     bool ok = true;
     for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
-      if (!(ok = wait_for(smem_u32(&S.q_full), it & 1, abort, 40, P.status))) break;
+      ok = wait_for(smem_u32(&S.q_full), it & 1, abort, 40, P.status);
       const uint64_t dq = smem_desc_sw128(smem_u32(S.q[it & 1]));
 #pragma unroll 1
       for (int b = 0; b < 2 * t.nb; ++b, ++g) {
         const int slot = g & 1;
         const uint32_t bit = 1u << slot;
-        if (!(ok = wait_for(smem_u32(&S.k_full[ks]), kp, abort, 41, P.status))) break;
-        if (used & bit) {
+        ok = ok && wait_for(smem_u32(&S.k_full[ks]), kp, abort, 41, P.status);
+        if (ok && (used & bit)) {
           const bool spent = (pass2 & bit) != 0;
-          if (!(ok = wait_for(spent ? smem_u32(&S.s_spent[slot]) : smem_u32(&S.s_empty[slot]), ((spent ? ph_spent : ph_empty) >> slot) & 1u,
-                               abort, 42, P.status))) break;
+          ok = wait_for(spent ? smem_u32(&S.s_spent[slot]) : smem_u32(&S.s_empty[slot]), ((spent ? ph_spent : ph_empty) >> slot) & 1u, abort, 42,
+                        P.status);
           if (spent) ph_spent ^= bit; else ph_empty ^= bit;
         }
+        if (!(ok = __all_sync(0xffffffffu, ok))) break;   // (all lanes leave together)
         used |= bit;
         pass2 = b >= t.nb ? pass2 | bit : pass2 & ~bit;
         tc_fence_after();
-        {
+        if (issues) {
           const uint64_t dk = dk0 + uint64_t(ks * (Shared::kKBytes >> 4));
           const uint32_t d = tmem_base + uint32_t(slot * kKeys);
 #pragma unroll
@@ -285,15 +288,16 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
           umma_commit(smem_u32(&S.s_full[slot]));
           umma_commit(smem_u32(&S.k_empty[ks]));
         }
+        __syncwarp();
         if (++ks == kK) { ks = 0; kp ^= 1u; }
       }
     }
-    umma_commit(smem_u32(&S.done_s));
+    if (issues) umma_commit(smem_u32(&S.done_s));
+    __syncwarp();
     mbar_drain(smem_u32(&S.done_s), 0);
-    }
   } else if (warp == kWork + 1) {
     // ---------------------------------------------------------------- P.V MMAs
-    if (lane == 0) {
+    const bool issues = elect_one();
     // D = f32, A (tensor memory) and B = bf16 or e4m3, B MN-major, N = n_pad, M = 128
     const uint32_t idesc = (kLut ? (1u << 4) | (1u << 7) | (1u << 10) : (1u << 4)) | (1u << 16) | (uint32_t(P.n_pad >> 3) << 17) |
                            (uint32_t(kRows >> 4) << 24);
@@ -305,15 +309,16 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     bool ok = true;
     for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
       g += t.nb;
-      if (it > 0 && !(ok = wait_for(smem_u32(&S.acc_empty), (it - 1) & 1, abort, 50, P.status))) break;
+      if (it > 0) ok = wait_for(smem_u32(&S.acc_empty), (it - 1) & 1, abort, 50, P.status);
 #pragma unroll 1
       for (int j = 0; j < t.nb; ++j, ++g) {
         const int slot = g & 1;
-        if (!(ok = wait_for(smem_u32(&S.p_full[slot]), (ph_p >> slot) & 1u, abort, 43, P.status))) break;
+        ok = ok && wait_for(smem_u32(&S.p_full[slot]), (ph_p >> slot) & 1u, abort, 43, P.status);
+        if (!(ok = __all_sync(0xffffffffu, ok))) break;
         ph_p ^= 1u << slot;
         tc_fence_after();
         const int left = t.k_end - j * kKeys;             // keys from the visit's first on
-        {
+        if (issues) {
           const uint64_t dv = dv0 + uint64_t(vs * (NB * Shared::kVBlockBytes >> 4));
           const uint32_t a_base = tmem_base + uint32_t(slot * kKeys);
 #pragma unroll
@@ -335,36 +340,40 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
           umma_commit(smem_u32(&S.v_empty[vs]));
           if (j + 1 == t.nb) umma_commit(smem_u32(&S.acc_full));
         }
+        __syncwarp();
         if (++vs == kV) vs = 0;
       }
     }
-    umma_commit(smem_u32(&S.done_pv));
+    if (issues) umma_commit(smem_u32(&S.done_pv));
+    __syncwarp();
     mbar_drain(smem_u32(&S.done_pv), 0);
-    }
   } else if (warp == kWork + 2) {
     // ---------------------------------------------------------------- K tiles by bulk tensor copies
-    if (lane == 0) {
-      uint32_t ks = 0, kp = 0;
-      int issued = 0;
-      bool ok = true;
-      for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
+    const bool issues = elect_one();
+    uint32_t ks = 0, kp = 0;
+    int issued = 0;
+    bool ok = true;
+    for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
 #pragma unroll 1
-        for (int b = 0; b < 2 * t.nb; ++b) {
-          if (!(ok = wait_for(smem_u32(&S.k_empty[ks]), kp ^ 1u, abort, 48, P.status))) break;
-          const uint32_t bar = smem_u32(&S.k_full[ks]);
+      for (int b = 0; b < 2 * t.nb; ++b) {
+        ok = wait_for(smem_u32(&S.k_empty[ks]), kp ^ 1u, abort, 48, P.status);
+        if (!(ok = __all_sync(0xffffffffu, ok))) break;
+        const uint32_t bar = smem_u32(&S.k_full[ks]);
+        // box: 128 bytes of the head's row (bytes past d_h meet zero bytes of the Q tile), the visit's keys (rows past Lk
+        // are zero-filled), one batch item
+        if (issues) {
           mbar_expect_tx(bar, Shared::kKBytes);
-          // box: 128 bytes of the head's row (bytes past d_h meet zero bytes of the Q tile), the visit's keys (rows past Lk
-          // are zero-filled), one batch item
           tma_load_3d(smem_u32(S.k[ks]), &map_k, bar, t.bi * int(P.k_si), (b < t.nb ? b : b - t.nb) * kKeys, t.bo);
-          ++issued;
-          if (++ks == kK) { ks = 0; kp ^= 1u; }
         }
+        __syncwarp();
+        ++issued;
+        if (++ks == kK) { ks = 0; kp ^= 1u; }
       }
-      // the copies issued last must have landed before this CTA may exit
-      for (int i = issued < kK ? issued : kK; i > 0; --i) {
-        if (ks == 0) { ks = kK - 1; kp ^= 1u; } else { --ks; }
-        mbar_drain(smem_u32(&S.k_full[ks]), kp);
-      }
+    }
+    // the copies issued last must have landed before this CTA may exit
+    for (int i = issued < kK ? issued : kK; i > 0; --i) {
+      if (ks == 0) { ks = kK - 1; kp ^= 1u; } else { --ks; }
+      mbar_drain(smem_u32(&S.k_full[ks]), kp);
     }
   } else {
     // ---------------------------------------------------------------- Softmax arithmetic, V tiles, epilogue

@@ -72,6 +72,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   return false;
 }
 
+// One lane of a converged warp (the same one every time).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 // Wait without side effects, for draining copies or MMAs that are still in flight before the CTA exits.
 __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity) {
   const long long t0 = clock64();
