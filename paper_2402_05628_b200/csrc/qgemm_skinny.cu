@@ -6,20 +6,25 @@
 // rate, and below some 2 MB of weights the latency of one tile.  Both ask for many CTAs with many bytes in flight each:
 //  - a tile's K range is split over the CTAs of a cluster (1, 2, 4 or 8); the int32 partial sums are exchanged through
 //    distributed shared memory, every CTA finishing an equal share of the tile's tokens (integer sums: the result does
-//    not depend on the split);
-//  - two CTAs per SM where the ring of operand stages allows it, at least 64 KB of weights in flight per CTA;
+//    not depend on the split).  They are sent as soon as a CTA has them, by stores that a barrier of the receiver counts: 1.4 us from
+//    the last MMA to the sums (48 x 4096 x 4096, clusters of four), 2.4 with two barriers of the cluster around plain stores;
+//  - two CTAs per SM of 110 KB where a call has more CTAs than SMs.  Calls of fewer take 200 KB each: a deeper ring, and no two CTAs on
+//    one SM while others idle (128 CTAs sat on 90 SMs; block pass of 48 tokens 72.1 -> 69.5 us);
+//  - what stands behind the main loop is run through once before it ends (`dry` below): the code (24-45 KB, out of L2 since the
+//    weights of a layer passed through it) and a chunk's residual and rotation values are near when the sums arrive;
 //  - inside a block, while the kernel before it in the stream still runs, every CTA asks for its first weights
 //    (activations and outputs, and weights that the kernel before may have written, are touched only behind the dependency).
 // The epilogue has one output channel per thread (the channel's terms live in registers), tokens along the accumulator
 // columns; for one token the 32 lanes of a warp are 32 neighbouring outputs, so loads and stores are coalesced without
 // staging.  The arithmetic is epilogue.cuh's, element by element.
 //
-// Measured (block passes, 7B-shaped decoder layer of 48 tokens, one byte per weight code): 1860 -> 75 us against the warp-MMA
-// kernel (2.7 TB/s of weights over the whole pass, all seven kernels included); one image through a ViT-S block 52 -> 32 us
-// against 128-row tiles, of which so small a layer fills only a handful of SMs.
+// Measured (block passes, 7B-shaped decoder layer of 48 tokens, one byte per weight code): 1860 -> 69.5 us against the warp-MMA
+// kernel (2.9 TB/s of weights over the whole pass, all seven kernels included); one image through a ViT-S block 52 -> 30 us
+// against 128-row tiles, of which so small a layer fills only a handful of SMs.  Of the 69.5, weights stream for 34 (at 4.9 to 6.7 TB/s);
+// 16 to 96 MB of the widest layer's weights brought into L2 while attention runs changed nothing (-0.3 to +3.6).
 //
-// Every wait on an mbarrier is bounded as in the other tensor-core kernels; all threads reach the two cluster barriers
-// whether or not a wait ran out.
+// Every wait on an mbarrier is bounded as in the other tensor-core kernels; all threads reach the two cluster barriers, and every
+// CTA sends its sums, whether or not a wait ran out.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -40,17 +45,20 @@ constexpr int kThreads = 32 * (kEpiWarps + 2);
 constexpr int kTok = 8;                     // tokens per tensor-memory load
 constexpr int kMaxStages = 8;
 constexpr uint32_t kWBytes = kRowsW * kBK;
+constexpr uint32_t kChunkBytes = kTok * kRowsW * 4;      // partial sums of a chunk
 constexpr int kMaxTokens = 128;           // tokens per tile at most
 constexpr int kPrefetch = 8;                // k-blocks of weights brought into L2 ahead of the dependency wait (all of a
                                             // CTA's blocks at once crowd out the running kernel's own loads: 83 -> 88 us for
                                             // a 7B-shaped decoder block of 48 tokens)
-constexpr int kSmemRing = 110 * 1024;       // operand ring with two resident CTAs (227 KB per SM less the static part)
+constexpr int kSmemTwo = 110 * 1024;        // shared memory of a CTA, two resident (227 KB per SM less the static part)
+constexpr int kSmemOne = 200 * 1024;        // ... where no SM needs to take two
 
 struct SkinnyParams {
   int M, N, K;
   int mt;                      // tokens per tile (multiple of 16)
   int stages, kblocks, split;
   int weights_settled;         // the weights may be read ahead of the dependency wait
+  int over_ring;               // the partial sums of a cluster's CTAs are exchanged over the ring instead of behind it
   uint32_t stage_bytes, a_bytes;
   uint32_t tmem_cols;
   const int32_t* asum;
@@ -63,8 +71,10 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
 }
-__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+// 16 bytes into the shared memory of a CTA of the cluster, counted by a barrier of that CTA
+__device__ __forceinline__ void st_async_v4(uint32_t addr, uint32_t bar, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%2, %3, %4, %5}, [%1];"
+               ::"r"(addr), "r"(bar), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, int y) {
   asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
@@ -75,13 +85,13 @@ enum : int { kStepNone = 0, kStepGelu = 1, kStepResidual = 2, kStepRope = 3, kSt
 enum : int { kOutF32 = 0, kOutBf16 = 1, kOutC4 = 2, kOutC8 = 3 };
 
 // One chunk of kTok tokens of the thread's output channel j: the accumulators at `taddr` plus the partial sums the other
-// CTAs of the cluster left (`part`, one block of `part_stride` pieces per CTA), then the epilogue.  What an element needs
-// from global memory (residual, rotation table) is requested for the whole chunk before any of it is used.
-template <int OUT, int STEP, bool kWholeChunk>
+// CTAs of the cluster left (`part`, one block of `part_stride` pieces per CTA), then the epilogue of its first `live` tokens (those inside
+// the matrix, at least one).  What an element needs from global memory (residual, rotation table) is requested for the whole chunk
+// before any of it is used.  `dry`: what the chunk will need is brought near and nothing else happens.
+template <int OUT, int STEP>
 __device__ __forceinline__ void finish_chunk(const SkinnyParams& P, const ColumnTerms& ct, uint32_t taddr, const int32_t* asum,
-                                             const uint4* part, int parts, int part_stride, int mc, int j, bool col_ok, int lane) {
+                                             const uint4* part, int parts, int part_stride, int mc, int live, int j, bool col_ok, int lane, bool dry) {
   const EpilogueParams& ep = P.ep;
-  const int live = kWholeChunk ? kTok : min(kTok, P.M - mc);                    // tokens of the chunk inside the matrix (at least one)
   float res[kTok];
   float2 cs[kTok];
   if constexpr (STEP == kStepResidual) {
@@ -101,17 +111,23 @@ __device__ __forceinline__ void finish_chunk(const SkinnyParams& P, const Column
       if (++pos == ep.rope_period) pos = 0;
     }
   }
-  uint32_t r[kTok];
+  uint32_t r[kTok] = {};
   __syncwarp();
-  tmem_ld8(taddr, r);
-  tmem_ld_wait();
+  if (!dry) {
+    tmem_ld8(taddr, r);
+    tmem_ld_wait();
+  }
+#pragma unroll 1
   for (int s = 0; s < parts; ++s) {
     const uint4 lo = part[s * part_stride], hi = part[s * part_stride + kRowsW];
     r[0] += lo.x; r[1] += lo.y; r[2] += lo.z; r[3] += lo.w;
     r[4] += hi.x; r[5] += hi.y; r[6] += hi.z; r[7] += hi.w;
   }
-  if (ep.acc_debug != nullptr && col_ok)
-    for (int e = 0; e < live; ++e) ep.acc_debug[int64_t(mc + e) * P.N + j] = int32_t(r[e]);
+  if (ep.acc_debug != nullptr && col_ok && !dry) {
+#pragma unroll
+    for (int e = 0; e < kTok; ++e)
+      if (e < live) ep.acc_debug[int64_t(mc + e) * P.N + j] = int32_t(r[e]);
+  }
   float v[kTok];
   const int4 as0 = *reinterpret_cast<const int4*>(asum), as1 = *reinterpret_cast<const int4*>(asum + 4);
   const int32_t as[kTok] = {as0.x, as0.y, as0.z, as0.w, as1.x, as1.y, as1.z, as1.w};
@@ -137,6 +153,7 @@ __device__ __forceinline__ void finish_chunk(const SkinnyParams& P, const Column
       v[e] = silu_mul(v[e], up);
     }
   }
+  if (dry) live = 0;
   const bool store = col_ok && !(STEP == kStepGlu && (j & 1));
   const int64_t at0 = int64_t(mc) * ep.ldo + (STEP == kStepGlu || OUT == kOutC4 ? j >> 1 : j);
   if constexpr (OUT == kOutF32 || OUT == kOutBf16) {
@@ -144,7 +161,7 @@ __device__ __forceinline__ void finish_chunk(const SkinnyParams& P, const Column
     T* o = static_cast<T*>(ep.out) + at0;
 #pragma unroll
     for (int e = 0; e < kTok; ++e) {
-      if (store && (kWholeChunk || e < live)) {
+      if (store && e < live) {
         if constexpr (OUT == kOutF32) *o = v[e]; else *o = __float2bfloat16_rn(v[e]);
       }
       o += ep.ldo;
@@ -158,9 +175,9 @@ __device__ __forceinline__ void finish_chunk(const SkinnyParams& P, const Column
     for (int e = 0; e < kTok; ++e) {
       if constexpr (OUT == kOutC4) {
         const int next = __shfl_down_sync(0xffffffffu, code[e], 1);
-        if (col_ok && !(j & 1) && (kWholeChunk || e < live)) *o = uint8_t(code[e] | (next << 4));
+        if (col_ok && !(j & 1) && e < live) *o = uint8_t(code[e] | (next << 4));
       } else {
-        if (store && (kWholeChunk || e < live)) *o = uint8_t(code[e]);
+        if (store && e < live) *o = uint8_t(code[e]);
       }
       o += ep.ldo;
     }
@@ -180,7 +197,7 @@ template <int OUT, int STEP>
 __global__ void __launch_bounds__(kThreads, 2)
 qgemm_skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_a, const __grid_constant__ SkinnyParams P) {
   extern __shared__ __align__(1024) uint8_t ring[];
-  __shared__ alignas(8) uint64_t s_full[kMaxStages], s_empty[kMaxStages], s_acc, s_done;
+  __shared__ alignas(8) uint64_t s_full[kMaxStages], s_empty[kMaxStages], s_acc, s_done, s_part;
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   __shared__ alignas(16) int32_t s_asum[kMaxTokens];
@@ -191,17 +208,26 @@ qgemm_skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
   const int n0 = int(blockIdx.x) / split * kRowsW, m0 = int(blockIdx.y) * P.mt;
   const int kb0 = rank * P.kblocks / split, kb1 = (rank + 1) * P.kblocks / split;
   const int stages = P.stages;
+  // The tile's chunks of kTok tokens are dealt to the cluster's CTAs in contiguous shares; a CTA sends its partial sums of the other
+  // shares to their owners, into a part of shared memory of their own: [source][chunk of the share][half of 4 tokens][channel] x 16 B.
+  const int chunks = P.mt / kTok, share = (chunks + split - 1) / split;
+  const int c_first = rank * share, c_end = min(chunks, c_first + share);
+  // (or, where a ring of three stages leaves no room for that, over the ring, once all CTAs have finished with theirs).
+  uint8_t* exchange = P.over_ring ? ring : ring + uint32_t(stages) * P.stage_bytes;
 
+  if (warp == kEpiWarps && lane == 0) { tma_prefetch_map(&map_w); tma_prefetch_map(&map_a); }
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) { mbar_init(smem_u32(&s_full[s]), 1); mbar_init(smem_u32(&s_empty[s]), 1); }
     mbar_init(smem_u32(&s_acc), 1);
     mbar_init(smem_u32(&s_done), 1);
+    mbar_init(smem_u32(&s_part), 1);
     s_abort = 0;
     if (smem_u32(ring) & 1023u) {                          // the swizzled tiles need this alignment
       atomicCAS(P.status, 0, 69);
       s_abort = 1;
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (c_end > c_first) mbar_expect_tx(smem_u32(&s_part), uint32_t((split - 1) * (c_end - c_first)) * kChunkBytes);
   }
   if (warp == kEpiWarps + 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(P.tmem_cols) : "memory");
@@ -209,6 +235,7 @@ qgemm_skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
   }
   tc_fence_before();
   __syncthreads();
+  if (split > 1 && !P.over_ring) cluster_arrive();         // (this CTA's barriers are set up)
   tc_fence_after();
   const uint32_t tmem = s_tmem;
   volatile int* abort = &s_abort;
@@ -235,23 +262,27 @@ qgemm_skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
   const bool col_ok = j < P.N;
   ColumnTerms ct{};
 
-  bool ok = true;
   if (warp == kEpiWarps) {
-    // ---------------------------------------------------------------- bulk copies
-    if (lane == 0) {
-      uint32_t stage = 0, phase = 0;
-      int issued = 0;
-      for (int kb = kb0; kb < kb1; ++kb) {
-        if (!mbar_wait(smem_u32(&s_empty[stage]), phase ^ 1, abort, 61, P.status)) break;
-        const uint32_t bar = smem_u32(&s_full[stage]);
-        const uint32_t base = smem_u32(ring) + stage * P.stage_bytes;
+    // ---------------------------------------------------------------- bulk copies (the warp walks the loop, one lane issues)
+    const bool issues = elect_one();
+    uint32_t stage = 0, phase = 0;
+    int issued = 0;
+    for (int kb = kb0; kb < kb1; ++kb) {
+      const bool free = mbar_wait(smem_u32(&s_empty[stage]), phase ^ 1, abort, 61, P.status);
+      if (!__all_sync(0xffffffffu, free)) break;
+      const uint32_t bar = smem_u32(&s_full[stage]);
+      const uint32_t base = smem_u32(ring) + stage * P.stage_bytes;
+      if (issues) {
         mbar_expect_tx(bar, early ? P.a_bytes : kWBytes + P.a_bytes);
         if (early == 0) tma_load_2d(base, &map_w, bar, kb * kBK, n0);
         tma_load_2d(base + kWBytes, &map_a, bar, kb * kBK, m0);
-        ++issued;
-        if (++stage == uint32_t(stages)) { stage = 0; phase ^= 1; }
       }
-      // the copies issued last must have landed before the ring is reused and the CTA may exit
+      __syncwarp();
+      ++issued;
+      if (++stage == uint32_t(stages)) { stage = 0; phase ^= 1; }
+    }
+    if (lane == 0) {
+      // the copies issued last must have landed before the CTA may exit
       for (int i = issued < stages ? issued : stages; i > 0; --i) {
         if (stage == 0) { stage = uint32_t(stages) - 1; phase ^= 1; } else { --stage; }
         mbar_drain(smem_u32(&s_full[stage]), phase);
@@ -261,73 +292,89 @@ qgemm_skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
     }
   } else if (warp == kEpiWarps + 1) {
     // ---------------------------------------------------------------- MMA issue: D = s32, A = B = unsigned bytes, K-major
-    if (lane == 0) {
-      const uint32_t idesc = (2u << 4) | (uint32_t(P.mt >> 3) << 17) | (uint32_t(kRowsW >> 4) << 24);
-      uint32_t stage = 0, phase = 0;
-      bool go = true;
-      for (int kb = kb0; kb < kb1; ++kb) {
-        if (!mbar_wait(smem_u32(&s_full[stage]), phase, abort, 62, P.status)) { go = false; break; }
-        tc_fence_after();
-        const uint32_t base = smem_u32(ring) + stage * P.stage_bytes;
-        const uint64_t dw = smem_desc_sw128(base), da = smem_desc_sw128(base + kWBytes);
+    const bool issues = elect_one();
+    const uint32_t idesc = (2u << 4) | (uint32_t(P.mt >> 3) << 17) | (uint32_t(kRowsW >> 4) << 24);
+    uint32_t stage = 0, phase = 0;
+    bool go = true;
+    for (int kb = kb0; kb < kb1; ++kb) {
+      go = mbar_wait(smem_u32(&s_full[stage]), phase, abort, 62, P.status);
+      if (!(go = __all_sync(0xffffffffu, go))) break;
+      tc_fence_after();
+      const uint32_t base = smem_u32(ring) + stage * P.stage_bytes;
+      const uint64_t dw = smem_desc_sw128(base), da = smem_desc_sw128(base + kWBytes);
+      if (issues) {
 #pragma unroll
         for (int k = 0; k < kBK / 32; ++k) umma_i8(tmem, dw + uint64_t(2 * k), da + uint64_t(2 * k), idesc, (kb != kb0 || k != 0) ? 1u : 0u);
         umma_commit(smem_u32(&s_empty[stage]));
-        if (++stage == uint32_t(stages)) { stage = 0; phase ^= 1; }
       }
+      __syncwarp();
+      if (++stage == uint32_t(stages)) { stage = 0; phase ^= 1; }
+    }
+    if (issues) {
       if (go) umma_commit(smem_u32(&s_acc));
       umma_commit(smem_u32(&s_done));                      // all MMAs have completed before tensor memory is freed
-      mbar_drain(smem_u32(&s_done), 0);
     }
+    __syncwarp();
+    mbar_drain(smem_u32(&s_done), 0);
   } else {
+    // ---------------------------------------------------------------- epilogue
     // the tile's token sums and the channel's terms, behind the main loop
     for (int i = threadIdx.x; i < P.mt; i += 32 * kEpiWarps) s_asum[i] = m0 + i < P.M ? __ldg(P.asum + m0 + i) : 0;
     if (col_ok) ct = column_terms(ep, j, __ldg(P.wsum + j));
     if (ep.glu) { const ColumnTerms q = column_terms(ep, 0, 0); ct.inv_so = q.inv_so; ct.zo_lo = q.zo_lo; ct.zo_hi = q.zo_hi; ct.zo = q.zo; }
     asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
-    ok = mbar_wait(smem_u32(&s_acc), 0, abort, 63, P.status);
-    tc_fence_after();
-  }
-  __syncwarp();
-
-  // ---------------------------------------------------------------- exchange of partial sums
-  // The tile's chunks of kTok tokens are dealt to the cluster's CTAs in contiguous shares; a CTA writes its partial sums
-  // of the other shares into their owners' shared memory: [source][chunk of the share][half of 4 tokens][channel] x 16 B.
-  const int chunks = P.mt / kTok;
-  const int share = (chunks + split - 1) / split;
-  const uint32_t tquarter = tmem + (uint32_t(quarter * 32) << 16);
-  const int row = quarter * 32 + lane;
-  if (split > 1) {
-    cluster_sync();                                        // every CTA of the cluster has finished with its ring
-    if (warp < kEpiWarps) {
-      for (int c = half; c < chunks; c += kEpiWarps / 4) {
-        const int owner = c / share;
-        if (owner == rank) continue;
-        uint32_t r[kTok];
-        tmem_ld8(tquarter + uint32_t(c * kTok), r);
-        tmem_ld_wait();
-        const int src = rank - (rank > owner ? 1 : 0);     // 0 .. split - 2
-        const uint32_t at = smem_u32(ring) + uint32_t((src * share + (c - owner * share)) * 2 * kRowsW + row) * 16u;
-        const uint32_t to = map_to_rank(at, uint32_t(owner));
-        st_cluster_v4(to, r[0], r[1], r[2], r[3]);
-        st_cluster_v4(to + kRowsW * 16u, r[4], r[5], r[6], r[7]);
+    const uint32_t tquarter = tmem + (uint32_t(quarter * 32) << 16);
+    const int row = quarter * 32 + lane;
+    // The first round runs dry, while the main loop waits for its operands: its code, and the residual and rotation values of the first
+    // chunk, are then near (48 tokens x 12288 x 4096 with rotation: last MMA to end of the kernel 3.1 -> 1.1 us).
+#pragma unroll 1
+    for (int round = 0; round < 2; ++round) {
+      if (round != 0) {
+        bool ok = mbar_wait(smem_u32(&s_acc), 0, abort, 63, P.status);
+        tc_fence_after();
+        if (split > 1) {
+          __syncwarp();
+          if (P.over_ring) cluster_arrive();               // (this CTA's main loop is through)
+          cluster_wait();                                  // (and so far are the others)
+#pragma unroll 1
+          for (int c = half; c < chunks; c += kEpiWarps / 4) {
+            const int owner = c / share;
+            if (owner == rank) continue;
+            uint32_t r[kTok];
+            __syncwarp();
+            tmem_ld8(tquarter + uint32_t(c * kTok), r);
+            tmem_ld_wait();
+            const int src = rank - (rank > owner ? 1 : 0);     // 0 .. split - 2
+            const uint32_t at = smem_u32(exchange) + uint32_t((src * (min(chunks, (owner + 1) * share) - owner * share) + (c - owner * share)) * 2 * kRowsW + row) * 16u;
+            const uint32_t to = map_to_rank(at, uint32_t(owner)), bar = map_to_rank(smem_u32(&s_part), uint32_t(owner));
+            st_async_v4(to, bar, r[0], r[1], r[2], r[3]);
+            st_async_v4(to + kRowsW * 16u, bar, r[4], r[5], r[6], r[7]);
+          }
+          if (c_end > c_first) ok = mbar_wait(smem_u32(&s_part), 0, abort, 64, P.status) && ok;
+          __syncwarp();
+          cluster_arrive();                                // (nothing more comes to this CTA, and it sends nothing more)
+        }
+        if (!ok || *abort) break;
+      }
+      for (int c = c_first + half; c < c_end; c += kEpiWarps / 4) {
+        const int mc = m0 + c * kTok;
+        if (mc >= P.M) break;
+        const uint4* part = reinterpret_cast<const uint4*>(exchange) + (c - c_first) * 2 * kRowsW + row;
+        finish_chunk<OUT, STEP>(P, ct, tquarter + uint32_t(c * kTok), s_asum + c * kTok, part, round != 0 ? split - 1 : 0,
+                                (c_end - c_first) * 2 * kRowsW, mc, min(kTok, P.M - mc), j, col_ok, lane, round == 0);
+        if (round == 0) break;
       }
     }
-    cluster_sync();
   }
-
-  // ---------------------------------------------------------------- epilogue of this CTA's share
-  if (warp < kEpiWarps && ok && !*abort) {
-    const int c_end = min(chunks, (rank + 1) * share);
-    for (int c = rank * share + half; c < c_end; c += kEpiWarps / 4) {
-      const int mc = m0 + c * kTok;
-      if (mc >= P.M) break;
-      const uint4* part = reinterpret_cast<const uint4*>(ring) + (c - rank * share) * 2 * kRowsW + row;
-      if (mc + kTok <= P.M)
-        finish_chunk<OUT, STEP, true>(P, ct, tquarter + uint32_t(c * kTok), s_asum + c * kTok, part, split - 1, share * 2 * kRowsW, mc, j, col_ok, lane);
-      else
-        finish_chunk<OUT, STEP, false>(P, ct, tquarter + uint32_t(c * kTok), s_asum + c * kTok, part, split - 1, share * 2 * kRowsW, mc, j, col_ok, lane);
+  __syncwarp();
+  if (split > 1) {
+    // no CTA leaves before the sums sent to it have arrived, whether or not a wait ran out
+    if (warp >= kEpiWarps) {
+      if (P.over_ring) cluster_arrive();
+      cluster_wait();
+      cluster_arrive();
     }
+    cluster_wait();
   }
 
   tc_fence_before();
@@ -354,7 +401,7 @@ repq_status make_map(CUtensorMap* map, const uint8_t* base, int64_t rows, int64_
 
 template <int OUT, int STEP>
 repq_status launch(dim3 grid, uint32_t smem, const CUtensorMap& map_w, const CUtensorMap& map_a, const SkinnyParams& P, cudaStream_t st) {
-  REPQ_TRY((allow_smem<qgemm_skinny_kernel<OUT, STEP>>(kSmemRing)));
+  REPQ_TRY((allow_smem<qgemm_skinny_kernel<OUT, STEP>>(kSmemOne)));
   REPQ_CUDA(launch_chained_cluster(qgemm_skinny_kernel<OUT, STEP>, grid, dim3(kThreads), smem, st, P.split, map_w, map_a, P));
   note_launch();
   return REPQ_OK;
@@ -379,7 +426,7 @@ repq_status launch_step(int step, dim3 grid, uint32_t smem, const CUtensorMap& m
 //   operands                k-blocks of a CTA x 0.295 (a ring's latency over its stages) or, with two CTAs on an SM, x (16 KB of
 //                           weights + tokens) at 160 KB per us and SM; or all weights at 4.6 TB/s, whichever is longer
 //   epilogue                0.024 per token of a CTA's share, 0.039 with GELU or a step on column pairs, 0.046 with a residual
-//   exchange in a cluster   1.15 and 0.031 per token that leaves the CTA
+//   exchange in a cluster   1.15 and 0.031 per token that leaves the CTA (fitted to the exchange behind two barriers of the cluster)
 //   two CTAs on an SM       0.5, and 1.53 x the epilogue and the exchange
 // Clusters fill the SMs less evenly: those of four and eight share SMs from 0.91 and 0.75 CTAs per SM on, and beyond 1.8 and 1.62
 // per SM (two without a cluster) the last ones wait for a second wave, which costs more than it brings.
@@ -432,15 +479,20 @@ repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, cons
   P.a_bytes = uint32_t(mt) * kBK;
   P.stage_bytes = kWBytes + P.a_bytes;
   const int per = (P.kblocks + split - 1) / split;         // k-blocks of a CTA
-  int stages = kSmemRing / int(P.stage_bytes);             // at least three
-  if (stages > kMaxStages) stages = kMaxStages;
-  if (stages > per) stages = per;
+  // behind the ring: the partial sums that the other CTAs of the cluster send
+  const uint32_t exchange = uint32_t(split - 1) * uint32_t((mt / kTok + split - 1) / split) * kChunkBytes;
+  auto ring_of = [&](uint32_t bytes) {
+    const int n = int(bytes / P.stage_bytes), useful = per < kMaxStages ? per : kMaxStages;
+    return n < useful ? n : useful;
+  };
+  const uint32_t most = n_tiles * m_tiles * split <= sm_count() ? kSmemOne : kSmemTwo;
+  int stages = ring_of(most - exchange);
+  P.over_ring = stages < 3 && stages < per;
+  if (P.over_ring) stages = ring_of(most);                 // (at least three, or all k-blocks)
   P.stages = stages;
-  // the ring also holds the partial sums of the exchange
-  const int share = (mt / kTok + split - 1) / split;
-  const uint32_t exchange = uint32_t(split - 1) * uint32_t(share) * 2u * kRowsW * 16u;
   uint32_t smem = uint32_t(stages) * P.stage_bytes;
-  if (smem < exchange) smem = exchange;
+  if (!P.over_ring) smem += exchange;
+  else if (smem < exchange) smem = exchange;
   P.tmem_cols = 32;
   while (P.tmem_cols < uint32_t(mt)) P.tmem_cols *= 2;
   CUtensorMap map_w, map_a;
