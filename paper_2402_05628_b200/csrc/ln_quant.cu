@@ -256,9 +256,7 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
 
   const float inv_d = 1.f / float(D);
   const uint32_t qmax4 = uint32_t(qmax) * 0x01010101u;
-  constexpr uint32_t kMagicBits = 0x4B400000u;   // 1.5 * 2^23
-  const f32x2 magic2 = splat2(__uint_as_float(kMagicBits));
-  const int z_less_magic = z - int(kMagicBits);
+  const f32x2 tiny2 = splat2(__uint_as_float(1u)), z2 = splat2(z < 0 ? -__uint_as_float(uint32_t(-z)) : __uint_as_float(uint32_t(z)));
 
   // the warp's slice of a row, and the slice its lane merges
   const int lane_w = threadIdx.x & 31;
@@ -417,10 +415,11 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
           if (!guard) {
 #pragma unroll
             for (int e = 0; e < kChunk / 2; ++e) {
+              const f32x2 t = fma2(normalised(v[r][i][e], r), g[e], b[e]);
               float u0, u1;
-              unpack2(add2(fma2(normalised(v[r][i][e], r), g[e], b[e]), magic2), u0, u1);
-              q[2 * e] = __float_as_int(u0) + z_less_magic;
-              q[2 * e + 1] = __float_as_int(u1) + z_less_magic;
+              unpack2(add2(mul2(t, tiny2), z2), u0, u1);
+              q[2 * e] = __float_as_int(u0);
+              q[2 * e + 1] = __float_as_int(u1);
             }
           } else {
             float t[kChunk];
