@@ -8,24 +8,25 @@
 // warp centres its slice on the slice's own mean, the means and squares are merged behind the barrier, and the code sums wait
 // for the next one.
 //
-// What bounds it: HBM for float input and for rows of one warp (5.1-6.3 TB/s of 6.46); for longer bf16 rows the latencies of a
-// row's chain at the 16 warps per SM that the registers leave (ncu, 32768 x 4096: DRAM 43 % of its peak, issue slots 56 %, first
-// stall the factors' reads from shared memory and the shuffles, then waits of known length; 76-80 us against 51 at the copy rate).
+// What bounds it: HBM for float input and for rows of one warp (5.1-6.3 TB/s of 6.46); for longer bf16 rows instructions and the latencies
+// of a row's chain at the 16 warps per SM that the registers leave (ncu, 32768 x 4096: 10.9 instructions per element, DRAM 43 % of its peak,
+// issue slots 56 %).  Calls of many rows of 2048 or 4096 elements take ln_rows_kernel below.
 // Measured against three barriers per iteration: 65536 bf16 rows of 1536 53 -> 45 us, 32768 float rows of 2048 83 -> 48, 16384 of
 // 4096 76 -> 49; 32768 bf16 rows of 4096 gained nothing (80).
 // The per-channel factors gamma~/s~ and beta~/s~ are staged once per CTA in shared memory (halves of the 8-element
 // chunks apart, so that a warp's 16-byte reads are free of bank conflicts).
 //
-// The float work runs on packed pairs (two elements per add / mul / fma issue slot).  Rounding is done by the
-// float adder: t + 1.5 * 2^23 leaves rint(t) (half to even, on t itself, as Eq. 4 has it) in the low mantissa
-// bits while |t| < 2^22; inputs that cannot guarantee that bound are clamped and converted with cvt.rni
-// instead.  z is added as an integer and the clip of Eq. 4 is the saturation of the packing instruction.
+// The float work runs on packed pairs (two elements per add / mul / fma issue slot).  t times 2^-149 is a denormal whose bit pattern is
+// rint(t) (half to even, on t itself, as Eq. 4 has it); z is added exactly as another denormal, and the clip of Eq. 4 is the saturation of
+// the packing instruction (negative values are negative integers, large ones are no longer denormals but large integers still).  Against
+// t + 1.5 * 2^23 and integer additions: 32768 x 4096 74.1 -> 72.7 us, 131072 x 1024 63.4 -> 60.7.
 #include <cuda_bf16.h>
 
 #include <type_traits>
 
 #include "f32x2.cuh"
 #include "kernels.h"
+#include "tc_ptx.cuh"
 
 namespace repq {
 namespace {
@@ -225,9 +226,10 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
 
   float* s_g = s_gb;
   float* s_b = s_gb + D;
-  // |t| <= sqrt(D) |gamma~/s~| + |beta~/s~|.  While that bound stays below 2^22 the round operation is one packed
-  // float add of 1.5 * 2^23 (round half to even by the adder, rint(t) left in the low mantissa bits); otherwise t
-  // is clamped and converted, so that adding z cannot wrap (a whole-kernel decision, taken here once).
+  // Rows of one warp keep a second form of the code for factors so large that |t| might reach 2^22: with the branch between the
+  // chunks their loop runs faster than without (100000 x 768 39.5 against 40.3 us, 60000 x 1536 46.0 and 47.9); longer rows do without it
+  // (16384 x 8192 67.9 and 65.0).  The two give the same codes, but for a NaN.
+  constexpr bool kGuard = !kWide;
   const float root_d = sqrtf(float(D));
   bool wide = false;
   // layout: the first halves (4 floats) of all chunks, then the second halves, so that the 16-byte reads of
@@ -241,11 +243,14 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
       const float bi[4] = {b4[k].x * inv_s, b4[k].y * inv_s, b4[k].z * inv_s, b4[k].w * inv_s};
       *reinterpret_cast<float4*>(s_g + at) = make_float4(gi[0], gi[1], gi[2], gi[3]);
       *reinterpret_cast<float4*>(s_b + at) = make_float4(bi[0], bi[1], bi[2], bi[3]);
+      if constexpr (kGuard) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) wide = wide || !(fabsf(gi[e]) * root_d + fabsf(bi[e]) < 4.0e6f);
+        for (int e = 0; e < 4; ++e) wide = wide || !(fabsf(gi[e]) * root_d + fabsf(bi[e]) < 4.0e6f);
+      }
     }
   }
-  const bool guard = __syncthreads_or(wide) != 0;
+  const bool guard = kGuard && __syncthreads_or(wide) != 0;
+  if (!kGuard) __syncthreads();
   // x and the outputs belong to the chain of kernels
   if (settled) {
     grid_dependency_wait();
@@ -478,6 +483,200 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
   }
 }
 
+
+// ---- bf16 rows of 2048 or 4096 elements, many of them: a row per warp
+//
+// With a row over several warps 4.4 of 10.9 instructions per element were what a row costs beside its elements (shuffles, merges, a barrier,
+// addresses, paid per warp), and 16 warps per SM waited for one another.  Here a lane holds all of a row's chunks of 8 elements that
+// its namesakes in the kSlices warps of ln_quant_kernel hold, as packed float pairs (64 or 128 registers), and there is no barrier in the
+// loop.  The registers leave no room for a row in flight, so a warp's next two rows are under way in shared memory, by one bulk copy
+// each.  A buffer is filled again one iteration after it was read: by then everything computed from it has been issued, so its loads
+// have returned.  The sums are formed slice by slice in the order of ln_quant_kernel, so that a row's codes do not depend on how many
+// rows share the call.
+// Input partly in L2, groups of warps -> this: 32768 x 4096 to packed codes 72.7 -> 59.0 us, to bytes 79.1 -> 65.5, 20000 x 4096 RMS 48.4 -> 44,
+// 65536 x 2048 68.6 -> 56.7.  A branch per chunk (to a second form for large factors, which the rounding into denormals does not
+// need) cost 10 us at 4096; eight warps of 200 registers 66.  Two rows per warp with half of a row each, which reads the factors half as
+// often, took 89 us: twelve warps are few, and each then waits on twice the work of one iteration.
+template <int kSlices> constexpr int row_warps() { return kSlices == 4 ? 12 : 20; }      // by 168 and 96 registers a thread
+template <int kSlices, bool kPack4>
+__global__ void __launch_bounds__(32 * row_warps<kSlices>(), 1)
+ln_rows_kernel(const __nv_bfloat16* __restrict__ x, uint32_t rows, int64_t ldx, const float* __restrict__ gamma_t,
+               const float* __restrict__ beta_t, float eps, int rms, float inv_s, int z, int qmax, uint8_t* __restrict__ codes, int64_t ldc,
+               int32_t* __restrict__ row_sum, int32_t* __restrict__ clear, int64_t n_clear, bool settled, int32_t* status) {
+  constexpr int kWarps = row_warps<kSlices>(), kBlock = 32 * kWarps, kPer = 4, kVPT = kSlices * kPer;
+  constexpr int D = 32 * kVPT * kChunk;
+  constexpr uint32_t kRowBytes = D * 2u;
+  extern __shared__ __align__(128) float s_gb[];         // gamma~/s~, beta~/s~ (halves of chunks apart), then two rows per warp
+  __shared__ alignas(8) uint64_t full[kWarps][2];
+  __shared__ volatile int abort;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t buf = tc::smem_u32(s_gb + 2 * D) + uint32_t(warp) * 2u * kRowBytes;
+  if (lane < 2) tc::mbar_init(tc::smem_u32(&full[warp][lane]), 1);
+  if (tid == 0) abort = 0;
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  __syncwarp();
+
+  constexpr int kPieces = D / 4;
+  const int rot = int(blockIdx.x * 32u % uint32_t(kPieces));
+  const bool vec = ((reinterpret_cast<uintptr_t>(gamma_t) | reinterpret_cast<uintptr_t>(beta_t)) & 15) == 0;
+  auto load4 = [&](const float* p) {
+    return vec ? __ldcg(reinterpret_cast<const float4*>(p)) : make_float4(__ldcg(p), __ldcg(p + 1), __ldcg(p + 2), __ldcg(p + 3));
+  };
+  const uint32_t stride = gridDim.x * kWarps, first = uint32_t(warp) * gridDim.x + blockIdx.x;
+  auto request = [&](uint32_t row, int k) {
+    if (lane == 0 && row < rows) {
+      const uint32_t bar = tc::smem_u32(&full[warp][k & 1]);
+      tc::mbar_expect_tx(bar, kRowBytes);
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                   ::"r"(buf + uint32_t(k & 1) * kRowBytes), "l"(x + int64_t(row) * ldx), "r"(kRowBytes), "r"(bar) : "memory");
+    }
+  };
+  auto begin = [&] {
+    grid_dependency_wait();
+    grid_dependency_trigger();
+    request(first, 0);
+    request(first + stride, 1);
+  };
+  if (!settled) begin();               // (factors that the kernel ahead may have written are read behind the wait, as in ln_quant_kernel)
+  for (int k = tid; k < kPieces; k += kBlock) {
+    const int q = (k + rot) % kPieces, at = (q & 1) * (D / 2) + (q >> 1) * 4;
+    const float4 g = load4(gamma_t + 4 * q), b = load4(beta_t + 4 * q);
+    *reinterpret_cast<float4*>(s_gb + at) = make_float4(g.x * inv_s, g.y * inv_s, g.z * inv_s, g.w * inv_s);
+    *reinterpret_cast<float4*>(s_gb + D + at) = make_float4(b.x * inv_s, b.y * inv_s, b.z * inv_s, b.w * inv_s);
+  }
+  __syncthreads();
+  if (settled) begin();
+  for (int64_t i = int64_t(blockIdx.x) * kBlock + tid; i < n_clear; i += int64_t(gridDim.x) * kBlock) clear[i] = 0;
+
+  // Totals over the lanes for every slice: the first steps of the tree split the slices between the halves of the warp (the pairs that
+  // are added are those of a tree per slice); lane l ends with slice l / 8 or l / 16.
+  auto totals = [&](const float (&t)[kSlices]) {
+    const bool high = lane & 16;
+    float u;
+    if constexpr (kSlices == 4) {
+      const float a = (high ? t[2] : t[0]) + __shfl_xor_sync(0xffffffffu, high ? t[0] : t[2], 16);
+      const float b = (high ? t[3] : t[1]) + __shfl_xor_sync(0xffffffffu, high ? t[1] : t[3], 16);
+      const bool next = lane & 8;
+      u = (next ? b : a) + __shfl_xor_sync(0xffffffffu, next ? a : b, 8);
+    } else {
+      u = (high ? t[1] : t[0]) + __shfl_xor_sync(0xffffffffu, high ? t[0] : t[1], 16);
+      u += __shfl_xor_sync(0xffffffffu, u, 8);
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
+    return u;
+  };
+  auto over_slices = [&](float u) {    // sum over the slices, in the order of their distance
+    u += __shfl_xor_sync(0xffffffffu, u, 16);
+    if constexpr (kSlices == 4) u += __shfl_xor_sync(0xffffffffu, u, 8);
+    return u;
+  };
+  constexpr float kSliceSize = float(32 * kPer * kChunk);
+  const float inv_d = 1.f / float(D);
+  const uint32_t qmax4 = uint32_t(qmax) * 0x01010101u;
+  const f32x2 tiny2 = splat2(__uint_as_float(1u)), z2 = splat2(z < 0 ? -__uint_as_float(uint32_t(-z)) : __uint_as_float(uint32_t(z)));
+  int k = 0;
+  uint32_t row = first;
+  for (; row < rows; row += stride, ++k) {
+    if (k > 0) request(row + stride, k + 1);
+    const bool came = tc::mbar_wait(tc::smem_u32(&full[warp][k & 1]), (k >> 1) & 1, &abort, 91, status);
+    if (!__all_sync(0xffffffffu, came)) break;
+    f32x2 v[kVPT][kChunk / 2];
+    const uint32_t at = buf + uint32_t(k & 1) * kRowBytes + uint32_t(lane) * 16u;
+#pragma unroll
+    for (int i = 0; i < kVPT; ++i) {
+      RawChunk<__nv_bfloat16> raw;
+      asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(raw.a.x), "=r"(raw.a.y), "=r"(raw.a.z), "=r"(raw.a.w) : "r"(at + uint32_t(i) * 512u));
+      expand(raw, v[i]);
+    }
+    // (a slice's mean, and later the rest of the way to the row's, stays with the lanes that own the slice and is fetched where it is
+    // used: 128 registers of values leave no room for all of them)
+    float t[kSlices], own_sum = 0.f;
+    if (!rms) {
+#pragma unroll
+      for (int w = 0; w < kSlices; ++w) {
+        f32x2 acc = 0ull;
+#pragma unroll
+        for (int i = w; i < kVPT; i += kSlices)
+#pragma unroll
+          for (int e = 0; e < kChunk / 2; ++e) acc = add2(acc, v[i][e]);
+        float lo, hi;
+        unpack2(acc, lo, hi);
+        t[w] = lo + hi;
+      }
+      own_sum = totals(t);
+    }
+    const float own_mean = own_sum * (1.f / kSliceSize);
+#pragma unroll
+    for (int w = 0; w < kSlices; ++w) {
+      const f32x2 neg_mu = splat2(-__shfl_sync(0xffffffffu, own_mean, (32 / kSlices) * w));
+      f32x2 acc = 0ull;
+#pragma unroll
+      for (int i = w; i < kVPT; i += kSlices)
+#pragma unroll
+        for (int e = 0; e < kChunk / 2; ++e) {
+          v[i][e] = add2(v[i][e], neg_mu);
+          acc = fma2(v[i][e], v[i][e], acc);
+        }
+      float lo, hi;
+      unpack2(acc, lo, hi);
+      t[w] = lo + hi;
+    }
+    const float mean = rms ? 0.f : over_slices(own_sum) * inv_d;
+    const float off = rms ? 0.f : own_mean - mean;
+    const float m2 = over_slices(fmaf(kSliceSize * off, off, totals(t)));
+    const float rs = rsqrtf(m2 * inv_d + eps);
+    const f32x2 rstd = splat2(rs);
+    const float own_rest = (own_mean - mean) * rs;
+    int csum[1] = {0};
+    uint8_t* out = codes + int64_t(row) * ldc;
+#pragma unroll
+    for (int w = 0; w < kSlices; ++w) {
+      const f32x2 rest = splat2(__shfl_sync(0xffffffffu, own_rest, (32 / kSlices) * w));
+#pragma unroll
+      for (int i = w; i < kVPT; i += kSlices) {
+        const int c = lane + 32 * i;
+        const float4 g0 = *reinterpret_cast<const float4*>(s_gb + c * 4), g1 = *reinterpret_cast<const float4*>(s_gb + D / 2 + c * 4);
+        const float4 b0 = *reinterpret_cast<const float4*>(s_gb + D + c * 4), b1 = *reinterpret_cast<const float4*>(s_gb + D + D / 2 + c * 4);
+        const f32x2 g[kChunk / 2] = {pack2(g0.x, g0.y), pack2(g0.z, g0.w), pack2(g1.x, g1.y), pack2(g1.z, g1.w)};
+        const f32x2 b[kChunk / 2] = {pack2(b0.x, b0.y), pack2(b0.z, b0.w), pack2(b1.x, b1.y), pack2(b1.z, b1.w)};
+        int q[kChunk];
+#pragma unroll
+        for (int e = 0; e < kChunk / 2; ++e) {
+          const f32x2 u = fma2(fma2(v[i][e], rstd, rest), g[e], b[e]);
+          float u0, u1;
+          unpack2(add2(mul2(u, tiny2), z2), u0, u1);
+          q[2 * e] = __float_as_int(u0);
+          q[2 * e + 1] = __float_as_int(u1);
+        }
+        if constexpr (kSlices == 4) __syncwarp();        // keeps the chunks apart: interleaved, they spill (67.7 us instead of 59.0)
+        if constexpr (kPack4) {
+          uint32_t p = 0;
+#pragma unroll
+          for (int e = kChunk - 2; e >= 0; e -= 2) p = push_pair_u4(q[e], q[e + 1], p);
+          reinterpret_cast<uint32_t*>(out)[c] = p;
+          csum[0] = int(__dp4a(p & 0x0F0F0F0Fu, 0x01010101u, __dp4a((p >> 4) & 0x0F0F0F0Fu, 0x01010101u, uint32_t(csum[0]))));
+        } else {
+          uint2 p;
+          p.x = __vminu4(push_pair_u8(q[0], q[1], push_pair_u8(q[2], q[3], 0u)), qmax4);      // 4- and 6-bit quantizers in byte containers
+          p.y = __vminu4(push_pair_u8(q[4], q[5], push_pair_u8(q[6], q[7], 0u)), qmax4);
+          reinterpret_cast<uint2*>(out)[c] = p;
+          csum[0] = int(__dp4a(p.x, 0x01010101u, __dp4a(p.y, 0x01010101u, uint32_t(csum[0]))));
+        }
+      }
+    }
+    if (row_sum != nullptr) {
+      group_sum<32, 1>(csum);
+      if (lane == 0) row_sum[row] = csum[0];
+    }
+  }
+  // given up: the copies under way must have landed before the block may exit
+  if (row < rows && lane == 0) {
+    tc::mbar_drain(tc::smem_u32(&full[warp][k & 1]), (k >> 1) & 1);
+    if (row + stride < rows) tc::mbar_drain(tc::smem_u32(&full[warp][(k + 1) & 1]), ((k + 1) >> 1) & 1);
+  }
+}
+
 template <typename T>
 struct Call {
   const T* x;
@@ -518,6 +717,25 @@ repq_status launch(const Call<T>& c, cudaStream_t st) {
   return REPQ_OK;
 }
 
+template <int kSlices, bool kPack4>
+repq_status launch_rows(const Call<__nv_bfloat16>& c, cudaStream_t st) {
+  constexpr int kWarps = row_warps<kSlices>(), kD = 1024 * kSlices, kSmem = kD * 8 + kWarps * 2 * kD * 2;
+  static_assert(kSmem <= 226 * 1024, "rows and factors exceed shared memory");
+  REPQ_TRY((allow_smem<ln_rows_kernel<kSlices, kPack4>>(kSmem)));
+  int32_t* status = device_status_word();
+  REPQ_REQUIRE(status != nullptr, REPQ_CUDA_ERROR, "ln_quant: device status word unavailable");
+  REPQ_CUDA(launch_chained(ln_rows_kernel<kSlices, kPack4>, dim3(sm_count()), dim3(32 * kWarps), size_t(kSmem), st, c.x, uint32_t(c.rows), c.ldx, c.gamma_t,
+                           c.beta_t, c.eps, c.rms, 1.f / c.s_t, c.z, code_max(c.bits), c.codes, c.ldc, c.row_sum, c.clear.at, c.clear.n,
+                           c.settled, status));
+  note_launch();
+  return REPQ_OK;
+}
+// Rows of a call from which a row per warp is ahead: about four and a half turns of the warps at 4096 elements (4096 rows 12.7 us by groups of
+// warps, 14.9 by single ones, 7000 18.3 and 19.3, 8192 23.2 and 21.7, 10000 24.9 and 23.8), five at 2048 (14000 17.3 and 17.6, 16000 22.0
+// and 20.0).  3072 elements gained nothing (63.9 and 63.8), rows that do not fill the chunks lost.
+template <int kSlices>
+bool many_rows(int64_t rows) { return rows < (int64_t(1) << 31) && 2 * rows >= int64_t(kSlices == 4 ? 9 : 10) * row_warps<kSlices>() * sm_count(); }
+
 // Chunks per thread kVPT .. kMost, the row lengths that narrower groups leave to groups of TPR threads.
 template <typename T, int TPR, int kVPT, int kMost>
 repq_status launch_group(const Call<T>& c, cudaStream_t st) {
@@ -538,6 +756,10 @@ repq_status dispatch(const Call<T>& c, cudaStream_t st) {
   if (nchunks <= 8 * 4) return launch_group<T, 8, 1, 4>(c, st);
   if (nchunks <= 16 * 4) return launch_group<T, 16, 3, 4>(c, st);
   if (nchunks <= 32 * 6) return launch_group<T, 32, 3, 6>(c, st);
+  if constexpr (sizeof(T) == 2) {
+    if (c.D == 2048 && many_rows<2>(c.rows)) return packed4(c.bits) ? launch_rows<2, true>(c, st) : launch_rows<2, false>(c, st);
+    if (c.D == 4096 && many_rows<4>(c.rows)) return packed4(c.bits) ? launch_rows<4, true>(c, st) : launch_rows<4, false>(c, st);
+  }
   if (nchunks <= 64 * 6) return launch_group<T, 64, 4, 6>(c, st);
   if (nchunks <= 128 * 6) return launch_group<T, 128, 4, 6>(c, st);
   if (nchunks <= 256 * 4) return launch_group<T, 256, 4, 4>(c, st);
