@@ -9,7 +9,9 @@ namespace repq {
 // no, like every other operand they may be the work of the kernel just ahead in the stream (the entry points of the library
 // promise stream order).  `settled`: a kernel of the same chain that waited for everything before the chain has started
 // already, so whatever wrote the parameters has completed (the kernels of a block behind its first one).
-enum class Params { streamed, settled };
+// `beside` (the first LayerNorm of a block): the kernel just ahead in the stream has waited for everything before it and does work that
+// this kernel does not need; the two run side by side, and this kernel ends only when the one ahead has.
+enum class Params { streamed, settled, beside };
 
 // LayerNorm + quantization (repq_ln_quant), which can also set a run of words to zero: row-sum accumulators that later
 // kernels of a chain add into, without a launch of their own.
@@ -56,6 +58,14 @@ repq_status qgemm_tc(const repq_gemm_desc& d, const EpilogueParams& ep, const Tc
 struct SkinnyPlan { int mt = 0, split = 0; float us = 0.f; };
 SkinnyPlan qgemm_skinny_plan(const repq_gemm_desc& d);
 repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, const SkinnyPlan& plan, Params params, cudaStream_t st);
+
+// Packed weights of a plain product in the form the GEMM kernels take, one code per byte: the same problem on byte codes (its w_codes still
+// to be set), the scratch it needs then and the bytes of its weights.  False: the problem has no such form.
+bool qgemm_byte_form(const repq_gemm_desc& d, repq_gemm_desc* as_bytes, size_t* scratch, size_t* bytes);
+// The packed weights of several products written in that form by one kernel, which reads them behind its dependency wait.
+constexpr int kMostExpansions = 4;
+struct Expansion { const uint8_t* src; int rows, k; int64_t ld_src; uint8_t* dst; int64_t ld_dst; };
+repq_status launch_expand_all(const Expansion* e, int n, int bits, cudaStream_t st);
 
 // Workspace of a GEMM: with room for a byte copy of packed weights, and the least it can run in.
 size_t qgemm_workspace(const repq_gemm_desc& d);

@@ -136,7 +136,8 @@ __global__ void __launch_bounds__((TPR > 256 ? TPR : 256), min_blocks(kVPT, TPR,
 ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
                 const float* __restrict__ gamma_t, const float* __restrict__ beta_t, float eps, int rms,
                 float inv_s, int z, int qmax, uint8_t* __restrict__ codes, int64_t ldc,
-                int32_t* __restrict__ row_sum, int32_t* __restrict__ clear, int64_t n_clear, bool settled) {
+                int32_t* __restrict__ row_sum, int32_t* __restrict__ clear, int64_t n_clear, Params params) {
+  const bool settled = params == Params::settled, beside = params == Params::beside;
   constexpr int kRows = rows_in_flight(kVPT, TPR, sizeof(T));
   constexpr int kBlock = TPR > 256 ? TPR : 256;
   constexpr int kGroups = kBlock / TPR;
@@ -193,7 +194,7 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
     return q < n4 ? q : q - n4;
   };
   if (!settled) {
-    grid_dependency_wait();
+    if (!beside) grid_dependency_wait();
     grid_dependency_trigger();
   }
   float4 g4[kPieces], b4[kPieces];
@@ -481,6 +482,7 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
       }
     }
   }
+  if (beside) grid_dependency_wait();
 }
 
 
@@ -502,7 +504,8 @@ template <int kSlices, bool kPack4>
 __global__ void __launch_bounds__(32 * row_warps<kSlices>(), 1)
 ln_rows_kernel(const __nv_bfloat16* __restrict__ x, uint32_t rows, int64_t ldx, const float* __restrict__ gamma_t,
                const float* __restrict__ beta_t, float eps, int rms, float inv_s, int z, int qmax, uint8_t* __restrict__ codes, int64_t ldc,
-               int32_t* __restrict__ row_sum, int32_t* __restrict__ clear, int64_t n_clear, bool settled, int32_t* status) {
+               int32_t* __restrict__ row_sum, int32_t* __restrict__ clear, int64_t n_clear, Params params, int32_t* status) {
+  const bool settled = params == Params::settled, beside = params == Params::beside;
   constexpr int kWarps = row_warps<kSlices>(), kBlock = 32 * kWarps, kPer = 4, kVPT = kSlices * kPer;
   constexpr int D = 32 * kVPT * kChunk;
   constexpr uint32_t kRowBytes = D * 2u;
@@ -532,7 +535,7 @@ ln_rows_kernel(const __nv_bfloat16* __restrict__ x, uint32_t rows, int64_t ldx, 
     }
   };
   auto begin = [&] {
-    grid_dependency_wait();
+    if (!beside) grid_dependency_wait();
     grid_dependency_trigger();
     request(first, 0);
     request(first + stride, 1);
@@ -675,6 +678,7 @@ ln_rows_kernel(const __nv_bfloat16* __restrict__ x, uint32_t rows, int64_t ldx, 
     tc::mbar_drain(tc::smem_u32(&full[warp][k & 1]), (k >> 1) & 1);
     if (row + stride < rows) tc::mbar_drain(tc::smem_u32(&full[warp][(k + 1) & 1]), ((k + 1) >> 1) & 1);
   }
+  if (beside) grid_dependency_wait();
 }
 
 template <typename T>
@@ -692,7 +696,7 @@ struct Call {
   int64_t ldc;
   int32_t* row_sum;
   ClearWords clear;
-  bool settled;
+  Params params;
 };
 
 template <typename T, int TPR, int kVPT, bool kPack4, bool kFull>
@@ -712,7 +716,7 @@ repq_status launch(const Call<T>& c, cudaStream_t st) {
   const int64_t cap = int64_t(sm_count()) * resident;
   const int grid = int(need < cap ? need : cap);
   REPQ_CUDA(launch_chained(kern, dim3(grid), dim3(kBlock), smem, st, c.x, c.rows, c.D, c.ldx, c.gamma_t, c.beta_t, c.eps, c.rms, 1.f / c.s_t,
-                           c.z, code_max(c.bits), c.codes, c.ldc, c.row_sum, c.clear.at, c.clear.n, c.settled));
+                           c.z, code_max(c.bits), c.codes, c.ldc, c.row_sum, c.clear.at, c.clear.n, c.params));
   note_launch();
   return REPQ_OK;
 }
@@ -726,7 +730,7 @@ repq_status launch_rows(const Call<__nv_bfloat16>& c, cudaStream_t st) {
   REPQ_REQUIRE(status != nullptr, REPQ_CUDA_ERROR, "ln_quant: device status word unavailable");
   REPQ_CUDA(launch_chained(ln_rows_kernel<kSlices, kPack4>, dim3(sm_count()), dim3(32 * kWarps), size_t(kSmem), st, c.x, uint32_t(c.rows), c.ldx, c.gamma_t,
                            c.beta_t, c.eps, c.rms, 1.f / c.s_t, c.z, code_max(c.bits), c.codes, c.ldc, c.row_sum, c.clear.at, c.clear.n,
-                           c.settled, status));
+                           c.params, status));
   note_launch();
   return REPQ_OK;
 }
@@ -792,7 +796,7 @@ repq_status launch_ln_quant(const void* x, int x_dtype, int64_t rows, int D, int
   auto run = [&](auto* typed) {
     return dispatch(Call<std::remove_const_t<std::remove_pointer_t<decltype(typed)>>>{
         typed, rows, D, ldx, gamma_t, beta_t, eps, norm_kind == REPQ_NORM_RMS, s_t, z_t, bits, codes, ld_codes_bytes, row_sum, clear,
-        params == Params::settled}, st);
+        params}, st);
   };
   return x_dtype == REPQ_F32 ? run(static_cast<const float*>(x)) : run(static_cast<const __nv_bfloat16*>(x));
 }

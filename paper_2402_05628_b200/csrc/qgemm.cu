@@ -147,6 +147,42 @@ __global__ void __launch_bounds__(256) expand_weights_kernel(const uint8_t* __re
   if (!waited) grid_dependency_wait();
 }
 
+// The same for several matrices, as one run of 64-code units.  Everything is read and written behind the dependency wait, and the next
+// kernel may start as soon as that is over.
+struct ExpandSet {
+  const uint8_t* src[kMostExpansions]; uint8_t* dst[kMostExpansions];
+  int64_t ld_src[kMostExpansions], ld_dst[kMostExpansions];
+  int groups[kMostExpansions], end[kMostExpansions];       // units of a row; units up to the end of this matrix
+};
+template <int kBits>
+__global__ void __launch_bounds__(256) expand_all_kernel(const __grid_constant__ ExpandSet E) {
+  constexpr int kIn = 8 * kBits;
+  grid_dependency_wait();
+  grid_dependency_trigger();
+  for (int u = int(blockIdx.x) * 256 + int(threadIdx.x); u < E.end[kMostExpansions - 1]; u += int(gridDim.x) * 256) {
+    const uint8_t* src = E.src[0];
+    uint8_t* dst = E.dst[0];
+    int64_t ld_src = E.ld_src[0], ld_dst = E.ld_dst[0];
+    int groups = E.groups[0], first = 0;
+#pragma unroll
+    for (int m = 1; m < kMostExpansions; ++m)
+      if (u >= E.end[m - 1]) { src = E.src[m]; dst = E.dst[m]; ld_src = E.ld_src[m]; ld_dst = E.ld_dst[m]; groups = E.groups[m]; first = E.end[m - 1]; }
+    const int r = (u - first) / groups, g = u - first - r * groups;
+    uint32_t w[2 * kBits], o[16];
+#pragma unroll
+    for (int q = 0; q < kIn / 16; ++q) {                   // (a row ends on a 16-byte boundary)
+      uint4 v = make_uint4(0u, 0u, 0u, 0u);
+      if (int64_t(g) * kIn + 16 * q < ld_src) v = __ldcg(reinterpret_cast<const uint4*>(src + r * ld_src + int64_t(g) * kIn) + q);
+      w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
+    }
+    expand_words<kBits>(w, o);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (int64_t(g) * 64 + 16 * q < ld_dst)
+        *(reinterpret_cast<uint4*>(dst + r * ld_dst + int64_t(g) * 64) + q) = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+  }
+}
+
 // The byte form of packed weights in the caller's workspace, where it has the room (repq_qgemm_workspace_bytes asks for it): one
 // pass over the weights, after which every GEMM kernel takes them.  The GEMM that expands the tiles it copies (bound by its
 // converters' shared-memory traffic, once per row tile) remains for smaller workspaces.  Measured (packed against that form):
@@ -266,6 +302,34 @@ EpilogueParams make_epilogue(const repq_gemm_desc& d) {
 }
 
 }  // namespace
+
+bool qgemm_byte_form(const repq_gemm_desc& d, repq_gemm_desc* as_bytes, size_t* scratch, size_t* bytes) {
+  ByteWeights B;
+  if (!byte_weights(d, as_bytes, &B)) return false;
+  *scratch = B.offset;
+  *bytes = B.total - B.offset;
+  return true;
+}
+
+repq_status launch_expand_all(const Expansion* e, int n, int bits, cudaStream_t st) {
+  ExpandSet E{};
+  int64_t units = 0;
+  for (int m = 0; m < kMostExpansions; ++m) {
+    if (m < n) {
+      E.src[m] = e[m].src; E.dst[m] = e[m].dst; E.ld_src[m] = e[m].ld_src; E.ld_dst[m] = e[m].ld_dst;
+      E.groups[m] = (e[m].k + 63) / 64;
+      units += int64_t(e[m].rows) * E.groups[m];
+    }
+    E.end[m] = int(units);
+  }
+  REPQ_REQUIRE(units < (int64_t(1) << 30), REPQ_UNSUPPORTED, "qgemm: too many weights to expand at once");
+  // (four blocks per SM: they leave room for the kernel that runs beside this one)
+  const int64_t blocks = (units + 255) / 256, most = int64_t(sm_count()) * 4;
+  auto kern = packed4(bits) ? expand_all_kernel<4> : expand_all_kernel<6>;
+  REPQ_CUDA(launch_chained(kern, dim3(unsigned(blocks < most ? blocks : most)), dim3(256), 0, st, E));
+  note_launch();
+  return REPQ_OK;
+}
 
 size_t qgemm_workspace_least(const repq_gemm_desc& d) {
   return !scores_supported(d) && qgemm_tc_supported(d) ? qgemm_tc_workspace(d) : 0;
