@@ -263,6 +263,28 @@ __device__ __forceinline__ uint32_t code_word(const ChunkQuant& q, f32x2 r01, f3
   const uint32_t p = push_pair_u8(__float_as_int(u0), __float_as_int(u1), push_pair_u8(__float_as_int(u2), __float_as_int(u3), 0u));
   return (p >> q.shift) & q.mask;
 }
+// 16 lanes x 32 columns of the accumulator: thread t gets columns 8 g + 2 (t % 4) + {0, 1} of lane t / 4 in r[4 g + {0, 1}], of lane
+// t / 4 + 8 in r[4 g + {2, 3}].
+__device__ __forceinline__ void tmem_ld_quads(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr) : "memory");
+}
+// A lane holds two bytes (columns 2 j + {0, 1}, j = lane % 4) of each of four groups of eight columns, groups 0 and 1 in w0, 2 and 3 in
+// w1; its quad holds 32 columns of a row.  Afterwards lane q has group q's eight bytes.
+__device__ __forceinline__ void quad_bytes(uint32_t w0, uint32_t w1, bool b0, bool b1, uint32_t& lo, uint32_t& hi) {
+  const uint32_t keep = b1 ? w1 : w0, got = __shfl_xor_sync(0xffffffffu, b1 ? w0 : w1, 2);
+  // keep: this lane's bytes of groups 2 b1 + {0, 1}; got: those of lane q ^ 2
+  const uint32_t mine = __byte_perm(keep, got, b0 ? 0x7632 : 0x5410), other = __shfl_xor_sync(0xffffffffu, __byte_perm(keep, got, b0 ? 0x5410 : 0x7632), 1);
+  // mine: group q from lanes q (low half) and q ^ 2; other: from lanes q ^ 1 and q ^ 3
+  const uint32_t even = b0 ? other : mine, odd = b0 ? mine : other;        // from the quad's even lanes, from its odd ones
+  const uint32_t first = b1 ? 0x7632 : 0x5410, second = b1 ? 0x5410 : 0x7632;
+  lo = __byte_perm(even, odd, first);                                      // lanes 0, 1
+  hi = __byte_perm(even, odd, second);                                     // lanes 2, 3
+}
 __device__ __forceinline__ void sts64(uint32_t addr, uint32_t a, uint32_t b) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
@@ -766,7 +788,72 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         if (!mbar_wait(res_bar, uint32_t(it) & 1u, abort, 6)) break;
         res_pending = false;
       }
-      if (fast) {
+      // Plain epilogues to byte codes: a thread takes two columns of each eight, of four rows, instead of all columns of one row, and reads
+      // a quarter of the column terms (16 bytes a column; reads of shared memory paced the chunk loop, 45 % of its wavefronts).  The
+      // bytes of a row then meet in one lane of its quad by two shuffles.  12608 x 2304 x 768 24.5 -> 24.3 us, block pass of 64 x 197
+      // tokens 186.9 -> 183.5; with GELU, where instructions set the pace, the shuffles cost more (12608 x 3072 x 768 43.0 and 44.1).
+      constexpr bool kQuads = OUT == kOutC8 && PAIR == kPairNone && !RES && !W4 && EPI == kEpiPlain;
+      // the row whose code sum the thread holds in the end
+      int64_t m_sum = m;
+      if (kQuads && fast) {
+        const int row_q = lane >> 2, col_q = 2 * (lane & 3);
+        const bool b0 = lane & 1, b1 = lane & 2;
+        int as[4], sums[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) as[k] = C.asum[quarter * 32 + row_q + 8 * k];
+        const uint32_t buf = smem_u32(S.epi[ew]);
+#pragma unroll 1
+        for (int cp = 0; cp < 2; ++cp) {
+          const int cl = cl0 + 32 * cp;
+          uint32_t r[2][16];
+          tmem_ld_quads(taddr0 + 32 * cp, r[0]);
+          tmem_ld_quads(taddr0 + (16u << 16) + 32 * cp, r[1]);
+          tmem_ld_wait(r[0]);
+          tmem_ld_wait(r[1]);
+          uint32_t w[2][4];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const ChunkQuant& q = C.quant[cl / kChunk + h];
+            f32x2 t[2][4];                               // [group of the chunk][row]
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const int g = 2 * h + u, at = cl + 8 * g + col_q;
+              const float2 sc = *reinterpret_cast<const float2*>(&C.sc[at]), bi = *reinterpret_cast<const float2*>(&C.bi[at]);
+              const int2 nz = *reinterpret_cast<const int2*>(&C.nzw[at]), kw = *reinterpret_cast<const int2*>(&C.kw[at]);
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                const int a0 = int(r[k >> 1][4 * g + 2 * (k & 1)]), a1 = int(r[k >> 1][4 * g + 2 * (k & 1) + 1]);
+                t[u][k] = fma2(pack2(sc.x, sc.y), pack2(float(a0 + nz.x * as[k] + kw.x), float(a1 + nz.y * as[k] + kw.y)), pack2(bi.x, bi.y));
+              }
+            }
+            const f32x2 magic2 = splat2(__uint_as_float(kMagicBits)), mult2 = splat2(q.mult);
+            const bool scaled = direct || !sat;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              f32x2 x0 = t[0][k], x1 = t[1][k];
+              if (!direct && !sat) { x0 = mul2(x0, mult2); x1 = mul2(x1, mult2); }
+              w[h][k] = code_word(q, scaled ? add2(x0, magic2) : fma2(x0, mult2, magic2), scaled ? add2(x1, magic2) : fma2(x1, mult2, magic2));
+              sums[k] = int(__dp4a(w[h][k], 0x01010101u, uint32_t(sums[k])));
+            }
+          }
+          box_begin(lane);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            uint32_t lo, hi;
+            quad_bytes(w[0][k], w[1][k], b0, b1, lo, hi);
+            const int row = row_q + 8 * k;               // 16-byte slot j of row r sits at r * 32 + ((j ^ ((r >> 2) & 1)) << 4)
+            sts64(buf + uint32_t(row) * 32u + ((uint32_t((lane & 3) >> 1) ^ uint32_t((row >> 2) & 1)) << 4) + uint32_t(lane & 1) * 8u, lo, hi);
+          }
+          box_end(&map_out, buf, lane, n0 + cl, m0 + quarter * 32);
+        }
+        // a row's sum over its quad: lane q of the quad ends with row row_q + 8 q
+        {
+          const int k0 = b0 ? sums[1] : sums[0], s0 = b0 ? sums[0] : sums[1], k1 = b0 ? sums[3] : sums[2], s1 = b0 ? sums[2] : sums[3];
+          const int a = k0 + __shfl_xor_sync(0xffffffffu, s0, 1), b = k1 + __shfl_xor_sync(0xffffffffu, s1, 1);
+          code_sum = (b1 ? b : a) + __shfl_xor_sync(0xffffffffu, b1 ? a : b, 2);
+          m_sum = int64_t(m0) + quarter * 32 + row_q + 8 * (lane & 3);
+        }
+      } else if (!kQuads && fast) {
         // (two chunks per trip: unrolled further, the 16 values of four chunks in flight spill at 96 registers)
         static_assert(kSliceChunks % 2 == 0, "the chunk loop takes two chunks per trip");
 #pragma unroll 1
@@ -908,7 +995,7 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         else mbar_arrive(smem_u32(&S.tmem_empty[acc]));
       }
       fetch_residual(tile + tile_step);               // every lane has read this tile's box (the __syncwarp above)
-      if (ep.out_row_sum != nullptr && row_ok && code_sum != 0) atomicAdd(ep.out_row_sum + m, code_sum);
+      if (ep.out_row_sum != nullptr && m_sum < P.M && code_sum != 0) atomicAdd(ep.out_row_sum + m_sum, code_sum);
     }
     if (RES && res_pending) mbar_drain(res_bar, uint32_t(it) & 1u);              // left the loop early: the copy must land
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");     // bulk stores complete
