@@ -74,9 +74,11 @@ __device__ __forceinline__ ColumnTerms column_terms(const EpilogueParams& p, int
 //     erfc(t) = 2^(-t q(t)),   Phi(v) = h for v < 0,   1 - h otherwise,   h = erfc(t) / 2 = 2^(-t q(t) - 1),
 // so v Phi(v) = max(v, 0) - |v| h, one multiply-add (a select between h and 1 - h, then a product: 12608 x 3072 x 768 42.7 us, 41.5 so),
 // and q, which is smooth (q(0) = 2 / (sqrt(pi) ln 2), q(t) ~ t / ln 2), is a degree-6 polynomial fitted so that
-// the error of erf stays below 1e-7.  Against the float64 erf form the float32 result is within 1.2e-7 |v|, and within 2e-7 of itself
-// for v > 0; of the small values of the negative tail it is off by 1.5e-6 at -2, 3e-5 at -3, 1.2e-3 at -4 and 10 % at the clamp
-// (1.6e-7 in absolute terms at most).
+// the error of erf stays below 1e-7.  It is evaluated in n = -|v| directly: -t q(t) = n p(n) with p(n) = q(-n / sqrt2) / sqrt2, whose
+// coefficients are q's times powers of 1 / sqrt2 (one product less per value: 12608 x 3072 x 768 43.2 -> 41.8 us, 18464 x 4096 x 1024 76.8 ->
+// 74.2).  Against the float64 erf form the float32 result is within 1.2e-7 |v| (4 million values: 1.09e-7, 1.12e-7 by way of t), and
+// within 2e-7 of itself for v > 0; of the small values of the negative tail it is off by 1e-6 at -2, 3e-5 at -3, 1.2e-3 at -4 and 10 % at the
+// clamp (1.6e-7 in absolute terms at most).
 constexpr float kGeluLow = -5.65685424949238f;                               // -4 sqrt2
 __device__ __forceinline__ float max_nan(float a, float b) {                 // (fmaxf drops a NaN)
   float d;
@@ -84,16 +86,16 @@ __device__ __forceinline__ float max_nan(float a, float b) {                 // 
   return d;
 }
 __device__ __forceinline__ float gelu_erf(float v) {
-  const float n = fmaxf(fminf(v, -v), kGeluLow), t = n * -0.70710678118654752f;
-  float q = -1.002269491e-04f;
-  q = fmaf(q, t, 4.616116930e-04f);
-  q = fmaf(q, t, 2.302142326e-03f);
-  q = fmaf(q, t, -2.945240214e-02f);
-  q = fmaf(q, t, 1.489636004e-01f);
-  q = fmaf(q, t, 9.183286428e-01f);
-  q = fmaf(q, t, 1.627913713e+00f);
+  const float n = fmaxf(fminf(v, -v), kGeluLow);                             // -|v|, clamped; -t q(t) = n p(n)
+  float p = -8.858894034e-06f;
+  p = fmaf(p, n, -5.770146163e-05f);
+  p = fmaf(p, n, 4.069651186e-04f);
+  p = fmaf(p, n, 7.363100536e-03f);
+  p = fmaf(p, n, 5.266658589e-02f);
+  p = fmaf(p, n, -4.591643214e-01f);
+  p = fmaf(p, n, 1.151108861e+00f);
   float h;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(h) : "f"(fmaf(-t, q, -1.f)));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(h) : "f"(fmaf(n, p, -1.f)));
   return fmaf(n, h, max_nan(v, 0.f));
 }
 
@@ -101,18 +103,17 @@ __device__ __forceinline__ float gelu_erf(float v) {
 // the operations of gelu_erf in the same order, so the results are the same bits.
 __device__ __forceinline__ void gelu_erf_pair(float& v0, float& v1) {
   const f32x2 n = pack2(fmaxf(fminf(v0, -v0), kGeluLow), fmaxf(fminf(v1, -v1), kGeluLow));
-  const f32x2 t = mul2(n, splat2(-0.70710678118654752f));
-  f32x2 q = splat2(-1.002269491e-04f);
-  q = fma2(q, t, splat2(4.616116930e-04f));
-  q = fma2(q, t, splat2(2.302142326e-03f));
-  q = fma2(q, t, splat2(-2.945240214e-02f));
-  q = fma2(q, t, splat2(1.489636004e-01f));
-  q = fma2(q, t, splat2(9.183286428e-01f));
-  q = fma2(q, t, splat2(1.627913713e+00f));
+  f32x2 p = splat2(-8.858894034e-06f);
+  p = fma2(p, n, splat2(-5.770146163e-05f));
+  p = fma2(p, n, splat2(4.069651186e-04f));
+  p = fma2(p, n, splat2(7.363100536e-03f));
+  p = fma2(p, n, splat2(5.266658589e-02f));
+  p = fma2(p, n, splat2(-4.591643214e-01f));
+  p = fma2(p, n, splat2(1.151108861e+00f));
   float e0, e1, h0, h1;
-  unpack2(fma2(t, q, splat2(1.f)), e0, e1);                                  // fma(-t, q, -1) = -fma(t, q, 1)
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(h0) : "f"(-e0));
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(h1) : "f"(-e1));
+  unpack2(fma2(n, p, splat2(-1.f)), e0, e1);
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(h0) : "f"(e0));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(h1) : "f"(e1));
   unpack2(fma2(n, pack2(h0, h1), pack2(max_nan(v0, 0.f), max_nan(v1, 0.f))), v0, v1);
 }
 
