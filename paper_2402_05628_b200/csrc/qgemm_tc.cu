@@ -78,40 +78,42 @@ struct alignas(16) ChunkQuant {
 
 // What the epilogue needs beside the accumulators of a tile, prepared one tile ahead by a warp of its own (by every epilogue warp
 // for its own 64 columns the same work took 2000-2200 of 7300 cycles per tile at K = 768).
+template <int BN>
 struct alignas(16) TileTerms {
-  int32_t nzw[kMaxBN];  // -z_w[j]
-  int32_t kw[kMaxBN];   // -z_a * wsum[j]
-  float sc[kMaxBN];     // alpha s_a s_w[j]   (times 1/s_o in direct re-quantization mode)
-  float bi[kMaxBN];     // bias[j]            (times 1/s_o in direct re-quantization mode)
+  int32_t nzw[BN];      // -z_w[j]
+  int32_t kw[BN];       // -z_a * wsum[j]
+  float sc[BN];         // alpha s_a s_w[j]   (times 1/s_o in direct re-quantization mode)
+  float bi[BN];         // bias[j]            (times 1/s_o in direct re-quantization mode)
   int32_t asum[BM];     // row sum - K z_a
   int32_t pos[BM];      // rotary embedding: the row's position
-  ChunkQuant quant[kMaxBN / kChunk];
+  ChunkQuant quant[BN / kChunk];
   int32_t m0, n0;       // first row (of this CTA) and column
 };
 
 constexpr uint32_t kResBytes = 32 * 128;            // bf16 residual of one warp and tile: 32 rows x 64 columns
 
 // RES (bf16 output with a bf16 residual, tiles of at most 192 columns): the residual of a tile comes in by bulk tensor
-// copies, one 32 x 64 box per epilogue warp, asked for one tile ahead; the output values are written over the residual
+// copies, one 32 x 64 box per epilogue warp, asked for one tile ahead (RES = 1: into the box that this tile has left from; RES = 2: into
+// the other of two, before this tile's epilogue); the output values are written over the residual
 // values they were computed from and the box leaves by one bulk tensor store (no staging buffer beside it)
 // WP: 0 = weight tiles arrive as bytes; 4 / 6 = packed (64 / 96 bytes per row of 128 codes), expanded by the converters
-template <int BN, bool RES, int WP, bool TWO = false>
+template <int BN, int RES, int WP, bool TWO = false>
 struct SharedStorage {
   static constexpr bool W4 = WP != 0;               // (any packed form)
   // kStages: ring of the bulk copies (activation tile + weight tile as it arrives).  kStagesB: ring of byte weight
   // tiles the MMA reads: the same ring when the weights arrive as bytes; with packed weights a short ring of its own
   // (the hop from converter to MMA is short), which leaves room for a deeper copy ring ahead of the converters.
-  static constexpr int kStages = TWO ? 6 : WP == 4 ? 5 : 4;
+  static constexpr int kStages = TWO ? 6 : WP == 4 ? 5 : RES == 2 && BN == 192 ? 3 : 4;
   static constexpr int kPackedRow = BK * (WP ? WP : 8) / 8;        // bytes of a packed tile row
   static constexpr int kStagesB = W4 ? 2 : kStages;
   static constexpr int kEpi = W4 ? kEpiWarpsW4 : kEpiWarps;
   alignas(1024) uint8_t a[kStages][kABytes];
   static constexpr int kBRows = TWO ? BN / 2 : BN;                // weight rows of this CTA's stage (a pair: half of the tile's)
   alignas(1024) uint8_t b[kStagesB][kBRows * BK];
-  alignas(1024) uint8_t res[RES ? (BN / kSliceCols) * 4 * kResBytes : 1024];   // one box per active epilogue warp
-  uint64_t res_full[kEpiWarps];
-  alignas(1024) uint8_t epi[RES ? 1 : kEpi][1024]; // per-warp staging box of the epilogue's bulk stores (RES: the residual box itself)
-  TileTerms terms[2];
+  alignas(1024) uint8_t res[RES ? RES * (BN / kSliceCols) * 4 * kResBytes : 1024];   // RES boxes per active epilogue warp
+  uint64_t res_full[2][kEpiWarps];
+  alignas(RES ? 16 : 1024) uint8_t epi[RES ? 1 : kEpi][RES ? 16 : 1024]; // per-warp staging box of the epilogue's bulk stores (RES: the residual box itself)
+  TileTerms<BN> terms[2];
   alignas(128) uint8_t bp[W4 ? kStages : 1][W4 ? BN * kPackedRow : 128];   // packed weight tiles: unswizzled rows
   alignas(8) uint64_t full[kStages];
   uint64_t empty[kStages];
@@ -125,9 +127,9 @@ struct SharedStorage {
   volatile int abort;
 };
 
-static_assert(sizeof(SharedStorage<kMaxBN, false, 0>) <= 227 * 1024 && sizeof(SharedStorage<kMaxBNW4, false, 4>) <= 227 * 1024 &&
-              sizeof(SharedStorage<kMaxBNW4, false, 6>) <= 227 * 1024 && sizeof(SharedStorage<192, true, 0>) <= 227 * 1024 &&
-              sizeof(SharedStorage<kMaxBN, false, 0, true>) <= 227 * 1024,
+static_assert(sizeof(SharedStorage<kMaxBN, 0, 0>) <= 227 * 1024 && sizeof(SharedStorage<kMaxBNW4, 0, 4>) <= 227 * 1024 &&
+              sizeof(SharedStorage<kMaxBNW4, 0, 6>) <= 227 * 1024 && sizeof(SharedStorage<192, 2, 0>) <= 227 * 1024 &&
+              sizeof(SharedStorage<kMaxBN, 0, 0, true>) <= 227 * 1024,
               "shared storage exceeds the 227 KB a CTA may use");
 
 using namespace tc;
@@ -191,7 +193,7 @@ struct TcParams {
   int w_packed4;               // weight tiles arrive packed (4: two codes per byte, 6: four in three bytes) and are
                                // expanded in shared memory; 0: byte tiles
   int pair;                    // 256-row tiles by pairs of CTAs
-  int res_boxes;               // bf16 residual by bulk-copied boxes (tiles of at most 192 columns)
+  int res_boxes;               // bf16 residual by bulk-copied boxes (tiles of at most 192 columns): boxes per warp
   TileOrder order;             // panels of row tiles (see TileOrder)
   EpilogueParams ep;
 };
@@ -368,7 +370,8 @@ __device__ __forceinline__ void emit_chunk(const CUtensorMap* map_out, uint32_t 
 
 // General path for one chunk of one thread (ragged rows / columns, float32 residual, accumulator dump):
 // element by element, kept out of line so that the common path stays small.
-__device__ __noinline__ void slow_chunk(const EpilogueParams& ep, const TcParams& P, const TileTerms& C, const uint32_t* r,
+template <int BN>
+__device__ __noinline__ void slow_chunk(const EpilogueParams& ep, const TcParams& P, const TileTerms<BN>& C, const uint32_t* r,
                                         int cl, int64_t m, int col0, int32_t asum_c, int* code_sum) {
   const ChunkQuant q = chunk_quant(ep, P, col0);
   const float magic = __uint_as_float(kMagicBits);
@@ -440,7 +443,7 @@ enum : int { kPairNone = 0, kPairRope = 1, kPairGlu = 2 };
 // 18464 x 3072 x 1024 45.0 -> 41.6; bf16 residual, 18464 x 1024 x 4096 61.5 -> 59.1, 8192 x 4096 x 4096 97.7 -> 93.5.
 enum : int { kEpiAny = 0, kEpiPlain = 1, kEpiGelu = 2, kEpiResidual = 3 };
 
-template <int BN, int OUT, bool RES, int PAIR, int WP, bool TWO, int EPI>
+template <int BN, int OUT, int RES, int PAIR, int WP, bool TWO, int EPI>
 __global__ void __launch_bounds__(kThreads, 1)
 qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                 const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res, const __grid_constant__ TcParams P) {
@@ -473,7 +476,7 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     for (int s = 0; s < Storage::kStagesB; ++s) { mbar_init(smem_u32(&S.ready[s]), kConvWarps); mbar_init(smem_u32(&S.bfree[s]), 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(smem_u32(&S.tmem_full[a]), 1); mbar_init(smem_u32(&S.tmem_empty[a]), TWO ? 2 * EW : EW); }
     for (int a = 0; a < 2; ++a) { mbar_init(smem_u32(&S.terms_full[a]), 1); mbar_init(smem_u32(&S.terms_empty[a]), EW); }
-    for (int w = 0; w < kEpiWarps; ++w) mbar_init(smem_u32(&S.res_full[w]), 1);
+    for (int w = 0; w < 2 * kEpiWarps; ++w) mbar_init(smem_u32(&S.res_full[0][w]), 1);
     mbar_init(smem_u32(&S.done), 1);
     S.abort = 0;
     if (smem_u32(smem_raw) & 1023u) {              // the swizzled tiles need the alignment asked for above
@@ -597,7 +600,7 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     for (int tile = tile0; tile < tiles && !*abort; tile += tile_step, ++it) {
       const TileOrigin o = tile_origin(tile, P.order, kTileM, BN);
       const int m0 = o.m0 + rank * BM, n0 = o.n0;
-      TileTerms& C = S.terms[it & 1];
+      TileTerms<BN>& C = S.terms[it & 1];
       // loads from clamped indices, all in flight before the buffer is waited for
       int zw[kPer], ws[kPer], rows[BM / 32];
       float sw[kPer], bs[kPer];
@@ -727,27 +730,30 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     const bool direct = EPI == kEpiAny ? P.direct_requant != 0 : EPI == kEpiPlain && PAIR != kPairGlu;
     const int cl0 = slice * kSliceCols;          // first column of this warp inside the tile
     // bulk copy of the residual box of tile t (rows and columns outside the matrix are zero-filled)
-    const uint32_t res_buf = smem_u32(S.res) + uint32_t(RES ? ew : 0) * kResBytes;
-    const uint32_t res_bar = smem_u32(&S.res_full[ew]);
+    // tile number n of this CTA takes box n % RES of the warp
+    auto box_of = [](int n) { return RES == 2 ? n & 1 : 0; };
+    auto box_phase = [](int n) { return uint32_t(RES == 2 ? n >> 1 : n) & 1u; };
+    auto res_box = [&](int n) { return smem_u32(S.res) + uint32_t(RES ? RES * ew + box_of(n) : 0) * kResBytes; };
+    auto res_bar = [&](int n) { return smem_u32(&S.res_full[box_of(n)][ew]); };
     bool res_pending = false;
-    auto fetch_residual = [&](int t) {
+    auto fetch_residual = [&](int t, int n) {
       if (!RES || t >= tiles || !slice_on) return;
       const TileOrigin o = tile_origin(t, P.order, kTileM, BN);
       const int tm0 = o.m0 + rank * BM, tn0 = o.n0;
       if (lane == 0) {
         // the box's last content may still be on its way out (the bulk store of the previous tile reads it)
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-        mbar_expect_tx(res_bar, kResBytes);
-        tma_load_2d(res_buf, &map_res, res_bar, tn0 + cl0, tm0 + quarter * 32);
+        mbar_expect_tx(res_bar(n), kResBytes);
+        tma_load_2d(res_box(n), &map_res, res_bar(n), tn0 + cl0, tm0 + quarter * 32);
       }
       res_pending = true;
     };
-    fetch_residual(tile0);
+    fetch_residual(tile0, 0);
     int it = 0;
     for (int tile = tile0; tile < tiles && !*abort; tile += tile_step, ++it) {
       const uint32_t acc = it & 1, acc_phase = (it >> 1) & 1;
       if (!mbar_wait(smem_u32(&S.terms_full[acc]), acc_phase, abort, 10)) break;
-      const TileTerms& C = S.terms[acc];
+      const TileTerms<BN>& C = S.terms[acc];
       const int m0 = C.m0, n0 = C.n0;
       const int64_t m = int64_t(m0) + quarter * 32 + lane;
       const bool row_ok = m < P.M;
@@ -785,9 +791,11 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       tc_fence_after();
       const uint32_t taddr0 = tmem_base + (uint32_t(quarter * 32) << 16) + acc * kAccStride + cl0;
       if (RES && res_pending) {
-        if (!mbar_wait(res_bar, uint32_t(it) & 1u, abort, 6)) break;
+        if (!mbar_wait(res_bar(it), box_phase(it), abort, 6)) break;
         res_pending = false;
       }
+      if (RES == 2) fetch_residual(tile + tile_step, it + 1);      // into the box that the tile before left from
+      const uint32_t res_buf = res_box(it);
       // Plain epilogues to byte codes: a thread takes two columns of each eight, of four rows, instead of all columns of one row, and reads
       // a quarter of the column terms (16 bytes a column; reads of shared memory paced the chunk loop, 45 % of its wavefronts).  The
       // bytes of a row then meet in one lane of its quad by two shuffles.  12608 x 2304 x 768 24.5 -> 24.3 us, block pass of 64 x 197
@@ -994,10 +1002,10 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         if constexpr (TWO) mbar_arrive_cluster(map_to_rank(smem_u32(&S.tmem_empty[acc]), 0));
         else mbar_arrive(smem_u32(&S.tmem_empty[acc]));
       }
-      fetch_residual(tile + tile_step);               // every lane has read this tile's box (the __syncwarp above)
+      if (RES != 2) fetch_residual(tile + tile_step, it + 1);      // every lane has read this tile's box (the __syncwarp above)
       if (ep.out_row_sum != nullptr && m_sum < P.M && code_sum != 0) atomicAdd(ep.out_row_sum + m_sum, code_sum);
     }
-    if (RES && res_pending) mbar_drain(res_bar, uint32_t(it) & 1u);              // left the loop early: the copy must land
+    if (RES && res_pending) mbar_drain(res_bar(it), box_phase(it));              // left the loop early: the copy must land
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");     // bulk stores complete
   }
 
@@ -1095,7 +1103,7 @@ repq_status make_box_map(CUtensorMap* map, const TcParams& P, const void* base, 
   return REPQ_OK;
 }
 
-template <int BN, int OUT, bool RES, int PAIR, int WP, bool TWO, int EPI>
+template <int BN, int OUT, int RES, int PAIR, int WP, bool TWO, int EPI>
 repq_status launch_tc_e(const CUtensorMap& map_a, const CUtensorMap& map_b, const TcParams& P, int sms, cudaStream_t st) {
   CUtensorMap map_out, map_res;
   if (RES) {
@@ -1117,7 +1125,7 @@ repq_status launch_tc_e(const CUtensorMap& map_a, const CUtensorMap& map_b, cons
   return REPQ_OK;
 }
 
-template <int BN, int OUT, bool RES, int PAIR, int WP, bool TWO = false>
+template <int BN, int OUT, int RES, int PAIR, int WP, bool TWO = false>
 repq_status launch_tc_w(const CUtensorMap& map_a, const CUtensorMap& map_b, const TcParams& P, int sms, cudaStream_t st) {
   // (packed weights and codes two per byte: one kernel each)
   if constexpr (WP == 0 && OUT != kOutC4) {
@@ -1135,11 +1143,11 @@ repq_status launch_tc_w(const CUtensorMap& map_a, const CUtensorMap& map_b, cons
   else return fail(REPQ_UNSUPPORTED, "qgemm: rope / glu are for plain products without gelu or residual");
 }
 
-template <int BN, int OUT, bool RES, int PAIR = kPairNone>
+template <int BN, int OUT, int RES, int PAIR = kPairNone>
 repq_status launch_tc_res(const CUtensorMap& map_a, const CUtensorMap& map_b, const TcParams& P, int sms, cudaStream_t st) {
   if constexpr (!RES && BN <= kMaxBNW4) {
-    if (P.w_packed4 == 4) return launch_tc_w<BN, OUT, false, PAIR, 4>(map_a, map_b, P, sms, st);
-    if (P.w_packed4 == 6) return launch_tc_w<BN, OUT, false, PAIR, 6>(map_a, map_b, P, sms, st);
+    if (P.w_packed4 == 4) return launch_tc_w<BN, OUT, 0, PAIR, 4>(map_a, map_b, P, sms, st);
+    if (P.w_packed4 == 6) return launch_tc_w<BN, OUT, 0, PAIR, 6>(map_a, map_b, P, sms, st);
   }
   if constexpr (!RES && BN == kMaxBN) {
     if (P.pair) return launch_tc_w<BN, OUT, RES, PAIR, 0, true>(map_a, map_b, P, sms, st);
@@ -1152,10 +1160,12 @@ repq_status launch_tc_out(const CUtensorMap& map_a, const CUtensorMap& map_b, co
   // bf16 outputs with a bf16 residual on tiles of at most 192 columns: the residual boxes, which also carry the output,
   // fit beside the four stages
   if constexpr (BN <= 192 && OUT == kOutBf16) {
-    if (P.res_boxes)
-      return launch_tc_res<BN, OUT, true>(map_a, map_b, P, sms, st);
+    if constexpr (BN == 192) {
+      if (P.res_boxes == 2) return launch_tc_res<BN, OUT, 2>(map_a, map_b, P, sms, st);
+    }
+    if (P.res_boxes) return launch_tc_res<BN, OUT, 1>(map_a, map_b, P, sms, st);
   }
-  return launch_tc_res<BN, OUT, false>(map_a, map_b, P, sms, st);
+  return launch_tc_res<BN, OUT, 0>(map_a, map_b, P, sms, st);
 }
 
 template <int BN>
@@ -1163,8 +1173,8 @@ repq_status launch_tc(const CUtensorMap& map_a, const CUtensorMap& map_b, const 
   if (P.ep.out_kind == REPQ_OUT_F32) return launch_tc_out<BN, kOutF32>(map_a, map_b, P, sms, st);
   if (P.ep.out_kind == REPQ_OUT_BF16) return launch_tc_out<BN, kOutBf16>(map_a, map_b, P, sms, st);
   if (P.ep.pack4) return launch_tc_out<BN, kOutC4>(map_a, map_b, P, sms, st);
-  if (P.ep.rope != nullptr) return launch_tc_res<BN, kOutC8, false, kPairRope>(map_a, map_b, P, sms, st);
-  if (P.ep.glu) return launch_tc_res<BN, kOutC8, false, kPairGlu>(map_a, map_b, P, sms, st);
+  if (P.ep.rope != nullptr) return launch_tc_res<BN, kOutC8, 0, kPairRope>(map_a, map_b, P, sms, st);
+  if (P.ep.glu) return launch_tc_res<BN, kOutC8, 0, kPairGlu>(map_a, map_b, P, sms, st);
   return launch_tc_out<BN, kOutC8>(map_a, map_b, P, sms, st);
 }
 
@@ -1300,7 +1310,11 @@ repq_status qgemm_tc(const repq_gemm_desc& d, const EpilogueParams& ep, const Tc
   const int sms = sm_count();
   const int bn = plan.bn;
   P.pair = plan.pair;
-  P.res_boxes = residual_boxes(d);
+  // A second box per warp, for the stage of the ring that it takes, where the next tile's residual paces the tiles: short K and more tiles
+  // than SMs (residual, one box and two: 12608 x 768 x 768 17.0 and 16.1 us, 12608 x 384 x 384 9.3 and 8.7; 18464 x 1024 x 1024 28.1 and 30.1,
+  // 12608 x 768 x 3072 33.7 and 38.0, one round of tiles, 3152 x 768 x 768, 7.2 and 7.3).
+  const int64_t all_tiles = ((int64_t(d.M) + BM - 1) / BM) * ((int64_t(d.N) + bn - 1) / bn);
+  P.res_boxes = !residual_boxes(d) ? 0 : bn == 192 && d.K <= 768 && all_tiles > sm_count() ? 2 : 1;
   {
     // panels of activations: all row tiles while the activations take at most 40 MB (a third of the L2 capacity),
     // else about 24 MB (measured at 8192 x 4096 x 11008 with residual: 248 us with 40 MB panels, 240-242 with

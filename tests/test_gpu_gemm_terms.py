@@ -68,3 +68,10 @@ def test_gemm_of_long_k_over_many_tiles(M, N, K, out_kind):
         low, high = (torch.clamp(torch.round(t + e) + z_o, 0, 15) for e in (-open_, open_))
         assert bool(((out >= low) & (out <= high)).all())
         assert bool(torch.equal(sums, out.int().sum(1, dtype=torch.int32)))
+
+
+@pytest.mark.parametrize("M,N,K", [(12608, 384, 384), (9601, 768, 768), (9500, 560, 700), (19001, 192, 768)])
+def test_residual_in_two_boxes_matches_oracle(M, N, K):
+    """Short K and more tiles of 192 columns than SMs: the next tile's residual comes while this one's leaves; ragged rows and columns."""
+    b = 4 | parity.BYTE_CODES
+    parity.check_qgemm(M, N, K, b, b, out_kind="bf16", residual="bf16", want_acc=False, give_sums=True, seed=M)
