@@ -56,7 +56,7 @@ class QuantBlock:
     def __init__(self, w, device="cuda:0", out_dtype: Optional[torch.dtype] = None, staged_attention: bool = False,
                  weight_storage: str = "bytes"):
         """weight_storage: "packed" keeps 4-bit weight codes two per byte and 6-bit codes four to three bytes in device
-        memory (the GEMM expands them, a layer at a time, into the workspace); "bytes" keeps one code per byte, the tensor-core operand
+        memory (every pass expands them into the workspace); "bytes" keeps one code per byte, the tensor-core operand
         format."""
         assert weight_storage in ("packed", "bytes")
         self.weight_storage = weight_storage
