@@ -551,11 +551,20 @@ ln_rows_kernel(const __nv_bfloat16* __restrict__ x, uint32_t rows, int64_t ldx, 
     request(first + stride, 1);
   };
   if (!settled) begin();               // (factors that the kernel ahead may have written are read behind the wait, as in ln_quant_kernel)
-  for (int k = tid; k < kPieces; k += kBlock) {
-    const int q = (k + rot) % kPieces, at = (q & 1) * (D / 2) + (q >> 1) * 4;
-    const float4 g = load4(gamma_t + 4 * q), b = load4(beta_t + 4 * q);
-    *reinterpret_cast<float4*>(s_gb + at) = make_float4(g.x * inv_s, g.y * inv_s, g.z * inv_s, g.w * inv_s);
-    *reinterpret_cast<float4*>(s_gb + D + at) = make_float4(b.x * inv_s, b.y * inv_s, b.z * inv_s, b.w * inv_s);
+  constexpr int kOwn = (kPieces + kBlock - 1) / kBlock;  // a thread's pieces, all in flight at once
+  float4 g4[kOwn], b4[kOwn];
+#pragma unroll
+  for (int i = 0; i < kOwn; ++i) {
+    const int q = (tid + i * kBlock + rot) % kPieces;
+    if (tid + i * kBlock < kPieces) { g4[i] = load4(gamma_t + 4 * q); b4[i] = load4(beta_t + 4 * q); }
+  }
+#pragma unroll
+  for (int i = 0; i < kOwn; ++i) {
+    const int q = (tid + i * kBlock + rot) % kPieces, at = (q & 1) * (D / 2) + (q >> 1) * 4;
+    if (tid + i * kBlock < kPieces) {
+      *reinterpret_cast<float4*>(s_gb + at) = make_float4(g4[i].x * inv_s, g4[i].y * inv_s, g4[i].z * inv_s, g4[i].w * inv_s);
+      *reinterpret_cast<float4*>(s_gb + D + at) = make_float4(b4[i].x * inv_s, b4[i].y * inv_s, b4[i].z * inv_s, b4[i].w * inv_s);
+    }
   }
   __syncthreads();
   if (settled) begin();
