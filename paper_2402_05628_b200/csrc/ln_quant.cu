@@ -227,13 +227,11 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
 
   float* s_g = s_gb;
   float* s_b = s_gb + D;
-  // Rows of one warp keep a second form of the code for factors so large that |t| might reach 2^22: with the branch between the
-  // chunks their loop runs faster than without (100000 x 768 39.5 against 40.3 us, 60000 x 1536 46.0 and 47.9); longer rows do without it
-  // (16384 x 8192 67.9 and 65.0).  The two give the same codes, but for a NaN.
-  constexpr bool kGuard = !kWide;
+  // |t| <= sqrt(D) |gamma~/s~| + |beta~/s~|.  Where that bound may reach 2^22, t is clamped and converted instead, which gives a NaN the
+  // lowest code (a whole-kernel decision, taken here once).
   // One form rounds by the float adder instead (t + 1.5 * 2^23 leaves rint(t) in the low bits while |t| < 2^22) and adds z as an integer:
   // float rows of 1536 to byte codes, where the denormals' constants are the registers too many for a second block (5000 rows 9.5 us, 10.1).
-  constexpr bool kMagic = kGuard && sizeof(T) == 4 && kVPT == 6 && kFull && !kPack4;
+  constexpr bool kMagic = !kWide && sizeof(T) == 4 && kVPT == 6 && kFull && !kPack4;
   constexpr int kMagicBits = 0x4B400000;
   const float root_d = sqrtf(float(D));
   bool wide = false;
@@ -248,14 +246,14 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
       const float bi[4] = {b4[k].x * inv_s, b4[k].y * inv_s, b4[k].z * inv_s, b4[k].w * inv_s};
       *reinterpret_cast<float4*>(s_g + at) = make_float4(gi[0], gi[1], gi[2], gi[3]);
       *reinterpret_cast<float4*>(s_b + at) = make_float4(bi[0], bi[1], bi[2], bi[3]);
-      if constexpr (kGuard) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) wide = wide || !(fabsf(gi[e]) * root_d + fabsf(bi[e]) < 4.0e6f);
-      }
+      for (int e = 0; e < 4; ++e) wide = wide || !(fabsf(gi[e]) * root_d + fabsf(bi[e]) < 4.0e6f);
     }
   }
-  const bool guard = kGuard && __syncthreads_or(wide) != 0;
-  if (!kGuard) __syncthreads();
+  const bool guard = __syncthreads_or(wide) != 0;
+  // The branch to the second form is taken once per row, around the chunks; float rows of one warp take it per chunk, where it costs them
+  // fewer registers.
+  constexpr bool kPerRow = kWide || sizeof(T) == 2;
   // x and the outputs belong to the chain of kernels
   if (settled) {
     grid_dependency_wait();
@@ -406,6 +404,7 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
       live[r] = row0 + r < rows;
       out[r] = codes + (row0 + r) * ldc;
     }
+    auto chunks = [&](auto guarded) {
 #pragma unroll
     for (int i = 0; i < kVPT; ++i) {
       const int c = tig + i * TPR;
@@ -422,7 +421,7 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
           // Eq. 4: clip(round(t) + z, 0, qmax): round half to even by the float -> int conversion, then the
           // packing instruction saturates to the container ([0, 15] or [0, 255])
           int q[kChunk];
-          if (!guard) {
+          if (kPerRow ? !decltype(guarded)::value : !guard) {
 #pragma unroll
             for (int e = 0; e < kChunk / 2; ++e) {
               const f32x2 t = fma2(normalised(v[r][i][e], r), g[e], b[e]);
@@ -463,6 +462,9 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
         }
       }
     }
+    };
+    if (kPerRow && guard) chunks(std::true_type{});
+    else chunks(std::false_type{});
     if (row_sum != nullptr) {
       if constexpr (!kWide) {
         group_sum<TPR, kRows>(csum);
@@ -553,6 +555,8 @@ ln_rows_kernel(const __nv_bfloat16* __restrict__ x, uint32_t rows, int64_t ldx, 
   if (!settled) begin();               // (factors that the kernel ahead may have written are read behind the wait, as in ln_quant_kernel)
   constexpr int kOwn = (kPieces + kBlock - 1) / kBlock;  // a thread's pieces, all in flight at once
   float4 g4[kOwn], b4[kOwn];
+  const float root_d = sqrtf(float(D));
+  bool wide = false;
 #pragma unroll
   for (int i = 0; i < kOwn; ++i) {
     const int q = (tid + i * kBlock + rot) % kPieces;
@@ -562,11 +566,15 @@ ln_rows_kernel(const __nv_bfloat16* __restrict__ x, uint32_t rows, int64_t ldx, 
   for (int i = 0; i < kOwn; ++i) {
     const int q = (tid + i * kBlock + rot) % kPieces, at = (q & 1) * (D / 2) + (q >> 1) * 4;
     if (tid + i * kBlock < kPieces) {
-      *reinterpret_cast<float4*>(s_gb + at) = make_float4(g4[i].x * inv_s, g4[i].y * inv_s, g4[i].z * inv_s, g4[i].w * inv_s);
-      *reinterpret_cast<float4*>(s_gb + D + at) = make_float4(b4[i].x * inv_s, b4[i].y * inv_s, b4[i].z * inv_s, b4[i].w * inv_s);
+      const float gi[4] = {g4[i].x * inv_s, g4[i].y * inv_s, g4[i].z * inv_s, g4[i].w * inv_s};
+      const float bi[4] = {b4[i].x * inv_s, b4[i].y * inv_s, b4[i].z * inv_s, b4[i].w * inv_s};
+      *reinterpret_cast<float4*>(s_gb + at) = make_float4(gi[0], gi[1], gi[2], gi[3]);
+      *reinterpret_cast<float4*>(s_gb + D + at) = make_float4(bi[0], bi[1], bi[2], bi[3]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) wide = wide || !(fabsf(gi[e]) * root_d + fabsf(bi[e]) < 4.0e6f);
     }
   }
-  __syncthreads();
+  const bool guard = __syncthreads_or(wide) != 0;          // (as in ln_quant_kernel)
   if (settled) begin();
   for (int64_t i = int64_t(blockIdx.x) * kBlock + tid; i < n_clear; i += int64_t(gridDim.x) * kBlock) clear[i] = 0;
 
@@ -652,6 +660,7 @@ ln_rows_kernel(const __nv_bfloat16* __restrict__ x, uint32_t rows, int64_t ldx, 
     const float own_rest = (own_mean - mean) * rs;
     int csum[1] = {0};
     uint8_t* out = codes + int64_t(row) * ldc;
+    auto chunks = [&](auto guarded) {
 #pragma unroll
     for (int w = 0; w < kSlices; ++w) {
       const f32x2 rest = splat2(__shfl_sync(0xffffffffu, own_rest, (32 / kSlices) * w));
@@ -667,9 +676,15 @@ ln_rows_kernel(const __nv_bfloat16* __restrict__ x, uint32_t rows, int64_t ldx, 
         for (int e = 0; e < kChunk / 2; ++e) {
           const f32x2 u = fma2(fma2(v[i][e], rstd, rest), g[e], b[e]);
           float u0, u1;
-          unpack2(add2(mul2(u, tiny2), z2), u0, u1);
-          q[2 * e] = __float_as_int(u0);
-          q[2 * e + 1] = __float_as_int(u1);
+          if constexpr (decltype(guarded)::value) {
+            unpack2(u, u0, u1);
+            q[2 * e] = __float2int_rn(fminf(fmaxf(u0, -1.0e9f), 1.0e9f)) + z;
+            q[2 * e + 1] = __float2int_rn(fminf(fmaxf(u1, -1.0e9f), 1.0e9f)) + z;
+          } else {
+            unpack2(add2(mul2(u, tiny2), z2), u0, u1);
+            q[2 * e] = __float_as_int(u0);
+            q[2 * e + 1] = __float_as_int(u1);
+          }
         }
         if constexpr (kSlices == 4) __syncwarp();        // keeps the chunks apart: interleaved, they spill (67.7 us instead of 59.0)
         if constexpr (kPack4) {
@@ -687,6 +702,9 @@ ln_rows_kernel(const __nv_bfloat16* __restrict__ x, uint32_t rows, int64_t ldx, 
         }
       }
     }
+    };
+    if (guard) chunks(std::true_type{});
+    else chunks(std::false_type{});
     if (row_sum != nullptr) {
       group_sum<32, 1>(csum);
       if (lane == 0) row_sum[row] = csum[0];
