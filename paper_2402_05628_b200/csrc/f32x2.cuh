@@ -1,5 +1,6 @@
 // Two float32 lanes in one 64-bit register, for the packed add / mul / fma instructions of sm_100
-// (each handles two elements per issue slot; IEEE round-to-nearest, same results as the scalar forms).
+// (each handles two elements per issue slot; IEEE round-to-nearest, same results as the scalar forms).  One thing differs: add2 of a mul2
+// may be compiled into a single fused operation, which rounds once, so neither may be relied on to round by itself there.
 #pragma once
 #include <cstdint>
 

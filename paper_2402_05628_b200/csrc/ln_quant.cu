@@ -16,10 +16,12 @@
 // The per-channel factors gamma~/s~ and beta~/s~ are staged once per CTA in shared memory (halves of the 8-element
 // chunks apart, so that a warp's 16-byte reads are free of bank conflicts).
 //
-// The float work runs on packed pairs (two elements per add / mul / fma issue slot).  t times 2^-149 is a denormal whose bit pattern is
-// rint(t) (half to even, on t itself, as Eq. 4 has it); z is added exactly as another denormal, and the clip of Eq. 4 is the saturation of
-// the packing instruction (negative values are negative integers, large ones are no longer denormals but large integers still).  Against
-// t + 1.5 * 2^23 and integer additions: 32768 x 4096 74.1 -> 72.7 us, 131072 x 1024 63.4 -> 60.7.
+// The float work runs on packed pairs (two elements per add / mul / fma issue slot).  Rounding is done by the
+// float adder: t + 1.5 * 2^23 leaves rint(t) (half to even, on t itself, as Eq. 4 has it) in the low mantissa
+// bits while |t| < 2^22; inputs that cannot guarantee that bound are clamped and converted with cvt.rni
+// instead.  z is added as an integer and the clip of Eq. 4 is the saturation of the packing instruction.  (t times 2^-149, a denormal whose
+// bits are rint(t), plus z as another denormal saves two integer additions per pair, but the compiler makes one fused operation of the packed
+// product and the packed sum, although both ask for their own rounding: t + z is then rounded, and a tie falls the other way for odd z.)
 #include <cuda_bf16.h>
 
 #include <type_traits>
@@ -32,6 +34,7 @@ namespace repq {
 namespace {
 
 constexpr int kChunk = 8;   // elements per 128-bit bf16 load
+constexpr int kMagicBits = 0x4B400000;   // float 1.5 * 2^23
 
 // Rows a thread group works on at a time (the loads of the next ones are always in flight as well): two, except where the
 // chunks per thread leave the registers for one.  bf16: from four chunks on in groups that share an SM with others (2048 / 4096
@@ -229,10 +232,6 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
   float* s_b = s_gb + D;
   // |t| <= sqrt(D) |gamma~/s~| + |beta~/s~|.  Where that bound may reach 2^22, t is clamped and converted instead, which gives a NaN the
   // lowest code (a whole-kernel decision, taken here once).
-  // One form rounds by the float adder instead (t + 1.5 * 2^23 leaves rint(t) in the low bits while |t| < 2^22) and adds z as an integer:
-  // float rows of 1536 to byte codes, where the denormals' constants are the registers too many for a second block (5000 rows 9.5 us, 10.1).
-  constexpr bool kMagic = !kWide && sizeof(T) == 4 && kVPT == 6 && kFull && !kPack4;
-  constexpr int kMagicBits = 0x4B400000;
   const float root_d = sqrtf(float(D));
   bool wide = false;
   // layout: the first halves (4 floats) of all chunks, then the second halves, so that the 16-byte reads of
@@ -251,8 +250,9 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
     }
   }
   const bool guard = __syncthreads_or(wide) != 0;
-  // The branch to the second form is taken once per row, around the chunks; float rows of one warp take it per chunk, where it costs them
-  // fewer registers.
+  // The branch to the second form is taken once per row, around the chunks (per chunk and per row: bf16, 16384 x 8192 74.6 and 72.5 us,
+  // 10000 x 6152 52.9 and 46.7, 12608 x 768 8.6 and 8.4, 131072 x 1024 66.1 and 65.2, but 18464 x 1024 13.1 and 13.6); float rows of one
+  // warp take it per chunk (12608 x 384 7.1 and 7.2, 30000 x 1536 36.0 and 36.8).
   constexpr bool kPerRow = kWide || sizeof(T) == 2;
   // x and the outputs belong to the chain of kernels
   if (settled) {
@@ -264,7 +264,8 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
 
   const float inv_d = 1.f / float(D);
   const uint32_t qmax4 = uint32_t(qmax) * 0x01010101u;
-  const f32x2 tiny2 = splat2(__uint_as_float(1u)), z2 = splat2(z < 0 ? -__uint_as_float(uint32_t(-z)) : __uint_as_float(uint32_t(z)));
+  const f32x2 magic2 = splat2(__int_as_float(kMagicBits));
+  const int z_less_magic = z - kMagicBits;
 
   // the warp's slice of a row, and the slice its lane merges
   const int lane_w = threadIdx.x & 31;
@@ -424,17 +425,10 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
           if (kPerRow ? !decltype(guarded)::value : !guard) {
 #pragma unroll
             for (int e = 0; e < kChunk / 2; ++e) {
-              const f32x2 t = fma2(normalised(v[r][i][e], r), g[e], b[e]);
               float u0, u1;
-              if constexpr (kMagic) {
-                unpack2(add2(t, splat2(__int_as_float(kMagicBits))), u0, u1);
-                q[2 * e] = __float_as_int(u0) + (z - kMagicBits);
-                q[2 * e + 1] = __float_as_int(u1) + (z - kMagicBits);
-              } else {
-                unpack2(add2(mul2(t, tiny2), z2), u0, u1);
-                q[2 * e] = __float_as_int(u0);
-                q[2 * e + 1] = __float_as_int(u1);
-              }
+              unpack2(add2(fma2(normalised(v[r][i][e], r), g[e], b[e]), magic2), u0, u1);
+              q[2 * e] = __float_as_int(u0) + z_less_magic;
+              q[2 * e + 1] = __float_as_int(u1) + z_less_magic;
             }
           } else {
             float t[kChunk];
@@ -507,9 +501,9 @@ ln_quant_kernel(const T* __restrict__ x, int64_t rows, int D, int64_t ldx,
 // each.  A buffer is filled again one iteration after it was read: by then everything computed from it has been issued, so its loads
 // have returned.  The sums are formed slice by slice in the order of ln_quant_kernel, so that a row's codes do not depend on how many
 // rows share the call.
-// Input partly in L2, groups of warps -> this: 32768 x 4096 to packed codes 72.7 -> 59.0 us, to bytes 79.1 -> 65.5, 20000 x 4096 RMS 48.4 -> 44,
-// 65536 x 2048 68.6 -> 56.7.  A branch per chunk (to a second form for large factors, which the rounding into denormals does not
-// need) cost 10 us at 4096; eight warps of 200 registers 66.  Two rows per warp with half of a row each, which reads the factors half as
+// New inputs, groups of warps -> this: 32768 x 4096 to packed codes 77.1 -> 63.4 us, to bytes 83.1 -> 69.4, 20000 x 4096 RMS 46.5 -> 40.1,
+// 65536 x 2048 73.5 -> 63.1.  The form for large factors is chosen once per row: a branch per chunk cost 10 us at 4096.  Eight warps of 200
+// registers took 66 us where this took 59.0.  Two rows per warp with half of a row each, which reads the factors half as
 // often, took 89 us: twelve warps are few, and each then waits on twice the work of one iteration.
 template <int kSlices> constexpr int row_warps() { return kSlices == 4 ? 12 : 20; }      // by 168 and 96 registers a thread
 template <int kSlices, bool kPack4>
@@ -604,7 +598,8 @@ ln_rows_kernel(const __nv_bfloat16* __restrict__ x, uint32_t rows, int64_t ldx, 
   constexpr float kSliceSize = float(32 * kPer * kChunk);
   const float inv_d = 1.f / float(D);
   const uint32_t qmax4 = uint32_t(qmax) * 0x01010101u;
-  const f32x2 tiny2 = splat2(__uint_as_float(1u)), z2 = splat2(z < 0 ? -__uint_as_float(uint32_t(-z)) : __uint_as_float(uint32_t(z)));
+  const f32x2 magic2 = splat2(__int_as_float(kMagicBits));
+  const int z_less_magic = z - kMagicBits;
   int k = 0;
   uint32_t row = first;
   for (; row < rows; row += stride, ++k) {
@@ -681,9 +676,9 @@ ln_rows_kernel(const __nv_bfloat16* __restrict__ x, uint32_t rows, int64_t ldx, 
             q[2 * e] = __float2int_rn(fminf(fmaxf(u0, -1.0e9f), 1.0e9f)) + z;
             q[2 * e + 1] = __float2int_rn(fminf(fmaxf(u1, -1.0e9f), 1.0e9f)) + z;
           } else {
-            unpack2(add2(mul2(u, tiny2), z2), u0, u1);
-            q[2 * e] = __float_as_int(u0);
-            q[2 * e + 1] = __float_as_int(u1);
+            unpack2(add2(u, magic2), u0, u1);
+            q[2 * e] = __float_as_int(u0) + z_less_magic;
+            q[2 * e + 1] = __float_as_int(u1) + z_less_magic;
           }
         }
         if constexpr (kSlices == 4) __syncwarp();        // keeps the chunks apart: interleaved, they spill (67.7 us instead of 59.0)

@@ -1,4 +1,4 @@
-"""LayerNorm + quantization, element by element where the general tests look away: values that are not numbers."""
+"""LayerNorm + quantization, element by element where the general tests look away: values that are not numbers, and exact ties."""
 import numpy as np
 import pytest
 
@@ -34,3 +34,19 @@ def test_codes_of_rows_that_are_not_numbers(D, rows, bf16, bits):
     for gamma, code in ((3.0, (1 << bits) - 1), (1.0e9, 0)):
         got = _codes(x, torch.full((D,), gamma, device=dev), beta, 6, bits)[[3, 7, 9]]
         assert bool((got == code).all()), (gamma, got[:, :8])
+
+
+@pytest.mark.parametrize("bits", [4, 6, 8])
+@pytest.mark.parametrize("bf16", [True, False])
+@pytest.mark.parametrize("D,rows", FORMS)
+def test_ties_round_to_even_before_the_zero_point_is_added(D, rows, bf16, bits):
+    """t = k + 1/2 exactly (gamma~ = 0, so that t = beta~): Eq. 4 rounds t to the even neighbour and adds z afterwards, odd or even."""
+    import torch
+    dev, top = "cuda:0", (1 << bits) - 1
+    x = torch.randn(rows, D, device=dev, generator=torch.Generator(dev).manual_seed(D)).to(torch.bfloat16 if bf16 else torch.float32)
+    gamma, k = torch.zeros(D, device=dev), torch.arange(D, device=dev) % (2 * top + 7)
+    for zero in (0, 6, 7, -3, 101):
+        beta = k.float() - zero - 2.5
+        want = (torch.round(beta.double()) + zero).clamp(0, top).to(torch.uint8)
+        got = _codes(x, gamma, beta, zero, bits, rms=zero == 6)
+        assert bool((got == want).all()), (zero, (got != want).nonzero()[:4])
