@@ -176,7 +176,14 @@ static repq_status block_forward_impl(const repq_block_desc* dp, const repq_bloc
     at_once = aligned(linear[i]->w_codes, 16) && linear[i]->ldw_bytes % 16 == 0;
     byte_forms[i] = Expansion{linear[i]->w_codes, n_of[i], k_of[i], linear[i]->ldw_bytes, ws + L.off_bytes[i], round_up(k_of[i], 16)};
   }
-  if (at_once) REPQ_TRY(launch_expand_all(byte_forms, 4, d.bits_w, st));
+  if (at_once) {
+    // (the products check the byte forms only)
+    for (const Expansion& e : byte_forms) {
+      REPQ_REQUIRE(e.src, REPQ_INVALID_ARG, "block_forward: NULL weight codes");
+      REPQ_REQUIRE(e.ld_src >= code_row_bytes(e.k, d.bits_w), REPQ_INVALID_ARG, "block_forward: weight row stride shorter than its codes");
+    }
+    REPQ_TRY(launch_expand_all(byte_forms, 4, d.bits_w, st));
+  }
   auto run_linear = [&](repq_gemm_desc& g, int i, Params params) {
     if (!at_once) return run_qgemm(g, gws, gws_bytes, Params::settled, st);
     g.w_codes = byte_forms[i].dst;

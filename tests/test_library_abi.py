@@ -132,3 +132,36 @@ def test_pack_weights_six_bit_layout(B):
     assert np.array_equal(c6, pack_codes(c8[:, :53], 6 | PACKED6, c6.shape[1]))
     bits = np.unpackbits(c6, axis=1, bitorder="little")[:, : 53 * 6].reshape(9, 53, 6)
     assert np.array_equal((bits * (1 << np.arange(6))).sum(axis=2), c8[:, :53])
+
+
+@pytest.mark.parametrize("bits_w", [4, 6 | 0x200])
+def test_block_refuses_packed_weights_it_cannot_read(B, bits_w):
+    """A missing matrix, or a row stride shorter than its codes, is refused before anything is launched, also where all packed matrices
+    are expanded ahead of the first product."""
+    import ctypes as C
+    D, mlp = 768, 3072
+    d = B.BlockDesc()
+    d.batch, d.seq, d.dim, d.heads, d.mlp, d.bits_a, d.bits_w, d.bits_p, d.eps = 2, 197, D, D // 64, mlp, 4, bits_w, 4, 1e-6
+    d.act_dtype = d.out_dtype = B.REPQ_BF16
+    total = B.repq_block_workspace_bytes(d)
+    at = 1 << 20                                            # (addresses of the right alignment that nothing looks at)
+
+    def params():
+        p = B.BlockParams()
+        for name, _ in B.BlockParams._fields_:
+            if name.endswith("_t"):
+                setattr(p, name, at)
+            elif name.startswith("s_") or name in ("ln1_s", "ln2_s", "softmax_s"):
+                setattr(p, name, 1.0)
+        for name, k in (("qkv", D), ("proj", D), ("fc1", D), ("fc2", mlp)):
+            w = getattr(p, name)
+            w.w_codes = w.s_w = w.z_w = w.w_row_sum = w.bias = at
+            w.ldw_bytes = B.code_row_bytes(k, bits_w)
+        return p
+
+    for name in ("qkv", "proj", "fc1", "fc2"):
+        for field, value, word in (("w_codes", None, "NULL"), ("ldw_bytes", 0, "stride"), ("ldw_bytes", 16, "stride")):
+            p = params()
+            setattr(getattr(p, name), field, value)
+            rc = B.lib().repq_block_forward(C.byref(d), C.byref(p), C.c_void_p(at), C.c_void_p(at), C.c_void_p(at), C.c_size_t(total), None)
+            assert rc == B.REPQ_INVALID_ARG and word in B.repq_last_error(), (name, field, value, rc, B.repq_last_error())
