@@ -350,11 +350,15 @@ qgemm_skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
             st_async_v4(to, bar, r[0], r[1], r[2], r[3]);
             st_async_v4(to + kRowsW * 16u, bar, r[4], r[5], r[6], r[7]);
           }
-          if (c_end > c_first) ok = mbar_wait(smem_u32(&s_part), 0, abort, 64, P.status) && ok;
+          if (c_end > c_first && !mbar_wait(smem_u32(&s_part), 0, abort, 64, P.status)) {
+            // given up, here or by a role that raised the flag: the sums still come (every CTA sends), and have to land before this one leaves
+            mbar_drain(smem_u32(&s_part), 0);
+            ok = false;
+          }
           __syncwarp();
           cluster_arrive();                                // (nothing more comes to this CTA, and it sends nothing more)
         }
-        if (!ok || *abort) break;
+        if (!__all_sync(0xffffffffu, ok && !*abort)) break;      // (all lanes leave together)
       }
       for (int c = c_first + half; c < c_end; c += kEpiWarps / 4) {
         const int mc = m0 + c * kTok;
