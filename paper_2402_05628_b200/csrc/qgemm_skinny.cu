@@ -10,7 +10,7 @@
 //    the last MMA to the sums (48 x 4096 x 4096, clusters of four), 2.4 with two barriers of the cluster around plain stores;
 //  - two CTAs per SM of 110 KB where a call has more CTAs than SMs.  Calls of fewer take 200 KB each: a deeper ring, and no two CTAs on
 //    one SM while others idle (128 CTAs sat on 90 SMs; block pass of 48 tokens 72.1 -> 69.5 us);
-//  - what stands behind the main loop is run through once before it ends (`dry` below): the code (24-45 KB, out of L2 since the
+//  - what stands behind the main loop is run through once before it ends where it is long enough (`dry` below): the code (24-45 KB, out of L2 since the
 //    weights of a layer passed through it) and a chunk's residual and rotation values are near when the sums arrive;
 //  - inside a block, while the kernel before it in the stream still runs, every CTA asks for its first weights
 //    (activations and outputs, and weights that the kernel before may have written, are touched only behind the dependency).
@@ -58,6 +58,7 @@ struct SkinnyParams {
   int mt;                      // tokens per tile (multiple of 16)
   int stages, kblocks, split;
   int weights_settled;         // the weights may be read ahead of the dependency wait
+  int dry;                     // the epilogue's code and first values are brought near while the main loop runs
   int over_ring;               // the partial sums of a cluster's CTAs are exchanged over the ring instead of behind it
   uint32_t stage_bytes, a_bytes;
   uint32_t tmem_cols;
@@ -326,9 +327,10 @@ qgemm_skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
     const uint32_t tquarter = tmem + (uint32_t(quarter * 32) << 16);
     const int row = quarter * 32 + lane;
     // The first round runs dry, while the main loop waits for its operands: its code, and the residual and rotation values of the first
-    // chunk, are then near (48 tokens x 12288 x 4096 with rotation: last MMA to end of the kernel 3.1 -> 1.1 us).
+    // chunk, are then near (48 tokens x 12288 x 4096 with rotation: last MMA to end of the kernel 3.1 -> 1.1 us).  Short main loops have
+    // no time for it, and start with the second.
 #pragma unroll 1
-    for (int round = 0; round < 2; ++round) {
+    for (int round = P.dry ? 0 : 1; round < 2; ++round) {
       if (round != 0) {
         bool ok = mbar_wait(smem_u32(&s_acc), 0, abort, 63, P.status);
         tc_fence_after();
@@ -494,6 +496,10 @@ repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, cons
   P.over_ring = stages < 3 && stages < per;
   if (P.over_ring) stages = ring_of(most);                 // (at least three, or all k-blocks)
   P.stages = stages;
+  // Where the dry round pays: never, always, this line; 197 x 1536 x 384 with GELU 3.84, 4.08, 3.92 us, 64 x 1024 x 128 with residual 2.99, 3.68,
+  // 2.91, 48 x 4096 x 4096 with residual 8.43, 8.20, 8.08, 197 x 2304 x 768 with residual 6.48, 6.22, 6.02; block passes of 197 x 384 27.5, 28.4,
+  // 27.7, of 16 tokens x 4096 60.3, 59.8, 59.7.
+  P.dry = per >= (d.residual ? 6 : 8);
   uint32_t smem = uint32_t(stages) * P.stage_bytes;
   if (!P.over_ring) smem += exchange;
   else if (smem < exchange) smem = exchange;
