@@ -54,8 +54,8 @@ size_t qgemm_tc_workspace(const repq_gemm_desc& d);
 repq_status qgemm_tc(const repq_gemm_desc& d, const EpilogueParams& ep, const TcPlan& plan, void* ws, size_t ws_bytes,
                      cudaStream_t st);
 // Few tokens (weights on the M side of the tensor-core instruction): plain products, byte codes, both row sums given.  mt:
-// tokens per tile, 0 where the kernel does not take the problem; split: CTAs that share a tile's K range.
-struct SkinnyPlan { int mt = 0, split = 0; float us = 0.f; };
+// tokens per tile, 0 where the kernel does not take the problem; split: CTAs that share a tile's K range; two: SMs take two CTAs.
+struct SkinnyPlan { int mt = 0, split = 0; bool two = false; float us = 0.f; };
 SkinnyPlan qgemm_skinny_plan(const repq_gemm_desc& d);
 repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, const SkinnyPlan& plan, Params params, cudaStream_t st);
 

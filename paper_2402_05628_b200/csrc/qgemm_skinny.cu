@@ -8,8 +8,8 @@
 //    distributed shared memory, every CTA finishing an equal share of the tile's tokens (integer sums: the result does
 //    not depend on the split).  They are sent as soon as a CTA has them, by stores that a barrier of the receiver counts: 1.4 us from
 //    the last MMA to the sums (48 x 4096 x 4096, clusters of four), 2.4 with two barriers of the cluster around plain stores;
-//  - two CTAs per SM of 110 KB where a call has more CTAs than SMs.  Calls of fewer take 200 KB each: a deeper ring, and no two CTAs on
-//    one SM while others idle (128 CTAs sat on 90 SMs; block pass of 48 tokens 72.1 -> 69.5 us);
+//  - two CTAs per SM of 110 KB where the CTAs of a call do not all find an SM of their own.  Where they do they take 200 KB each: a deeper ring,
+//    and no two CTAs on one SM while others idle (128 CTAs sat on 90 SMs; block pass of 48 tokens 72.1 -> 69.5 us);
 //  - what stands behind the main loop is run through once before it ends where it is long enough (`dry` below): the code (24-45 KB, out of L2 since the
 //    weights of a layer passed through it) and a chunk's residual and rotation values are near when the sums arrive;
 //  - inside a block, while the kernel before it in the stream still runs, every CTA asks for its first weights
@@ -462,7 +462,7 @@ SkinnyPlan qgemm_skinny_plan(const repq_gemm_desc& d) {
       if (load < hbm) load = hbm;
       float us = 1.9f + load + (two ? 0.49f : 0.f) + (two ? 1.53f : 1.f) * share * per_token;
       if (split > 1) us += 1.15f + (two ? 1.53f : 1.f) * 0.0314f * float(mt) * (1.f - 1.f / float(split));
-      if (best.mt == 0 || us < best.us) { best.mt = mt; best.split = split; best.us = us; }
+      if (best.mt == 0 || us < best.us) { best.mt = mt; best.split = split; best.two = two; best.us = us; }
     }
     if (mt >= d.M) break;
   }
@@ -491,7 +491,9 @@ repq_status qgemm_skinny(const repq_gemm_desc& d, const EpilogueParams& ep, cons
     const int n = int(bytes / P.stage_bytes), useful = per < kMaxStages ? per : kMaxStages;
     return n < useful ? n : useful;
   };
-  const uint32_t most = n_tiles * m_tiles * split <= sm_count() ? kSmemOne : kSmemTwo;
+  // (by the plan's limits: fewer CTAs than SMs do not all fit one per SM in clusters, and with 200 KB each the rest wait for a second wave,
+  // 16 x 2048 x 8192, 128 CTAs in clusters of eight, 12.2 us; with 110 KB 7.4)
+  const uint32_t most = plan.two ? kSmemTwo : kSmemOne;
   int stages = ring_of(most - exchange);
   P.over_ring = stages < 3 && stages < per;
   if (P.over_ring) stages = ring_of(most);                 // (at least three, or all k-blocks)
