@@ -270,7 +270,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     uint32_t ph_empty = 0, ph_spent = 0, used = 0, pass2 = 0;
     uint32_t ks = 0, kp = 0;                              // K ring: slot and parity
     bool ok = true;
-    for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
+    for (int it = 0; ok && !given_up(abort) && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
       ok = wait_for(smem_u32(&S.q_full), it & 1, abort, 40, P.status);
       const uint64_t dq = smem_desc_sw128(smem_u32(S.q[it & 1]));
 #pragma unroll 1
@@ -320,7 +320,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     int g = 0;
     uint32_t ph_p = 0, vs = 0;
     bool ok = true;
-    for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
+    for (int it = 0; ok && !given_up(abort) && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
       g += t.nb;
       if (it > 0) ok = wait_for(smem_u32(&S.acc_empty), (it - 1) & 1, abort, 50, P.status);
 #pragma unroll 1
@@ -366,7 +366,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     uint32_t ks = 0, kp = 0;
     int issued = 0;
     bool ok = true;
-    for (int it = 0; ok && !*abort && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
+    for (int it = 0; ok && !given_up(abort) && tile_at<kKeys>(P, it, blockIdx.x, gridDim.x, t); ++it) {
 #pragma unroll 1
       for (int b = 0; b < 2 * t.nb; ++b) {
         ok = wait_for(smem_u32(&S.k_empty[ks]), kp ^ 1u, abort, 48, P.status);

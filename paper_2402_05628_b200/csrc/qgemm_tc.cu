@@ -512,7 +512,7 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     const bool issues = elect_one();
     uint32_t stage = 0, phase = 0;
     int issued = 0;
-    for (int tile = tile0; tile < tiles && !*abort; tile += tile_step) {
+    for (int tile = tile0; tile < tiles && !given_up(abort); tile += tile_step) {
       const TileOrigin o = tile_origin(tile, P.order, kTileM, BN);
       const int m0 = o.m0 + rank * BM, n0 = o.n0 + rank * (BN / 2);
       for (int kb = 0; kb < kblocks; ++kb) {
@@ -554,7 +554,7 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       };
       uint32_t stage = 0, phase = 0, bstage = 0, bphase = 0;
       int it = 0;
-      for (int tile = tile0; tile < tiles && !*abort; tile += tile_step, ++it) {
+      for (int tile = tile0; tile < tiles && !given_up(abort); tile += tile_step, ++it) {
         const uint32_t acc = it & 1, acc_phase = (it >> 1) & 1;
         bool ok = mbar_wait(smem_u32(&S.tmem_empty[acc]), acc_phase ^ 1, abort, 2);
         if (!__all_sync(0xffffffffu, ok)) break;

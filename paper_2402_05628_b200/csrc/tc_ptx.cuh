@@ -79,6 +79,9 @@ __device__ __forceinline__ bool elect_one() {
   return p != 0;
 }
 
+// The abort flag, alike for all lanes (which may read it at different moments, and then vote or leave together).
+__device__ __forceinline__ bool given_up(const volatile int* abort) { return __any_sync(0xffffffffu, *abort != 0); }
+
 // Wait without side effects, for draining copies or MMAs that are still in flight before the CTA exits.
 __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity) {
   const long long t0 = clock64();
