@@ -328,9 +328,11 @@ qgemm_skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
     const int row = quarter * 32 + lane;
     // The first round runs dry, while the main loop waits for its operands: its code, and the residual and rotation values of the first
     // chunk, are then near (48 tokens x 12288 x 4096 with rotation: last MMA to end of the kernel 3.1 -> 1.1 us).  Short main loops have
-    // no time for it, and start with the second.
+    // no time for it, and start with the second.  Codes two per byte do without the code for it: products of a block have no such output,
+    // and by themselves they lose 4 to 11 % by it (2000 x 1000 x 512 6.0 and 6.4 us, 1000 x 1000 x 1024 with GELU 6.5 and 6.9).
+    constexpr bool kDry = OUT != kOutC4;
 #pragma unroll 1
-    for (int round = P.dry ? 0 : 1; round < 2; ++round) {
+    for (int round = kDry && P.dry ? 0 : 1; round < 2; ++round) {
       if (round != 0) {
         bool ok = mbar_wait(smem_u32(&s_acc), 0, abort, 63, P.status);
         tc_fence_after();
@@ -367,7 +369,7 @@ qgemm_skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
         if (mc >= P.M) break;
         const uint4* part = reinterpret_cast<const uint4*>(exchange) + (c - c_first) * 2 * kRowsW + row;
         finish_chunk<OUT, STEP>(P, ct, tquarter + uint32_t(c * kTok), s_asum + c * kTok, part, round != 0 ? split - 1 : 0,
-                                (c_end - c_first) * 2 * kRowsW, mc, min(kTok, P.M - mc), j, col_ok, lane, round == 0);
+                                (c_end - c_first) * 2 * kRowsW, mc, min(kTok, P.M - mc), j, col_ok, lane, kDry && round == 0);
         if (round == 0) break;
       }
     }
