@@ -834,13 +834,10 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
                 t[u][k] = fma2(pack2(sc.x, sc.y), pack2(float(a0 + nz.x * as[k] + kw.x), float(a1 + nz.y * as[k] + kw.y)), pack2(bi.x, bi.y));
               }
             }
-            const f32x2 magic2 = splat2(__uint_as_float(kMagicBits)), mult2 = splat2(q.mult);
-            const bool scaled = direct || !sat;
+            const f32x2 magic2 = splat2(__uint_as_float(kMagicBits));
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              f32x2 x0 = t[0][k], x1 = t[1][k];
-              if (!direct && !sat) { x0 = mul2(x0, mult2); x1 = mul2(x1, mult2); }
-              w[h][k] = code_word(q, scaled ? add2(x0, magic2) : fma2(x0, mult2, magic2), scaled ? add2(x1, magic2) : fma2(x1, mult2, magic2));
+              w[h][k] = code_word(q, add2(t[0][k], magic2), add2(t[1][k], magic2));      // (plain epilogue: the terms hold 1 / s_o)
               sums[k] = int(__dp4a(w[h][k], 0x01010101u, uint32_t(sums[k])));
             }
           }
