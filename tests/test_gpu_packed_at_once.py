@@ -64,3 +64,33 @@ def test_packed_weights_of_a_block_written_just_ahead(bits, batch):
     assert B.repq_device_status() == 0
     assert not torch.equal(got[0][0], got[0][1])
     assert all(torch.equal(a, b) for a, b in zip(*got))
+
+
+@pytest.mark.parametrize("bits,batch", [(4, 1), (6, 6)])
+def test_input_and_factors_of_a_block_written_just_ahead(bits, batch):
+    """The first LayerNorm runs beside the expansion and has no wait of its own: its input and factors are the work of the kernels just
+    ahead, other ones in every pass; compared with the device idle in between."""
+    import torch
+    from paper_2402_05628_b200 import binding as B
+    blk, x = _block(bits, batch)
+    d, p = blk.desc(batch), blk.params()
+    ws = torch.empty(B.repq_block_workspace_bytes(d), dtype=torch.uint8, device=x.device)
+    g = torch.Generator(x.device).manual_seed(bits)
+    sets = [(torch.randn(x.shape, device=x.device, generator=g).to(x.dtype), 1.0 + torch.randn(blk.ln1_g.shape, device=x.device, generator=g),
+             torch.randn(blk.ln1_b.shape, device=x.device, generator=g)) for _ in range(8)]
+    got = []
+    for idle in (True, False):
+        outs = []
+        for s in sets:
+            for t, v in zip((x, blk.ln1_g, blk.ln1_b), s):
+                t.copy_(v)
+            if idle:
+                torch.cuda.synchronize()
+            y = torch.empty(x.shape, dtype=blk.out_dtype, device=x.device)
+            B.repq_block_forward(d, p, x, y, ws)
+            outs.append(y)
+        torch.cuda.synchronize()
+        got.append(outs)
+    assert B.repq_device_status() == 0
+    assert not torch.equal(got[0][0], got[0][1])
+    assert all(torch.equal(a, b) for a, b in zip(*got))
