@@ -111,12 +111,6 @@ __device__ __forceinline__ void umma_f8_ts(uint32_t d_tmem, uint32_t a_tmem, uin
       "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], [%1], %2, %3, p;\n\t}"
       ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
-// Two codes (the first in the low nibble) clipped to [0, 15] and pushed into the low byte of a word of codes that follow them.
-__device__ __forceinline__ uint32_t push_pair_u4(int q0, int q1, uint32_t following) {
-  uint32_t d;
-  asm("cvt.pack.sat.u4.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(q1), "r"(q0), "r"(following));
-  return d;
-}
 // Four bytes out of the eight of (b, a), chosen by the low three bits of a nibble of `sel`; a nibble's fourth bit replicates the sign.
 __device__ __forceinline__ uint32_t select_bytes(uint32_t a, uint32_t b, uint32_t sel) {
   uint32_t d;

@@ -78,20 +78,6 @@ __device__ __forceinline__ void expand(const RawChunk<__nv_bfloat16>& r, f32x2 (
   for (int i = 0; i < 4; ++i) v[i] = pack2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xffff0000u));
 }
 
-// Two consecutive codes (even index e0 in the low nibble) pushed into the low byte of a word that already
-// holds the codes of the following pairs: d = (c << 8) | sat4(e1) << 4 | sat4(e0), saturation to [0, 15].
-__device__ __forceinline__ uint32_t push_pair_u4(int e0, int e1, uint32_t c) {
-  uint32_t d;
-  asm("cvt.pack.sat.u4.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(e1), "r"(e0), "r"(c));
-  return d;
-}
-// The same for byte codes: d = (c << 16) | sat8(e1) << 8 | sat8(e0), saturation to [0, 255].
-__device__ __forceinline__ uint32_t push_pair_u8(int e0, int e1, uint32_t c) {
-  uint32_t d;
-  asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(e1), "r"(e0), "r"(c));
-  return d;
-}
-
 // Reductions inside a warp are xor shuffles (integers of a whole warp take the warp-wide reduction instruction).
 // Barrier of one thread group: the whole block where a group is the block, else a named barrier of the group's own (the
 // groups of a block then no longer wait for one another).

@@ -252,11 +252,6 @@ __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, ui
 // stays far outside the codes).  The pack instruction clips 2^(8 - b) q to [0, 255], the shift drops the low bits again:
 // clip(q, 0, 2^b - 1).  36 instructions for 16 codes against 60 with a saturating multiply-add and byte permutes (12608 x 2304 x
 // 768, 4 bits: 30.0 -> 29.5 us, 8 bits 31.8 -> 29.7, 18464 x 4096 x 1024 with GELU, 4 bits, 91.6 -> 89.9).
-__device__ __forceinline__ uint32_t push_pair_u8(int e0, int e1, uint32_t c) {       // c << 16 | sat(e1) << 8 | sat(e0)
-  uint32_t d;
-  asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(e1), "r"(e0), "r"(c));
-  return d;
-}
 __device__ __forceinline__ uint32_t code_word(const ChunkQuant& q, f32x2 r01, f32x2 r23) {
   const f32x2 unit2 = splat2(q.unit), z2 = splat2(q.z_unit);
   float u0, u1, u2, u3;

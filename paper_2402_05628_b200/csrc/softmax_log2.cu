@@ -76,19 +76,6 @@ __device__ __noinline__ ChunkPairs load_ragged(const __nv_bfloat16* row, int idx
   return ChunkPairs{pack2(f[0], f[1]), pack2(f[2], f[3]), pack2(f[4], f[5]), pack2(f[6], f[7])};
 }
 
-// Two consecutive codes (even index first) pushed into the low byte / low half of a word that already holds the
-// codes after them, with saturation to [0, 15] / [0, 255] (cvt.pack.sat: d = c << 8 | sat(e1) << 4 | sat(e0)).
-__device__ __forceinline__ uint32_t push_pair_u4(int e0, int e1, uint32_t c) {
-  uint32_t d;
-  asm("cvt.pack.sat.u4.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(e1), "r"(e0), "r"(c));
-  return d;
-}
-__device__ __forceinline__ uint32_t push_pair_u8(int e0, int e1, uint32_t c) {
-  uint32_t d;
-  asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(e1), "r"(e0), "r"(c));
-  return d;
-}
-
 // Eq. 15 for the 8 scores of a chunk: clip(round(t), 0, qmax) with t = k1 (S - m) + k0.  t 2^-149 is a denormal float whose
 // bits are t rounded half to even, so one packed multiply makes two integers; both clips are the saturation of the pack
 // (negative t, possible for s < 1 only, has the sign bit: a negative integer; t = +inf for keys past the row and underflowed
