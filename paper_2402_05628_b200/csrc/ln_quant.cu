@@ -752,9 +752,9 @@ repq_status launch_rows(const Call<__nv_bfloat16>& c, cudaStream_t st) {
   note_launch();
   return REPQ_OK;
 }
-// Rows of a call from which a row per warp is ahead: about four and a half turns of the warps at 4096 elements (4096 rows 12.7 us by groups of
-// warps, 14.9 by single ones, 7000 18.3 and 19.3, 8192 23.2 and 21.7, 10000 24.9 and 23.8), five at 2048 (14000 17.3 and 17.6, 16000 22.0
-// and 20.0).  3072 elements gained nothing (63.9 and 63.8), rows that do not fill the chunks lost.
+// Rows of a call from which a row per warp is ahead: about four and a half turns of the warps at 4096 elements (new inputs, packed codes, by groups
+// of warps and by single ones: 4096 rows 12.9 and 14.6 us, 7000 19.7 and 19.8, 7992 22.2 and 21.5, 10000 26.7 and 25.0), five at 2048 (12000 16.4 and
+// 16.6, 14000 18.8 and 18.0, 14800 19.9 and 18.6, 16000 21.1 and 19.7).  3072 elements gained nothing (63.9 and 63.8), rows that do not fill the chunks lost.
 template <int kSlices>
 bool many_rows(int64_t rows) { return rows < (int64_t(1) << 31) && 2 * rows >= int64_t(kSlices == 4 ? 9 : 10) * row_warps<kSlices>() * sm_count(); }
 
